@@ -112,10 +112,6 @@ __host__ __device__ inline dfloat::operator double() const
     return (double)hi + (double)lo;
 }
 
-struct __align__(16) dfloat2 {
-    dfloat x, y;
-};
-
 __host__ __device__ __forceinline__ dfloat dd_fast_two_sum(float a, float b)
 {
     const float s = a + b;
@@ -161,20 +157,5 @@ __host__ __device__ __forceinline__ dfloat dd_recip(dfloat x)
 }
 
 __device__ __forceinline__ dfloat recip(dfloat x) { return dd_recip(x); }
-
-template <> struct C2<dfloat> { using T = dfloat2; };
-
-// A small constant exactly representable in a float, in the arithmetic type K, built without a
-// conversion from double.
-template <typename K> __host__ __device__ __forceinline__ K kconst(float c) { return K(c); }
-template <> __host__ __device__ __forceinline__ dfloat kconst<dfloat>(float c)
-{
-    return dfloat(c, 0.0f);
-}
-
-// Arithmetic type of the three-pass FFT for a grid precision: FP32 grids compute in FP32, FP64
-// grids in double-float.
-template <typename R> struct FftCompute { using type = R; };
-template <> struct FftCompute<double> { using type = dfloat; };
 
 }  // namespace mbk

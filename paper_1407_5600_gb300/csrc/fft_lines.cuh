@@ -209,18 +209,5 @@ __device__ __forceinline__ void store4(double* p, const double v[4])
     reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
     reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
 }
-// FP64 grids read into, and written from, double-float values.
-__device__ __forceinline__ void load4(const double* p, dfloat v[4])
-{
-    double d[4];
-    load4(p, d);
-    for (int i = 0; i < 4; ++i) v[i] = dfloat(d[i]);
-}
-__device__ __forceinline__ void store4(double* p, const dfloat v[4])
-{
-    const double d[4] = {(double)v[0], (double)v[1], (double)v[2], (double)v[3]};
-    store4(p, d);
-}
-
 }  // namespace
 }  // namespace mbk

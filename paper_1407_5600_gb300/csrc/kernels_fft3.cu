@@ -1,5 +1,6 @@
-// Fluid update in three passes over HBM (Eq. vf with the viscous stress, Crank-Nicolson in
-// time, exact discrete projection), each component transformed on its own index grid:
+// Fluid update of FP32 grids in three passes over HBM (Eq. vf with the viscous stress,
+// Crank-Nicolson in time, exact discrete projection), each component transformed on its own
+// index grid (FP64 grids: kernels_fft64.cu):
 //
 //   pass A  per (box, component, z) plane: rhs = (rho/dt) v + (eta/2) L v + f + f_body, then
 //           the 2-D real-to-complex FFT of the plane in shared memory     -> spec [z][kx][ky]
@@ -21,7 +22,7 @@ namespace mbk {
 
 namespace {
 
-template <typename T> __device__ __forceinline__ void load_table(T* dst, const T* src, int n)
+__device__ __forceinline__ void load_table(float2* dst, const float2* src, int n)
 {
     for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
@@ -46,12 +47,12 @@ struct PadPlane {
     __device__ __forceinline__ int row(int p) const { return p * S; }
     __device__ __forceinline__ int off(int j) const { return j + (j >> sx); }
     __device__ __forceinline__ int at(int p, int j) const { return p * S + j + (j >> sx); }
-    template <bool INV, typename T> __device__ __forceinline__ void rows(T* P, const T* tw) const
+    template <bool INV> __device__ __forceinline__ void rows(float2* P, const float2* tw) const
     {
         const int S_ = S, sx_ = sx;
         lines_fft_n<INV>(nx, P, ny / 2, [S_, sx_](int l, int j) { return l * S_ + j + (j >> sx_); }, tw);
     }
-    template <bool INV, typename T> __device__ __forceinline__ void cols(T* P, const T* tw) const
+    template <bool INV> __device__ __forceinline__ void cols(float2* P, const float2* tw) const
     {
         const int S_ = S, sx_ = sx;
         lines_fft_n<INV>(ny, P, nx / 2, [S_, sx_](int k, int y) {
@@ -131,11 +132,11 @@ struct Skew128 {
         const int sub = COL ? lane >> 3 : lane & 3, t = COL ? lane & 7 : lane >> 2;
         for (int l0 = warp * 4; l0 < 64; l0 += nw * 4) line_round<INV, COL>(P, l0 + sub, t, tw);
     }
-    template <bool INV, typename T> __device__ __forceinline__ void rows(T* P, const T* tw) const
+    template <bool INV> __device__ __forceinline__ void rows(float2* P, const float2* tw) const
     {
         lines<INV, false>(P, tw);
     }
-    template <bool INV, typename T> __device__ __forceinline__ void cols(T* P, const T* tw) const
+    template <bool INV> __device__ __forceinline__ void cols(float2* P, const float2* tw) const
     {
         lines<INV, true>(P, tw);
     }
@@ -149,44 +150,43 @@ template <> struct PlaneSlots<Skew128> { static size_t count(int, int) { return 
 // Pass A.  Plane buffer P[p][pad(j)], p < ny/2: first rows 2p, 2p+1 packed as re + i im; after
 // the row FFT and the in-place separation, logical slot 2k + e of row p holds X_{2p+e}[k],
 // k <= nx/2.  pad(j) = j + (j >> pad_shift(nx)).
-template <typename R, typename K, typename L>
-__global__ void __launch_bounds__(sizeof(R) == 4 ? 256 : 512, sizeof(R) == 4 ? 3 : 1)
-k_plane_fwd(FluidArgs<R> a, GridGeo g)
+template <typename L>
+__global__ void __launch_bounds__(256, 3)
+k_plane_fwd(FluidArgs<float> a, GridGeo g)
 {
     dep_wait();
     dep_release();
-    using T = typename C2<K>::T;     // K: arithmetic type (FP32, or double-float for FP64)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
     const L lay(nx, ny);
-    T* P = reinterpret_cast<T*>(smem_raw);
-    const T* twx = reinterpret_cast<const T*>(a.twk[0]);      // twiddles through L1
-    const T* twy = reinterpret_cast<const T*>(a.twk[1]);
+    float2* P = reinterpret_cast<float2*>(smem_raw);
+    const float2* twx = reinterpret_cast<const float2*>(a.twk[0]);      // twiddles through L1
+    const float2* twy = reinterpret_cast<const float2*>(a.twk[1]);
     const int z = blockIdx.x, bc = blockIdx.y, comp = bc % 3;
-    const R* vc = a.v + (size_t)bc * g.N;
-    const R* fc = a.f ? a.f + (size_t)bc * g.N : nullptr;
-    const K ih2 = kparam<K>(a.inv_h2, a.inv_h2_32), rho_dt = kparam<K>(a.rho_dt, a.rho_dt32),
-            half_eta = kparam<K>(a.half_eta, a.half_eta32);
+    const float* vc = a.v + (size_t)bc * g.N;
+    const float* fc = a.f ? a.f + (size_t)bc * g.N : nullptr;
+    const float ih2 = kparam<float>(a.inv_h2, a.inv_h2_32), rho_dt = kparam<float>(a.rho_dt, a.rho_dt32),
+            half_eta = kparam<float>(a.half_eta, a.half_eta32);
     const bool body = a.body_prof && comp == a.body_axis;
-    const R* pz = vc + (size_t)z * ny * nx;
-    const R* pzp = vc + (size_t)((z + 1) & (nz - 1)) * ny * nx;
-    const R* pzm = vc + (size_t)((z - 1) & (nz - 1)) * ny * nx;
-    const R* pf = fc ? fc + (size_t)z * ny * nx : nullptr;
-    R* pclr = a.f_clear && fc ? a.f_clear + (size_t)bc * g.N + (size_t)z * ny * nx : nullptr;
+    const float* pz = vc + (size_t)z * ny * nx;
+    const float* pzp = vc + (size_t)((z + 1) & (nz - 1)) * ny * nx;
+    const float* pzm = vc + (size_t)((z - 1) & (nz - 1)) * ny * nx;
+    const float* pf = fc ? fc + (size_t)z * ny * nx : nullptr;
+    float* pclr = a.f_clear && fc ? a.f_clear + (size_t)bc * g.N + (size_t)z * ny * nx : nullptr;
     // each work unit: 4 consecutive x of the two rows 2p, 2p+1
     const int qx = nx / 4, lq = 31 - __clz(qx);   // nx is a power of two
     for (int u = threadIdx.x; u < qx * (ny / 2) && a.no_v; u += blockDim.x) {
         // Stokes limit: the right-hand side is the force density (and body force) alone
         const int x0 = 4 * (u & (qx - 1)), p = u >> lq;
         const int y0 = 2 * p, y1 = y0 + 1;
-        const K z0 = kconst<K>(0.0f);
-        K r0[4] = {z0, z0, z0, z0}, r1[4] = {z0, z0, z0, z0};
+        const float z0 = 0.0f;
+        float r0[4] = {z0, z0, z0, z0}, r1[4] = {z0, z0, z0, z0};
         if (pf) {
             load4(pf + (size_t)y0 * nx + x0, r0);
             load4(pf + (size_t)y1 * nx + x0, r1);
             if (pclr) {
-                const K zero[4] = {kconst<K>(0.0f), kconst<K>(0.0f), kconst<K>(0.0f),
-                                   kconst<K>(0.0f)};
+                const float zero[4] = {0.0f, 0.0f, 0.0f,
+                                   0.0f};
                 store4(pclr + (size_t)y0 * nx + x0, zero);
                 store4(pclr + (size_t)y1 * nx + x0, zero);
             }
@@ -194,26 +194,26 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
         if (body) {
             for (int i = 0; i < 4; ++i) {
                 const int x = x0 + i;
-                r0[i] += K(a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y0 : z)]);
-                r1[i] += K(a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y1 : z)]);
+                r0[i] += (a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y0 : z)]);
+                r1[i] += (a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y1 : z)]);
             }
         }
-        T* rowp = P + lay.row(p);
-        for (int i = 0; i < 4; ++i) rowp[lay.off(x0 + i)] = T{r0[i], r1[i]};
+        float2* rowp = P + lay.row(p);
+        for (int i = 0; i < 4; ++i) rowp[lay.off(x0 + i)] = float2{r0[i], r1[i]};
     }
     for (int u = threadIdx.x; u < qx * (ny / 2) && !a.no_v; u += blockDim.x) {
         const int x0 = 4 * (u & (qx - 1)), p = u >> lq;
         const int y0 = 2 * p, y1 = y0 + 1;
         const int ym = (y0 - 1) & (ny - 1), yp = (y1 + 1) & (ny - 1);
-        K c0[4], c1[4], am[4], ap[4], t[4];
+        float c0[4], c1[4], am[4], ap[4], t[4];
         load4(pz + (size_t)y0 * nx + x0, c0);
         load4(pz + (size_t)y1 * nx + x0, c1);
         load4(pz + (size_t)ym * nx + x0, am);
         load4(pz + (size_t)yp * nx + x0, ap);
-        K l0[4], l1[4];
+        float l0[4], l1[4];
         for (int i = 0; i < 4; ++i) {
-            l0[i] = am[i] + c1[i] - kconst<K>(6.0f) * c0[i];
-            l1[i] = c0[i] + ap[i] - kconst<K>(6.0f) * c1[i];
+            l0[i] = am[i] + c1[i] - 6.0f * c0[i];
+            l1[i] = c0[i] + ap[i] - 6.0f * c1[i];
         }
         load4(pzp + (size_t)y0 * nx + x0, t);
         for (int i = 0; i < 4; ++i) l0[i] += t[i];
@@ -224,13 +224,13 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
         load4(pzm + (size_t)y1 * nx + x0, t);
         for (int i = 0; i < 4; ++i) l1[i] += t[i];
         const int xm = (x0 - 1) & (nx - 1), xp = (x0 + 4) & (nx - 1);
-        const K e0m = K(pz[(size_t)y0 * nx + xm]), e0p = K(pz[(size_t)y0 * nx + xp]);
-        const K e1m = K(pz[(size_t)y1 * nx + xm]), e1p = K(pz[(size_t)y1 * nx + xp]);
+        const float e0m = (pz[(size_t)y0 * nx + xm]), e0p = (pz[(size_t)y0 * nx + xp]);
+        const float e1m = (pz[(size_t)y1 * nx + xm]), e1p = (pz[(size_t)y1 * nx + xp]);
         for (int i = 0; i < 4; ++i) {
             l0[i] += (i == 0 ? e0m : c0[i - 1]) + (i == 3 ? e0p : c0[i + 1]);
             l1[i] += (i == 0 ? e1m : c1[i - 1]) + (i == 3 ? e1p : c1[i + 1]);
         }
-        K r0[4], r1[4];
+        float r0[4], r1[4];
         for (int i = 0; i < 4; ++i) {
             r0[i] = rho_dt * c0[i] + half_eta * (l0[i] * ih2);
             r1[i] = rho_dt * c1[i] + half_eta * (l1[i] * ih2);
@@ -241,8 +241,8 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
             load4(pf + (size_t)y1 * nx + x0, t);
             for (int i = 0; i < 4; ++i) r1[i] += t[i];
             if (pclr) {                  // leave f zeroed for the next accumulation
-                const K zero[4] = {kconst<K>(0.0f), kconst<K>(0.0f), kconst<K>(0.0f),
-                                   kconst<K>(0.0f)};
+                const float zero[4] = {0.0f, 0.0f, 0.0f,
+                                   0.0f};
                 store4(pclr + (size_t)y0 * nx + x0, zero);
                 store4(pclr + (size_t)y1 * nx + x0, zero);
             }
@@ -250,12 +250,12 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
         if (body) {
             for (int i = 0; i < 4; ++i) {
                 const int x = x0 + i;
-                r0[i] += K(a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y0 : z)]);
-                r1[i] += K(a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y1 : z)]);
+                r0[i] += (a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y0 : z)]);
+                r1[i] += (a.body_prof[a.body_dir == 0 ? x : (a.body_dir == 1 ? y1 : z)]);
             }
         }
-        T* rowp = P + lay.row(p);
-        for (int i = 0; i < 4; ++i) rowp[lay.off(x0 + i)] = T{r0[i], r1[i]};
+        float2* rowp = P + lay.row(p);
+        for (int i = 0; i < 4; ++i) rowp[lay.off(x0 + i)] = float2{r0[i], r1[i]};
     }
     __syncthreads();
     lay.template rows<false>(P, twx);
@@ -264,16 +264,16 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
     {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
         for (int p = warp; p < ny / 2; p += nw) {
-            T* rowp = P + lay.row(p);
-            T ev[3], od[3];        // nx/2 + 1 <= 65 values: at most 3 per lane
+            float2* rowp = P + lay.row(p);
+            float2 ev[3], od[3];        // nx/2 + 1 <= 65 values: at most 3 per lane
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 const int k = lane + 32 * r;
                 if (k < nxh) {
                     const int kr = (nx - k) & (nx - 1);
-                    const T Z = rowp[lay.off(k)], Zr = rowp[lay.off(kr)];
-                    ev[r] = T{(Z.x + Zr.x) * kconst<K>(0.5f), (Z.y - Zr.y) * kconst<K>(0.5f)};
-                    od[r] = T{(Z.y + Zr.y) * kconst<K>(0.5f), (Zr.x - Z.x) * kconst<K>(0.5f)};
+                    const float2 Z = rowp[lay.off(k)], Zr = rowp[lay.off(kr)];
+                    ev[r] = float2{(Z.x + Zr.x) * 0.5f, (Z.y - Zr.y) * 0.5f};
+                    od[r] = float2{(Z.y + Zr.y) * 0.5f, (Zr.x - Z.x) * 0.5f};
                 }
             }
             __syncwarp();
@@ -293,20 +293,20 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
     // columns k = 0 and k = nx/2 are real: transform them as one complex column
     // Z_y = X_y[0] + i X_y[nx/2], so that nx/2 column lines remain
     for (int y = threadIdx.x; y < ny; y += blockDim.x)
-        P[col(0, y)] = T{P[col(0, y)].x, P[col(nx / 2, y)].x};
+        P[col(0, y)] = float2{P[col(0, y)].x, P[col(nx / 2, y)].x};
     __syncthreads();
     lay.template cols<false>(P, twy);
     __syncthreads();
     // A = FFT X[0] = (Z_k + conj Z_-k) / 2,  B = FFT X[nx/2] = (Z_k - conj Z_-k) / (2i)
     if (threadIdx.x < 32) {
-        T av[4], bv[4];            // ny <= 128: at most 4 per lane
+        float2 av[4], bv[4];            // ny <= 128: at most 4 per lane
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int k = threadIdx.x + 32 * r;
             if (k < ny) {
-                const T Zk = P[col(0, k)], Zr = P[col(0, (ny - k) & (ny - 1))];
-                av[r] = T{(Zk.x + Zr.x) * kconst<K>(0.5f), (Zk.y - Zr.y) * kconst<K>(0.5f)};
-                bv[r] = T{(Zk.y + Zr.y) * kconst<K>(0.5f), (Zr.x - Zk.x) * kconst<K>(0.5f)};
+                const float2 Zk = P[col(0, k)], Zr = P[col(0, (ny - k) & (ny - 1))];
+                av[r] = float2{(Zk.x + Zr.x) * 0.5f, (Zk.y - Zr.y) * 0.5f};
+                bv[r] = float2{(Zk.y + Zr.y) * 0.5f, (Zr.x - Zk.x) * 0.5f};
             }
         }
         __syncwarp();
@@ -320,12 +320,12 @@ k_plane_fwd(FluidArgs<R> a, GridGeo g)
         }
     }
     __syncthreads();
-    T* out = reinterpret_cast<T*>(a.spec) + ((size_t)bc * nz + z) * (size_t)nxh * ny;
+    float2* out = reinterpret_cast<float2*>(a.spec) + ((size_t)bc * nz + z) * (size_t)nxh * ny;
     const int ly = 31 - __clz(ny);
     if (blockDim.x % ny == 0) {
         // a thread keeps its y (so its packed row and parity) and steps through k
         const int y = threadIdx.x & (ny - 1), e = y & 1, dk = blockDim.x >> ly;
-        const T* rowp = P + lay.row(y >> 1);
+        const float2* rowp = P + lay.row(y >> 1);
         for (int k = threadIdx.x >> ly; k < nxh; k += dk) out[k * ny + y] = rowp[lay.off(2 * k + e)];
     } else {
         for (int i = threadIdx.x; i < nxh * ny; i += blockDim.x) out[i] = P[col(i >> ly, i & (ny - 1))];
@@ -379,35 +379,34 @@ __device__ __forceinline__ void zlines128(float2* Bf, const float2* tw)
 // ------------------------------------------------------------------------------------------
 // Pass B.  CTA = (ky block of width C, kx, box); shared buffer [3][pad(nz)][C + 4].  C is a
 // compile-time width (16 FP32, 8 FP64) and the block has 3 C N2 threads, one round of lines.
-template <typename R, typename K, int C>
-__global__ void __launch_bounds__(3 * C * 8, sizeof(R) == 4 ? 768 / (3 * C * 8) : 1)
-k_zsolve(FluidArgs<R> a, GridGeo g)
+template <int C>
+__global__ void __launch_bounds__(3 * C * 8, 768 / (3 * C * 8))
+k_zsolve(FluidArgs<float> a, GridGeo g)
 {
-    using T = typename C2<K>::T;
     constexpr int Cp = C + 4;                    // 4 z-rows x 4 lines per half-warp: distinct banks
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
     const int lz = 31 - __clz(nz);
     const int sz = pad_shift(nz), nzp = padded_len(nz);
-    T* Bf = reinterpret_cast<T*>(smem_raw);
-    T* twz = Bf + 3 * nzp * Cp;
-    load_table(twz, reinterpret_cast<const T*>(a.twk[2]), nz);   // set up once: no wait
+    float2* Bf = reinterpret_cast<float2*>(smem_raw);
+    float2* twz = Bf + 3 * nzp * Cp;
+    load_table(twz, reinterpret_cast<const float2*>(a.twk[2]), nz);   // set up once: no wait
     dep_wait();
     dep_release();
     const int ky0 = blockIdx.x * C, kx = blockIdx.y, box = blockIdx.z;
     const size_t zstride = (size_t)nxh * ny;
     const size_t cstride = (size_t)nz * zstride;
-    T* base = reinterpret_cast<T*>(a.spec) + (size_t)(box * 3) * cstride + (size_t)kx * ny + ky0;
+    float2* base = reinterpret_cast<float2*>(a.spec) + (size_t)(box * 3) * cstride + (size_t)kx * ny + ky0;
     auto at = [=](int c, int z, int k) { return (c * nzp + z + (z >> sz)) * Cp + k; };
     const int total = 3 * nz * C;
-    constexpr bool z128 = sizeof(T) == 8 && C == 8;     // FP32 complex, eight columns
+    constexpr bool z128 = C == 8;
     // 128-point z-lines with 192 threads: thread (zr = tid / 8, k = tid % 8) moves the elements
     // (c = zr / 8, z = zr % 8 + 8 j, k), j < 16, at a fixed stride on both sides
     const bool fast = z128 && nz == 128 && blockDim.x == 3 * 8 * C;
     if (fast) {
         const int k = threadIdx.x & 7, zr = threadIdx.x >> 3, c = zr >> 3, z0 = zr & 7;
-        T* sb = Bf + (c * 144 + z0) * 12 + k;
-        const T* gb = base + c * cstride + (size_t)z0 * zstride + k;
+        float2* sb = Bf + (c * 144 + z0) * 12 + k;
+        const float2* gb = base + c * cstride + (size_t)z0 * zstride + k;
 #pragma unroll
         for (int j = 0; j < 16; ++j) async_copy(sb + 108 * j, gb + (size_t)(8 * j) * zstride);
     } else {
@@ -426,26 +425,26 @@ k_zsolve(FluidArgs<R> a, GridGeo g)
         lines_fft_n<false>(nz, Bf, 3 * C, idx, twz);
     }
     __syncthreads();
-    const K* sym = reinterpret_cast<const K*>(a.symk);     // [9][256] cos, sin, lambda
-    const K ih = kparam<K>(a.inv_h, a.inv_h32);
-    const K csx = sym[0 * 256 + kx], snx = sym[1 * 256 + kx], lx = sym[2 * 256 + kx];
-    const K rho_dt = kparam<K>(a.rho_dt, a.rho_dt32);
-    const K half_eta = kparam<K>(a.half_eta, a.half_eta32);
+    const float* sym = reinterpret_cast<const float*>(a.symk);     // [9][256] cos, sin, lambda
+    const float ih = kparam<float>(a.inv_h, a.inv_h32);
+    const float csx = sym[0 * 256 + kx], snx = sym[1 * 256 + kx], lx = sym[2 * 256 + kx];
+    const float rho_dt = kparam<float>(a.rho_dt, a.rho_dt32);
+    const float half_eta = kparam<float>(a.half_eta, a.half_eta32);
     // with blockDim a multiple of C a thread keeps its column k (and ky's symbols) throughout
     const int kfix = threadIdx.x % C;
-    const K csy = sym[3 * 256 + ky0 + kfix], sny = sym[4 * 256 + ky0 + kfix];
-    const K lxy = lx + sym[5 * 256 + ky0 + kfix];
+    const float csy = sym[3 * 256 + ky0 + kfix], sny = sym[4 * 256 + ky0 + kfix];
+    const float lxy = lx + sym[5 * 256 + ky0 + kfix];
     const bool colfix = blockDim.x % C == 0;
     for (int i = threadIdx.x; i < nz * C; i += blockDim.x) {
         const int k = colfix ? kfix : i % C, kz = i / C, ky = ky0 + k;
-        const K cs[3] = {csx, colfix ? csy : sym[3 * 256 + ky], sym[6 * 256 + kz]};
-        const K sn[3] = {snx, colfix ? sny : sym[4 * 256 + ky], sym[7 * 256 + kz]};
-        const K lam = (colfix ? lxy : lx + sym[5 * 256 + ky]) + sym[8 * 256 + kz];
-        const K cinv = recip(rho_dt + half_eta * lam);
-        T W[3];
+        const float cs[3] = {csx, colfix ? csy : sym[3 * 256 + ky], sym[6 * 256 + kz]};
+        const float sn[3] = {snx, colfix ? sny : sym[4 * 256 + ky], sym[7 * 256 + kz]};
+        const float lam = (colfix ? lxy : lx + sym[5 * 256 + ky]) + sym[8 * 256 + kz];
+        const float cinv = recip(rho_dt + half_eta * lam);
+        float2 W[3];
         for (int c = 0; c < 3; ++c) {
-            const T v = Bf[at(c, kz, k)];
-            W[c] = T{v.x * cinv, v.y * cinv};
+            const float2 v = Bf[at(c, kz, k)];
+            W[c] = float2{v.x * cinv, v.y * cinv};
         }
         if (kx == 0 && ky == 0 && kz == 0) {
             for (int c = 0; c < 3; ++c) {
@@ -453,27 +452,27 @@ k_zsolve(FluidArgs<R> a, GridGeo g)
                     double m = a.mean_state[3 * box + c];
                     if (a.mean_force) m += a.mean_scale * a.mean_force[3 * box + c];
                     a.mean_state[3 * box + c] = m;
-                    W[c] = T{K((double)g.N * m), kconst<K>(0.0f)};
+                    W[c] = float2{(float)((double)g.N * m), 0.0f};
                 } else if (a.mean_override) {
-                    W[c] = T{K((double)g.N * a.mean_override[3 * box + c]), kconst<K>(0.0f)};
+                    W[c] = float2{(float)((double)g.N * a.mean_override[3 * box + c]), 0.0f};
                 } else if (a.mean_mode == 1) {
-                    W[c] = T{kconst<K>(0.0f), kconst<K>(0.0f)};
+                    W[c] = float2{0.0f, 0.0f};
                 }
             }
         } else {
             // D_a = (e^{i th} - 1)/h, G_a = (1 - e^{-i th})/h, D.G = -lambda:
             // P W = W + G (D.W) / lambda
-            K dr = kconst<K>(0.0f), di = kconst<K>(0.0f);
+            float dr = 0.0f, di = 0.0f;
             for (int c = 0; c < 3; ++c) {
-                const K Dr = (cs[c] - kconst<K>(1.0f)) * ih, Di = sn[c] * ih;
+                const float Dr = (cs[c] - 1.0f) * ih, Di = sn[c] * ih;
                 dr += Dr * W[c].x - Di * W[c].y;
                 di += Dr * W[c].y + Di * W[c].x;
             }
-            const K il = recip(lam);
+            const float il = recip(lam);
             dr *= il;
             di *= il;
             for (int c = 0; c < 3; ++c) {
-                const K Gr = (kconst<K>(1.0f) - cs[c]) * ih, Gi = sn[c] * ih;
+                const float Gr = (1.0f - cs[c]) * ih, Gi = sn[c] * ih;
                 W[c].x += Gr * dr - Gi * di;
                 W[c].y += Gr * di + Gi * dr;
             }
@@ -490,8 +489,8 @@ k_zsolve(FluidArgs<R> a, GridGeo g)
     __syncthreads();
     if (fast) {
         const int k = threadIdx.x & 7, zr = threadIdx.x >> 3, c = zr >> 3, z0 = zr & 7;
-        const T* sb = Bf + (c * 144 + z0) * 12 + k;
-        T* gb = base + c * cstride + (size_t)z0 * zstride + k;
+        const float2* sb = Bf + (c * 144 + z0) * 12 + k;
+        float2* gb = base + c * cstride + (size_t)z0 * zstride + k;
 #pragma unroll
         for (int j = 0; j < 16; ++j) gb[(size_t)(8 * j) * zstride] = sb[108 * j];
     } else {
@@ -505,28 +504,27 @@ k_zsolve(FluidArgs<R> a, GridGeo g)
 // ------------------------------------------------------------------------------------------
 // Pass C.  Inverse of pass A: columns, then the packed rows Z = X_{2p} + i X_{2p+1} (with the
 // Hermitian extension X[nx - k] = conj X[k]), then the real rows, scaled by 1/N.
-template <typename R, typename K, typename L>
-__global__ void __launch_bounds__(sizeof(R) == 4 ? 256 : 512, sizeof(R) == 4 ? 3 : 1)
-k_plane_inv(FluidArgs<R> a, GridGeo g)
+template <typename L>
+__global__ void __launch_bounds__(256, 3)
+k_plane_inv(FluidArgs<float> a, GridGeo g)
 {
     // no early release: the next kernel (the interpolation's persistent grid, which splits the
     // blobs evenly over its warps) then starts all its blocks together, not first on the SMs
     // this pass leaves early
     dep_wait();
-    using T = typename C2<K>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
     const L lay(nx, ny);
-    T* P = reinterpret_cast<T*>(smem_raw);
-    const T* twx = reinterpret_cast<const T*>(a.twk[0]);      // twiddles through L1
-    const T* twy = reinterpret_cast<const T*>(a.twk[1]);
+    float2* P = reinterpret_cast<float2*>(smem_raw);
+    const float2* twx = reinterpret_cast<const float2*>(a.twk[0]);      // twiddles through L1
+    const float2* twy = reinterpret_cast<const float2*>(a.twk[1]);
     const int z = blockIdx.x, bc = blockIdx.y;
-    const T* in = reinterpret_cast<const T*>(a.spec) + ((size_t)bc * nz + z) * (size_t)nxh * ny;
+    const float2* in = reinterpret_cast<const float2*>(a.spec) + ((size_t)bc * nz + z) * (size_t)nxh * ny;
     auto col = [lay](int k, int y) { return lay.at(y >> 1, 2 * k + (y & 1)); };
     const int ly = 31 - __clz(ny);
     if (blockDim.x % ny == 0) {
         const int y = threadIdx.x & (ny - 1), e = y & 1, dk = blockDim.x >> ly;
-        T* rowp = P + lay.row(y >> 1);
+        float2* rowp = P + lay.row(y >> 1);
         for (int k = threadIdx.x >> ly; k < nxh; k += dk) async_copy(&rowp[lay.off(2 * k + e)], &in[k * ny + y]);
     } else {
         for (int i = threadIdx.x; i < nxh * ny; i += blockDim.x) async_copy(&P[col(i >> ly, i & (ny - 1))], &in[i]);
@@ -536,18 +534,18 @@ k_plane_inv(FluidArgs<R> a, GridGeo g)
     // columns k = 0 and k = nx/2 invert to real sequences: transform their Hermitian parts as
     // one complex column Z = herm(A) + i herm(B), whose inverse is Re(IFFT A) + i Re(IFFT B)
     if (threadIdx.x < 32) {
-        T zv[4];
+        float2 zv[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int k = threadIdx.x + 32 * r;
             if (k < ny) {
                 const int kr = (ny - k) & (ny - 1);
-                const T A = P[col(0, k)], Ar = P[col(0, kr)];
-                const T Bv = P[col(nx / 2, k)], Br = P[col(nx / 2, kr)];
+                const float2 A = P[col(0, k)], Ar = P[col(0, kr)];
+                const float2 Bv = P[col(nx / 2, k)], Br = P[col(nx / 2, kr)];
                 // herm(A) = (A_k + conj A_-k) / 2, herm(B) likewise; Z = herm(A) + i herm(B)
-                const T ha = T{(A.x + Ar.x) * kconst<K>(0.5f), (A.y - Ar.y) * kconst<K>(0.5f)};
-                const T hb = T{(Bv.x + Br.x) * kconst<K>(0.5f), (Bv.y - Br.y) * kconst<K>(0.5f)};
-                zv[r] = T{ha.x - hb.y, ha.y + hb.x};
+                const float2 ha = float2{(A.x + Ar.x) * 0.5f, (A.y - Ar.y) * 0.5f};
+                const float2 hb = float2{(Bv.x + Br.x) * 0.5f, (Bv.y - Br.y) * 0.5f};
+                zv[r] = float2{ha.x - hb.y, ha.y + hb.x};
             }
         }
         __syncwarp();
@@ -561,25 +559,25 @@ k_plane_inv(FluidArgs<R> a, GridGeo g)
     lay.template cols<true>(P, twy);
     __syncthreads();
     for (int y = threadIdx.x; y < ny; y += blockDim.x) {
-        const T zc = P[col(0, y)];
-        P[col(0, y)] = T{zc.x, kconst<K>(0.0f)};
-        P[col(nx / 2, y)] = T{zc.y, kconst<K>(0.0f)};
+        const float2 zc = P[col(0, y)];
+        P[col(0, y)] = float2{zc.x, 0.0f};
+        P[col(nx / 2, y)] = float2{zc.y, 0.0f};
     }
     __syncthreads();
     {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
         for (int p = warp; p < ny / 2; p += nw) {
-            T* rowp = P + lay.row(p);
-            T zv[4];              // nx <= 128 values: at most 4 per lane
+            float2* rowp = P + lay.row(p);
+            float2 zv[4];              // nx <= 128 values: at most 4 per lane
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int k = lane + 32 * r;
                 if (k < nx) {
                     const int kk = k <= nx / 2 ? k : nx - k;
-                    T e = rowp[lay.off(2 * kk)], o = rowp[lay.off(2 * kk + 1)];
-                    if (k == 0 || k == nx / 2) { e.y = kconst<K>(0.0f); o.y = kconst<K>(0.0f); }
+                    float2 e = rowp[lay.off(2 * kk)], o = rowp[lay.off(2 * kk + 1)];
+                    if (k == 0 || k == nx / 2) { e.y = 0.0f; o.y = 0.0f; }
                     if (k > nx / 2) { e.y = -e.y; o.y = -o.y; }
-                    zv[r] = T{e.x - o.y, e.y + o.x};
+                    zv[r] = float2{e.x - o.y, e.y + o.x};
                 }
             }
             __syncwarp();
@@ -594,15 +592,15 @@ k_plane_inv(FluidArgs<R> a, GridGeo g)
     __syncthreads();
     lay.template rows<true>(P, twx);
     __syncthreads();
-    const K scale = kparam<K>(a.inv_n, a.inv_n32);
-    R* out = a.v_out + (size_t)bc * g.N + (size_t)z * ny * nx;
+    const float scale = kparam<float>(a.inv_n, a.inv_n32);
+    float* out = a.v_out + (size_t)bc * g.N + (size_t)z * ny * nx;
     const int qx = nx / 4, lq = 31 - __clz(qx);   // nx is a power of two
     for (int u = threadIdx.x; u < qx * (ny / 2); u += blockDim.x) {
         const int x0 = 4 * (u & (qx - 1)), p = u >> lq;
-        K r0[4], r1[4];
-        const T* rowp = P + lay.row(p);
+        float r0[4], r1[4];
+        const float2* rowp = P + lay.row(p);
         for (int i = 0; i < 4; ++i) {
-            const T zv = rowp[lay.off(x0 + i)];
+            const float2 zv = rowp[lay.off(x0 + i)];
             r0[i] = zv.x * scale;
             r1[i] = zv.y * scale;
         }
@@ -610,7 +608,7 @@ k_plane_inv(FluidArgs<R> a, GridGeo g)
         store4(out + (size_t)(2 * p + 1) * nx + x0, r1);
         if (a.v_sum_out) {               // v^n + v^{n+1} for the corrector's single gather
             const size_t o0 = (size_t)bc * g.N + (size_t)z * ny * nx + (size_t)(2 * p) * nx + x0;
-            K b0[4], b1[4];
+            float b0[4], b1[4];
             load4(a.v_sum_base + o0, b0);
             load4(a.v_sum_base + o0 + nx, b1);
             for (int i = 0; i < 4; ++i) {
@@ -623,28 +621,23 @@ k_plane_inv(FluidArgs<R> a, GridGeo g)
     }
 }
 
-template <typename R>
-cudaError_t launch_fluid3(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a_in,
+template <>
+cudaError_t launch_fluid3<float>(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<float>& a_in,
                           cudaEvent_t* marks)
 {
-    const FluidArgs<R> a = with_derived(a_in, g);
-    using K = typename FftCompute<R>::type;
-    using T = typename C2<K>::T;
-    // plane blocks: FP64 planes (one block per SM) take 512 threads to hide latency
-    constexpr int PT = sizeof(R) == 4 ? 256 : 512;
+    const FluidArgs<float> a = with_derived(a_in, g);
+    constexpr int PT = 256;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
     constexpr int CZ = 8;                             // ky columns per z-pass block
     static std::atomic<unsigned> attr{0};     // per instantiation
     if (first_on_device(attr)) {
         const int lim = 200 * 1024;
-        cudaFuncSetAttribute(k_plane_fwd<R, K, PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zsolve<R, K, CZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zsolve<R, K, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_inv<R, K, PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        if constexpr (sizeof(R) == 4) {
-            cudaFuncSetAttribute(k_plane_fwd<R, K, Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-            cudaFuncSetAttribute(k_plane_inv<R, K, Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        }
+        cudaFuncSetAttribute(k_plane_fwd<PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_zsolve<CZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_zsolve<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_inv<PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_fwd<Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_inv<Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     }
     // FP32 planes of 128 x 128 take the conflict-free layout (MB_PLANE_LAYOUT=pad keeps the
     // padded one, for comparison)
@@ -652,42 +645,30 @@ cudaError_t launch_fluid3(cudaStream_t st, int B, const GridGeo& g, const FluidA
         const char* e = std::getenv("MB_PLANE_LAYOUT");
         return e && std::string(e) == "pad";
     }();
-    const bool skew = sizeof(R) == 4 && nx == 128 && ny == 128 && !skew_off;
+    const bool skew = nx == 128 && ny == 128 && !skew_off;
     const size_t smem_plane = (skew ? PlaneSlots<Skew128>::count(nx, ny)
-                                    : PlaneSlots<PadPlane>::count(nx, ny)) * sizeof(T);
+                                    : PlaneSlots<PadPlane>::count(nx, ny)) * sizeof(float2);
     const int C = ny >= CZ ? CZ : 4;
-    const size_t smem_z = ((size_t)3 * padded_len(nz) * (C + 4) + nz) * sizeof(T);
+    const size_t smem_z = ((size_t)3 * padded_len(nz) * (C + 4) + nz) * sizeof(float2);
     auto mark = [&](int i) { if (marks) cudaEventRecord(marks[i], st); };
     mark(0);
     cudaError_t e;
     const dim3 gp(nz, 3 * B), gz(ny / C, nxh, B);
-    if constexpr (sizeof(R) == 4) {
-        if (skew) e = launch_dep(k_plane_fwd<R, K, Skew128>, gp, dim3(PT), smem_plane, st, a, g);
-        else e = launch_dep(k_plane_fwd<R, K, PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
-    } else {
-        e = launch_dep(k_plane_fwd<R, K, PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
-    }
+    if (skew) e = launch_dep(k_plane_fwd<Skew128>, gp, dim3(PT), smem_plane, st, a, g);
+    else e = launch_dep(k_plane_fwd<PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
     if (e != cudaSuccess) return e;
     mark(1);
     mark(2);
-    if (C == CZ) e = launch_dep(k_zsolve<R, K, CZ>, gz, dim3(3 * CZ * 8), smem_z, st, a, g);
-    else e = launch_dep(k_zsolve<R, K, 4>, gz, dim3(3 * 4 * 8), smem_z, st, a, g);
+    if (C == CZ) e = launch_dep(k_zsolve<CZ>, gz, dim3(3 * CZ * 8), smem_z, st, a, g);
+    else e = launch_dep(k_zsolve<4>, gz, dim3(3 * 4 * 8), smem_z, st, a, g);
     if (e != cudaSuccess) return e;
     mark(3);
     mark(4);
-    if constexpr (sizeof(R) == 4) {
-        if (skew) e = launch_dep(k_plane_inv<R, K, Skew128>, gp, dim3(PT), smem_plane, st, a, g);
-        else e = launch_dep(k_plane_inv<R, K, PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
-    } else {
-        e = launch_dep(k_plane_inv<R, K, PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
-    }
+    if (skew) e = launch_dep(k_plane_inv<Skew128>, gp, dim3(PT), smem_plane, st, a, g);
+    else e = launch_dep(k_plane_inv<PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
     if (e != cudaSuccess) return e;
     mark(5);
     return cudaGetLastError();
 }
-template cudaError_t launch_fluid3<float>(cudaStream_t, int, const GridGeo&,
-                                          const FluidArgs<float>&, cudaEvent_t*);
-template cudaError_t launch_fluid3<double>(cudaStream_t, int, const GridGeo&,
-                                           const FluidArgs<double>&, cudaEvent_t*);
 
 }  // namespace mbk

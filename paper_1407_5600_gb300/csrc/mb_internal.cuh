@@ -249,11 +249,17 @@ template <typename R>
 cudaError_t launch_fluid(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a,
                          cudaEvent_t* marks = nullptr);
 constexpr int FLUID_KERNELS = 5;
-// Three-pass variant (plane R2C, z solve, plane C2R); marks as for launch_fluid, with the
-// y-pass marks recorded back to back.
+// Three-pass variant (plane R2C, z solve, plane C2R; FP32 grids in kernels_fft3.cu, FP64 grids
+// in kernels_fft64.cu); marks as for launch_fluid, with the y-pass marks recorded back to back.
 template <typename R>
 cudaError_t launch_fluid3(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a,
                           cudaEvent_t* marks = nullptr);
+template <>
+cudaError_t launch_fluid3<float>(cudaStream_t st, int B, const GridGeo& g,
+                                 const FluidArgs<float>& a, cudaEvent_t* marks);
+template <>
+cudaError_t launch_fluid3<double>(cudaStream_t st, int B, const GridGeo& g,
+                                  const FluidArgs<double>& a, cudaEvent_t* marks);
 constexpr int FLUID3_KERNELS = 3;
 
 // Thermal and convective stress (kernels_noise.cu): W = amp * normals of step *step_index
