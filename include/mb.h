@@ -22,8 +22,8 @@
  *    passes; no caller pointer is used by work enqueued after the call returns.
  *  - Environment (read when a context is created; for comparisons and tuning, the defaults
  *    are the fast path): MB_FFT_PASSES=5 runs the fluid solve as five one-axis passes instead
- *    of three; MB_NO_GRAPH=1 launches every FP32-grid step directly instead of replaying its
- *    captured CUDA graph; MB_NO_AUTOTUNE=1 keeps the default spreading tile;
+ *    of three; MB_NO_GRAPH=1 launches every step directly instead of replaying its captured CUDA
+ *    graph; MB_NO_AUTOTUNE=1 keeps the default spreading tile;
  *    MB_NO_FUSE_INTERP=1 runs the corrector and the next predictor as separate passes.
  *    MB_FAULT_ALLOC=k makes the k-th device allocation fail (tests of the error paths).
  *  - Layouts: blob arrays are [n][3] row-major FP64 (x, y, z).  A velocity or force grid of

@@ -30,14 +30,14 @@ class _Rollout(torch.autograd.Function):
         chk = []
         for s in range(K):
             if s % checkpoint == 0:
-                chk.append((sim.blob_positions().clone(), sim.velocity_field().clone()))
+                chk.append((sim.blob_positions(), sim.velocity_field()))
             step(sim.ctx, 1, ext, body)
         U, _ = sim.particle_velocities()
         fctx.sim, fctx.topo, fctx.K, fctx.checkpoint = sim, topo, K, checkpoint
         fctx.ext, fctx.body, fctx.chk = ext, body, chk
-        fctx.qK = sim.blob_positions().clone()
-        fctx.vK = sim.velocity_field().clone()
-        return U.clone()
+        fctx.qK = sim.blob_positions()
+        fctx.vK = sim.velocity_field()
+        return U
 
     @staticmethod
     def backward(fctx, gU):
@@ -47,7 +47,8 @@ class _Rollout(torch.autograd.Function):
         particle_velocity_adjoint(sim.ctx, fctx.qK, fctx.vK,
                                   gU.to(dtype=torch.float64, device=sim.device).contiguous(),
                                   gq, gv)
-        gk = np.zeros(1, dtype=np.float64)
+        # on the device, so that no step of the backward pass waits for the host
+        gk = torch.zeros(1, dtype=torch.float64, device=sim.device)
         K, chk_every = fctx.K, fctx.checkpoint
         for seg in reversed(range(len(fctx.chk))):
             q_s, v_s = fctx.chk[seg]
@@ -56,12 +57,11 @@ class _Rollout(torch.autograd.Function):
             n_seg = min(chk_every, K - seg * chk_every)
             states = []
             for _ in range(n_seg):
-                states.append((sim.blob_positions().clone(), sim.velocity_field().clone()))
+                states.append((sim.blob_positions(), sim.velocity_field()))
                 step(sim.ctx, 1, fctx.ext, fctx.body)
             for qn, vn in reversed(states):
                 adjoint_step(sim.ctx, qn, vn, fctx.ext, fctx.body, gq, gv, gk)
-        gk_t = torch.tensor(gk[0], dtype=torch.float64, device=sim.device)
-        return gq, gk_t, None, None, None, None, None, None
+        return gq, gk[0], None, None, None, None, None, None
 
 
 def rollout_particle_velocities(sim: Multiblob, q0: torch.Tensor, k_spring: torch.Tensor,

@@ -14,61 +14,162 @@ namespace mbk {
 
 namespace {
 
-// Window weights and their derivatives with respect to x = q/h - shift (see peskin_window):
-// with t = x - i0 and s = sqrt(1 - 3t^2): dPhi/dt at i0-1, i0, i0+1 = (t/s - 1)/2, -t/s,
-// (1 + t/s)/2.
-__device__ __forceinline__ int peskin_window_d(double x, double w[3], double dw[3])
+// Sums over the 27 nodes of a window of one grid (+ a second one): the interpolated value and
+// the sums with the weights' derivatives along x, y, z, taken by rows and planes (90 products
+// a component instead of 243).
+struct WinD {
+    double w[3], d[3];
+    int o[3];
+    __device__ __forceinline__ void set(double x, int mask, int stride)
+    {
+        const int i = peskin_window_d(x, w, d);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o[k] = ((i + k) & mask) * stride;
+    }
+};
+__device__ __forceinline__ void window_grad(const double* __restrict__ c0,
+                                            const double* __restrict__ c1, const WinD& wx,
+                                            const WinD& wy, const WinD& wz, double& val,
+                                            double gr[3])
 {
-    const double fl = floor(x + 0.5);
-    const double t = x - fl;
-    const double s = sqrt(1.0 - 3.0 * t * t);
-    w[0] = (2.0 - 3.0 * t - s) / 6.0;
-    w[1] = (1.0 + s) / 3.0;
-    w[2] = (2.0 + 3.0 * t - s) / 6.0;
-    const double ts = t / s;
-    dw[0] = 0.5 * (ts - 1.0);
-    dw[1] = -ts;
-    dw[2] = 0.5 * (1.0 + ts);
-    return (int)fl - 1;
+    val = gr[0] = gr[1] = gr[2] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double pv = 0.0, px = 0.0, py = 0.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int row = wz.o[c] + wy.o[b];
+            double rv = 0.0, rx = 0.0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                double v = __ldg(c0 + (row + wx.o[a]));
+                if (c1) v += __ldg(c1 + (row + wx.o[a]));
+                rv += wx.w[a] * v;
+                rx += wx.d[a] * v;
+            }
+            pv += wy.w[b] * rv;
+            px += wy.w[b] * rx;
+            py += wy.d[b] * rv;
+        }
+        val += wz.w[c] * pv;
+        gr[0] += wz.w[c] * px;
+        gr[1] += wz.w[c] * py;
+        gr[2] += wz.d[c] * pv;
+    }
 }
 
-// out_i += scale * sum_a c_ia grad_{q_i} sum_nodes prod_b Phi_a(node - q_i) w_a(node)
-__global__ void __launch_bounds__(256)
-k_grad_interp(int64_t nb, const double* __restrict__ q, const double* __restrict__ w,
-              const double* __restrict__ c, GridGeo g, double scale, double* __restrict__ out)
+// The windows of component `comp` at position x (in mesh units, x h = q).
+__device__ __forceinline__ void windows_of(int comp, const double x[3], const GridGeo& g, WinD w[3])
 {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    w[0].set(x[0] - (comp == 0 ? 0.0 : 0.5), g.n[0] - 1, 1);
+    w[1].set(x[1] - (comp == 1 ? 0.0 : 0.5), g.n[1] - 1, g.n[0]);
+    w[2].set(x[2] - (comp == 2 ? 0.0 : 0.5), g.n[2] - 1, g.n[0] * g.n[1]);
+}
+
+// These two kernels take one thread per blob and component, 32 blobs a block: the component
+// sums of a blob's gradient meet in shared memory.
+constexpr int ADJ_BLOBS = 32, ADJ_THREADS = 3 * ADJ_BLOBS;
+
+__device__ __forceinline__ double component_sum(const double gr[3], double (*sh)[3], int mine)
+{
+    for (int d = 0; d < 3; ++d) sh[threadIdx.x][d] = gr[d];
+    __syncthreads();
+    const int j = (int)threadIdx.x - mine;
+    return sh[j][mine] + sh[j + 1][mine] + sh[j + 2][mine];
+}
+
+// At the midpoints q: with gf = T dL/dv^{n+1} (the transpose of the fluid update in f),
+//   gF  = S^T gf = h^-3 J gf
+//   gqh = d/dq [ <gf, S(q) F> + sum dt gq . J(q) (v0 + v1)/2 ]
+__global__ void __launch_bounds__(ADJ_THREADS)
+k_adjoint_midpoint(int64_t nb, const double* __restrict__ q, const double* __restrict__ gf,
+                   const double* __restrict__ F, const double* __restrict__ v0,
+                   const double* __restrict__ v1, const double* __restrict__ gq, double dt,
+                   GridGeo g, double* __restrict__ gF, double* __restrict__ gqh)
+{
+    __shared__ double sh[ADJ_THREADS][3];
+    const int64_t t = blockIdx.x * (int64_t)ADJ_THREADS + threadIdx.x;
+    const int64_t b = t / 3;
+    const int mine = (int)(t - 3 * b);
+    const bool live = b < nb;
+    const double inv_h3 = g.inv_h * g.inv_h * g.inv_h;
     double gr[3] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 3; ++a) {
-        const double ca = c[3 * b + a];
-        if (ca == 0.0) continue;
-        double wx[3], wy[3], wz[3], dx[3], dy[3], dz[3];
-        const int ix = peskin_window_d(q[3 * b] * g.inv_h - mac_shift(a, 0), wx, dx);
-        const int iy = peskin_window_d(q[3 * b + 1] * g.inv_h - mac_shift(a, 1), wy, dy);
-        const int iz = peskin_window_d(q[3 * b + 2] * g.inv_h - mac_shift(a, 2), wz, dz);
-        const double* wa = w + (size_t)a * g.N;
-        double sx = 0.0, sy = 0.0, sz = 0.0;
-        for (int kz = 0; kz < 3; ++kz) {
-            const int zz = (iz + kz) & (nz - 1);
-            for (int ky = 0; ky < 3; ++ky) {
-                const int yy = (iy + ky) & (ny - 1);
-                const size_t row = ((size_t)zz * ny + yy) * nx;
-                for (int kx = 0; kx < 3; ++kx) {
-                    const double val = wa[row + ((ix + kx) & (nx - 1))];
-                    sx += dx[kx] * wy[ky] * wz[kz] * val;
-                    sy += wx[kx] * dy[ky] * wz[kz] * val;
-                    sz += wx[kx] * wy[ky] * dz[kz] * val;
-                }
-            }
-        }
-        gr[0] += ca * sx;
-        gr[1] += ca * sy;
-        gr[2] += ca * sz;
+    if (live) {
+        const double x[3] = {q[3 * b] * g.inv_h, q[3 * b + 1] * g.inv_h, q[3 * b + 2] * g.inv_h};
+        WinD w[3];
+        windows_of(mine, x, g, w);
+        const size_t base = (size_t)mine * g.N;
+        double val, d1[3], d2[3];
+        window_grad(gf + base, nullptr, w[0], w[1], w[2], val, d1);
+        gF[t] = val * inv_h3;
+        const double c1 = F[t] * inv_h3, c2 = 0.5 * dt * gq[t];
+        window_grad(v0 + base, v1 + base, w[0], w[1], w[2], val, d2);
+        for (int d = 0; d < 3; ++d) gr[d] = (c1 * d1[d] + c2 * d2[d]) * g.inv_h;
     }
-    // dt/dq = 1/h
-    for (int d = 0; d < 3; ++d) out[3 * b + d] += scale * g.inv_h * gr[d];
+    const double s = component_sum(gr, sh, mine);
+    if (live) gqh[t] = s;
+}
+
+// Transpose of u = J(q) v with gradient gu = scale * gu_in:
+//   out = base (+ base2) + (du/dq)^T gu,  gv += J(q)^T gu
+__global__ void __launch_bounds__(ADJ_THREADS)
+k_adjoint_velocity(int64_t nb, const double* __restrict__ q, const double* __restrict__ v,
+                   const double* gu_in, double scale, const double* base, const double* base2,
+                   GridGeo g, double* out, double* gv)
+{
+    __shared__ double sh[ADJ_THREADS][3];
+    const int64_t t = blockIdx.x * (int64_t)ADJ_THREADS + threadIdx.x;
+    const int64_t b = t / 3;
+    const int mine = (int)(t - 3 * b);
+    const bool live = b < nb;
+    double gr[3] = {0.0, 0.0, 0.0};
+    double at = 0.0;
+    if (live) {
+        double x[3];
+        for (int d = 0; d < 3; ++d) x[d] = wrap_any(q[3 * b + d], g.L[d]) * g.inv_h;
+        const double gu = scale * gu_in[t];
+        at = base2 ? base[t] + base2[t] : base[t];
+        if (gu != 0.0) {
+            WinD w[3];
+            windows_of(mine, x, g, w);
+            const size_t comp = (size_t)mine * g.N;
+            double val;
+            window_grad(v + comp, nullptr, w[0], w[1], w[2], val, gr);
+            for (int d = 0; d < 3; ++d) gr[d] *= gu * g.inv_h;
+            double* f = gv + comp;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const double wyz = w[1].w[k] * w[2].w[c] * gu;
+                    const int row = w[2].o[c] + w[1].o[k];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) atomicAdd(f + (row + w[0].o[a]), w[0].w[a] * wyz);
+                }
+        }
+    }
+    const double s = component_sum(gr, sh, mine);
+    if (live) out[t] = at + s;
+}
+
+// (rho/dt + (eta/2) L) x: A = (rho/dt + (eta/2) L) T for the fluid update v' = A v + T f, all
+// three diagonal in Fourier space, so that A^T g is this stencil of T g and needs no second
+// solve.
+__global__ void __launch_bounds__(256)
+k_viscous_stencil(GridGeo g, const double* __restrict__ x, double a, double c, double* __restrict__ out)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= 3 * g.N) return;
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const int comp = (int)(i / g.N), m = (int)(i - comp * g.N);
+    const int ix = m & (nx - 1), row = m - ix, iy = (row / nx) & (ny - 1), iz = row / (nx * ny);
+    const int plane = row - iy * nx, col = m - iz * nx * ny;
+    const double* s = x + (size_t)comp * g.N;
+    const double v = s[m];
+    const double sum = (s[row + ((ix - 1) & (nx - 1))] + s[row + ((ix + 1) & (nx - 1))]) +
+                       (s[plane + ((iy - 1) & (ny - 1)) * nx + ix] + s[plane + ((iy + 1) & (ny - 1)) * nx + ix]) +
+                       (s[col + ((iz - 1) & (nz - 1)) * nx * ny] + s[col + ((iz + 1) & (nz - 1)) * nx * ny]);
+    out[i] = a * v + c * (sum - 6.0 * v);
 }
 
 // Hessian-vector product of the blob forces and the spring-stiffness derivative.
@@ -76,7 +177,11 @@ k_grad_interp(int64_t nb, const double* __restrict__ q, const double* __restrict
 //   J_s = -k [(1 - r0/|r|) I + (r0/|r|) rhat rhat^T]
 //   J_r = k_rep [(r_cut/|r| - 1) I - (r_cut/|r|) rhat rhat^T]         (|r| < r_cut)
 //   dL/dk += (1/2) sum_b sum_bonds (f_bond(r_bj)/k) . (g_b - g_j)    (each bond seen twice)
-__global__ void __launch_bounds__(256)
+// Eight lanes a blob over its bonds and then its neighbour cells: the centre of an icosahedron
+// has twelve bonds, which one thread took in turn (101 us for 832 blobs).
+constexpr int JVP_LANES = 8, JVP_BLOCK = 128;
+
+__global__ void __launch_bounds__(JVP_BLOCK)
 k_force_jvp(int64_t nb, const double* __restrict__ q, const double* __restrict__ gF,
             const int32_t* __restrict__ pid, const int32_t* __restrict__ adj_start,
             const int32_t* __restrict__ adj_j, const double* __restrict__ adj_rest,
@@ -84,93 +189,112 @@ k_force_jvp(int64_t nb, const double* __restrict__ q, const double* __restrict__
             const int32_t* __restrict__ sorted, const int32_t* __restrict__ blob_cell,
             GridGeo g, BinGeo bg, double* __restrict__ out, double* __restrict__ gk)
 {
-    __shared__ double sh[32];
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    __shared__ double sh[JVP_BLOCK / 32];
+    const int lane = threadIdx.x % JVP_LANES;
     double dk = 0.0;
-    if (b < nb) {
-        const double qb[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
-        const double gb[3] = {gF[3 * b], gF[3 * b + 1], gF[3 * b + 2]};
+    for (int64_t b0 = blockIdx.x * (int64_t)(JVP_BLOCK / JVP_LANES); b0 < nb;
+         b0 += (int64_t)gridDim.x * (JVP_BLOCK / JVP_LANES)) {
+        const int64_t b = b0 + threadIdx.x / JVP_LANES;
         double acc[3] = {0.0, 0.0, 0.0};
-        for (int e = adj_start[b]; e < adj_start[b + 1]; ++e) {
-            const int j = adj_j[e];
-            double r[3], dg[3];
-            for (int d = 0; d < 3; ++d) {
-                r[d] = min_image(qb[d] - q[3 * j + d], g.L[d]);
-                dg[d] = gb[d] - gF[3 * j + d];
+        if (b < nb) {
+            const double qb[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
+            const double gb[3] = {gF[3 * b], gF[3 * b + 1], gF[3 * b + 2]};
+            for (int e = adj_start[b] + lane; e < adj_start[b + 1]; e += JVP_LANES) {
+                const int j = adj_j[e];
+                double r[3], dg[3];
+                for (int d = 0; d < 3; ++d) {
+                    r[d] = min_image(qb[d] - q[3 * j + d], g.L[d]);
+                    dg[d] = gb[d] - gF[3 * j + d];
+                }
+                const Length l(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+                const double dot = r[0] * dg[0] + r[1] * dg[1] + r[2] * dg[2];
+                const double ratio = l.divide(adj_rest[e]);
+                const double a0 = -k_spring * (1.0 - ratio);
+                const double a1 = -k_spring * ratio * l.divide(l.divide(dot));
+                for (int d = 0; d < 3; ++d) acc[d] += a0 * dg[d] + a1 * r[d];
+                dk -= 0.5 * l.divide(l.len - adj_rest[e]) * dot;      // f_bond / k
             }
-            const double len = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-            const double rdg = (r[0] * dg[0] + r[1] * dg[1] + r[2] * dg[2]) / len;
-            const double a0 = -k_spring * (1.0 - adj_rest[e] / len);
-            const double a1 = -k_spring * (adj_rest[e] / len);
-            for (int d = 0; d < 3; ++d) acc[d] += a0 * dg[d] + a1 * rdg * r[d] / len;
-            // f_bond / k = -(|r| - r0) r/|r|
-            const double fk = -(len - adj_rest[e]) / len;
-            dk += 0.5 * fk * (r[0] * dg[0] + r[1] * dg[1] + r[2] * dg[2]);
-        }
-        if (k_rep != 0.0 && r_cut > 0.0) {
-            const int cell = blob_cell[b];
-            const int c[3] = {cell % bg.nc[0], (cell / bg.nc[0]) % bg.nc[1],
-                              cell / (bg.nc[0] * bg.nc[1])};
-            int lo[3], hi[3];
-            for (int d = 0; d < 3; ++d) {
-                if (bg.nc[d] >= 3) { lo[d] = -1; hi[d] = 1; }
-                else { lo[d] = 0; hi[d] = bg.nc[d] - 1; }
-            }
-            for (int dz = lo[2]; dz <= hi[2]; ++dz)
-                for (int dy = lo[1]; dy <= hi[1]; ++dy)
-                    for (int dx = lo[0]; dx <= hi[0]; ++dx) {
-                        const int cx = bg.nc[0] >= 3 ? (c[0] + dx + bg.nc[0]) % bg.nc[0] : dx;
-                        const int cy = bg.nc[1] >= 3 ? (c[1] + dy + bg.nc[1]) % bg.nc[1] : dy;
-                        const int cz = bg.nc[2] >= 3 ? (c[2] + dz + bg.nc[2]) % bg.nc[2] : dz;
-                        const int64_t cc = ((int64_t)cz * bg.nc[1] + cy) * bg.nc[0] + cx;
-                        for (int t = cell_start[cc]; t < cell_start[cc + 1]; ++t) {
-                            const int j = sorted[t];
-                            if (j == b || pid[j] == pid[b]) continue;
-                            double r[3];
-                            for (int d = 0; d < 3; ++d) r[d] = min_image(qb[d] - q[3 * j + d], g.L[d]);
-                            const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                            if (r2 >= r_cut * r_cut || r2 == 0.0) continue;
-                            const double len = sqrt(r2);
-                            double dg[3];
-                            for (int d = 0; d < 3; ++d) dg[d] = gb[d] - gF[3 * j + d];
-                            const double rdg = (r[0] * dg[0] + r[1] * dg[1] + r[2] * dg[2]) / len;
-                            const double a0 = k_rep * (r_cut / len - 1.0);
-                            const double a1 = -k_rep * (r_cut / len);
-                            for (int d = 0; d < 3; ++d) acc[d] += a0 * dg[d] + a1 * rdg * r[d] / len;
-                        }
+            if (k_rep != 0.0 && r_cut > 0.0) {
+                const int cell = blob_cell[b];
+                const int c[3] = {cell % bg.nc[0], (cell / bg.nc[0]) % bg.nc[1],
+                                  cell / (bg.nc[0] * bg.nc[1])};
+                int lo[3], cnt[3];
+                for (int d = 0; d < 3; ++d) {
+                    lo[d] = bg.nc[d] >= 3 ? -1 : 0;
+                    cnt[d] = bg.nc[d] >= 3 ? 3 : bg.nc[d];
+                }
+                for (int k = lane; k < cnt[0] * cnt[1] * cnt[2]; k += JVP_LANES) {
+                    const int dd[3] = {lo[0] + k % cnt[0], lo[1] + (k / cnt[0]) % cnt[1],
+                                       lo[2] + k / (cnt[0] * cnt[1])};
+                    int cc[3];
+                    for (int d = 0; d < 3; ++d)
+                        cc[d] = bg.nc[d] >= 3 ? (c[d] + dd[d] + bg.nc[d]) % bg.nc[d] : dd[d];
+                    const int at = (cc[2] * bg.nc[1] + cc[1]) * bg.nc[0] + cc[0];
+                    for (int t = cell_start[at]; t < cell_start[at + 1]; ++t) {
+                        const int j = sorted[t];
+                        if (j == b || pid[j] == pid[b]) continue;
+                        double r[3], dg[3];
+                        for (int d = 0; d < 3; ++d) r[d] = min_image(qb[d] - q[3 * j + d], g.L[d]);
+                        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+                        if (r2 >= r_cut * r_cut || r2 == 0.0) continue;
+                        const Length l(r2);
+                        for (int d = 0; d < 3; ++d) dg[d] = gb[d] - gF[3 * j + d];
+                        const double dot = r[0] * dg[0] + r[1] * dg[1] + r[2] * dg[2];
+                        const double ratio = l.divide(r_cut);
+                        const double a0 = k_rep * (ratio - 1.0);
+                        const double a1 = -k_rep * ratio * l.divide(l.divide(dot));
+                        for (int d = 0; d < 3; ++d) acc[d] += a0 * dg[d] + a1 * r[d];
                     }
+                }
+            }
         }
-        for (int d = 0; d < 3; ++d) out[3 * b + d] += acc[d];
+#pragma unroll
+        for (int o = JVP_LANES / 2; o > 0; o >>= 1)
+            for (int d = 0; d < 3; ++d) acc[d] += __shfl_xor_sync(0xffffffffu, acc[d], o);
+        if (b < nb && lane == 0)
+            for (int d = 0; d < 3; ++d) out[3 * b + d] += acc[d];
     }
+    if (!gk) return;
     // block sum of dk, one double atomic per block
     for (int o = 16; o > 0; o >>= 1) dk += __shfl_down_sync(0xffffffffu, dk, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = dk;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double x = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (threadIdx.x == 0 && gk) atomicAdd(gk, x);
+    if (threadIdx.x == 0) {
+        double x = 0.0;
+        for (int w = 0; w < JVP_BLOCK / 32; ++w) x += sh[w];
+        atomicAdd(gk, x);
     }
 }
 
-// out = a x + b y (elementwise), y may be null (then out = a x).
-__global__ void k_axpby(int64_t n, double a, const double* __restrict__ x, double b,
-                        const double* __restrict__ y, double* __restrict__ out)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    out[i] = a * x[i] + (y ? b * y[i] : 0.0);
-}
-
-inline unsigned nblk(int64_t n) { return (unsigned)((n + 255) / 256); }
+inline unsigned nblk(int64_t n, int per) { return (unsigned)((n + per - 1) / per); }
 
 }  // namespace
 
-cudaError_t launch_grad_interp(cudaStream_t st, int64_t nb, const double* q, const double* w,
-                               const double* c, const GridGeo& g, double scale, double* out)
+cudaError_t launch_adjoint_midpoint(cudaStream_t st, int64_t nb, const double* q, const double* gf,
+                                    const double* F, const double* v0, const double* v1,
+                                    const double* gq, double dt, const GridGeo& g, double* gF,
+                                    double* gqh)
 {
     if (nb <= 0) return cudaSuccess;
-    k_grad_interp<<<nblk(nb), 256, 0, st>>>(nb, q, w, c, g, scale, out);
+    k_adjoint_midpoint<<<nblk(nb, ADJ_BLOBS), ADJ_THREADS, 0, st>>>(nb, q, gf, F, v0, v1, gq, dt, g,
+                                                                   gF, gqh);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_velocity(cudaStream_t st, int64_t nb, const double* q, const double* v,
+                                    const double* gu, double scale, const double* base,
+                                    const double* base2, const GridGeo& g, double* out, double* gv)
+{
+    if (nb <= 0) return cudaSuccess;
+    k_adjoint_velocity<<<nblk(nb, ADJ_BLOBS), ADJ_THREADS, 0, st>>>(nb, q, v, gu, scale, base, base2,
+                                                                   g, out, gv);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_viscous_stencil(cudaStream_t st, const GridGeo& g, const double* x, double a,
+                                   double c, double* out)
+{
+    k_viscous_stencil<<<nblk(3 * g.N, 256), 256, 0, st>>>(g, x, a, c, out);
     return cudaGetLastError();
 }
 
@@ -182,17 +306,11 @@ cudaError_t launch_force_jvp(cudaStream_t st, int64_t nb, const double* q, const
                              double* out, double* gk)
 {
     if (nb <= 0) return cudaSuccess;
-    k_force_jvp<<<nblk(nb), 256, 0, st>>>(nb, q, gF, pid, adj_start, adj_j, adj_rest, k_spring,
-                                          k_rep, r_cut, cell_start, sorted, blob_cell, g, bg, out,
-                                          gk);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_axpby(cudaStream_t st, int64_t n, double a, const double* x, double b,
-                         const double* y, double* out)
-{
-    if (n <= 0) return cudaSuccess;
-    k_axpby<<<nblk(n), 256, 0, st>>>(n, a, x, b, y, out);
+    // at most 2048 blocks, so that as few atomics meet on gk
+    const unsigned blocks = nblk(nb, JVP_BLOCK / JVP_LANES);
+    k_force_jvp<<<blocks < 2048 ? blocks : 2048, JVP_BLOCK, 0, st>>>(
+        nb, q, gF, pid, adj_start, adj_j, adj_rest, k_spring, k_rep, r_cut, cell_start, sorted,
+        blob_cell, g, bg, out, gk);
     return cudaGetLastError();
 }
 

@@ -6,101 +6,15 @@
 namespace mbk {
 
 // ==========================================================================================
-// Interpolation J (Eq. ju): u_a = sum over the 3x3x3 window of Phi Phi Phi v_a(node).
-// One thread per blob; each component reads its own staggered grid.
-template <typename R, int MODE>
-__global__ void __launch_bounds__(256)
-k_interp(int64_t nb, const double* __restrict__ q, const double* q_base,
-         const R* __restrict__ v0, const R* __restrict__ v1, const int32_t* __restrict__ box_of,
-         GridGeo g, double dt, double* __restrict__ u_out, double* q_out)
-{
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const int box = box_of ? box_of[b] : 0;
-    const double p[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    double u[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        R wx[3], wy[3], wz[3];
-        const int ix = peskin_window<R>(p[0] * g.inv_h - mac_shift(a, 0), wx);
-        const int iy = peskin_window<R>(p[1] * g.inv_h - mac_shift(a, 1), wy);
-        const int iz = peskin_window<R>(p[2] * g.inv_h - mac_shift(a, 2), wz);
-        const size_t base = ((size_t)box * 3 + a) * (size_t)g.N;
-        const R* c0 = v0 + base;
-        const R* c1 = MODE == 2 ? v1 + base : nullptr;
-        // 32-bit offsets inside the component grid (at most 2^24 nodes), the wrapped node
-        // indices computed once per dimension
-        int xo[3], yo[3], zo[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            xo[d] = (ix + d) & (nx - 1);
-            yo[d] = ((iy + d) & (ny - 1)) * nx;
-            zo[d] = ((iz + d) & (nz - 1)) * (ny * nx);
-        }
-        R acc = R(0);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-#pragma unroll
-            for (int bb = 0; bb < 3; ++bb) {
-                const int row = zo[c] + yo[bb];
-                R r = R(0);
-#pragma unroll
-                for (int aa = 0; aa < 3; ++aa) {
-                    R val = __ldg(c0 + (row + xo[aa]));
-                    if (MODE == 2) val += __ldg(c1 + (row + xo[aa]));
-                    r += wx[aa] * val;
-                }
-                acc += wy[bb] * wz[c] * r;
-            }
-        }
-        u[a] = MODE == 2 ? 0.5 * (double)acc : (double)acc;
-    }
-    // position updates round like the plain expression q + (c dt) u (no contraction)
-    if (MODE == 0) {
-        for (int a = 0; a < 3; ++a) u_out[3 * b + a] = u[a];
-    } else if (MODE == 1) {
-        for (int a = 0; a < 3; ++a) {
-            if (u_out) u_out[3 * b + a] = u[a];
-            q_out[3 * b + a] = wrap_position(__dadd_rn(p[a], __dmul_rn(0.5 * dt, u[a])), g.L[a]);
-        }
-    } else {
-        for (int a = 0; a < 3; ++a) {
-            const double qb = q_base[3 * b + a];
-            if (u_out) u_out[3 * b + a] = u[a];
-            q_out[3 * b + a] = wrap_position(__dadd_rn(qb, __dmul_rn(dt, u[a])), g.L[a]);
-        }
-    }
-}
-
-template <typename R>
-cudaError_t launch_interp(cudaStream_t st, int mode, int64_t nb, const double* q,
-                          const double* q_base, const R* v0, const R* v1,
-                          const int32_t* box_of, const GridGeo& g, double dt, double* u_out,
-                          double* q_out)
-{
-    if (nb <= 0) return cudaSuccess;
-    const int T = 256;
-    const unsigned blocks = (unsigned)((nb + T - 1) / T);
-    if (mode == 0)
-        k_interp<R, 0><<<blocks, T, 0, st>>>(nb, q, q_base, v0, v1, box_of, g, dt, u_out, q_out);
-    else if (mode == 1)
-        k_interp<R, 1><<<blocks, T, 0, st>>>(nb, q, q_base, v0, v1, box_of, g, dt, u_out, q_out);
-    else
-        k_interp<R, 2><<<blocks, T, 0, st>>>(nb, q, q_base, v0, v1, box_of, g, dt, u_out, q_out);
-    return cudaGetLastError();
-}
-template cudaError_t launch_interp<float>(cudaStream_t, int, int64_t, const double*,
-                                          const double*, const float*, const float*,
-                                          const int32_t*, const GridGeo&, double, double*,
-                                          double*);
-template cudaError_t launch_interp<double>(cudaStream_t, int, int64_t, const double*,
-                                           const double*, const double*, const double*,
-                                           const int32_t*, const GridGeo&, double, double*,
-                                           double*);
-
-// ==========================================================================================
-// Cell binning (counting sort of blobs by bin cell, box-major).
+// Launch shapes of the FP64 blob kernels.  GB300 issues two FP64 lanes a cycle and SM, so these
+// kernels are bound by that pipe on every SM they reach, and below a few thousand blobs by the
+// latency of one thread's chain: few blobs are spread over as many SMs as there are warps.
+// Blocks of 32 threads up to 16384 blobs (512 blocks, over three for each SM), larger ones
+// after that; a thread per blob and component (split) up to 4096 blobs, where the 3 x 128
+// warps still fit one or two an SM: 832 blobs at 64^3, predictor 26.8 -> 5.0 us.
+inline int blob_block(int64_t nb) { return nb <= 16384 ? 32 : 128; }
+inline bool split_components(int64_t nb) { return nb <= 4096; }
+inline unsigned blocks_of(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 __device__ __forceinline__ int bin_coord(double x, double inv_w, int nc)
 {
@@ -111,138 +25,215 @@ __device__ __forceinline__ int bin_coord(double x, double inv_w, int nc)
     return c;
 }
 
+// Counts a blob at p into its bin cell; its rank there is its place in the cell.
+__device__ __forceinline__ void count_blob(const BinCount& c, int64_t b, int box, const double* p)
+{
+    const int cx = bin_coord(p[0], c.bg.inv_w, c.bg.nc[0]);
+    const int cy = bin_coord(p[1], c.bg.inv_w, c.bg.nc[1]);
+    const int cz = bin_coord(p[2], c.bg.inv_w, c.bg.nc[2]);
+    const int cell = (int)(box * c.bg.ncell + ((int64_t)cz * c.bg.nc[1] + cy) * c.bg.nc[0] + cx);
+    c.blob_cell[b] = cell;
+    c.blob_rank[b] = atomicAdd(c.count + cell, 1);
+}
+
+// Sum over a blob's 27 nodes of the weights times c0 (+ c1 when not null).
+template <typename R>
+__device__ __forceinline__ R window_sum(const R* __restrict__ c0, const R* __restrict__ c1,
+                                        const Win<R>& wx, const Win<R>& wy, const Win<R>& wz)
+{
+    R acc = R(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        R plane = R(0);
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) {
+            const int row = wz.o[c] + wy.o[bb];
+            R r = R(0);
+#pragma unroll
+            for (int aa = 0; aa < 3; ++aa) {
+                R val = __ldg(c0 + (row + wx.o[aa]));
+                if (c1) val += __ldg(c1 + (row + wx.o[aa]));
+                r += wx.w[aa] * val;
+            }
+            // FP64: products summed by rows and planes (39 instructions instead of 45)
+            if constexpr (sizeof(R) == 8) plane += wy.w[bb] * r;
+            else acc += wy.w[bb] * wz.w[c] * r;
+        }
+        if constexpr (sizeof(R) == 8) acc += wz.w[c] * plane;
+    }
+    return acc;
+}
+
+// Interpolation J (Eq. ju): u_a = sum over the 3x3x3 window of Phi Phi Phi v_a(node), each
+// component on its own staggered grid.  One thread per blob, its windows at both MAC shifts
+// computed once per dimension (6 instead of 9); with SPLIT one per blob and component, three
+// windows each.  v1 = null: v0 alone; otherwise the mean of v0 and v1.  WRAP: positions from
+// anywhere (standalone calls).  With `count` the new position is counted into its bin cell.
+struct InterpArgs {
+    int64_t nb;
+    const double* q;
+    const double* q_base;
+    const int32_t* box_of;
+    double dt;
+    double* u_out;
+    double* q_out;
+    BinCount bin;
+};
+
+template <typename R, int MODE, bool SPLIT, bool WRAP>
+__global__ void __launch_bounds__(128)
+k_interp(InterpArgs a, const R* __restrict__ v0, const R* __restrict__ v1, GridGeo g)
+{
+    __shared__ double moved[MODE == 1 && SPLIT ? 96 : 1];       // [32 blobs][3]
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    int64_t b = SPLIT ? t / 3 : t;
+    const int mine = SPLIT ? (int)(t - 3 * b) : 0;
+    const bool live = b < a.nb;
+    if (!live) {
+        if (!(MODE == 1 && SPLIT)) return;
+        b = a.nb - 1;                      // stays for the block's barrier, stores nothing
+    }
+    const int box = a.box_of ? a.box_of[b] : 0;
+    double p[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        p[d] = a.q[3 * b + d];
+        if (WRAP) p[d] = wrap_any(p[d], g.L[d]);
+    }
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const int mask[3] = {nx - 1, ny - 1, nz - 1}, stride[3] = {1, nx, ny * nx};
+    double u[3] = {0.0, 0.0, 0.0};
+    const R half = MODE == 2 && v1 ? R(0.5) : R(1);
+    if (SPLIT) {
+        Win<R> w[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            w[d].set(p[d] * g.inv_h - (d == mine ? 0.0 : 0.5), mask[d], stride[d]);
+        const size_t base = ((size_t)box * 3 + mine) * (size_t)g.N;
+        const R acc = window_sum(v0 + base, v1 ? v1 + base : nullptr, w[0], w[1], w[2]);
+        u[0] = (double)half * (double)acc;
+    } else {
+        Win<R> own[3], across[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            own[d].set(p[d] * g.inv_h - 0.0, mask[d], stride[d]);
+            across[d].set(p[d] * g.inv_h - 0.5, mask[d], stride[d]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t base = ((size_t)box * 3 + c) * (size_t)g.N;
+            const R acc = window_sum(v0 + base, v1 ? v1 + base : nullptr,
+                                     c == 0 ? own[0] : across[0], c == 1 ? own[1] : across[1],
+                                     c == 2 ? own[2] : across[2]);
+            u[c] = (double)half * (double)acc;
+        }
+    }
+    // position updates round like the plain expression q + (c dt) u (no contraction)
+    double nq[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if ((SPLIT && c > 0) || !live) break;
+        const int d = SPLIT ? mine : c;
+        if (a.u_out) a.u_out[3 * b + d] = u[c];
+        if (MODE == 0) continue;
+        const double base = MODE == 1 ? (SPLIT ? (mine == 0 ? p[0] : mine == 1 ? p[1] : p[2]) : p[c])
+                                      : a.q_base[3 * b + d];
+        nq[c] = wrap_position(__dadd_rn(base, __dmul_rn(MODE == 1 ? 0.5 * a.dt : a.dt, u[c])), g.L[d]);
+        a.q_out[3 * b + d] = nq[c];
+    }
+    if (MODE == 1 && a.bin.count) {
+        if constexpr (SPLIT) {
+            moved[threadIdx.x] = nq[0];
+            __syncthreads();
+            const int64_t mb = (int64_t)blockIdx.x * 32 + threadIdx.x;
+            if (threadIdx.x < 32 && mb < a.nb)
+                count_blob(a.bin, mb, a.box_of ? a.box_of[mb] : 0, moved + 3 * threadIdx.x);
+        } else {
+            count_blob(a.bin, b, box, nq);
+        }
+    }
+}
+
+template <typename R>
+cudaError_t launch_interp(cudaStream_t st, int mode, int64_t nb, const double* q,
+                          const double* q_base, const R* v0, const R* v1,
+                          const int32_t* box_of, const GridGeo& g, double dt, double* u_out,
+                          double* q_out, bool wrap, const BinCount* bin)
+{
+    if (nb <= 0) return cudaSuccess;
+    InterpArgs a{nb, q, q_base, box_of, dt, u_out, q_out, bin ? *bin : BinCount{}};
+    const bool split = split_components(nb);
+    const int T = split ? 96 : blob_block(nb);           // split: 32 blobs a block
+    const unsigned blocks = blocks_of(split ? 3 * nb : nb, T);
+    auto go = [&](auto k) { k<<<blocks, T, 0, st>>>(a, v0, mode == 2 ? v1 : nullptr, g); };
+    if (mode == 0) {
+        if (wrap) split ? go(k_interp<R, 0, true, true>) : go(k_interp<R, 0, false, true>);
+        else split ? go(k_interp<R, 0, true, false>) : go(k_interp<R, 0, false, false>);
+    } else if (mode == 1) {
+        if (wrap) split ? go(k_interp<R, 1, true, true>) : go(k_interp<R, 1, false, true>);
+        else split ? go(k_interp<R, 1, true, false>) : go(k_interp<R, 1, false, false>);
+    } else {
+        split ? go(k_interp<R, 2, true, false>) : go(k_interp<R, 2, false, false>);
+    }
+    return cudaGetLastError();
+}
+template cudaError_t launch_interp<float>(cudaStream_t, int, int64_t, const double*,
+                                          const double*, const float*, const float*,
+                                          const int32_t*, const GridGeo&, double, double*,
+                                          double*, bool, const BinCount*);
+template cudaError_t launch_interp<double>(cudaStream_t, int, int64_t, const double*,
+                                           const double*, const double*, const double*,
+                                           const int32_t*, const GridGeo&, double, double*,
+                                           double*, bool, const BinCount*);
+
+// ==========================================================================================
+// Cell binning (counting sort of blobs by bin cell, box-major): counts (by the predictor or
+// k_bin_count), the scan of kernels_blob32.cu, and the placement.
 __global__ void k_bin_count(int64_t nb, const double* __restrict__ q,
-                            const int32_t* __restrict__ box_of, BinGeo bg,
-                            int32_t* __restrict__ count, int32_t* __restrict__ blob_cell,
-                            int32_t* __restrict__ blob_rank)
+                            const int32_t* __restrict__ box_of, BinCount c)
 {
     const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (b >= nb) return;
-    const int box = box_of ? box_of[b] : 0;
-    const int cx = bin_coord(q[3 * b], bg.inv_w, bg.nc[0]);
-    const int cy = bin_coord(q[3 * b + 1], bg.inv_w, bg.nc[1]);
-    const int cz = bin_coord(q[3 * b + 2], bg.inv_w, bg.nc[2]);
-    const int cell = (int)(box * bg.ncell + ((int64_t)cz * bg.nc[1] + cy) * bg.nc[0] + cx);
-    blob_cell[b] = cell;
-    blob_rank[b] = atomicAdd(count + cell, 1);
+    const double p[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
+    count_blob(c, b, box_of ? box_of[b] : 0, p);
 }
 
-constexpr int SCAN_THREADS = 1024;
-constexpr int SCAN_TILE = 4 * SCAN_THREADS;
-
-// Exclusive scan of one tile of 4096 ints; writes the tile total to tile_sums.
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_scan_tile(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n,
-            int32_t* __restrict__ tile_sums)
+// The position of blob b (of bin cell `cell`) relative to the lower corner of its cell (FP32,
+// |x| < cell side) and its particle id, for the FP32 prefilter of the pair search.
+__device__ __forceinline__ float4 cell_local(int b, int cell, const double* __restrict__ q,
+                                             const int32_t* __restrict__ pid, const BinGeo& bg)
 {
-    __shared__ int32_t warp_tot[32];
-    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + 4 * threadIdx.x;
-    int32_t v[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = base + i < n ? in[base + i] : 0;
-    const int32_t s = v[0] + v[1] + v[2] + v[3];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int32_t x = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_tot[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        int32_t w = warp_tot[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        warp_tot[lane] = w;
-    }
-    __syncthreads();
-    int32_t run = x - s + (warp > 0 ? warp_tot[warp - 1] : 0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (base + i < n) out[base + i] = run;
-        run += v[i];
-    }
-    if (threadIdx.x == SCAN_THREADS - 1) tile_sums[blockIdx.x] = run;
+    const int local = (int)(cell % bg.ncell);
+    const int c[3] = {local % bg.nc[0], (local / bg.nc[0]) % bg.nc[1],
+                      local / (bg.nc[0] * bg.nc[1])};
+    float r[3];
+    for (int d = 0; d < 3; ++d) r[d] = (float)(q[3 * b + d] - c[d] * bg.w);
+    return make_float4(r[0], r[1], r[2], __int_as_float(pid ? pid[b] : 0));
 }
 
-// Exclusive scan of the tile totals (one block, sequential chunks); total goes to *total.
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_scan_tops(int32_t* __restrict__ tile_sums, int ntiles, int32_t* __restrict__ total)
-{
-    __shared__ int32_t warp_tot[32];
-    __shared__ int32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c0 = 0; c0 < ntiles; c0 += SCAN_THREADS) {
-        const int i = c0 + threadIdx.x;
-        const int32_t s = i < ntiles ? tile_sums[i] : 0;
-        int32_t x = s;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) warp_tot[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            int32_t w = warp_tot[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            warp_tot[lane] = w;
-        }
-        __syncthreads();
-        const int32_t excl = carry + x - s + (warp > 0 ? warp_tot[warp - 1] : 0);
-        if (i < ntiles) tile_sums[i] = excl;
-        __syncthreads();
-        if (threadIdx.x == SCAN_THREADS - 1) carry = excl + s;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total = carry;
-}
-
-__global__ void k_scan_add(int32_t* __restrict__ out, int64_t n,
-                           const int32_t* __restrict__ tile_offsets)
+// Cell starts from the scan's two levels, and every blob's slot.
+__global__ void __launch_bounds__(256)
+k_bin_place(int64_t nb, int64_t ncells, const int32_t* __restrict__ local,
+            const int32_t* __restrict__ tile_off, int32_t* __restrict__ cell_start,
+            const int32_t* __restrict__ blob_cell, const int32_t* __restrict__ blob_rank,
+            int32_t* __restrict__ sorted, const double* __restrict__ q,
+            const int32_t* __restrict__ pid, BinGeo bg, float4* __restrict__ loc)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] += tile_offsets[i / SCAN_TILE];
-}
-
-// Scatter into sorted order; optionally record each blob's position relative to the lower
-// corner of its bin cell (FP32, |x| < cell side) and its particle id, for the FP32 prefilter of
-// the pair search.
-__global__ void k_bin_scatter(int64_t nb, const int32_t* __restrict__ blob_cell,
-                              const int32_t* __restrict__ blob_rank,
-                              const int32_t* __restrict__ cell_start, int32_t* __restrict__ sorted,
-                              const double* __restrict__ q, const int32_t* __restrict__ pid,
-                              BinGeo bg, float4* __restrict__ loc)
-{
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const int cell = blob_cell[b];
-    const int slot = cell_start[cell] + blob_rank[b];
-    sorted[slot] = (int32_t)b;
-    if (loc) {
-        const int local = (int)(cell % bg.ncell);
-        const int c[3] = {local % bg.nc[0], (local / bg.nc[0]) % bg.nc[1],
-                          local / (bg.nc[0] * bg.nc[1])};
-        const double w = bg.w;   // cell side
-        float r[3];
-        for (int d = 0; d < 3; ++d) r[d] = (float)(q[3 * b + d] - c[d] * w);
-        loc[slot] = make_float4(r[0], r[1], r[2], __int_as_float(pid ? pid[b] : 0));
+    if (i < ncells) cell_start[i] = local[i] + tile_off[i >> BIN_SCAN_LOG];
+    if (i < nb) {
+        const int cell = blob_cell[i];
+        const int slot = local[cell] + tile_off[cell >> BIN_SCAN_LOG] + blob_rank[i];
+        sorted[slot] = (int32_t)i;
+        if (loc) loc[slot] = cell_local((int)i, cell, q, pid, bg);
     }
 }
 
-// Deterministic order inside each cell: ascending blob index (cells hold a handful of blobs).
+// Deterministic order inside each cell: ascending blob index (cells hold a handful of blobs),
+// then the cell-local coordinates in that order.
 __global__ void k_cell_order(int64_t ncells, const int32_t* __restrict__ cell_start,
-                             int32_t* __restrict__ sorted)
+                             int32_t* __restrict__ sorted, const double* __restrict__ q,
+                             const int32_t* __restrict__ pid, BinGeo bg, float4* __restrict__ loc)
 {
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (c >= ncells) return;
@@ -256,62 +247,31 @@ __global__ void k_cell_order(int64_t ncells, const int32_t* __restrict__ cell_st
         }
         sorted[j + 1] = key;
     }
-}
-
-// Cell-local coordinates in the final (reordered) slot order.
-__global__ void k_fill_loc(int64_t nb, const int32_t* __restrict__ sorted,
-                           const int32_t* __restrict__ blob_cell, const double* __restrict__ q,
-                           const int32_t* __restrict__ pid, BinGeo bg, float4* __restrict__ loc)
-{
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nb) return;
-    const int b = sorted[t];
-    const int local = (int)(blob_cell[b] % bg.ncell);
-    const int c[3] = {local % bg.nc[0], (local / bg.nc[0]) % bg.nc[1],
-                      local / (bg.nc[0] * bg.nc[1])};
-    const double w = bg.w;
-    float r[3];
-    for (int d = 0; d < 3; ++d) r[d] = (float)(q[3 * b + d] - c[d] * w);
-    loc[t] = make_float4(r[0], r[1], r[2], __int_as_float(pid ? pid[b] : 0));
-}
-
-cudaError_t launch_exclusive_scan(cudaStream_t st, const int32_t* in, int32_t* out, int64_t n,
-                                  int32_t* tile_tmp)
-{
-    const int T = 256;
-    const int ntiles = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
-    k_scan_tile<<<ntiles, SCAN_THREADS, 0, st>>>(in, out, n, tile_tmp);
-    k_scan_tops<<<1, SCAN_THREADS, 0, st>>>(tile_tmp, ntiles, out + n);
-    k_scan_add<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(out, n, tile_tmp);
-    return cudaGetLastError();
+    if (loc)
+        for (int i = s; i < e; ++i) loc[i] = cell_local(sorted[i], (int)c, q, pid, bg);
 }
 
 cudaError_t launch_bin(cudaStream_t st, int64_t nb, const double* q, const int32_t* box_of,
-                       int B, const BinGeo& bg, int32_t* cell_count, int32_t* cell_start,
-                       int32_t* blob_cell, int32_t* blob_rank, int32_t* sorted,
-                       int32_t* scan_tmp, bool deterministic, const int32_t* pid, float4* loc)
+                       int B, const BinCount& c, int32_t* cell_start, int32_t* sorted,
+                       int32_t* scan_tmp, bool deterministic, const int32_t* pid, float4* loc,
+                       bool counted)
 {
+    const BinGeo& bg = c.bg;
     const int64_t ncells = (int64_t)B * bg.ncell;
-    cudaError_t e = cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, st);
-    if (e != cudaSuccess) return e;
-    const int T = 256;
-    if (nb > 0)
-        k_bin_count<<<(unsigned)((nb + T - 1) / T), T, 0, st>>>(nb, q, box_of, bg, cell_count,
-                                                                blob_cell, blob_rank);
-    const int ntiles = (int)((ncells + SCAN_TILE - 1) / SCAN_TILE);
-    k_scan_tile<<<ntiles, SCAN_THREADS, 0, st>>>(cell_count, cell_start, ncells, scan_tmp);
-    k_scan_tops<<<1, SCAN_THREADS, 0, st>>>(scan_tmp, ntiles, cell_start + ncells);
-    k_scan_add<<<(unsigned)((ncells + T - 1) / T), T, 0, st>>>(cell_start, ncells, scan_tmp);
-    if (nb > 0)
-        k_bin_scatter<<<(unsigned)((nb + T - 1) / T), T, 0, st>>>(nb, blob_cell, blob_rank,
-                                                                  cell_start, sorted, q, pid, bg,
-                                                                  deterministic ? nullptr : loc);
-    if (deterministic) {
-        k_cell_order<<<(unsigned)((ncells + T - 1) / T), T, 0, st>>>(ncells, cell_start, sorted);
-        if (loc && nb > 0)
-            k_fill_loc<<<(unsigned)((nb + T - 1) / T), T, 0, st>>>(nb, sorted, blob_cell, q, pid,
-                                                                   bg, loc);
+    cudaError_t e;
+    if (!counted) {
+        e = cudaMemsetAsync(c.count, 0, sizeof(int32_t) * ncells, st);
+        if (e != cudaSuccess) return e;
+        if (nb > 0) k_bin_count<<<blocks_of(nb, 256), 256, 0, st>>>(nb, q, box_of, c);
     }
+    e = launch_bin_scan(st, c.count, ncells, scan_tmp, cell_start + ncells);
+    if (e != cudaSuccess) return e;
+    k_bin_place<<<blocks_of(nb > ncells ? nb : ncells, 256), 256, 0, st>>>(
+        nb, ncells, c.count, scan_tmp, cell_start, c.blob_cell, c.blob_rank, sorted, q, pid, bg,
+        deterministic ? nullptr : loc);
+    if (deterministic)
+        k_cell_order<<<blocks_of(ncells, 256), 256, 0, st>>>(ncells, cell_start, sorted, q, pid, bg,
+                                                             loc);
     return cudaGetLastError();
 }
 
@@ -343,65 +303,47 @@ __device__ __forceinline__ void block_sum3(double v[3], double* sh /*[3][32]*/)
     }
 }
 
-// Spring force on blob b from bond (b, j): -k (|r| - r0) r/|r|, r = q_b - q_j (minimum image).
-// PRECISE: FP64 with the operations in the plain order and no contraction, so that a blob's
-// spring force is the same bits however the work is scheduled.  Otherwise: r, |r|^2 and
-// |r|^2 - r0^2 in FP64 (the only cancellation), the rest in FP32, accumulated in FP64.
-template <bool PRECISE>
+// Spring force on blob b from bond (b, j): -k (|r| - r0) r/|r|, r = q_b - q_j (minimum image),
+// in FP64 with the operations in the plain order and no contraction, so that a blob's spring
+// force is the same bits however the work is scheduled.
 __device__ __forceinline__ void spring_term(const double qb[3], const double* __restrict__ qj,
-                                            double r0, double k, const double L[3],
-                                            const double halfL[3], double F[3])
+                                            double r0, double k, const double L[3], double F[3])
 {
     double r[3];
     for (int d = 0; d < 3; ++d) {
         double x = __dsub_rn(qb[d], qj[d]);
-        if (x > halfL[d]) x = __dsub_rn(x, L[d]);
-        else if (x < -halfL[d]) x = __dadd_rn(x, L[d]);
+        // beyond half the box (by the high words; exactly below): the other image
+        if ((__double2hiint(x) & 0x7fffffff) >= __double2hiint(L[d]) - (1 << 20)) {
+            const double half = 0.5 * L[d];
+            if (x > half) x = __dsub_rn(x, L[d]);
+            else if (x < -half) x = __dadd_rn(x, L[d]);
+        }
         r[d] = x;
     }
-    if (PRECISE) {
-        const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])),
-                                    __dmul_rn(r[2], r[2]));
-        const double len = __dsqrt_rn(r2);
-        const double mag = __ddiv_rn(__dmul_rn(-k, __dsub_rn(len, r0)), len);
-        for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], __dmul_rn(mag, r[d]));
-    } else {
-        const double r2 = fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2]));
-        const float d2 = (float)(r2 - r0 * r0);               // |r|^2 - r0^2
-        const float len = sqrtf((float)r2);
-        const float mag = -(float)k * d2 / ((len + (float)r0) * len);
-        for (int d = 0; d < 3; ++d) F[d] += (double)(mag * (float)r[d]);
-    }
+    const Length l(__dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])),
+                             __dmul_rn(r[2], r[2])));
+    const double mag = l.divide(__dmul_rn(-k, __dsub_rn(l.len, r0)));
+    for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], __dmul_rn(mag, r[d]));
 }
 
 // Repulsion k_rep (r_cut - |r|) r/|r| for |r| < r_cut, r = q_b - q_j.
-template <bool PRECISE>
 __device__ __forceinline__ void pair_term(const double qb[3], const double* __restrict__ qj,
-                                          const float rf[3], double k_rep, double r_cut,
-                                          const double L[3], double Fp[3])
+                                          double k_rep, double r_cut, const double L[3],
+                                          double Fp[3])
 {
-    if (PRECISE) {
-        double r[3];
-        for (int d = 0; d < 3; ++d) r[d] = min_image(__dsub_rn(qb[d], qj[d]), L[d]);
-        const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])),
-                                    __dmul_rn(r[2], r[2]));
-        if (r2 >= r_cut * r_cut || r2 == 0.0) return;
-        const double len = __dsqrt_rn(r2);
-        const double mag = __ddiv_rn(__dmul_rn(k_rep, __dsub_rn(r_cut, len)), len);
-        for (int d = 0; d < 3; ++d) Fp[d] = __dadd_rn(Fp[d], __dmul_rn(mag, r[d]));
-    } else {
-        const float r2 = rf[0] * rf[0] + rf[1] * rf[1] + rf[2] * rf[2];
-        const float rc = (float)r_cut;
-        if (r2 >= rc * rc || r2 == 0.0f) return;
-        const float len = sqrtf(r2);
-        const float mag = (float)k_rep * (rc - len) / len;
-        for (int d = 0; d < 3; ++d) Fp[d] += (double)(mag * rf[d]);
-    }
+    double r[3];
+    for (int d = 0; d < 3; ++d) r[d] = min_image(__dsub_rn(qb[d], qj[d]), L[d]);
+    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])),
+                                __dmul_rn(r[2], r[2]));
+    if (r2 >= r_cut * r_cut || r2 == 0.0) return;
+    const Length l(r2);
+    const double mag = l.divide(__dmul_rn(k_rep, __dsub_rn(r_cut, l.len)));
+    for (int d = 0; d < 3; ++d) Fp[d] = __dadd_rn(Fp[d], __dmul_rn(mag, r[d]));
 }
 
 // FP64 springs of a bond pattern shared by all particles (launch_springs64).  A block holds
 // whole particles (one thread per blob, blob order).  Each thread evaluates the bonds its
-// evaluation list names (spring_term<true> on a zero sum: the force on its own blob) into its
+// evaluation list names (spring_term on a zero sum: the force on its own blob) into its
 // shared-memory slots; after a barrier it sums ext and, in its adjacency order, its own slots
 // and the negated slots of the bonds its partners evaluated.  Negation is exact and the
 // evaluation of a bond from the other end gives the negated bits, so every sum equals the
@@ -419,7 +361,6 @@ k_springs64(int nb, int m, int S, const double* __restrict__ q, const double* __
     const int l = tid % m;
     if (live) {
         const double qb[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
-        const double halfL[3] = {0.5 * g.L[0], 0.5 * g.L[1], 0.5 * g.L[2]};
         const double k_spring = box_par[3 * (box_of ? box_of[b] : 0)];
         const int e0 = __ldg(tstart + 2 * l), e1 = __ldg(tstart + 2 * l + 1);
         for (int e = e0; e < e1; ++e) {
@@ -428,7 +369,7 @@ k_springs64(int nb, int m, int S, const double* __restrict__ q, const double* __
             const int slot = (ad.x >> 16) - 1;
             const double r0 = __hiloint2double(ad.z, ad.y);
             double f[3] = {0.0, 0.0, 0.0};
-            spring_term<true>(qb, q + 3 * j, r0, k_spring, g.L, halfL, f);
+            spring_term(qb, q + 3 * j, r0, k_spring, g.L, f);
             for (int d = 0; d < 3; ++d) slot_d[(tid * S + slot) * 3 + d] = f[d];
         }
     }
@@ -452,14 +393,16 @@ cudaError_t launch_springs64(cudaStream_t st, int64_t nb, int m, int slots, cons
                              double* Fout)
 {
     if (nb <= 0) return cudaSuccess;
-    const int threads = (256 / m) * m;                   // whole particles per block
+    // whole particles per block; few blobs in small blocks over more SMs
+    const int most = blob_block(nb) < 128 ? (m > 32 ? m : 32) : 256;
+    const int threads = (most / m) * m;
     const size_t smem = sizeof(double) * 3 * (size_t)threads * (slots > 0 ? slots : 1);
     k_springs64<<<(unsigned)((nb + threads - 1) / threads), threads, smem, st>>>(
         (int)nb, m, slots, q, ext, tmpl, tstart, box_of, box_par, g, Fout);
     return cudaGetLastError();
 }
 
-template <bool PRECISE>
+// Blob forces in slot order (blob order without bins: no repulsion then).
 __global__ void __launch_bounds__(256)
 k_forces(ForceArgs a, GridGeo g, BinGeo bg)
 {
@@ -470,9 +413,8 @@ k_forces(ForceArgs a, GridGeo g, BinGeo bg)
     double F[3] = {0.0, 0.0, 0.0};
     if (local < cnt) {
         const int64_t slot = s0 + local;
-        const int b = a.sorted[slot];
+        const int b = a.sorted ? a.sorted[slot] : (int)slot;
         const double qb[3] = {a.q[3 * b], a.q[3 * b + 1], a.q[3 * b + 2]};
-        const double halfL[3] = {0.5 * g.L[0], 0.5 * g.L[1], 0.5 * g.L[2]};
         const double k_rep = a.box_par[3 * box + 1];
         const double r_cut = a.box_par[3 * box + 2];
         if (a.Fpre) {
@@ -485,10 +427,9 @@ k_forces(ForceArgs a, GridGeo g, BinGeo bg)
             }
             const double k_spring = a.box_par[3 * box];
             for (int e = a.adj_start[b]; e < a.adj_start[b + 1]; ++e)
-                spring_term<PRECISE>(qb, a.q + 3 * a.adj_j[e], a.adj_rest[e], k_spring, g.L,
-                                     halfL, F);
+                spring_term(qb, a.q + 3 * a.adj_j[e], a.adj_rest[e], k_spring, g.L, F);
         }
-        if (k_rep != 0.0 && r_cut > 0.0) {
+        if (a.sorted && k_rep != 0.0 && r_cut > 0.0) {
             double Fp[3] = {0.0, 0.0, 0.0};
             const float4 lb = a.loc[slot];
             const int pb = __float_as_int(lb.w);
@@ -499,57 +440,76 @@ k_forces(ForceArgs a, GridGeo g, BinGeo bg)
             const float rcf = (float)r_cut;
             const float pre = rcf * rcf * 1.0001f + 1e-6f;     // conservative FP32 prefilter
             const bool wide = bg.nc[0] >= 3 && bg.nc[1] >= 3 && bg.nc[2] >= 3;
+            // neighbour cells along each axis; in the wide case only those on whose side the
+            // blob is within the prefilter's reach (the margin covers the rounding of loc), in
+            // the order of the full search: the partners met are the same
+            const float reach = sqrtf(pre) + 1e-3f * w, mine[3] = {lb.x, lb.y, lb.z};
             int lo[3], hi[3];
             for (int d = 0; d < 3; ++d) {
-                if (bg.nc[d] >= 3) { lo[d] = -1; hi[d] = 1; }
-                else { lo[d] = 0; hi[d] = bg.nc[d] - 1; }
+                if (wide) {
+                    lo[d] = mine[d] < reach ? -1 : 0;
+                    hi[d] = mine[d] > w - reach ? 1 : 0;
+                } else if (bg.nc[d] >= 3) {
+                    lo[d] = -1;
+                    hi[d] = 1;
+                } else {
+                    lo[d] = 0;
+                    hi[d] = bg.nc[d] - 1;
+                }
             }
+            auto nbr = [](int c0, int d, int nc) {
+                if (nc < 3) return d;
+                int x = c0 + d;
+                x += x < 0 ? nc : 0;
+                x -= x >= nc ? nc : 0;
+                return x;
+            };
             for (int dz = lo[2]; dz <= hi[2]; ++dz) {
-                const int cz = bg.nc[2] >= 3 ? (c[2] + dz + bg.nc[2]) % bg.nc[2] : dz;
+                const int cz = nbr(c[2], dz, bg.nc[2]);
                 for (int dy = lo[1]; dy <= hi[1]; ++dy) {
-                    const int cy = bg.nc[1] >= 3 ? (c[1] + dy + bg.nc[1]) % bg.nc[1] : dy;
+                    const int cy = nbr(c[1], dy, bg.nc[1]);
+                    const int row = (int)(box * bg.ncell) + (cz * bg.nc[1] + cy) * bg.nc[0];
                     for (int dx = lo[0]; dx <= hi[0]; ++dx) {
-                        const int cx = bg.nc[0] >= 3 ? (c[0] + dx + bg.nc[0]) % bg.nc[0] : dx;
-                        const int64_t cc = box * bg.ncell + ((int64_t)cz * bg.nc[1] + cy) * bg.nc[0] + cx;
+                        const int cc = row + nbr(c[0], dx, bg.nc[0]);
                         const float ox = dx * w, oy = dy * w, oz = dz * w;
                         for (int t = a.cell_start[cc]; t < a.cell_start[cc + 1]; ++t) {
                             if (t == slot) continue;
                             const float4 lj = a.loc[t];
                             if (__float_as_int(lj.w) == pb) continue;
-                            float rf[3] = {lb.x - lj.x - ox, lb.y - lj.y - oy, lb.z - lj.z - oz};
+                            const float rf[3] = {lb.x - lj.x - ox, lb.y - lj.y - oy, lb.z - lj.z - oz};
                             if (wide && rf[0] * rf[0] + rf[1] * rf[1] + rf[2] * rf[2] > pre) continue;
-                            const int j = a.sorted[t];
-                            if (!PRECISE && !wide) {
-                                for (int d = 0; d < 3; ++d)
-                                    rf[d] = (float)min_image(qb[d] - a.q[3 * j + d], g.L[d]);
-                            }
-                            pair_term<PRECISE>(qb, a.q + 3 * j, rf, k_rep, r_cut, g.L, Fp);
+                            pair_term(qb, a.q + 3 * a.sorted[t], k_rep, r_cut, g.L, Fp);
                         }
                     }
                 }
             }
             for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], Fp[d]);
         }
-        for (int d = 0; d < 3; ++d) {
-            a.F[3 * b + d] = F[d];
-            a.rec[6 * slot + d] = qb[d];
-            a.rec[6 * slot + 3 + d] = F[d];
-        }
+        for (int d = 0; d < 3; ++d) a.F[3 * b + d] = F[d];
+        if (a.rec)
+            for (int d = 0; d < 3; ++d) {
+                a.rec[6 * slot + d] = qb[d];
+                a.rec[6 * slot + 3 + d] = F[d];
+            }
     }
     block_sum3(F, sh);
     if (threadIdx.x == 0)
         for (int d = 0; d < 3; ++d)
-            a.partial[((int64_t)box * a.nchunk + blockIdx.x) * 3 + d] = F[d];
+            a.partial[((int64_t)box * gridDim.x + blockIdx.x) * 3 + d] = F[d];
 }
 
-cudaError_t launch_forces(cudaStream_t st, int B, int64_t max_box_blobs, const ForceArgs& a,
-                          const GridGeo& g, const BinGeo& bg, bool precise)
+int force_chunks(int64_t nb, int64_t max_box_blobs)
 {
-    if (a.nchunk <= 0) return cudaSuccess;
-    dim3 grid((unsigned)a.nchunk, (unsigned)B);
-    (void)max_box_blobs;
-    if (precise) k_forces<true><<<grid, 256, 0, st>>>(a, g, bg);
-    else k_forces<false><<<grid, 256, 0, st>>>(a, g, bg);
+    const int T = blob_block(nb);
+    return (int)((max_box_blobs + T - 1) / T);
+}
+
+cudaError_t launch_forces(cudaStream_t st, int B, int64_t nb, int64_t max_box_blobs,
+                          const ForceArgs& a, const GridGeo& g, const BinGeo& bg)
+{
+    const int chunks = force_chunks(nb, max_box_blobs);
+    if (chunks <= 0) return cudaSuccess;
+    k_forces<<<dim3((unsigned)chunks, (unsigned)B), blob_block(nb), 0, st>>>(a, g, bg);
     return cudaGetLastError();
 }
 
@@ -589,33 +549,10 @@ cudaError_t launch_force_sum(cudaStream_t st, int B, int nchunk, const double* p
     return cudaGetLastError();
 }
 
-__global__ void k_make_rec(int64_t nb, const int32_t* __restrict__ sorted,
-                           const double* __restrict__ q, const double* __restrict__ F,
-                           double* __restrict__ rec)
-{
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nb) return;
-    const int b = sorted[s];
-    for (int d = 0; d < 3; ++d) {
-        rec[6 * s + d] = q[3 * b + d];
-        rec[6 * s + 3 + d] = F[3 * b + d];
-    }
-}
-
-cudaError_t launch_make_rec(cudaStream_t st, int64_t nb, const int32_t* sorted, const double* q,
-                            const double* F, double* rec)
-{
-    if (nb <= 0) return cudaSuccess;
-    k_make_rec<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(nb, sorted, q, F, rec);
-    return cudaGetLastError();
-}
-
 // ==========================================================================================
-// Spreading S as tile-owner accumulation: each CTA owns a TX x TY x TZ block of nodes of all
-// three components, gathers every blob whose 3x3x3 window can reach it from the bin cells of
-// the block plus its halo, accumulates the in-block part of f = sum delta_h F in shared
-// memory, and writes the block once.  No global atomics; every node is written by exactly one
-// CTA.
+// Deterministic spreading (FP64 grids): tile-owner accumulation in 64-bit fixed point.  Each CTA
+// owns a TX x TY x TZ block of nodes of all three components and gathers every blob whose 3x3x3
+// window can reach it from the bin cells of the block plus its halo.
 
 __host__ __device__ __forceinline__ int floor_div(int a, int b)
 {
@@ -642,175 +579,99 @@ __host__ __device__ __forceinline__ void halo_cells(int T0, int T, int bs, int n
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_spread(const double* __restrict__ rec, const int32_t* __restrict__ cell_start, GridGeo g,
-         BinGeo bg, int TX, int TY, int TZ, int max_ranges, R* __restrict__ f)
+// Blob-owner spreading with global atomics, straight from the caller's order: each blob adds its
+// 81 node contributions into f (zeroed beforehand) with the native FP64 global atomic add, or on
+// FP32 grids with two aligned 8-byte vector adds a row of three nodes (the spare node gets zero;
+// nx is even, so a pair never wraps).  One thread per blob, or with SPLIT one per blob and
+// component.
+template <typename R, bool SPLIT, bool WRAP>
+__global__ void __launch_bounds__(128)
+k_spread_atomic(int64_t nb, const double* __restrict__ q, const double* __restrict__ F,
+                const int32_t* __restrict__ box_of, GridGeo g, double scale, R* __restrict__ f)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tileN = TX * TY * TZ;
-    R* acc = reinterpret_cast<R*>(smem_raw);
-    int32_t* rbeg = reinterpret_cast<int32_t*>(acc + 3 * tileN);
-    int32_t* rpre = rbeg + max_ranges;    // max_ranges + 1 entries
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t b = SPLIT ? t / 3 : t;
+    if (b >= nb) return;
+    const int mine = SPLIT ? (int)(t - 3 * b) : 0;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int box = blockIdx.y;
-    const int ntx = nx / TX, nty = ny / TY;
-    const int tid = blockIdx.x;
-    const int T0[3] = {(tid % ntx) * TX, ((tid / ntx) % nty) * TY, (tid / (ntx * nty)) * TZ};
-    const int T[3] = {TX, TY, TZ};
-
-    for (int i = threadIdx.x; i < 3 * tileN; i += blockDim.x) acc[i] = R(0);
-    int lo[3], cnt[3];
-    for (int d = 0; d < 3; ++d) halo_cells(T0[d], T[d], bg.bs, bg.nc[d], lo[d], cnt[d]);
-    const int rows = cnt[1] * cnt[2];
-    const int nr = 2 * rows;
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-        const int cz = wrap_cell(lo[2] + r / cnt[1], bg.nc[2]);
-        const int cy = wrap_cell(lo[1] + r % cnt[1], bg.nc[1]);
-        const int64_t rowbase = box * bg.ncell + ((int64_t)cz * bg.nc[1] + cy) * bg.nc[0];
-        const int sx = wrap_cell(lo[0], bg.nc[0]);
-        const int ex = sx + cnt[0];
-        const int a1 = ex <= bg.nc[0] ? ex : bg.nc[0];
-        const int s0 = cell_start[rowbase + sx];
-        rbeg[2 * r] = s0;
-        rpre[2 * r] = cell_start[rowbase + a1] - s0;          // length, prefix-summed below
-        if (ex > bg.nc[0]) {
-            const int t0 = cell_start[rowbase];
-            rbeg[2 * r + 1] = t0;
-            rpre[2 * r + 1] = cell_start[rowbase + (ex - bg.nc[0])] - t0;
-        } else {
-            rbeg[2 * r + 1] = 0;
-            rpre[2 * r + 1] = 0;
-        }
+    const int mask[3] = {nx - 1, ny - 1, nz - 1}, stride[3] = {1, nx, ny * nx};
+    R* fb = f + (size_t)(box_of ? box_of[b] : 0) * 3 * (size_t)g.N;
+    double x[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        x[d] = q[3 * b + d];
+        if (WRAP) x[d] = wrap_any(x[d], g.L[d]);
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {       // exclusive prefix of the lengths (one warp)
-        const int lane = threadIdx.x;
-        int carry = 0;
-        for (int c0 = 0; c0 < nr; c0 += 32) {
-            const int i = c0 + lane;
-            const int len = i < nr ? rpre[i] : 0;
-            int x = len;
+    auto add = [&](int comp, const Win<R>& wx, const Win<R>& wy, const Win<R>& wz) {
+        const R Fa = static_cast<R>(F[3 * b + comp] * scale);
+        R* fa = fb + comp * (int)g.N;
+        const bool odd = (wx.o[0] & 1) != 0;
+        const int a0 = wx.o[0] & ~1, a1 = (a0 + 2) & (nx - 1);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (i < nr) rpre[i] = carry + x - len;
-            carry += __shfl_sync(0xffffffffu, x, 31);
-        }
-        if (lane == 0) rpre[nr] = carry;
-    }
-    __syncthreads();
-    const int total = rpre[nr];
-    const double inv_h3 = g.inv_h * g.inv_h * g.inv_h;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        int lo_r = 0, hi_r = nr - 1;
-        while (lo_r < hi_r) {
-            const int mid = (lo_r + hi_r + 1) >> 1;
-            if (rpre[mid] <= t) lo_r = mid; else hi_r = mid - 1;
-        }
-        const int64_t slot = rbeg[lo_r] + (t - rpre[lo_r]);
-        const double* rr = rec + 6 * slot;
-        const double p[3] = {rr[0], rr[1], rr[2]};
+        for (int c = 0; c < 3; ++c) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const R Fa = static_cast<R>(rr[3 + a] * inv_h3);
-            R wx[3], wy[3], wz[3];
-            const int ix = peskin_window<R>(p[0] * g.inv_h - mac_shift(a, 0), wx) - T0[0];
-            const int iy = peskin_window<R>(p[1] * g.inv_h - mac_shift(a, 1), wy) - T0[1];
-            const int iz = peskin_window<R>(p[2] * g.inv_h - mac_shift(a, 2), wz) - T0[2];
-            R* acc_a = acc + a * tileN;
+            for (int bb = 0; bb < 3; ++bb) {
+                const R wyz = wy.w[bb] * wz.w[c] * Fa;
+                R* row = fa + (wz.o[c] + wy.o[bb]);
+                if constexpr (sizeof(R) == 4) {
+                    const float v0 = wx.w[0] * wyz, v1 = wx.w[1] * wyz, v2 = wx.w[2] * wyz;
+                    atomicAdd(reinterpret_cast<float2*>(row + a0),
+                              odd ? make_float2(0.0f, v0) : make_float2(v0, v1));
+                    atomicAdd(reinterpret_cast<float2*>(row + a1),
+                              odd ? make_float2(v1, v2) : make_float2(v2, 0.0f));
+                } else {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int rz = (iz + c) & (nz - 1);
-                if (rz >= TZ) continue;
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb) {
-                    const int ry = (iy + bb) & (ny - 1);
-                    if (ry >= TY) continue;
-                    const R wyz = wy[bb] * wz[c] * Fa;
-#pragma unroll
-                    for (int aa = 0; aa < 3; ++aa) {
-                        const int rx = (ix + aa) & (nx - 1);
-                        if (rx < TX) atomicAdd(acc_a + (rz * TY + ry) * TX + rx, wx[aa] * wyz);
-                    }
+                    for (int aa = 0; aa < 3; ++aa) atomicAdd(row + wx.o[aa], wx.w[aa] * wyz);
                 }
             }
         }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 3 * tileN; i += blockDim.x) {
-        const int a = i / tileN, rem = i - a * tileN;
-        const int rz = rem / (TY * TX), ry = (rem / TX) % TY, rx = rem % TX;
-        f[((size_t)box * 3 + a) * (size_t)g.N +
-          ((size_t)(T0[2] + rz) * ny + (T0[1] + ry)) * nx + (T0[0] + rx)] = acc[i];
-    }
-}
-
-// Blob-owner spreading with global atomics: one thread per sorted slot adds its 81 node
-// contributions straight into f (zeroed beforehand) with the native FP64 (or FP32) global
-// atomic add; the sorted order keeps a warp's nodes close together in L2.
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_spread_atomic(const double* __restrict__ rec, const int32_t* __restrict__ cell_start,
-                GridGeo g, BinGeo bg, R* __restrict__ f)
-{
-    const int box = blockIdx.y;
-    const int64_t s0 = cell_start[box * bg.ncell], s1 = cell_start[(box + 1) * bg.ncell];
-    const int64_t slot = s0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (slot >= s1) return;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const double* rr = rec + 6 * slot;
-    const double p[3] = {rr[0], rr[1], rr[2]};
-    const double inv_h3 = g.inv_h * g.inv_h * g.inv_h;
-    R* fb = f + (size_t)box * 3 * (size_t)g.N;
-    const int N32 = (int)g.N;
+    };
+    if (SPLIT) {
+        Win<R> w[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const R Fa = static_cast<R>(rr[3 + a] * inv_h3);
-        R wx[3], wy[3], wz[3];
-        const int ix = peskin_window<R>(p[0] * g.inv_h - mac_shift(a, 0), wx);
-        const int iy = peskin_window<R>(p[1] * g.inv_h - mac_shift(a, 1), wy);
-        const int iz = peskin_window<R>(p[2] * g.inv_h - mac_shift(a, 2), wz);
-        int xo[3], yo[3], zo[3];
+        for (int d = 0; d < 3; ++d)
+            w[d].set(x[d] * g.inv_h - (d == mine ? 0.0 : 0.5), mask[d], stride[d]);
+        add(mine, w[0], w[1], w[2]);
+    } else {
+        Win<R> own[3], across[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            xo[d] = (ix + d) & (nx - 1);
-            yo[d] = ((iy + d) & (ny - 1)) * nx;
-            zo[d] = ((iz + d) & (nz - 1)) * (ny * nx);
+            own[d].set(x[d] * g.inv_h - 0.0, mask[d], stride[d]);
+            across[d].set(x[d] * g.inv_h - 0.5, mask[d], stride[d]);
         }
-        R* fa = fb + a * N32;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int bb = 0; bb < 3; ++bb) {
-                const R wyz = wy[bb] * wz[c] * Fa;
-#pragma unroll
-                for (int aa = 0; aa < 3; ++aa) atomicAdd(fa + (zo[c] + yo[bb] + xo[aa]), wx[aa] * wyz);
-            }
+            add(c, c == 0 ? own[0] : across[0], c == 1 ? own[1] : across[1],
+                c == 2 ? own[2] : across[2]);
     }
 }
 
 template <typename R>
-cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t max_box_blobs, const double* rec,
-                                 const int32_t* cell_start, const GridGeo& g, const BinGeo& bg,
-                                 R* f)
+cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t nb, const double* q,
+                                 const double* F, const int32_t* box_of, const GridGeo& g, R* f,
+                                 bool zeroed, bool wrap, double scale)
 {
-    cudaError_t e = cudaMemsetAsync(f, 0, sizeof(R) * 3 * (size_t)B * g.N, st);
-    if (e != cudaSuccess || max_box_blobs <= 0) return e;
-    dim3 grid((unsigned)((max_box_blobs + 255) / 256), (unsigned)B);
-    k_spread_atomic<R><<<grid, 256, 0, st>>>(rec, cell_start, g, bg, f);
+    if (!zeroed) {
+        const cudaError_t e = cudaMemsetAsync(f, 0, sizeof(R) * 3 * (size_t)B * g.N, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (nb <= 0) return cudaSuccess;
+    const bool split = split_components(nb);
+    const int T = split ? 96 : blob_block(nb);
+    const unsigned blocks = blocks_of(split ? 3 * nb : nb, T);
+    auto go = [&](auto k) { k<<<blocks, T, 0, st>>>(nb, q, F, box_of, g, scale, f); };
+    if (wrap) split ? go(k_spread_atomic<R, true, true>) : go(k_spread_atomic<R, false, true>);
+    else split ? go(k_spread_atomic<R, true, false>) : go(k_spread_atomic<R, false, false>);
     return cudaGetLastError();
 }
 template cudaError_t launch_spread_atomic<double>(cudaStream_t, int, int64_t, const double*,
-                                                  const int32_t*, const GridGeo&, const BinGeo&,
-                                                  double*);
+                                                  const double*, const int32_t*, const GridGeo&,
+                                                  double*, bool, bool, double);
 template cudaError_t launch_spread_atomic<float>(cudaStream_t, int, int64_t, const double*,
-                                                 const int32_t*, const GridGeo&, const BinGeo&,
-                                                 float*);
+                                                 const double*, const int32_t*, const GridGeo&,
+                                                 float*, bool, bool, double);
 
-// Deterministic FP64 spreading: the same tile-owner scheme, accumulated in 64-bit fixed point
+// The sums are 64-bit fixed point
 // (shared-memory integer atomics are associative, so the sums do not depend on the order in
 // which threads add).  The tile's scale is a power of two chosen from its largest force so that
 // no node can overflow: 2^62 over (candidates x max weight product x max |F| / h^3).
@@ -855,14 +716,22 @@ k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_st
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < nr; ++i) {
-            const int len = rpre[i];
-            rpre[i] = run;
-            run += len;
+    if (threadIdx.x < 32) {       // exclusive prefix of the lengths (one warp)
+        const int lane = threadIdx.x;
+        int carry = 0;
+        for (int c0 = 0; c0 < nr; c0 += 32) {
+            const int i = c0 + lane;
+            const int len = i < nr ? rpre[i] : 0;
+            int x = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (i < nr) rpre[i] = carry + x - len;
+            carry += __shfl_sync(0xffffffffu, x, 31);
         }
-        rpre[nr] = run;
+        if (lane == 0) rpre[nr] = carry;
     }
     __syncthreads();
     const int total = rpre[nr];
@@ -894,29 +763,32 @@ k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_st
     int ex2;
     frexp(bound, &ex2);                      // bound < 2^ex2
     const double scale = ldexp(1.0, 62 - max(ex2, -900));   // finite even for a zero tile
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+    // one thread per blob and component, or per plane of its window too when the tile has few
+    // blobs (a thread's chain of roots and conversions sets the time then)
+    const int parts = 9 * total <= (int)blockDim.x ? 9 : 3;
+    for (int i = threadIdx.x; i < parts * total; i += blockDim.x) {
+        const int t = i / parts, part = i - t * parts;
+        const int a = part % 3, c0 = part / 3, c1 = parts == 9 ? c0 + 1 : 3;
         const double* rr = rec + 6 * slot_of(t);
-        const double p[3] = {rr[0], rr[1], rr[2]};
-        for (int a = 0; a < 3; ++a) {
-            const double Fa = rr[3 + a] * inv_h3;
-            double wx[3], wy[3], wz[3];
-            const int ix = peskin_window<double>(p[0] * g.inv_h - mac_shift(a, 0), wx) - T0[0];
-            const int iy = peskin_window<double>(p[1] * g.inv_h - mac_shift(a, 1), wy) - T0[1];
-            const int iz = peskin_window<double>(p[2] * g.inv_h - mac_shift(a, 2), wz) - T0[2];
-            unsigned long long* acc_a = acc + a * tileN;
-            for (int c = 0; c < 3; ++c) {
-                const int rz = (iz + c) & (nz - 1);
-                if (rz >= TZ) continue;
-                for (int bb = 0; bb < 3; ++bb) {
-                    const int ry = (iy + bb) & (ny - 1);
-                    if (ry >= TY) continue;
-                    const double wyz = wy[bb] * wz[c] * Fa;
-                    for (int aa = 0; aa < 3; ++aa) {
-                        const int rx = (ix + aa) & (nx - 1);
-                        if (rx < TX) {
-                            const long long v = llrint(wx[aa] * wyz * scale);
-                            atomicAdd(acc_a + (rz * TY + ry) * TX + rx, (unsigned long long)v);
-                        }
+        const double Fa = rr[3 + a] * inv_h3;
+        double wx[3], wy[3], wz[3];
+        const int ix = peskin_window<double>(rr[0] * g.inv_h - mac_shift(a, 0), wx) - T0[0];
+        const int iy = peskin_window<double>(rr[1] * g.inv_h - mac_shift(a, 1), wy) - T0[1];
+        const int iz = peskin_window<double>(rr[2] * g.inv_h - mac_shift(a, 2), wz) - T0[2];
+        unsigned long long* acc_a = acc + a * tileN;
+        for (int c = c0; c < c1; ++c) {
+            const int rz = (iz + c) & (nz - 1);
+            if (rz >= TZ) continue;
+            const double wzc = c == 0 ? wz[0] : (c == 1 ? wz[1] : wz[2]);
+            for (int bb = 0; bb < 3; ++bb) {
+                const int ry = (iy + bb) & (ny - 1);
+                if (ry >= TY) continue;
+                const double wyz = wy[bb] * wzc * Fa;
+                for (int aa = 0; aa < 3; ++aa) {
+                    const int rx = (ix + aa) & (nx - 1);
+                    if (rx < TX) {
+                        const long long v = llrint(wx[aa] * wyz * scale);
+                        atomicAdd(acc_a + (rz * TY + ry) * TX + rx, (unsigned long long)v);
                     }
                 }
             }
@@ -958,111 +830,96 @@ cudaError_t launch_spread_det(cudaStream_t st, int B, const double* rec, const i
     return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t launch_spread(cudaStream_t st, int B, const double* rec, const int32_t* cell_start,
-                          const GridGeo& g, const BinGeo& bg, const int tile[3], R* f)
-{
-    const int TX = tile[0], TY = tile[1], TZ = tile[2];
-    int max_rows = 1;
-    for (int d = 1; d < 3; ++d) {
-        int most = 0;
-        for (int T0 = 0; T0 < g.n[d]; T0 += tile[d]) {
-            int lo, cnt;
-            halo_cells(T0, tile[d], bg.bs, bg.nc[d], lo, cnt);
-            most = cnt > most ? cnt : most;
-        }
-        max_rows *= most;
-    }
-    const int max_ranges = 2 * max_rows;
-    const size_t smem = 3 * (size_t)TX * TY * TZ * sizeof(R) + sizeof(int32_t) * (2 * max_ranges + 1);
-    static std::atomic<unsigned> attr{0};
-    if (first_on_device(attr))
-        cudaFuncSetAttribute(k_spread<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    const int ntiles = (g.n[0] / TX) * (g.n[1] / TY) * (g.n[2] / TZ);
-    dim3 grid((unsigned)ntiles, (unsigned)B);
-    k_spread<R><<<grid, 256, smem, st>>>(rec, cell_start, g, bg, TX, TY, TZ, max_ranges, f);
-    return cudaGetLastError();
-}
-template cudaError_t launch_spread<float>(cudaStream_t, int, const double*, const int32_t*,
-                                          const GridGeo&, const BinGeo&, const int[3], float*);
-template cudaError_t launch_spread<double>(cudaStream_t, int, const double*, const int32_t*,
-                                           const GridGeo&, const BinGeo&, const int[3], double*);
-
 // ==========================================================================================
 // Particle velocities: U0 = mean blob velocity; Omega from the least-squares rigid rotation,
 // I0 Omega = sum s x (u - U0) with I0 = sum (s.s 1 - s s) and s relative to the baricentre.
-__global__ void k_particle_reduce(int64_t np, const int32_t* __restrict__ part_start,
-                                  const int32_t* __restrict__ part_blobs,
-                                  const int32_t* __restrict__ box_of_part,
-                                  const double* __restrict__ q, const double* __restrict__ u,
-                                  GridGeo g, double* __restrict__ U, double* __restrict__ Omega)
+// One warp per particle, its blobs over the lanes (a thread per particle took 60 us for 64
+// particles, one chain of FP64 sums and image searches each).
+__device__ __forceinline__ double warp_sum(double x)
 {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+__global__ void __launch_bounds__(128)
+k_particle_reduce(int64_t np, const int32_t* __restrict__ part_start,
+                  const int32_t* __restrict__ part_blobs, const double* __restrict__ q,
+                  const double* __restrict__ u, GridGeo g, double* __restrict__ U,
+                  double* __restrict__ Omega)
+{
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (p >= np) return;
-    (void)box_of_part;
     const int s = part_start[p], e = part_start[p + 1];
-    double Um[3] = {0, 0, 0}, cm[3] = {0, 0, 0};
+    double Um[3] = {0, 0, 0}, Om[3] = {0, 0, 0};
     if (e > s) {
         const int b0 = part_blobs[s];
-        for (int i = s; i < e; ++i) {
+        const double inv = 1.0 / (double)(e - s);
+        double cm[3] = {0, 0, 0}, q0[3];
+        for (int d = 0; d < 3; ++d) q0[d] = q[3 * b0 + d];
+        for (int i = s + lane; i < e; i += 32) {
             const int b = part_blobs[i];
             for (int d = 0; d < 3; ++d) {
                 Um[d] += u[3 * b + d];
-                cm[d] += min_image(q[3 * b + d] - q[3 * b0 + d], g.L[d]);
+                cm[d] += min_image(q[3 * b + d] - q0[d], g.L[d]);
             }
         }
-        const double inv = 1.0 / (double)(e - s);
-        for (int d = 0; d < 3; ++d) { Um[d] *= inv; cm[d] *= inv; }
-        double I[6] = {0, 0, 0, 0, 0, 0};   // xx, yy, zz, xy, xz, yz
-        double tq[3] = {0, 0, 0};
-        for (int i = s; i < e; ++i) {
-            const int b = part_blobs[i];
-            double sv[3], w[3];
-            for (int d = 0; d < 3; ++d) {
-                sv[d] = min_image(q[3 * b + d] - q[3 * b0 + d], g.L[d]) - cm[d];
-                w[d] = u[3 * b + d] - Um[d];
+        for (int d = 0; d < 3; ++d) {
+            Um[d] = warp_sum(Um[d]) * inv;
+            cm[d] = warp_sum(cm[d]) * inv;
+        }
+        if (Omega) {
+            double I[6] = {0, 0, 0, 0, 0, 0};   // xx, yy, zz, xy, xz, yz
+            double tq[3] = {0, 0, 0};
+            for (int i = s + lane; i < e; i += 32) {
+                const int b = part_blobs[i];
+                double sv[3], w[3];
+                for (int d = 0; d < 3; ++d) {
+                    sv[d] = min_image(q[3 * b + d] - q0[d], g.L[d]) - cm[d];
+                    w[d] = u[3 * b + d] - Um[d];
+                }
+                const double s2 = sv[0] * sv[0] + sv[1] * sv[1] + sv[2] * sv[2];
+                I[0] += s2 - sv[0] * sv[0];
+                I[1] += s2 - sv[1] * sv[1];
+                I[2] += s2 - sv[2] * sv[2];
+                I[3] -= sv[0] * sv[1];
+                I[4] -= sv[0] * sv[2];
+                I[5] -= sv[1] * sv[2];
+                tq[0] += sv[1] * w[2] - sv[2] * w[1];
+                tq[1] += sv[2] * w[0] - sv[0] * w[2];
+                tq[2] += sv[0] * w[1] - sv[1] * w[0];
             }
-            const double s2 = sv[0] * sv[0] + sv[1] * sv[1] + sv[2] * sv[2];
-            I[0] += s2 - sv[0] * sv[0];
-            I[1] += s2 - sv[1] * sv[1];
-            I[2] += s2 - sv[2] * sv[2];
-            I[3] -= sv[0] * sv[1];
-            I[4] -= sv[0] * sv[2];
-            I[5] -= sv[1] * sv[2];
-            tq[0] += sv[1] * w[2] - sv[2] * w[1];
-            tq[1] += sv[2] * w[0] - sv[0] * w[2];
-            tq[2] += sv[0] * w[1] - sv[1] * w[0];
+            for (int k = 0; k < 6; ++k) I[k] = warp_sum(I[k]);
+            for (int k = 0; k < 3; ++k) tq[k] = warp_sum(tq[k]);
+            // symmetric 3x3 inverse through the adjugate
+            const double a = I[0], bq = I[1], c = I[2], xy = I[3], xz = I[4], yz = I[5];
+            const double A00 = bq * c - yz * yz, A01 = xz * yz - xy * c, A02 = xy * yz - xz * bq;
+            const double A11 = a * c - xz * xz, A12 = xy * xz - a * yz, A22 = a * bq - xy * xy;
+            const double det = a * A00 + xy * A01 + xz * A02;
+            const double tr = a + bq + c;
+            if (tr > 0.0 && fabs(det) > 1e-12 * tr * tr * tr) {
+                const double id = 1.0 / det;
+                Om[0] = (A00 * tq[0] + A01 * tq[1] + A02 * tq[2]) * id;
+                Om[1] = (A01 * tq[0] + A11 * tq[1] + A12 * tq[2]) * id;
+                Om[2] = (A02 * tq[0] + A12 * tq[1] + A22 * tq[2]) * id;
+            }
         }
-        // symmetric 3x3 inverse through the adjugate
-        const double a = I[0], bq = I[1], c = I[2], xy = I[3], xz = I[4], yz = I[5];
-        const double A00 = bq * c - yz * yz, A01 = xz * yz - xy * c, A02 = xy * yz - xz * bq;
-        const double A11 = a * c - xz * xz, A12 = xy * xz - a * yz, A22 = a * bq - xy * xy;
-        const double det = a * A00 + xy * A01 + xz * A02;
-        const double tr = a + bq + c;
-        double Om[3] = {0, 0, 0};
-        if (tr > 0.0 && fabs(det) > 1e-12 * tr * tr * tr) {
-            const double id = 1.0 / det;
-            Om[0] = (A00 * tq[0] + A01 * tq[1] + A02 * tq[2]) * id;
-            Om[1] = (A01 * tq[0] + A11 * tq[1] + A12 * tq[2]) * id;
-            Om[2] = (A02 * tq[0] + A12 * tq[1] + A22 * tq[2]) * id;
-        }
-        if (Omega)
-            for (int d = 0; d < 3; ++d) Omega[3 * p + d] = Om[d];
-    } else if (Omega) {
-        for (int d = 0; d < 3; ++d) Omega[3 * p + d] = 0.0;
     }
-    if (U)
-        for (int d = 0; d < 3; ++d) U[3 * p + d] = Um[d];
+    if (lane != 0) return;
+    for (int d = 0; d < 3; ++d) {
+        if (U) U[3 * p + d] = Um[d];
+        if (Omega) Omega[3 * p + d] = Om[d];
+    }
 }
 
 cudaError_t launch_particle_reduce(cudaStream_t st, int64_t np, const int32_t* part_start,
-                                   const int32_t* part_blobs, const int32_t* box_of_part,
-                                   const double* q, const double* u, const GridGeo& g,
-                                   double* U, double* Omega)
+                                   const int32_t* part_blobs, const double* q, const double* u,
+                                   const GridGeo& g, double* U, double* Omega)
 {
     if (np <= 0) return cudaSuccess;
-    k_particle_reduce<<<(unsigned)((np + 127) / 128), 128, 0, st>>>(
-        np, part_start, part_blobs, box_of_part, q, u, g, U, Omega);
+    k_particle_reduce<<<blocks_of(np, 4), 128, 0, st>>>(np, part_start, part_blobs, q, u, g, U,
+                                                        Omega);
     return cudaGetLastError();
 }
 
@@ -1097,31 +954,56 @@ cudaError_t launch_particle_mean_adjoint(cudaStream_t st, int64_t np, const int3
 }
 
 // ==========================================================================================
-// Mean of each component grid (FP64 accumulation, fixed order).
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_grid_mean(GridGeo g, const R* __restrict__ v, double* __restrict__ mean_out)
+// Mean of each component grid (FP64 accumulation, fixed order): partial sums of equal chunks,
+// then their sum.  (One block a component took 1.5 ms at 128^3.)
+__device__ __forceinline__ double block_sum(double s, double* sh)
 {
-    __shared__ double sh[256];
-    const int bc = blockIdx.x;
-    const R* c = v + (size_t)bc * g.N;
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < g.N; i += blockDim.x) s += (double)c[i];
     sh[threadIdx.x] = s;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
         if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) mean_out[bc] = sh[0] / (double)g.N;
+    return sh[0];
 }
 
 template <typename R>
-cudaError_t launch_grid_mean(cudaStream_t st, int B, const GridGeo& g, const R* v,
-                             double* mean_out, double* scratch)
+__global__ void __launch_bounds__(256)
+k_grid_partial(GridGeo g, const R* __restrict__ v, double* __restrict__ partial)
 {
-    (void)scratch;
-    k_grid_mean<R><<<B * 3, 256, 0, st>>>(g, v, mean_out);
+    __shared__ double sh[256];
+    const R* c = v + (size_t)blockIdx.y * g.N;
+    double s = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N;
+         i += (int64_t)gridDim.x * blockDim.x)
+        s += (double)c[i];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) partial[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
+}
+
+__global__ void __launch_bounds__(256)
+k_grid_mean(int chunks, int64_t N, const double* __restrict__ partial, double* __restrict__ mean_out)
+{
+    __shared__ double sh[256];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < chunks; i += blockDim.x) s += partial[(size_t)blockIdx.x * chunks + i];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) mean_out[blockIdx.x] = s / (double)N;
+}
+
+int grid_mean_chunks(int64_t N) { return (int)((N + 16383) / 16384); }
+
+template <typename R>
+cudaError_t launch_grid_mean(cudaStream_t st, int B, const GridGeo& g, const R* v,
+                             double* mean_out, double* partial)
+{
+    const int chunks = grid_mean_chunks(g.N);
+    for (int b0 = 0; b0 < 3 * B; b0 += 65535) {                 // the grid's y limit
+        const int nc = 3 * B - b0 < 65535 ? 3 * B - b0 : 65535;
+        k_grid_partial<R><<<dim3((unsigned)chunks, (unsigned)nc), 256, 0, st>>>(
+            g, v + (size_t)b0 * g.N, partial + (size_t)b0 * chunks);
+    }
+    k_grid_mean<<<B * 3, 256, 0, st>>>(chunks, g.N, partial, mean_out);
     return cudaGetLastError();
 }
 template cudaError_t launch_grid_mean<float>(cudaStream_t, int, const GridGeo&, const float*,

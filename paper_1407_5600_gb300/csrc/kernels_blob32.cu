@@ -425,7 +425,7 @@ __global__ void k_bin_count32(int64_t nb, const float4* __restrict__ A,
 // after a fence; no block waits for another) scans the block totals into tile offsets, writes
 // the grand total and resets the ticket for the next launch.  k_bin_place32: cell_start =
 // local scan + tile offset for every cell, and every blob's slot from the same two numbers.
-constexpr int BIN_SCAN_THREADS = 1024, BIN_SCAN_LOG = 12;          // 4096 cells per block
+constexpr int BIN_SCAN_THREADS = 1024;          // four cells a thread
 
 __global__ void __launch_bounds__(BIN_SCAN_THREADS)
 k_bin_scan32(int32_t* __restrict__ c, int64_t n, int32_t* __restrict__ tile_off,
@@ -1174,6 +1174,16 @@ cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, 
                       dim3(256), 0, st, nb, f, g, bg);
 }
 
+cudaError_t launch_bin_scan(cudaStream_t st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
+                            int32_t* total)
+{
+    // scan_tmp: [ntiles] tile offsets, then the ticket of the last-block scan (zero between
+    // launches)
+    const int ntiles = (int)((ncells + (1 << BIN_SCAN_LOG) - 1) >> BIN_SCAN_LOG);
+    return launch_dep(k_bin_scan32, dim3(ntiles), dim3(BIN_SCAN_THREADS), 0, st, count, ncells,
+                      scan_tmp, total, reinterpret_cast<unsigned*>(scan_tmp + ntiles));
+}
+
 cudaError_t launch_bin32(cudaStream_t st, int64_t nb, const float4* A, const int32_t* box_of,
                          int Bx, const BinGeo& bg, int32_t* cell_count, int32_t* cell_start,
                          int32_t* blob_cell, int32_t* blob_rank, int32_t* sorted,
@@ -1188,12 +1198,7 @@ cudaError_t launch_bin32(cudaStream_t st, int64_t nb, const float4* A, const int
             k_bin_count32<<<blocks_for(nb, 256), 256, 0, st>>>(nb, A, box_of, bg, cell_count,
                                                                blob_cell, blob_rank);
     }
-    // scan_tmp: [ntiles] tile offsets, then the ticket of the last-block scan (zero between
-    // launches)
-    const int ntiles = (int)((ncells + (1 << BIN_SCAN_LOG) - 1) >> BIN_SCAN_LOG);
-    e = launch_dep(k_bin_scan32, dim3(ntiles), dim3(BIN_SCAN_THREADS), 0, st, cell_count,
-                   ncells, scan_tmp, cell_start + ncells,
-                   reinterpret_cast<unsigned*>(scan_tmp + ntiles));
+    e = launch_bin_scan(st, cell_count, ncells, scan_tmp, cell_start + ncells);
     if (e != cudaSuccess) return e;
     const int64_t nthr = nb > ncells ? nb : ncells;
     return launch_dep(k_bin_place32, dim3(blocks_for(nthr, 256)), dim3(256), 0, st, nb, ncells,

@@ -159,6 +159,8 @@ struct mb_ctx {
     bool dirty = true;
     int64_t nb = 0, np = 0, max_box_blobs = 0;
     int nchunk = 0;
+    bool any_rep = false;      // some box has a repulsion
+    int direct64 = 0;          // FP64 steps launched directly since the last rebuild
     std::vector<int64_t> box_off_h, part_off_h;
     std::vector<float> box_par32_h;                // float copy of the box parameters
     DBuf q, qh, u, F, rec, ext, pid, box_of, adj_start, adj_j, adj_rest, part_start,
@@ -201,13 +203,13 @@ struct mb_ctx {
     bool graph_ext[2] = {false, false}, graph_body[2] = {false, false};
     int graph_hcur[2] = {0, 0};
     bool graph_fz[2] = {false, false};
+    bool graph_fz_after = false;       // f_zero after a replay (FP64 steps)
     int64_t graph_launches = 0;        // kernels per graph launch
     // adjoint scratch: blob vectors and grids (FP64 contexts)
-    DBuf a_qn, a_u, a_qh, a_gq, a_guc, a_gqh, a_gF, a_gu, a_gk, a_gU;
-    DBuf a_vn, a_vp, a_w, a_gw, a_gvp, a_gvn, a_gf, a_tmp, a_zero;
+    DBuf a_qn, a_qh, a_gq, a_gqh, a_gF, a_gu, a_gk, a_gU;
+    DBuf a_vn, a_vp, a_gvp, a_gvn, a_gf;
     // standalone-operator scratch
-    DBuf s_q, s_F, s_rec, s_cell_count, s_cell_start, s_blob_cell, s_blob_rank, s_sorted,
-        s_scan, s_u, s_g0, s_g1, s_g2, s_out;
+    DBuf s_F, s_g0, s_g1, s_g2, s_out;
 
     // stage timing (CUDA events on the context stream) and kernel launch count
     bool timing = false;
@@ -397,12 +399,17 @@ mb_status rebuild(mb_ctx* ctx)
     ctx->box_off_h.assign(B + 1, 0);
     ctx->part_off_h.assign(B + 1, 0);
     double rmax = 0.0;
+    bool any_rep = false;
     for (int b = 0; b < B; ++b) {
         const BoxData& bx = ctx->boxes[b];
         ctx->box_off_h[b + 1] = ctx->box_off_h[b] + (int64_t)bx.pid.size();
         ctx->part_off_h[b + 1] = ctx->part_off_h[b] + bx.np;
         if (bx.k_rep != 0.0) rmax = std::max(rmax, bx.r_cut);
+        any_rep = any_rep || (bx.k_rep != 0.0 && bx.r_cut > 0.0);
     }
+    ctx->any_rep = any_rep;
+    ctx->direct64 = 0;
+    ctx->f_zero = false;
     const int64_t nb = ctx->box_off_h[B], np = ctx->part_off_h[B];
     ctx->nb = nb;
     ctx->np = np;
@@ -487,7 +494,8 @@ mb_status rebuild(mb_ctx* ctx)
     MB_TRY(ensure(ctx->scan_tmp, sizeof(int32_t) * (ncells / 4096 + 2), E, "scan_tmp"));
     // the FP32 binning keeps a zero ticket after its tile offsets
     MB_CUDA(cudaMemsetAsync(ctx->scan_tmp.p, 0, sizeof(int32_t) * (ncells / 4096 + 2), ctx->st));
-    MB_TRY(ensure(ctx->partial, sizeof(double) * 3 * B * std::max(ctx->nchunk, 1), E, "partial"));
+    MB_TRY(ensure(ctx->partial, sizeof(double) * 3 * B * std::max({ctx->nchunk, force_chunks(nb, ctx->max_box_blobs), 1}),
+                  E, "partial"));
 
     cudaStream_t st = ctx->st;
     auto up = [&](DBuf& d, const void* h, size_t bytes) -> mb_status {
@@ -749,30 +757,124 @@ mb_status drain_stage_events(mb_ctx* ctx)
     return MB_OK;
 }
 
-// One time step of every box (see mb_step in include/mb.h).
-// FP64-mode spreading by blob-owner global atomics (MB_SPREAD64=tile keeps the tile-owner
-// shared-memory kernel).
-bool spread_atomic64()
+// FP64 blobs: the bin cells are needed by the repulsion and by the deterministic spreading.
+bool needs_bins(const mb_ctx* ctx) { return ctx->any_rep || ctx->d.deterministic != 0; }
+
+BinCount bin_count(const mb_ctx* ctx)
 {
-    static const bool on = [] {
-        const char* e = std::getenv("MB_SPREAD64");
-        return !(e && std::string(e) == "tile");
-    }();
-    return on;
+    return BinCount{static_cast<int32_t*>(ctx->cell_count.p),
+                    static_cast<int32_t*>(ctx->blob_cell.p),
+                    static_cast<int32_t*>(ctx->blob_rank.p), ctx->bg};
 }
 
-template <typename R>
-mb_status do_step(mb_ctx* ctx, const double* ext, const double* body)
+// FP64 blob forces F at x (and sorted records when the spreading is deterministic).  counted:
+// the blobs are in the bin counts already.  With one bond pattern for all particles the springs
+// run once per bond, summed with the external forces in the per-blob order (the same bits), on
+// the side stream beside the binning when `overlap`.
+template <typename Mark>
+mb_status forces64(mb_ctx* ctx, const double* x, const double* ext, bool counted, bool overlap,
+                   bool det, Mark&& mark)
+{
+    cudaStream_t st = ctx->st;
+    const int32_t* box_of = static_cast<const int32_t*>(ctx->box_of.p);
+    const bool bins = ctx->any_rep || det;
+    const bool pattern = ctx->tmpl_m > 0 && !springs_per_blob();
+    auto springs = [&](cudaStream_t s2) {
+        ctx->launches += 1;
+        return launch_springs64(s2, ctx->nb, ctx->tmpl_m, ctx->tmpl_slots, x, ext,
+                                static_cast<const int4*>(ctx->tmpl32.p),
+                                static_cast<const int32_t*>(ctx->tstart32.p), box_of,
+                                static_cast<const double*>(ctx->box_par.p), ctx->g,
+                                static_cast<double*>(ctx->Fpre64.p));
+    };
+    const bool side = pattern && bins && overlap;
+    if (side) {
+        MB_CUDA(cudaEventRecord(ctx->fork[0], st));
+        MB_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork[0], 0));
+        MB_CUDA(springs(ctx->side));
+        MB_CUDA(cudaEventRecord(ctx->fork[1], ctx->side));
+    }
+    mark(ST_BIN);
+    if (bins) {
+        MB_CUDA(launch_bin(st, ctx->nb, x, box_of, ctx->B, bin_count(ctx),
+                           static_cast<int32_t*>(ctx->cell_start.p),
+                           static_cast<int32_t*>(ctx->sorted.p),
+                           static_cast<int32_t*>(ctx->scan_tmp.p), det,
+                           static_cast<const int32_t*>(ctx->pid.p),
+                           static_cast<float4*>(ctx->loc.p), counted));
+        ctx->launches += (counted ? 2 : 3) + (det ? 1 : 0);
+    }
+    mark(ST_FORCES);
+    if (side) MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[1], 0));
+    else if (pattern) MB_CUDA(springs(st));
+    ForceArgs fa{};
+    fa.Fpre = pattern ? static_cast<const double*>(ctx->Fpre64.p) : nullptr;
+    fa.box_off = static_cast<const int64_t*>(ctx->box_off.p);
+    fa.sorted = bins ? static_cast<const int32_t*>(ctx->sorted.p) : nullptr;
+    fa.q = x;
+    fa.pid = static_cast<const int32_t*>(ctx->pid.p);
+    fa.adj_start = static_cast<const int32_t*>(ctx->adj_start.p);
+    fa.adj_j = static_cast<const int32_t*>(ctx->adj_j.p);
+    fa.adj_rest = static_cast<const double*>(ctx->adj_rest.p);
+    fa.box_par = static_cast<const double*>(ctx->box_par.p);
+    fa.cell_start = static_cast<const int32_t*>(ctx->cell_start.p);
+    fa.blob_cell = static_cast<const int32_t*>(ctx->blob_cell.p);
+    fa.ext = ext;
+    fa.loc = static_cast<const float4*>(ctx->loc.p);
+    fa.F = static_cast<double*>(ctx->F.p);
+    fa.rec = det ? static_cast<double*>(ctx->rec.p) : nullptr;
+    fa.partial = static_cast<double*>(ctx->partial.p);
+    MB_CUDA(launch_forces(st, ctx->B, ctx->nb, ctx->max_box_blobs, fa, ctx->g, ctx->bg));
+    ctx->launches += 1;
+    return MB_OK;
+}
+
+// f = S(x) F from forces64; the deterministic kernel writes every node, the atomic one adds.
+mb_status spread64(mb_ctx* ctx, const double* x, bool det)
+{
+    if (det)
+        MB_CUDA(launch_spread_det(ctx->st, ctx->B, static_cast<const double*>(ctx->rec.p),
+                                  static_cast<const int32_t*>(ctx->cell_start.p), ctx->g, ctx->bg,
+                                  ctx->tile, static_cast<double*>(ctx->f.p)));
+    else
+        MB_CUDA(launch_spread_atomic<double>(ctx->st, ctx->B, ctx->nb, x,
+                                             static_cast<const double*>(ctx->F.p),
+                                             static_cast<const int32_t*>(ctx->box_of.p), ctx->g,
+                                             static_cast<double*>(ctx->f.p), ctx->f_zero, false,
+                                             ctx->g.inv_h * ctx->g.inv_h * ctx->g.inv_h));
+    ctx->launches += 1;
+    return MB_OK;
+}
+
+// The FP64 fluid solve.  After an accumulating spreading the three-pass pipeline clears f as it
+// reads it, so that no memset runs before the next one.
+mb_status fluid64(mb_ctx* ctx, int boxes, FluidArgs<double> fa, bool clear_f, cudaEvent_t* marks)
+{
+    if (ctx->fft_passes == 5) {
+        MB_CUDA(launch_fluid<double>(ctx->st, boxes, ctx->g, fa, marks));
+        ctx->launches += FLUID_KERNELS;
+    } else {
+        if (clear_f) fa.f_clear = static_cast<double*>(ctx->f.p);
+        MB_CUDA(launch_fluid3<double>(ctx->st, boxes, ctx->g, fa, marks));
+        ctx->launches += FLUID3_KERNELS;
+    }
+    ctx->f_zero = clear_f && ctx->fft_passes == 3;
+    return MB_OK;
+}
+
+// One time step of every box in FP64 (see mb_step in include/mb.h).  Host-side state other than
+// f_zero and the launch count changes in finish_step64.
+mb_status do_step64(mb_ctx* ctx, const double* ext, const double* body)
 {
     cudaStream_t st = ctx->st;
     const GridGeo& g = ctx->g;
     const int B = ctx->B;
-    R* vcur = static_cast<R*>(ctx->v[ctx->cur].p);
-    R* vnext = static_cast<R*>(ctx->v[ctx->cur ^ 1].p);
+    double* vcur = static_cast<double*>(ctx->v[ctx->cur].p);
+    double* vnext = static_cast<double*>(ctx->v[ctx->cur ^ 1].p);
     double* q = static_cast<double*>(ctx->q.p);
     double* qh = static_cast<double*>(ctx->qh.p);
     const int32_t* box_of = static_cast<const int32_t*>(ctx->box_of.p);
-    const bool blobs = ctx->nb > 0;
+    const bool blobs = ctx->nb > 0, bins = blobs && needs_bins(ctx), det = ctx->d.deterministic != 0;
     if (ctx->timing) {
         if (ctx->ev_pending == mb_ctx::EV_RING) MB_TRY(drain_stage_events(ctx));
         ctx->ev = ctx->ev_ring.data() + (size_t)ctx->ev_pending * (NUM_STAGES + 1);
@@ -780,240 +882,130 @@ mb_status do_step(mb_ctx* ctx, const double* ext, const double* body)
     auto mark = [&](int i) { if (ctx->timing) cudaEventRecord(ctx->ev[i], st); };
     mark(ST_INTERP_PREDICT);
     if (blobs) {
-        // u^n = J(q^n) v^n ; q^{n+1/2} = q^n + dt/2 u^n
-        MB_CUDA(launch_interp<R>(st, 1, ctx->nb, q, nullptr, vcur, nullptr, box_of, g,
-                                 ctx->d.dt, nullptr, qh));
+        // u^n = J(q^n) v^n ; q^{n+1/2} = q^n + dt/2 u^n, counted into its bin cell on the way
+        const BinCount bin = bin_count(ctx);
+        if (bins) MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * B * ctx->bg.ncell, st));
+        MB_CUDA(launch_interp<double>(st, 1, ctx->nb, q, nullptr, vcur, nullptr, box_of, g,
+                                      ctx->d.dt, nullptr, qh, false, bins ? &bin : nullptr));
         ctx->launches += 1;
-    }
-    // FP64 grid, one bond pattern for all particles: the springs once per bond, summed with
-    // the external forces in the per-blob order (the same bits); without stage timing on the
-    // side stream, beside the binning
-    const bool pattern = blobs && ctx->rsz == 8 && ctx->tmpl_m > 0 && !springs_per_blob();
-    auto springs64 = [&](cudaStream_t s2) {
-        return launch_springs64(s2, ctx->nb, ctx->tmpl_m, ctx->tmpl_slots, qh, ext,
-                                static_cast<const int4*>(ctx->tmpl32.p),
-                                static_cast<const int32_t*>(ctx->tstart32.p), box_of,
-                                static_cast<const double*>(ctx->box_par.p), g,
-                                static_cast<double*>(ctx->Fpre64.p));
-    };
-    const bool side64 = pattern && !ctx->timing;
-    if (side64) {
-        MB_CUDA(cudaEventRecord(ctx->fork[0], st));
-        MB_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork[0], 0));
-        MB_CUDA(springs64(ctx->side));
-        MB_CUDA(cudaEventRecord(ctx->fork[1], ctx->side));
-        ctx->launches += 1;
-    }
-    mark(ST_BIN);
-    if (blobs) {
-        MB_CUDA(launch_bin(st, ctx->nb, qh, box_of, B, ctx->bg,
-                           static_cast<int32_t*>(ctx->cell_count.p),
-                           static_cast<int32_t*>(ctx->cell_start.p),
-                           static_cast<int32_t*>(ctx->blob_cell.p),
-                           static_cast<int32_t*>(ctx->blob_rank.p),
-                           static_cast<int32_t*>(ctx->sorted.p),
-                           static_cast<int32_t*>(ctx->scan_tmp.p), ctx->d.deterministic != 0,
-                           static_cast<const int32_t*>(ctx->pid.p),
-                           static_cast<float4*>(ctx->loc.p)));
-        ctx->launches += 5 + 2 * (ctx->d.deterministic != 0);
-    }
-    mark(ST_FORCES);
-    if (blobs) {
-        if (side64) {
-            MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[1], 0));
-        } else if (pattern) {
-            MB_CUDA(springs64(st));
-            ctx->launches += 1;
-        }
-        ForceArgs fa{};
-        fa.Fpre = pattern ? static_cast<const double*>(ctx->Fpre64.p) : nullptr;
-        fa.box_off = static_cast<const int64_t*>(ctx->box_off.p);
-        fa.sorted = static_cast<const int32_t*>(ctx->sorted.p);
-        fa.q = qh;
-        fa.pid = static_cast<const int32_t*>(ctx->pid.p);
-        fa.adj_start = static_cast<const int32_t*>(ctx->adj_start.p);
-        fa.adj_j = static_cast<const int32_t*>(ctx->adj_j.p);
-        fa.adj_rest = static_cast<const double*>(ctx->adj_rest.p);
-        fa.box_par = static_cast<const double*>(ctx->box_par.p);
-        fa.cell_start = static_cast<const int32_t*>(ctx->cell_start.p);
-        fa.blob_cell = static_cast<const int32_t*>(ctx->blob_cell.p);
-        fa.ext = ext;
-        fa.loc = static_cast<const float4*>(ctx->loc.p);
-        fa.F = static_cast<double*>(ctx->F.p);
-        fa.rec = static_cast<double*>(ctx->rec.p);
-        fa.partial = static_cast<double*>(ctx->partial.p);
-        fa.nchunk = ctx->nchunk;
-        MB_CUDA(launch_forces(st, B, ctx->max_box_blobs, fa, g, ctx->bg, ctx->rsz == 8));
-        ctx->launches += 1;
+        MB_TRY(forces64(ctx, qh, ext, true, !ctx->timing, det, mark));
+    } else {
+        mark(ST_BIN);
+        mark(ST_FORCES);
     }
     mark(ST_FORCE_SUM);
     if (blobs) {
         const double L3 = g.L[0] * g.L[1] * g.L[2];
-        MB_CUDA(launch_force_sum(st, B, ctx->nchunk, static_cast<const double*>(ctx->partial.p),
+        MB_CUDA(launch_force_sum(st, B, force_chunks(ctx->nb, ctx->max_box_blobs),
+                                 static_cast<const double*>(ctx->partial.p),
                                  static_cast<double*>(ctx->vbar.p),
                                  ctx->d.dt / (ctx->d.rho * L3), ctx->d.mean_mode,
                                  static_cast<double*>(ctx->fsum.p)));
         ctx->launches += 1;
     }
     mark(ST_SPREAD);
-    if (blobs) {
-        if (ctx->d.deterministic && sizeof(R) == 8)
-            MB_CUDA(launch_spread_det(st, B, static_cast<const double*>(ctx->rec.p),
-                                      static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
-                                      ctx->tile, reinterpret_cast<double*>(ctx->f.p)));
-        else if (spread_atomic64())
-            MB_CUDA(launch_spread_atomic<R>(st, B, ctx->max_box_blobs,
-                                            static_cast<const double*>(ctx->rec.p),
-                                            static_cast<const int32_t*>(ctx->cell_start.p), g,
-                                            ctx->bg, static_cast<R*>(ctx->f.p)));
-        else
-            MB_CUDA(launch_spread<R>(st, B, static_cast<const double*>(ctx->rec.p),
-                                     static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
-                                     ctx->tile, static_cast<R*>(ctx->f.p)));
-        ctx->launches += 1;
-    }
+    if (blobs) MB_TRY(spread64(ctx, qh, det));
     mark(ST_STRESS);
     const bool stress = ctx->thermal || ctx->advect;
     if (stress) {
-        MB_CUDA(launch_fluid_stress<R>(st, B, g, ctx->d.seed,
-                                       static_cast<uint64_t*>(ctx->step_index.p),
-                                       ctx->thermal_amp, ctx->advect ? vcur : nullptr,
-                                       ctx->d.rho, static_cast<R*>(ctx->W.p),
-                                       static_cast<R*>(ctx->f.p), blobs));
+        MB_CUDA(launch_fluid_stress<double>(st, B, g, ctx->d.seed,
+                                            static_cast<uint64_t*>(ctx->step_index.p),
+                                            ctx->thermal_amp, ctx->advect ? vcur : nullptr,
+                                            ctx->d.rho, static_cast<double*>(ctx->W.p),
+                                            static_cast<double*>(ctx->f.p), blobs));
         ctx->launches += STRESS_KERNELS;
     }
     const double* mean = ctx->d.mean_mode == 0 ? static_cast<const double*>(ctx->vbar.p) : nullptr;
-    FluidArgs<R> fa = fluid_args<R>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr, vnext,
-                                    ctx->body_prof.p, body, mean);
-    cudaEvent_t* fm = ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr;
-    if (ctx->fft_passes == 5) {
-        MB_CUDA(launch_fluid<R>(st, B, g, fa, fm));
-        ctx->launches += FLUID_KERNELS;
-    } else {
-        MB_CUDA(launch_fluid3<R>(st, B, g, fa, fm));
-        ctx->launches += FLUID3_KERNELS;
-    }
+    MB_TRY(fluid64(ctx, B,
+                   fluid_args<double>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr, vnext,
+                                      ctx->body_prof.p, body, mean),
+                   blobs && !det, ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr));
     if (blobs) {
         // q^{n+1} = q^n + dt J(q^{n+1/2}) (v^n + v^{n+1})/2
-        MB_CUDA(launch_interp<R>(st, 2, ctx->nb, qh, q, vcur, vnext, box_of, g, ctx->d.dt,
-                                 nullptr, q));
+        MB_CUDA(launch_interp<double>(st, 2, ctx->nb, qh, q, vcur, vnext, box_of, g, ctx->d.dt,
+                                      nullptr, q));
         ctx->launches += 1;
     }
     mark(NUM_STAGES);
     if (ctx->timing) ctx->ev_pending++;
-    ctx->cur ^= 1;
-    ctx->steps_taken++;
     return MB_OK;
 }
 
-// One Stokes-limit step of every box (integrator 1), FP64 blob positions in either grid
-// precision: two half steps, each binning the blobs, computing their forces, spreading them and
-// solving the steady zero-mean Stokes flow v = P (-eta L)^{-1} (S F + f_body) (the three-pass
-// FFT with the right-hand side f alone and the divide by eta lambda); then
-// q^{n+1/2} = q^n + dt/2 J(q^n) v(q^n) and q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2}).
-template <typename R>
-mb_status do_step_stokes(mb_ctx* ctx, const double* ext, const double* body)
+// One Stokes-limit step of every box (integrator 1) in FP64: two half steps, each binning the
+// blobs, computing their forces, spreading them and solving the steady zero-mean Stokes flow
+// v = P (-eta L)^{-1} (S F + f_body) (the FFT passes with the right-hand side f alone and the
+// divide by eta lambda); then q^{n+1/2} = q^n + dt/2 J(q^n) v(q^n) and
+// q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2}).
+mb_status do_step_stokes64(mb_ctx* ctx, const double* ext, const double* body)
 {
     cudaStream_t st = ctx->st;
     const GridGeo& g = ctx->g;
-    const int B = ctx->B;
-    R* v_half = static_cast<R*>(ctx->v[ctx->cur ^ 1].p);
-    R* v_full = static_cast<R*>(ctx->v[ctx->cur].p);
+    double* v_half = static_cast<double*>(ctx->v[ctx->cur ^ 1].p);
+    double* v_full = static_cast<double*>(ctx->v[ctx->cur].p);
     double* q = static_cast<double*>(ctx->q.p);
     double* qh = static_cast<double*>(ctx->qh.p);
     const int32_t* box_of = static_cast<const int32_t*>(ctx->box_of.p);
-    const bool blobs = ctx->nb > 0;
+    const bool blobs = ctx->nb > 0, bins = blobs && needs_bins(ctx), det = ctx->d.deterministic != 0;
     if (ctx->timing) {
         if (ctx->ev_pending == mb_ctx::EV_RING) MB_TRY(drain_stage_events(ctx));
         ctx->ev = ctx->ev_ring.data() + (size_t)ctx->ev_pending * (NUM_STAGES + 1);
     }
     auto mark = [&](int i) { if (ctx->timing) cudaEventRecord(ctx->ev[i], st); };
     // forces at x into ctx->f, then the Stokes flow into v_out (stage marks on the second half)
-    auto half = [&](const double* x, R* v_out, bool marks) -> mb_status {
-        if (marks) mark(ST_BIN);
+    auto half = [&](const double* x, bool counted, double* v_out, bool marks) -> mb_status {
+        auto m = [&](int i) { if (marks) mark(i); };
         if (blobs) {
-            MB_CUDA(launch_bin(st, ctx->nb, x, box_of, B, ctx->bg,
-                               static_cast<int32_t*>(ctx->cell_count.p),
-                               static_cast<int32_t*>(ctx->cell_start.p),
-                               static_cast<int32_t*>(ctx->blob_cell.p),
-                               static_cast<int32_t*>(ctx->blob_rank.p),
-                               static_cast<int32_t*>(ctx->sorted.p),
-                               static_cast<int32_t*>(ctx->scan_tmp.p), ctx->d.deterministic != 0,
-                               static_cast<const int32_t*>(ctx->pid.p),
-                               static_cast<float4*>(ctx->loc.p)));
-            ctx->launches += 5 + 2 * (ctx->d.deterministic != 0);
+            MB_TRY(forces64(ctx, x, ext, counted, !ctx->timing, det, m));
+        } else {
+            m(ST_BIN);
+            m(ST_FORCES);
         }
-        if (marks) mark(ST_FORCES);
-        if (blobs) {
-            ForceArgs fa{};
-            fa.box_off = static_cast<const int64_t*>(ctx->box_off.p);
-            fa.sorted = static_cast<const int32_t*>(ctx->sorted.p);
-            fa.q = x;
-            fa.pid = static_cast<const int32_t*>(ctx->pid.p);
-            fa.adj_start = static_cast<const int32_t*>(ctx->adj_start.p);
-            fa.adj_j = static_cast<const int32_t*>(ctx->adj_j.p);
-            fa.adj_rest = static_cast<const double*>(ctx->adj_rest.p);
-            fa.box_par = static_cast<const double*>(ctx->box_par.p);
-            fa.cell_start = static_cast<const int32_t*>(ctx->cell_start.p);
-            fa.blob_cell = static_cast<const int32_t*>(ctx->blob_cell.p);
-            fa.ext = ext;
-            fa.loc = static_cast<const float4*>(ctx->loc.p);
-            fa.F = static_cast<double*>(ctx->F.p);
-            fa.rec = static_cast<double*>(ctx->rec.p);
-            fa.partial = static_cast<double*>(ctx->partial.p);
-            fa.nchunk = ctx->nchunk;
-            MB_CUDA(launch_forces(st, B, ctx->max_box_blobs, fa, g, ctx->bg, ctx->rsz == 8));
-            ctx->launches += 1;
-        }
-        if (marks) mark(ST_FORCE_SUM);
-        if (marks) mark(ST_SPREAD);
-        if (blobs) {
-            if (ctx->d.deterministic && sizeof(R) == 8)
-                MB_CUDA(launch_spread_det(st, B, static_cast<const double*>(ctx->rec.p),
-                                          static_cast<const int32_t*>(ctx->cell_start.p), g,
-                                          ctx->bg, ctx->tile, reinterpret_cast<double*>(ctx->f.p)));
-            else
-                MB_CUDA(launch_spread<R>(st, B, static_cast<const double*>(ctx->rec.p),
-                                         static_cast<const int32_t*>(ctx->cell_start.p), g,
-                                         ctx->bg, ctx->tile, static_cast<R*>(ctx->f.p)));
-            ctx->launches += 1;
-        }
-        if (marks) mark(ST_STRESS);        // no thermal or convective stress in this integrator
-        FluidArgs<R> fa = fluid_args<R>(ctx, v_out, blobs ? ctx->f.p : nullptr, v_out,
-                                        ctx->body_prof.p, body, nullptr);
+        m(ST_FORCE_SUM);
+        m(ST_SPREAD);
+        if (blobs) MB_TRY(spread64(ctx, x, det));
+        m(ST_STRESS);        // no thermal or convective stress in this integrator
+        FluidArgs<double> fa = fluid_args<double>(ctx, v_out, blobs ? ctx->f.p : nullptr, v_out,
+                                                  ctx->body_prof.p, body, nullptr);
         fa.no_v = 1;                        // right-hand side S F + f_body
         fa.rho_dt = 0.0;                    // divide by eta lambda: steady Stokes
         fa.half_eta = ctx->d.eta;
         fa.mean_mode = 1;
-        cudaEvent_t* fm = marks && ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr;
-        if (ctx->fft_passes == 5) {
-            MB_CUDA(launch_fluid<R>(st, B, g, fa, fm));
-            ctx->launches += FLUID_KERNELS;
-        } else {
-            MB_CUDA(launch_fluid3<R>(st, B, g, fa, fm));
-            ctx->launches += FLUID3_KERNELS;
-        }
-        return MB_OK;
+        return fluid64(ctx, ctx->B, fa, blobs && !det,
+                       marks && ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr);
     };
     mark(ST_INTERP_PREDICT);
-    MB_TRY(half(q, v_half, false));
+    MB_TRY(half(q, false, v_half, false));
     if (blobs) {
         // q^{n+1/2} = q^n + dt/2 J(q^n) v(q^n)
-        MB_CUDA(launch_interp<R>(st, 1, ctx->nb, q, nullptr, v_half, nullptr, box_of, g,
-                                 ctx->d.dt, nullptr, qh));
+        const BinCount bin = bin_count(ctx);
+        if (bins)
+            MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * ctx->B * ctx->bg.ncell, st));
+        MB_CUDA(launch_interp<double>(st, 1, ctx->nb, q, nullptr, v_half, nullptr, box_of, g,
+                                      ctx->d.dt, nullptr, qh, false, bins ? &bin : nullptr));
         ctx->launches += 1;
     }
-    MB_TRY(half(qh, v_full, true));
+    MB_TRY(half(qh, true, v_full, true));
     if (blobs) {
-        // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})  (the mean of a field with itself)
-        MB_CUDA(launch_interp<R>(st, 2, ctx->nb, qh, q, v_full, v_full, box_of, g, ctx->d.dt,
-                                 nullptr, q));
+        // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})
+        MB_CUDA(launch_interp<double>(st, 2, ctx->nb, qh, q, v_full, nullptr, box_of, g, ctx->d.dt,
+                                      nullptr, q));
         ctx->launches += 1;
     }
     mark(NUM_STAGES);
     if (ctx->timing) ctx->ev_pending++;
-    ctx->steps_taken++;
     return MB_OK;
+}
+
+mb_status enqueue_step64(mb_ctx* ctx, const double* ext, const double* body)
+{
+    return ctx->d.integrator == 1 ? do_step_stokes64(ctx, ext, body) : do_step64(ctx, ext, body);
+}
+
+// Host-side state after an FP64 step has been enqueued (directly or as a graph replay).
+void finish_step64(mb_ctx* ctx)
+{
+    if (ctx->d.integrator == 0) ctx->cur ^= 1;
+    ctx->steps_taken++;
 }
 
 // One time step of every box in FP32-grid mode: blob positions as bin cell + float-float
@@ -1425,7 +1417,7 @@ mb_status autotune_spread(mb_ctx* ctx)
     return MB_OK;
 }
 
-// Captures one FP32-grid step from the current velocity buffer into a CUDA graph (on a private
+// Captures one step from the current velocity buffer into a CUDA graph (on a private
 // stream; nothing executes during the capture).
 mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
 {
@@ -1437,14 +1429,17 @@ mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
     cudaStream_t user = ctx->st;
     const int64_t steps0 = ctx->steps_taken, l0 = ctx->launches;
     const int hcur0 = ctx->hcur, hlast0 = ctx->hlast;
-    const bool ready0 = ctx->pred_ready, fz0 = ctx->f_zero;
+    const bool ready0 = ctx->pred_ready, fz0 = ctx->f_zero, sorted0 = ctx->sorted_valid;
     ctx->st = ctx->cap_stream;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(ctx->st, cudaStreamCaptureModeThreadLocal);
     mb_status s = MB_OK;
     if (e == cudaSuccess) {
-        s = ctx->d.integrator == 1 ? do_step_stokes_fast(ctx, ext, body)
-                                   : do_step_fast(ctx, ext, body);
+        if (ctx->rsz == 8)
+            s = enqueue_step64(ctx, ext ? static_cast<const double*>(ctx->ext.p) : nullptr, body);
+        else
+            s = ctx->d.integrator == 1 ? do_step_stokes_fast(ctx, ext, body)
+                                       : do_step_fast(ctx, ext, body);
         e = cudaStreamEndCapture(ctx->st, &graph);
     }
     ctx->st = user;
@@ -1453,7 +1448,9 @@ mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
     ctx->hcur = hcur0;
     ctx->hlast = hlast0;
     ctx->pred_ready = ready0;
+    ctx->graph_fz_after = ctx->f_zero;
     ctx->f_zero = fz0;
+    ctx->sorted_valid = sorted0;
     ctx->graph_launches = ctx->launches - l0;
     ctx->launches = l0;
     if (s != MB_OK) {
@@ -1528,6 +1525,30 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
         ctx->f_zero = false;
         ctx->sorted_valid = true;
         ctx->steps_taken++;
+        ctx->launches += ctx->graph_launches;
+    }
+    return MB_OK;
+}
+
+// n_steps FP64 steps: the first two after a rebuild launched directly (a capture costs as much
+// as a few steps), then replays of the captured graph of each velocity-buffer parity.
+mb_status run_steps64(mb_ctx* ctx, int n_steps, const double* ext, const double* body)
+{
+    const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0;
+    for (int s = 0; s < n_steps; ++s) {
+        if (!graphs || ctx->direct64 < 2) {
+            MB_TRY(enqueue_step64(ctx, ext, body));
+            finish_step64(ctx);
+            ctx->direct64++;
+            continue;
+        }
+        const int c = ctx->cur;
+        if (!ctx->graph_exec[c] || ctx->graph_ext[c] != (ext != nullptr) ||
+            ctx->graph_body[c] != (body != nullptr) || ctx->graph_fz[c] != ctx->f_zero)
+            MB_TRY(capture_graph(ctx, ext != nullptr, body));
+        MB_CUDA(cudaGraphLaunch(ctx->graph_exec[c], ctx->st));
+        finish_step64(ctx);
+        ctx->f_zero = ctx->graph_fz_after;
         ctx->launches += ctx->graph_launches;
     }
     return MB_OK;
@@ -1640,68 +1661,18 @@ void release(mb_ctx* ctx)
                    &ctx->adj_rest, &ctx->part_start, &ctx->part_blobs, &ctx->box_off,
                    &ctx->box_par, &ctx->cell_count, &ctx->cell_start, &ctx->blob_cell,
                    &ctx->blob_rank, &ctx->sorted, &ctx->loc, &ctx->scan_tmp, &ctx->partial,
-                   &ctx->staging_in, &ctx->staging_out, &ctx->mean_scratch, &ctx->s_q,
-                   &ctx->s_F, &ctx->s_rec, &ctx->s_cell_count, &ctx->s_cell_start,
-                   &ctx->s_blob_cell, &ctx->s_blob_rank, &ctx->s_sorted, &ctx->s_scan,
-                   &ctx->s_u, &ctx->s_g0, &ctx->s_g1, &ctx->s_g2, &ctx->s_out, &ctx->sA,
+                   &ctx->staging_in, &ctx->staging_out, &ctx->mean_scratch, 
+                   &ctx->s_F, &ctx->s_g0, &ctx->s_g1, &ctx->s_g2, &ctx->s_out, &ctx->sA,
                    &ctx->sB, &ctx->hA[0], &ctx->hA[1], &ctx->hB[0], &ctx->hB[1], &ctx->F32, &ctx->rec32, &ctx->ext32,
-                   &ctx->ext_sum, &ctx->ext_ticket, &ctx->adj32, &ctx->adj32_start, &ctx->tmpl32, &ctx->tstart32, &ctx->Fpre64, &ctx->Fs32, &ctx->u32, &ctx->a_qn, &ctx->a_u, &ctx->a_qh,
-                   &ctx->a_gq, &ctx->a_guc, &ctx->a_gqh, &ctx->a_gF, &ctx->a_gu, &ctx->a_gk, &ctx->a_gU,
-                   &ctx->a_vn, &ctx->a_vp, &ctx->a_w, &ctx->a_gw, &ctx->a_gvp, &ctx->a_gvn,
-                   &ctx->a_gf, &ctx->a_tmp, &ctx->a_zero, &ctx->W, &ctx->step_index,
+                   &ctx->ext_sum, &ctx->ext_ticket, &ctx->adj32, &ctx->adj32_start, &ctx->tmpl32, &ctx->tstart32, &ctx->Fpre64, &ctx->Fs32, &ctx->u32, &ctx->a_qn, &ctx->a_qh,
+                   &ctx->a_gq, &ctx->a_gqh, &ctx->a_gF, &ctx->a_gu, &ctx->a_gk, &ctx->a_gU,
+                   &ctx->a_vn, &ctx->a_vp, &ctx->a_gvp, &ctx->a_gvn,
+                   &ctx->a_gf, &ctx->W, &ctx->step_index,
                    &ctx->twk[0], &ctx->twk[1], &ctx->twk[2], &ctx->symk};
     for (DBuf* b : all) dfree(*b);
     for (cudaEvent_t& e : ctx->ev_ring)
         if (e) cudaEventDestroy(e);
     ctx->ev_ring.clear();
-}
-
-// Standalone spreading of n blobs into one box grid `out_dev` (device pointer).
-template <typename R>
-mb_status standalone_spread(mb_ctx* ctx, int64_t n, const double* qd, const double* Fd,
-                            R* out_dev)
-{
-    cudaStream_t st = ctx->st;
-    std::string& E = ctx->err;
-    BinGeo bg = ctx->bg;
-    // standalone operators bin with the default cell size
-    {
-        int bs = 2;
-        const int nmin = std::min(ctx->g.n[0], std::min(ctx->g.n[1], ctx->g.n[2]));
-        if (bs > nmin) bs = nmin;
-        bg.bs = bs;
-        for (int a = 0; a < 3; ++a) bg.nc[a] = ctx->g.n[a] / bs;
-        bg.ncell = (int64_t)bg.nc[0] * bg.nc[1] * bg.nc[2];
-        bg.inv_w = 1.0 / (bs * ctx->d.h);
-        set_float_geo(bg);
-    }
-    MB_TRY(ensure(ctx->s_q, sizeof(double) * 3 * n, E, "spread q"));
-    MB_TRY(ensure(ctx->s_rec, sizeof(double) * 6 * n, E, "spread rec"));
-    MB_TRY(ensure(ctx->s_cell_count, sizeof(int32_t) * bg.ncell, E, "spread cells"));
-    MB_TRY(ensure(ctx->s_cell_start, sizeof(int32_t) * (bg.ncell + 1), E, "spread cells"));
-    MB_TRY(ensure(ctx->s_blob_cell, sizeof(int32_t) * n, E, "spread cells"));
-    MB_TRY(ensure(ctx->s_blob_rank, sizeof(int32_t) * n, E, "spread cells"));
-    MB_TRY(ensure(ctx->s_sorted, sizeof(int32_t) * n, E, "spread cells"));
-    MB_TRY(ensure(ctx->s_scan, sizeof(int32_t) * (bg.ncell / 4096 + 2), E, "spread scan"));
-    double* q = static_cast<double*>(ctx->s_q.p);
-    if (n > 0) {
-        MB_CUDA(cudaMemcpyAsync(q, qd, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, st));
-        k_wrap<<<(unsigned)((3 * n + 255) / 256), 256, 0, st>>>(n, q, ctx->g.L[0], ctx->g.L[1],
-                                                                ctx->g.L[2]);
-        MB_CUDA(cudaGetLastError());
-    }
-    MB_CUDA(launch_bin(st, n, q, nullptr, 1, bg, static_cast<int32_t*>(ctx->s_cell_count.p),
-                       static_cast<int32_t*>(ctx->s_cell_start.p),
-                       static_cast<int32_t*>(ctx->s_blob_cell.p),
-                       static_cast<int32_t*>(ctx->s_blob_rank.p),
-                       static_cast<int32_t*>(ctx->s_sorted.p),
-                       static_cast<int32_t*>(ctx->s_scan.p), ctx->d.deterministic != 0));
-    MB_CUDA(launch_make_rec(st, n, static_cast<const int32_t*>(ctx->s_sorted.p), q, Fd,
-                            static_cast<double*>(ctx->s_rec.p)));
-    MB_CUDA(launch_spread<R>(st, 1, static_cast<const double*>(ctx->s_rec.p),
-                             static_cast<const int32_t*>(ctx->s_cell_start.p), ctx->g, bg,
-                             ctx->tile, out_dev));
-    return MB_OK;
 }
 
 }  // namespace
@@ -1931,9 +1902,12 @@ mb_status mb_step(mb_ctx* ctx, int n_steps, const double* ext_blob_force,
     if (n_steps < 0) return invalid(ctx, "n_steps must be >= 0");
     MB_TRY(ensure_ready(ctx));
     if (body_force) {
+        // captured steps hold the profile's buffer, axis and wave direction
         const void* before = ctx->body_prof.p;
+        const double axis = ctx->body_cached[1], dir = ctx->body_cached[2];
         MB_TRY(set_body(ctx, body_force, ctx->body_prof, true));
-        if (ctx->body_prof.p != before) drop_graph(ctx);   // captured steps hold the old buffer
+        if (ctx->body_prof.p != before || ctx->body_cached[1] != axis || ctx->body_cached[2] != dir)
+            drop_graph(ctx);
     }
     const double* ext = nullptr;
     if (ctx->d.integrator == 1 && ctx->rsz == 4) {
@@ -1963,8 +1937,7 @@ mb_status mb_step(mb_ctx* ctx, int n_steps, const double* ext_blob_force,
                                         cudaMemcpyDeviceToDevice, ctx->st));
             ext = static_cast<const double*>(ctx->ext.p);
         }
-        for (int s = 0; s < n_steps; ++s) MB_TRY(do_step_stokes<double>(ctx, ext, body_force));
-        return MB_OK;
+        return run_steps64(ctx, n_steps, ext, body_force);
     }
     if (ext_blob_force && ctx->nb > 0) {
         const void* src = nullptr;
@@ -2000,8 +1973,7 @@ mb_status mb_step(mb_ctx* ctx, int n_steps, const double* ext_blob_force,
         ctx->ext_src = nullptr;
         return st;
     }
-    for (int s = 0; s < n_steps; ++s) MB_TRY(do_step<double>(ctx, ext, body_force));
-    return MB_OK;
+    return run_steps64(ctx, n_steps, ext, body_force);
 }
 
 mb_status mb_get_forces(mb_ctx* ctx, double* blob_force, double* midpoint_pos)
@@ -2119,24 +2091,60 @@ mb_status mb_set_positions(mb_ctx* ctx, const double* pos)
     ctx->sorted_valid = false;
     ctx->pred_ready = false;
     ctx->steps_taken = 0;
-    MB_CUDA(cudaStreamSynchronize(ctx->st));
     return MB_OK;
 }
 
 namespace {
 
-// Copies a caller array (host or device) into a device scratch buffer.
-mb_status pull(mb_ctx* ctx, DBuf& dst, const void* src, size_t bytes, const char* what)
+// A caller array as device memory of this context: itself when it is there, otherwise (host
+// memory, another GPU) a copy in buf.
+mb_status pull(mb_ctx* ctx, DBuf& buf, const void* src, size_t bytes, const char* what,
+               const double** out)
 {
-    MB_TRY(ensure(dst, bytes, ctx->err, what));
-    MB_CUDA(cudaMemcpyAsync(dst.p, src, bytes, cudaMemcpyDefault, ctx->st));
+    cudaPointerAttributes at;
+    const bool known = cudaPointerGetAttributes(&at, src) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (known && (at.type == cudaMemoryTypeManaged ||
+                  (at.type == cudaMemoryTypeDevice && at.device == ctx->device))) {
+        *out = static_cast<const double*>(src);
+        return MB_OK;
+    }
+    MB_TRY(ensure(buf, bytes, ctx->err, what));
+    MB_CUDA(cudaMemcpyAsync(buf.p, src, bytes, cudaMemcpyDefault, ctx->st));
+    *out = static_cast<const double*>(buf.p);
     return MB_OK;
 }
 
-// Copies a device scratch buffer back to a caller array (host or device).
-mb_status push(mb_ctx* ctx, void* dst, const DBuf& src, size_t bytes)
+// An array that a call reads and overwrites: used in place where pull would, unless it shares
+// bytes with one of the call's inputs; then a copy in buf that push returns.
+struct Span {
+    const void* p;
+    size_t bytes;
+};
+mb_status pull_inout(mb_ctx* ctx, DBuf& buf, void* p, size_t bytes, const char* what,
+                     const std::vector<Span>& inputs, double** out)
 {
-    MB_CUDA(cudaMemcpyAsync(dst, src.p, bytes, cudaMemcpyDefault, ctx->st));
+    const double* dev = nullptr;
+    bool shared = false;
+    for (const Span& s : inputs)
+        if (s.p)
+            shared = shared || ((const char*)p < (const char*)s.p + s.bytes &&
+                                (const char*)s.p < (const char*)p + bytes);
+    if (!shared) MB_TRY(pull(ctx, buf, p, bytes, what, &dev));
+    if (shared) {
+        MB_TRY(ensure(buf, bytes, ctx->err, what));
+        MB_CUDA(cudaMemcpyAsync(buf.p, p, bytes, cudaMemcpyDefault, ctx->st));
+        dev = static_cast<const double*>(buf.p);
+    }
+    *out = const_cast<double*>(dev);
+    return MB_OK;
+}
+
+// Copies a result back to the caller's array unless it was computed there.
+mb_status push(mb_ctx* ctx, void* dst, const double* src, size_t bytes)
+{
+    if (src == dst) return MB_OK;
+    MB_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, ctx->st));
     if (!is_device_ptr(dst)) MB_CUDA(cudaStreamSynchronize(ctx->st));
     return MB_OK;
 }
@@ -2148,20 +2156,6 @@ mb_status adjoint_preconditions(mb_ctx* ctx)
     return ensure_ready(ctx);
 }
 
-// gq += G(q; v, gu) and gv += h^3 S(q) gu (the transpose of u = J(q) v), all on device buffers.
-mb_status velocity_adjoint_dev(mb_ctx* ctx, const double* q, const double* v, const double* gu,
-                               double* gq, double* gv)
-{
-    const int64_t n3N = 3 * ctx->g.N;
-    const double h3 = ctx->d.h * ctx->d.h * ctx->d.h;
-    MB_CUDA(launch_grad_interp(ctx->st, ctx->nb, q, v, gu, ctx->g, 1.0, gq));
-    MB_TRY(ensure(ctx->a_tmp, sizeof(double) * n3N, ctx->err, "adjoint grid"));
-    double* tmp = static_cast<double*>(ctx->a_tmp.p);
-    MB_TRY(standalone_spread<double>(ctx, ctx->nb, q, gu, tmp));
-    MB_CUDA(launch_axpby(ctx->st, n3N, 1.0, gv, h3, tmp, gv));
-    return MB_OK;
-}
-
 }  // namespace
 
 mb_status mb_velocity_adjoint(mb_ctx* ctx, const double* pos, const void* grid_v,
@@ -2171,23 +2165,18 @@ mb_status mb_velocity_adjoint(mb_ctx* ctx, const double* pos, const void* grid_v
     DeviceGuard dg(ctx->device);
     if (!pos || !grid_v || !grad_u || !grad_pos || !grad_v) return invalid(ctx, "null argument");
     MB_TRY(adjoint_preconditions(ctx));
-    const int64_t nb = ctx->nb;
-    const size_t bv = sizeof(double) * 3 * nb, bg = sizeof(double) * 3 * ctx->g.N;
-    MB_TRY(pull(ctx, ctx->a_qn, pos, bv, "adjoint q"));
-    MB_TRY(pull(ctx, ctx->a_vn, grid_v, bg, "adjoint v"));
-    MB_TRY(pull(ctx, ctx->a_gu, grad_u, bv, "adjoint gu"));
-    MB_TRY(pull(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq"));
-    MB_TRY(pull(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv"));
-    double* q = static_cast<double*>(ctx->a_qn.p);
-    k_wrap<<<(unsigned)((3 * nb + 255) / 256), 256, 0, ctx->st>>>(nb, q, ctx->g.L[0], ctx->g.L[1],
-                                                                 ctx->g.L[2]);
-    MB_CUDA(cudaGetLastError());
-    MB_TRY(velocity_adjoint_dev(ctx, q, static_cast<const double*>(ctx->a_vn.p),
-                                static_cast<const double*>(ctx->a_gu.p),
-                                static_cast<double*>(ctx->a_gq.p),
-                                static_cast<double*>(ctx->a_gvn.p)));
-    MB_TRY(push(ctx, grad_pos, ctx->a_gq, bv));
-    return push(ctx, grad_v, ctx->a_gvn, bg);
+    const size_t bv = sizeof(double) * 3 * ctx->nb, bg = sizeof(double) * 3 * ctx->g.N;
+    const std::vector<Span> in{{pos, bv}, {grid_v, bg}, {grad_u, bv}};
+    const double *q, *v, *gu;
+    double *gq, *gv;
+    MB_TRY(pull(ctx, ctx->a_qn, pos, bv, "adjoint q", &q));
+    MB_TRY(pull(ctx, ctx->a_vn, grid_v, bg, "adjoint v", &v));
+    MB_TRY(pull(ctx, ctx->a_gu, grad_u, bv, "adjoint gu", &gu));
+    MB_TRY(pull_inout(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq", in, &gq));
+    MB_TRY(pull_inout(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv", in, &gv));
+    MB_CUDA(launch_adjoint_velocity(ctx->st, ctx->nb, q, v, gu, 1.0, gq, nullptr, ctx->g, gq, gv));
+    MB_TRY(push(ctx, grad_pos, gq, bv));
+    return push(ctx, grad_v, gv, bg);
 }
 
 mb_status mb_particle_velocity_adjoint(mb_ctx* ctx, const double* pos, const void* grid_v,
@@ -2197,30 +2186,26 @@ mb_status mb_particle_velocity_adjoint(mb_ctx* ctx, const double* pos, const voi
     DeviceGuard dg(ctx->device);
     if (!pos || !grid_v || !grad_U || !grad_pos || !grad_v) return invalid(ctx, "null argument");
     MB_TRY(adjoint_preconditions(ctx));
-    const int64_t nb = ctx->nb, np = ctx->np;
-    const size_t bv = sizeof(double) * 3 * nb, bg = sizeof(double) * 3 * ctx->g.N;
-    MB_TRY(pull(ctx, ctx->a_qn, pos, bv, "adjoint q"));
-    MB_TRY(pull(ctx, ctx->a_vn, grid_v, bg, "adjoint v"));
-    MB_TRY(pull(ctx, ctx->a_gU, grad_U, sizeof(double) * 3 * (np > 0 ? np : 1), "adjoint gU"));
-    MB_TRY(pull(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq"));
-    MB_TRY(pull(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv"));
+    const int64_t np = ctx->np;
+    const size_t bv = sizeof(double) * 3 * ctx->nb, bg = sizeof(double) * 3 * ctx->g.N,
+                 bU = sizeof(double) * 3 * (np > 0 ? np : 1);
+    const std::vector<Span> in{{pos, bv}, {grid_v, bg}, {grad_U, bU}};
+    const double *q, *v, *gU;
+    double *gq, *gv;
+    MB_TRY(pull(ctx, ctx->a_qn, pos, bv, "adjoint q", &q));
+    MB_TRY(pull(ctx, ctx->a_vn, grid_v, bg, "adjoint v", &v));
+    MB_TRY(pull(ctx, ctx->a_gU, grad_U, bU, "adjoint gU", &gU));
+    MB_TRY(pull_inout(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq", in, &gq));
+    MB_TRY(pull_inout(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv", in, &gv));
     MB_TRY(ensure(ctx->a_gu, bv, ctx->err, "adjoint gu"));
-    MB_CUDA(cudaMemsetAsync(ctx->a_gu.p, 0, bv, ctx->st));
+    double* gu = static_cast<double*>(ctx->a_gu.p);
+    MB_CUDA(cudaMemsetAsync(gu, 0, bv, ctx->st));
     MB_CUDA(launch_particle_mean_adjoint(ctx->st, np,
                                          static_cast<const int32_t*>(ctx->part_start.p),
-                                         static_cast<const int32_t*>(ctx->part_blobs.p),
-                                         static_cast<const double*>(ctx->a_gU.p),
-                                         static_cast<double*>(ctx->a_gu.p)));
-    double* q = static_cast<double*>(ctx->a_qn.p);
-    k_wrap<<<(unsigned)((3 * nb + 255) / 256), 256, 0, ctx->st>>>(nb, q, ctx->g.L[0], ctx->g.L[1],
-                                                                 ctx->g.L[2]);
-    MB_CUDA(cudaGetLastError());
-    MB_TRY(velocity_adjoint_dev(ctx, q, static_cast<const double*>(ctx->a_vn.p),
-                                static_cast<const double*>(ctx->a_gu.p),
-                                static_cast<double*>(ctx->a_gq.p),
-                                static_cast<double*>(ctx->a_gvn.p)));
-    MB_TRY(push(ctx, grad_pos, ctx->a_gq, bv));
-    return push(ctx, grad_v, ctx->a_gvn, bg);
+                                         static_cast<const int32_t*>(ctx->part_blobs.p), gU, gu));
+    MB_CUDA(launch_adjoint_velocity(ctx->st, ctx->nb, q, v, gu, 1.0, gq, nullptr, ctx->g, gq, gv));
+    MB_TRY(push(ctx, grad_pos, gq, bv));
+    return push(ctx, grad_v, gv, bg);
 }
 
 mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n,
@@ -2238,105 +2223,69 @@ mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n
     if (body_force) MB_TRY(set_body(ctx, body_force, ctx->prof_scratch, false));
     cudaStream_t st = ctx->st;
     const GridGeo& g = ctx->g;
-    const int64_t nb = ctx->nb, n3N = 3 * g.N;
-    const size_t bv = sizeof(double) * 3 * nb, bg = sizeof(double) * n3N;
-    const double h = ctx->d.h, h3 = h * h * h, dt = ctx->d.dt;
+    const int64_t nb = ctx->nb;
+    const size_t bv = sizeof(double) * 3 * nb, bg = sizeof(double) * 3 * g.N;
+    const double dt = ctx->d.dt;
     std::string& E = ctx->err;
     // ---- inputs
-    MB_TRY(pull(ctx, ctx->a_qn, pos_n, bv, "adjoint q"));
-    MB_TRY(pull(ctx, ctx->a_vn, grid_v_n, bg, "adjoint v"));
-    MB_TRY(pull(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq"));
-    MB_TRY(pull(ctx, ctx->a_gvp, grad_v, bg, "adjoint gv"));   // becomes dL/dv^{n+1} + gw/2
-    const double* ext = nullptr;
-    if (ext_blob_force && nb > 0) {
-        MB_TRY(pull(ctx, ctx->ext, ext_blob_force, bv, "adjoint ext"));
-        ext = static_cast<const double*>(ctx->ext.p);
+    const bool has_ext = ext_blob_force && nb > 0;
+    const std::vector<Span> in{{pos_n, bv}, {grid_v_n, bg},
+                               {has_ext ? ext_blob_force : nullptr, bv}};
+    const double *qn, *vn, *ext = nullptr;
+    double *gq, *gv;
+    MB_TRY(pull(ctx, ctx->a_qn, pos_n, bv, "adjoint q", &qn));
+    MB_TRY(pull(ctx, ctx->a_vn, grid_v_n, bg, "adjoint v", &vn));
+    if (has_ext) MB_TRY(pull(ctx, ctx->ext, ext_blob_force, bv, "adjoint ext", &ext));
+    MB_TRY(pull_inout(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq", in, &gq));
+    MB_TRY(pull_inout(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv", in, &gv));
+    for (DBuf* b : {&ctx->a_qh, &ctx->a_gqh, &ctx->a_gF}) MB_TRY(ensure(*b, bv, E, "adjoint blobs"));
+    for (DBuf* b : {&ctx->a_vp, &ctx->a_gf}) MB_TRY(ensure(*b, bg, E, "adjoint grids"));
+    // dL/dk: added straight to device memory of this context, through a device scalar otherwise
+    double* gk_dev = nullptr;
+    bool gk_host = false;
+    if (grad_k_spring) {
+        MB_TRY(ensure(ctx->a_gk, sizeof(double), E, "adjoint gk"));
+        const double* p = nullptr;
+        MB_TRY(pull(ctx, ctx->a_gk, grad_k_spring, sizeof(double), "adjoint gk", &p));
+        gk_host = p != grad_k_spring;
+        gk_dev = const_cast<double*>(p);
     }
-    for (DBuf* b : {&ctx->a_u, &ctx->a_qh, &ctx->a_guc, &ctx->a_gqh, &ctx->a_gF, &ctx->a_gu})
-        MB_TRY(ensure(*b, bv, E, "adjoint blobs"));
-    for (DBuf* b : {&ctx->a_vp, &ctx->a_w, &ctx->a_gw, &ctx->a_gvn, &ctx->a_gf, &ctx->a_tmp,
-                    &ctx->a_zero})
-        MB_TRY(ensure(*b, bg, E, "adjoint grids"));
-    MB_TRY(ensure(ctx->a_gk, sizeof(double), E, "adjoint gk"));
-    MB_CUDA(cudaMemsetAsync(ctx->a_zero.p, 0, bg, st));
-    MB_CUDA(cudaMemsetAsync(ctx->a_gk.p, 0, sizeof(double), st));
-    MB_CUDA(cudaMemsetAsync(ctx->a_gqh.p, 0, bv, st));
-    double* qn = static_cast<double*>(ctx->a_qn.p);
     double* qh = static_cast<double*>(ctx->a_qh.p);
-    double* vn = static_cast<double*>(ctx->a_vn.p);
     double* vp = static_cast<double*>(ctx->a_vp.p);
-    double* w = static_cast<double*>(ctx->a_w.p);
-    double* f = static_cast<double*>(ctx->f.p);
-    double* gq = static_cast<double*>(ctx->a_gq.p);
     double* gqh = static_cast<double*>(ctx->a_gqh.p);
-    double* guc = static_cast<double*>(ctx->a_guc.p);
     double* gF = static_cast<double*>(ctx->a_gF.p);
-    double* gu = static_cast<double*>(ctx->a_gu.p);
-    double* gw = static_cast<double*>(ctx->a_gw.p);
-    double* gvp = static_cast<double*>(ctx->a_gvp.p);
-    double* gvn = static_cast<double*>(ctx->a_gvn.p);
     double* gf = static_cast<double*>(ctx->a_gf.p);
-    double* tmp = static_cast<double*>(ctx->a_tmp.p);
-    double* F = static_cast<double*>(ctx->F.p);
-    k_wrap<<<(unsigned)((3 * nb + 255) / 256), 256, 0, st>>>(nb, qn, g.L[0], g.L[1], g.L[2]);
-    MB_CUDA(cudaGetLastError());
+    const double* F = static_cast<const double*>(ctx->F.p);
     const BoxData& bx = ctx->boxes[0];
-    // ---- recompute the step: u^n, q^{n+1/2}, F, f, v^{n+1}, w = (v^n + v^{n+1})/2
-    MB_CUDA(launch_interp<double>(st, 1, nb, qn, nullptr, vn, nullptr, nullptr, g, dt,
-                                  static_cast<double*>(ctx->a_u.p), qh));
-    MB_CUDA(launch_bin(st, nb, qh, nullptr, 1, ctx->bg, static_cast<int32_t*>(ctx->cell_count.p),
-                       static_cast<int32_t*>(ctx->cell_start.p),
-                       static_cast<int32_t*>(ctx->blob_cell.p),
-                       static_cast<int32_t*>(ctx->blob_rank.p), static_cast<int32_t*>(ctx->sorted.p),
-                       static_cast<int32_t*>(ctx->scan_tmp.p), false,
-                       static_cast<const int32_t*>(ctx->pid.p), static_cast<float4*>(ctx->loc.p)));
-    ForceArgs fa{};
-    fa.box_off = static_cast<const int64_t*>(ctx->box_off.p);
-    fa.sorted = static_cast<const int32_t*>(ctx->sorted.p);
-    fa.q = qh;
-    fa.pid = static_cast<const int32_t*>(ctx->pid.p);
-    fa.adj_start = static_cast<const int32_t*>(ctx->adj_start.p);
-    fa.adj_j = static_cast<const int32_t*>(ctx->adj_j.p);
-    fa.adj_rest = static_cast<const double*>(ctx->adj_rest.p);
-    fa.box_par = static_cast<const double*>(ctx->box_par.p);
-    fa.cell_start = static_cast<const int32_t*>(ctx->cell_start.p);
-    fa.blob_cell = static_cast<const int32_t*>(ctx->blob_cell.p);
-    fa.ext = ext;
-    fa.loc = static_cast<const float4*>(ctx->loc.p);
-    fa.F = F;
-    fa.rec = static_cast<double*>(ctx->rec.p);
-    fa.partial = static_cast<double*>(ctx->partial.p);
-    fa.nchunk = ctx->nchunk;
-    MB_CUDA(launch_forces(st, 1, ctx->max_box_blobs, fa, g, ctx->bg, true));
-    MB_CUDA(launch_spread<double>(st, 1, static_cast<const double*>(ctx->rec.p),
-                                  static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
-                                  ctx->tile, f));
-    FluidArgs<double> fl = fluid_args<double>(ctx, vn, f, vp, ctx->prof_scratch.p, body_force, nullptr);
-    MB_CUDA(launch_fluid3<double>(st, 1, g, fl));
-    MB_CUDA(launch_axpby(st, n3N, 0.5, vn, 0.5, vp, w));
+    // ---- recompute the step: q^{n+1/2}, F, f, v^{n+1}
+    const BinCount bin = bin_count(ctx);
+    if (ctx->any_rep && nb > 0)
+        MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * ctx->bg.ncell, st));
+    MB_CUDA(launch_interp<double>(st, 1, nb, qn, nullptr, vn, nullptr, nullptr, g, dt, nullptr, qh,
+                                  true, ctx->any_rep ? &bin : nullptr));
+    if (nb > 0) {
+        MB_TRY(forces64(ctx, qh, ext, true, true, false, [](int) {}));
+        MB_TRY(spread64(ctx, qh, false));
+    }
+    MB_TRY(fluid64(ctx, 1,
+                   fluid_args<double>(ctx, vn, nb > 0 ? ctx->f.p : nullptr, vp,
+                                      ctx->prof_scratch.p, body_force, nullptr),
+                   nb > 0, nullptr));
     // ---- backward
-    // corrector q^{n+1} = q^n + dt J(q^{n+1/2}) w
-    MB_CUDA(launch_axpby(st, 3 * nb, dt, gq, 0.0, nullptr, guc));
-    MB_CUDA(launch_make_rec(st, nb, static_cast<const int32_t*>(ctx->sorted.p), qh, guc,
-                            static_cast<double*>(ctx->rec.p)));
-    MB_CUDA(launch_spread<double>(st, 1, static_cast<const double*>(ctx->rec.p),
-                                  static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
-                                  ctx->tile, gw));
-    MB_CUDA(launch_axpby(st, n3N, h3, gw, 0.0, nullptr, gw));                 // gw = J^T guc
-    MB_CUDA(launch_grad_interp(st, nb, qh, w, guc, g, 1.0, gqh));
-    MB_CUDA(launch_axpby(st, n3N, 1.0, gvp, 0.5, gw, gvp));                  // dL/dv^{n+1}
-    // fluid update v^{n+1} = A v^n + T f (A, T symmetric)
-    FluidArgs<double> fa1 = fluid_args<double>(ctx, gvp, nullptr, tmp, nullptr, nullptr, nullptr);
-    MB_CUDA(launch_fluid3<double>(st, 1, g, fa1));                           // A gvp
-    MB_CUDA(launch_axpby(st, n3N, 1.0, tmp, 0.5, gw, gvn));                  // + gw/2
-    FluidArgs<double> fa2 = fluid_args<double>(ctx, ctx->a_zero.p, gvp, gf, nullptr, nullptr, nullptr);
-    MB_CUDA(launch_fluid3<double>(st, 1, g, fa2));                           // T gvp
-    // spreading f = S(q^{n+1/2}) F
-    MB_CUDA(launch_interp<double>(st, 0, nb, qh, nullptr, gf, nullptr, nullptr, g, dt, gF, nullptr));
-    MB_CUDA(launch_axpby(st, 3 * nb, 1.0 / h3, gF, 0.0, nullptr, gF));       // gF = S^T gf
-    MB_CUDA(launch_grad_interp(st, nb, qh, gf, F, g, 1.0 / h3, gqh));
+    // corrector q^{n+1} = q^n + dt J(q^{n+1/2}) (v^n + v^{n+1})/2: half of J^T (dt gq) goes to
+    // dL/dv^{n+1}, half to dL/dv^n
+    MB_CUDA(launch_spread_atomic<double>(st, 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
+    // fluid update v^{n+1} = A v^n + T f (A, T symmetric): gf = T gv, and A gv is a stencil of gf
+    FluidArgs<double> fa = fluid_args<double>(ctx, vn, gv, gf, nullptr, nullptr, nullptr);
+    fa.no_v = 1;
+    if (ctx->fft_passes == 5) MB_CUDA(launch_fluid<double>(st, 1, g, fa));
+    else MB_CUDA(launch_fluid3<double>(st, 1, g, fa));
+    MB_CUDA(launch_viscous_stencil(st, g, gf, ctx->d.rho / dt,
+                                   0.5 * ctx->d.eta * g.inv_h * g.inv_h, gv));
+    MB_CUDA(launch_spread_atomic<double>(st, 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
+    // spreading f = S(q^{n+1/2}) F and the corrector's positions
+    MB_CUDA(launch_adjoint_midpoint(st, nb, qh, gf, F, vn, vp, gq, dt, g, gF, gqh));
     // forces F(q^{n+1/2}; k)
-    double* gk_dev = static_cast<double*>(ctx->a_gk.p);
     MB_CUDA(launch_force_jvp(st, nb, qh, gF, static_cast<const int32_t*>(ctx->pid.p),
                              static_cast<const int32_t*>(ctx->adj_start.p),
                              static_cast<const int32_t*>(ctx->adj_j.p),
@@ -2345,21 +2294,11 @@ mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n
                              static_cast<const int32_t*>(ctx->sorted.p),
                              static_cast<const int32_t*>(ctx->blob_cell.p), g, ctx->bg, gqh, gk_dev));
     // predictor q^{n+1/2} = q^n + dt/2 J(q^n) v^n
-    MB_CUDA(launch_axpby(st, 3 * nb, 1.0, gq, 1.0, gqh, gq));
-    MB_CUDA(launch_axpby(st, 3 * nb, 0.5 * dt, gqh, 0.0, nullptr, gu));
-    MB_TRY(velocity_adjoint_dev(ctx, qn, vn, gu, gq, gvn));
+    MB_CUDA(launch_adjoint_velocity(st, nb, qn, vn, gqh, 0.5 * dt, gq, gqh, g, gq, gv));
     // ---- outputs
-    MB_TRY(push(ctx, grad_pos, ctx->a_gq, bv));
-    MB_TRY(push(ctx, grad_v, ctx->a_gvn, bg));
-    if (grad_k_spring) {
-        double gk = 0.0;
-        MB_CUDA(cudaMemcpyAsync(&gk, gk_dev, sizeof(double), cudaMemcpyDeviceToHost, st));
-        MB_CUDA(cudaStreamSynchronize(st));
-        double prev = 0.0;
-        MB_CUDA(cudaMemcpy(&prev, grad_k_spring, sizeof(double), cudaMemcpyDefault));
-        prev += gk;
-        MB_CUDA(cudaMemcpy(grad_k_spring, &prev, sizeof(double), cudaMemcpyDefault));
-    }
+    MB_TRY(push(ctx, grad_pos, gq, bv));
+    MB_TRY(push(ctx, grad_v, gv, bg));
+    if (gk_host) MB_TRY(push(ctx, grad_k_spring, gk_dev, sizeof(double)));
     ctx->steps_taken = 0;     // the recomputation overwrote the last step's forces
     return MB_OK;
 }
@@ -2444,7 +2383,7 @@ mb_status mb_get_velocities(mb_ctx* ctx, double* blob_vel, double* blob_pos, dou
         MB_TRY(out_target(ctx, particle_U, by, ctx->staging_out, &dst, &host, "particle_U"));
         MB_CUDA(launch_particle_reduce(ctx->st, ctx->np,
                                        static_cast<const int32_t*>(ctx->part_start.p),
-                                       static_cast<const int32_t*>(ctx->part_blobs.p), nullptr,
+                                       static_cast<const int32_t*>(ctx->part_blobs.p),
                                        static_cast<const double*>(ctx->q.p),
                                        static_cast<const double*>(ctx->u.p), ctx->g,
                                        static_cast<double*>(dst), nullptr));
@@ -2475,7 +2414,7 @@ mb_status mb_get_particle_velocities(mb_ctx* ctx, double* particle_U, double* pa
     if (particle_U) MB_TRY(out_target(ctx, particle_U, by, ctx->staging_out, &dU, &hU, "U"));
     if (particle_Omega) MB_TRY(out_target(ctx, particle_Omega, by, ctx->s_out, &dW, &hW, "Omega"));
     MB_CUDA(launch_particle_reduce(ctx->st, ctx->np, static_cast<const int32_t*>(ctx->part_start.p),
-                                   static_cast<const int32_t*>(ctx->part_blobs.p), nullptr,
+                                   static_cast<const int32_t*>(ctx->part_blobs.p),
                                    static_cast<const double*>(ctx->q.p),
                                    static_cast<const double*>(ctx->u.p), ctx->g,
                                    static_cast<double*>(dU), static_cast<double*>(dW)));
@@ -2494,15 +2433,19 @@ mb_status mb_set_velocity_field(mb_ctx* ctx, const void* grid_v)
     MB_TRY(stage_in(ctx, grid_v, by, ctx->staging_in, &src, "grid_v"));
     MB_CUDA(cudaMemcpyAsync(ctx->v[ctx->cur].p, src, by, cudaMemcpyDeviceToDevice, ctx->st));
     ctx->pred_ready = false;              // the next predictor must see the new field
+    if (ctx->d.mean_mode == 1) {
+        MB_CUDA(cudaMemsetAsync(ctx->vbar.p, 0, sizeof(double) * 3 * ctx->B, ctx->st));
+        return MB_OK;
+    }
+    MB_TRY(ensure(ctx->mean_scratch, sizeof(double) * 3 * ctx->B * grid_mean_chunks(ctx->g.N),
+                  ctx->err, "mean"));
+    double* partial = static_cast<double*>(ctx->mean_scratch.p);
     if (ctx->rsz == 4)
         MB_CUDA(launch_grid_mean<float>(ctx->st, ctx->B, ctx->g, static_cast<const float*>(ctx->v[ctx->cur].p),
-                                        static_cast<double*>(ctx->vbar.p), nullptr));
+                                        static_cast<double*>(ctx->vbar.p), partial));
     else
         MB_CUDA(launch_grid_mean<double>(ctx->st, ctx->B, ctx->g, static_cast<const double*>(ctx->v[ctx->cur].p),
-                                         static_cast<double*>(ctx->vbar.p), nullptr));
-    if (ctx->d.mean_mode == 1)
-        MB_CUDA(cudaMemsetAsync(ctx->vbar.p, 0, sizeof(double) * 3 * ctx->B, ctx->st));
-    MB_CUDA(cudaStreamSynchronize(ctx->st));
+                                         static_cast<double*>(ctx->vbar.p), partial));
     return MB_OK;
 }
 
@@ -2520,12 +2463,15 @@ mb_status mb_spread(mb_ctx* ctx, int64_t n, const double* pos, const double* F, 
     void* dst;
     bool host;
     MB_TRY(out_target(ctx, grid_out, by, ctx->s_out, &dst, &host, "grid_out"));
+    const double scale = ctx->g.inv_h * ctx->g.inv_h * ctx->g.inv_h;
     if (ctx->rsz == 4)
-        MB_TRY(standalone_spread<float>(ctx, n, static_cast<const double*>(qd),
-                                        static_cast<const double*>(Fd), static_cast<float*>(dst)));
+        MB_CUDA(launch_spread_atomic<float>(ctx->st, 1, n, static_cast<const double*>(qd),
+                                            static_cast<const double*>(Fd), nullptr, ctx->g,
+                                            static_cast<float*>(dst), false, true, scale));
     else
-        MB_TRY(standalone_spread<double>(ctx, n, static_cast<const double*>(qd),
-                                         static_cast<const double*>(Fd), static_cast<double*>(dst)));
+        MB_CUDA(launch_spread_atomic<double>(ctx->st, 1, n, static_cast<const double*>(qd),
+                                             static_cast<const double*>(Fd), nullptr, ctx->g,
+                                             static_cast<double*>(dst), false, true, scale));
     return finish_out(ctx, grid_out, dst, by, host);
 }
 
@@ -2537,25 +2483,20 @@ mb_status mb_interp(mb_ctx* ctx, int64_t n, const double* pos, const void* grid_
     if (n == 0) return MB_OK;
     const void *qd = nullptr, *vd = nullptr;
     MB_TRY(stage_in(ctx, pos, sizeof(double) * 3 * n, ctx->s_g0, &qd, "pos"));
-    MB_TRY(ensure(ctx->s_q, sizeof(double) * 3 * n, ctx->err, "interp q"));
-    double* q = static_cast<double*>(ctx->s_q.p);
-    MB_CUDA(cudaMemcpyAsync(q, qd, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, ctx->st));
-    k_wrap<<<(unsigned)((3 * n + 255) / 256), 256, 0, ctx->st>>>(n, q, ctx->g.L[0], ctx->g.L[1],
-                                                                  ctx->g.L[2]);
-    MB_CUDA(cudaGetLastError());
     MB_TRY(stage_in(ctx, grid_v, grid_bytes(ctx, 1), ctx->s_g1, &vd, "grid_v"));
     const size_t by = sizeof(double) * 3 * n;
     void* dst;
     bool host;
     MB_TRY(out_target(ctx, u_out, by, ctx->s_out, &dst, &host, "u_out"));
+    const double* q = static_cast<const double*>(qd);
     if (ctx->rsz == 4)
         MB_CUDA(launch_interp<float>(ctx->st, 0, n, q, nullptr, static_cast<const float*>(vd),
                                      nullptr, nullptr, ctx->g, ctx->d.dt,
-                                     static_cast<double*>(dst), nullptr));
+                                     static_cast<double*>(dst), nullptr, true));
     else
         MB_CUDA(launch_interp<double>(ctx->st, 0, n, q, nullptr, static_cast<const double*>(vd),
                                       nullptr, nullptr, ctx->g, ctx->d.dt,
-                                      static_cast<double*>(dst), nullptr));
+                                      static_cast<double*>(dst), nullptr, true));
     return finish_out(ctx, u_out, dst, by, host);
 }
 

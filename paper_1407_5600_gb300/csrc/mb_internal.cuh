@@ -63,25 +63,43 @@ template <> struct C2<double> { using T = double2; };
 // ------------------------------------------------------------------------------------------
 // Launchers (each returns cudaGetLastError() after enqueuing).
 
+// Where blobs are counted into bin cells (a kernel that moves blobs can count them on the way);
+// count null: nowhere.  count must be zero before the first blob.
+struct BinCount {
+    int32_t* count = nullptr;
+    int32_t* blob_cell = nullptr;
+    int32_t* blob_rank = nullptr;
+    BinGeo bg{};
+};
+
 // Interpolation J of one or two grids at blob positions q.
 //   mode 0: u_out = J(q) v0
-//   mode 1: u_out = J(q) v0, q_out = wrap(q + 0.5 dt u)            (predictor)
-//   mode 2: u = J(q) (v0 + v1)/2, q_out = wrap(q_base + dt u), u_out = u if non-null (corrector)
+//   mode 1: u_out = J(q) v0, q_out = wrap(q + 0.5 dt u)            (predictor); with bin, the
+//           blobs are counted into the cells of q_out
+//   mode 2: u = J(q) v with v the mean of v0 and v1 (v0 when v1 is null),
+//           q_out = wrap(q_base + dt u)                            (corrector)
+// wrap (modes 0 and 1): q from anywhere, taken modulo the box.
 template <typename R>
 cudaError_t launch_interp(cudaStream_t st, int mode, int64_t nb, const double* q,
                           const double* q_base, const R* v0, const R* v1,
                           const int32_t* box_of, const GridGeo& g, double dt, double* u_out,
-                          double* q_out);
+                          double* q_out, bool wrap = false, const BinCount* bin = nullptr);
 
-// Cell binning: count, scan, scatter (and per-cell ordering when deterministic).
+// Cell binning: count (unless the blobs are `counted` already), scan, placement (and per-cell
+// ordering when deterministic).  scan_tmp: ncells / 4096 + 2 ints, the ticket among them zero.
 cudaError_t launch_bin(cudaStream_t st, int64_t nb, const double* q, const int32_t* box_of,
-                       int B, const BinGeo& bg, int32_t* cell_count, int32_t* cell_start,
-                       int32_t* blob_cell, int32_t* blob_rank, int32_t* sorted,
-                       int32_t* scan_tmp, bool deterministic, const int32_t* pid = nullptr,
-                       float4* loc = nullptr);
+                       int B, const BinCount& c, int32_t* cell_start, int32_t* sorted,
+                       int32_t* scan_tmp, bool deterministic, const int32_t* pid, float4* loc,
+                       bool counted);
+// The scan of the cell counts (kernels_blob32.cu): count scanned in place within tiles of
+// 2^BIN_SCAN_LOG cells, the tiles' offsets in scan_tmp, the grand total in *total.
+constexpr int BIN_SCAN_LOG = 12;
+cudaError_t launch_bin_scan(cudaStream_t st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
+                            int32_t* total);
 
-// Blob forces at q (springs, repulsion, external) in sorted-slot order; writes F (blob order),
-// rec (sorted order: q, F) and per-(box, block) partial force sums.
+// FP64 blob forces at q (springs, repulsion, external) in sorted-slot order, in the plain
+// operation order without contraction; writes F (blob order), rec (sorted order: q, F) and
+// per-(box, block) partial force sums.  sorted null: blob order and no repulsion.
 struct ForceArgs {
     const int64_t* box_off;    // [B+1]
     const int32_t* sorted;
@@ -96,16 +114,15 @@ struct ForceArgs {
     const double* ext;         // may be null
     const float4* loc;         // [nb] sorted-order cell-local coordinates and particle id
     double* F;
-    double* rec;
-    double* partial;           // [B][nchunk][3]
-    int nchunk;
+    double* rec;               // null: not written
+    double* partial;           // [B][force_chunks][3]
     // [nb][3] external plus spring forces already summed (launch_springs64); null: the kernel
     // sums them from ext and the adjacency lists
     const double* Fpre;
 };
-// precise: FP64 in the plain operation order without contraction (FP64 grid mode).
-cudaError_t launch_forces(cudaStream_t st, int B, int64_t max_box_blobs, const ForceArgs& a,
-                          const GridGeo& g, const BinGeo& bg, bool precise);
+cudaError_t launch_forces(cudaStream_t st, int B, int64_t nb, int64_t max_box_blobs,
+                          const ForceArgs& a, const GridGeo& g, const BinGeo& bg);
+int force_chunks(int64_t nb, int64_t max_box_blobs);     // blocks a box
 
 // FP64 spring forces when every particle shares one bond pattern (m blobs, blob l of particle
 // p is blob p m + l): each bond evaluated once, in the precise FP64 order, by the end the
@@ -125,30 +142,23 @@ cudaError_t launch_springs64(cudaStream_t st, int64_t nb, int m, int slots, cons
 cudaError_t launch_force_sum(cudaStream_t st, int B, int nchunk, const double* partial,
                              double* vbar, double scale, int mean_mode, double* fsum_out);
 
-// Sorted records from arbitrary q, F (standalone spreading).
-cudaError_t launch_make_rec(cudaStream_t st, int64_t nb, const int32_t* sorted, const double* q,
-                            const double* F, double* rec);
-
-// Tile-owner spreading from sorted records.
+// Blob-owner spreading with global atomic adds into f (zeroed by the launcher unless `zeroed`);
+// q, F, box_of in blob order (box_of null: one box); wrap: positions from anywhere; the node
+// sums of weights * F are multiplied by `scale` (1/h^3 for S, 1 for the transpose of J).
 template <typename R>
-cudaError_t launch_spread(cudaStream_t st, int B, const double* rec, const int32_t* cell_start,
-                          const GridGeo& g, const BinGeo& bg, const int tile[3], R* f);
+cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t nb, const double* q,
+                                 const double* F, const int32_t* box_of, const GridGeo& g, R* f,
+                                 bool zeroed, bool wrap, double scale);
 
-// Blob-owner spreading with global atomic adds into f (zeroed by the launcher).
-template <typename R>
-cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t max_box_blobs, const double* rec,
-                                 const int32_t* cell_start, const GridGeo& g, const BinGeo& bg,
-                                 R* f);
-
-// Deterministic FP64 spreading (64-bit fixed-point shared-memory accumulation).
+// Deterministic FP64 spreading from sorted records (64-bit fixed-point shared-memory
+// accumulation); writes every node of f.
 cudaError_t launch_spread_det(cudaStream_t st, int B, const double* rec, const int32_t* cell_start,
                               const GridGeo& g, const BinGeo& bg, const int tile[3], double* f);
 
 // Particle velocities U0, Omega from blob velocities (particle CSR).
 cudaError_t launch_particle_reduce(cudaStream_t st, int64_t np, const int32_t* part_start,
-                                   const int32_t* part_blobs, const int32_t* box_of_part,
-                                   const double* q, const double* u, const GridGeo& g,
-                                   double* U, double* Omega);
+                                   const int32_t* part_blobs, const double* q, const double* u,
+                                   const GridGeo& g, double* U, double* Omega);
 
 // Adjoint of U0 = (1/N_p) sum_i u_i: gu[i] = gU[p(i)] / N_p for every blob of every particle.
 cudaError_t launch_particle_mean_adjoint(cudaStream_t st, int64_t np, const int32_t* part_start,
@@ -271,10 +281,6 @@ cudaError_t launch_fluid_stress(cudaStream_t st, int B, const GridGeo& g, uint64
                                 R* f, bool accumulate, int parts = 3);
 constexpr int STRESS_KERNELS = 2;
 
-// Exclusive scan of n ints into out[0..n] (out[n] = total); tile_tmp holds n/4096 + 2 ints.
-cudaError_t launch_exclusive_scan(cudaStream_t st, const int32_t* in, int32_t* out, int64_t n,
-                                  int32_t* tile_tmp);
-
 // FP32-grid blob pipeline (kernels_blob32.cu): positions as bin cell + float-float offset,
 // A = {hi.xyz, packed cell}, B = {lo.xyz, 0} per blob.
 cudaError_t launch_split(cudaStream_t st, int64_t nb, const double* q, const GridGeo& g,
@@ -361,20 +367,29 @@ cudaError_t launch_vbar_step(cudaStream_t st, int Bx, const double* sum, double 
 cudaError_t launch_forces_to_fp64(cudaStream_t st, int64_t nb, const float4* F, double* out);
 
 // Adjoint kernels (adjoint.cu), FP64.
-cudaError_t launch_grad_interp(cudaStream_t st, int64_t nb, const double* q, const double* w,
-                               const double* c, const GridGeo& g, double scale, double* out);
+// At the midpoints q: gF = h^-3 J gf and gqh = d/dq [<gf, S(q) F> + sum dt gq . J(q) (v0 + v1)/2].
+cudaError_t launch_adjoint_midpoint(cudaStream_t st, int64_t nb, const double* q, const double* gf,
+                                    const double* F, const double* v0, const double* v1,
+                                    const double* gq, double dt, const GridGeo& g, double* gF,
+                                    double* gqh);
+// Transpose of u = J(q) v with gradient scale * gu: out = base (+ base2) + (du/dq)^T, in place if
+// out == base; gv += J(q)^T.  Positions from anywhere.
+cudaError_t launch_adjoint_velocity(cudaStream_t st, int64_t nb, const double* q, const double* v,
+                                    const double* gu, double scale, const double* base,
+                                    const double* base2, const GridGeo& g, double* out, double* gv);
+// out = a x + c (sum of the six neighbours - 6 x), one box grid.
+cudaError_t launch_viscous_stencil(cudaStream_t st, const GridGeo& g, const double* x, double a,
+                                   double c, double* out);
 cudaError_t launch_force_jvp(cudaStream_t st, int64_t nb, const double* q, const double* gF,
                              const int32_t* pid, const int32_t* adj_start, const int32_t* adj_j,
                              const double* adj_rest, double k_spring, double k_rep, double r_cut,
                              const int32_t* cell_start, const int32_t* sorted,
                              const int32_t* blob_cell, const GridGeo& g, const BinGeo& bg,
                              double* out, double* gk);
-cudaError_t launch_axpby(cudaStream_t st, int64_t n, double a, const double* x, double b,
-                         const double* y, double* out);
-
-// Reductions / utilities.
+// Mean of each component grid to mean_out [B][3]; partial: [B][3][grid_mean_chunks(N)].
 template <typename R>
 cudaError_t launch_grid_mean(cudaStream_t st, int B, const GridGeo& g, const R* v,
-                             double* mean_out /*[B][3]*/, double* scratch);
+                             double* mean_out, double* partial);
+int grid_mean_chunks(int64_t N);
 
 }  // namespace mbk
