@@ -87,6 +87,8 @@ k_adjoint_midpoint(int64_t nb, const double* __restrict__ q, const double* __res
                    const double* __restrict__ v1, const double* __restrict__ gq, double dt,
                    GridGeo g, double* __restrict__ gF, double* __restrict__ gqh)
 {
+    dep_wait();
+    dep_release();
     __shared__ double sh[ADJ_THREADS][3];
     const int64_t t = blockIdx.x * (int64_t)ADJ_THREADS + threadIdx.x;
     const int64_t b = t / 3;
@@ -117,6 +119,8 @@ k_adjoint_velocity(int64_t nb, const double* __restrict__ q, const double* __res
                    const double* gu_in, double scale, const double* base, const double* base2,
                    GridGeo g, double* out, double* gv)
 {
+    dep_wait();
+    dep_release();
     __shared__ double sh[ADJ_THREADS][3];
     const int64_t t = blockIdx.x * (int64_t)ADJ_THREADS + threadIdx.x;
     const int64_t b = t / 3;
@@ -158,6 +162,8 @@ k_adjoint_velocity(int64_t nb, const double* __restrict__ q, const double* __res
 __global__ void __launch_bounds__(256)
 k_viscous_stencil(GridGeo g, const double* __restrict__ x, double a, double c, double* __restrict__ out)
 {
+    dep_wait();
+    dep_release();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= 3 * g.N) return;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -189,6 +195,8 @@ k_force_jvp(int64_t nb, const double* __restrict__ q, const double* __restrict__
             const int32_t* __restrict__ sorted, const int32_t* __restrict__ blob_cell,
             GridGeo g, BinGeo bg, double* __restrict__ out, double* __restrict__ gk)
 {
+    dep_wait();
+    dep_release();
     __shared__ double sh[JVP_BLOCK / 32];
     const int lane = threadIdx.x % JVP_LANES;
     double dk = 0.0;
@@ -270,35 +278,32 @@ inline unsigned nblk(int64_t n, int per) { return (unsigned)((n + per - 1) / per
 
 }  // namespace
 
-cudaError_t launch_adjoint_midpoint(cudaStream_t st, int64_t nb, const double* q, const double* gf,
+cudaError_t launch_adjoint_midpoint(Chain st, int64_t nb, const double* q, const double* gf,
                                     const double* F, const double* v0, const double* v1,
                                     const double* gq, double dt, const GridGeo& g, double* gF,
                                     double* gqh)
 {
     if (nb <= 0) return cudaSuccess;
-    k_adjoint_midpoint<<<nblk(nb, ADJ_BLOBS), ADJ_THREADS, 0, st>>>(nb, q, gf, F, v0, v1, gq, dt, g,
+    return launch_on(st, k_adjoint_midpoint, dim3(nblk(nb, ADJ_BLOBS)), dim3(ADJ_THREADS), 0, nb, q, gf, F, v0, v1, gq, dt, g,
                                                                    gF, gqh);
-    return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_velocity(cudaStream_t st, int64_t nb, const double* q, const double* v,
+cudaError_t launch_adjoint_velocity(Chain st, int64_t nb, const double* q, const double* v,
                                     const double* gu, double scale, const double* base,
                                     const double* base2, const GridGeo& g, double* out, double* gv)
 {
     if (nb <= 0) return cudaSuccess;
-    k_adjoint_velocity<<<nblk(nb, ADJ_BLOBS), ADJ_THREADS, 0, st>>>(nb, q, v, gu, scale, base, base2,
+    return launch_on(st, k_adjoint_velocity, dim3(nblk(nb, ADJ_BLOBS)), dim3(ADJ_THREADS), 0, nb, q, v, gu, scale, base, base2,
                                                                    g, out, gv);
-    return cudaGetLastError();
 }
 
-cudaError_t launch_viscous_stencil(cudaStream_t st, const GridGeo& g, const double* x, double a,
+cudaError_t launch_viscous_stencil(Chain st, const GridGeo& g, const double* x, double a,
                                    double c, double* out)
 {
-    k_viscous_stencil<<<nblk(3 * g.N, 256), 256, 0, st>>>(g, x, a, c, out);
-    return cudaGetLastError();
+    return launch_on(st, k_viscous_stencil, dim3(nblk(3 * g.N, 256)), dim3(256), 0, g, x, a, c, out);
 }
 
-cudaError_t launch_force_jvp(cudaStream_t st, int64_t nb, const double* q, const double* gF,
+cudaError_t launch_force_jvp(Chain st, int64_t nb, const double* q, const double* gF,
                              const int32_t* pid, const int32_t* adj_start, const int32_t* adj_j,
                              const double* adj_rest, double k_spring, double k_rep, double r_cut,
                              const int32_t* cell_start, const int32_t* sorted,
@@ -308,10 +313,9 @@ cudaError_t launch_force_jvp(cudaStream_t st, int64_t nb, const double* q, const
     if (nb <= 0) return cudaSuccess;
     // at most 2048 blocks, so that as few atomics meet on gk
     const unsigned blocks = nblk(nb, JVP_BLOCK / JVP_LANES);
-    k_force_jvp<<<blocks < 2048 ? blocks : 2048, JVP_BLOCK, 0, st>>>(
+    return launch_on(st, k_force_jvp, dim3(blocks < 2048 ? blocks : 2048), dim3(JVP_BLOCK), 0, 
         nb, q, gF, pid, adj_start, adj_j, adj_rest, k_spring, k_rep, r_cut, cell_start, sorted,
         blob_cell, g, bg, out, gk);
-    return cudaGetLastError();
 }
 
 }  // namespace mbk

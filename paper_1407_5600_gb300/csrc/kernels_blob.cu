@@ -36,8 +36,8 @@ __device__ __forceinline__ void count_blob(const BinCount& c, int64_t b, int box
     c.blob_rank[b] = atomicAdd(c.count + cell, 1);
 }
 
-// Sum over a blob's 27 nodes of the weights times c0 (+ c1 when not null).
-template <typename R>
+// Sum over a blob's 27 nodes of the weights times c0 (+ c1 with TWO).
+template <bool TWO, typename R>
 __device__ __forceinline__ R window_sum(const R* __restrict__ c0, const R* __restrict__ c1,
                                         const Win<R>& wx, const Win<R>& wy, const Win<R>& wz)
 {
@@ -52,7 +52,7 @@ __device__ __forceinline__ R window_sum(const R* __restrict__ c0, const R* __res
 #pragma unroll
             for (int aa = 0; aa < 3; ++aa) {
                 R val = __ldg(c0 + (row + wx.o[aa]));
-                if (c1) val += __ldg(c1 + (row + wx.o[aa]));
+                if (TWO) val += __ldg(c1 + (row + wx.o[aa]));
                 r += wx.w[aa] * val;
             }
             // FP64: products summed by rows and planes (39 instructions instead of 45)
@@ -67,23 +67,26 @@ __device__ __forceinline__ R window_sum(const R* __restrict__ c0, const R* __res
 // Interpolation J (Eq. ju): u_a = sum over the 3x3x3 window of Phi Phi Phi v_a(node), each
 // component on its own staggered grid.  One thread per blob, its windows at both MAC shifts
 // computed once per dimension (6 instead of 9); with SPLIT one per blob and component, three
-// windows each.  v1 = null: v0 alone; otherwise the mean of v0 and v1.  WRAP: positions from
-// anywhere (standalone calls).  With `count` the new position is counted into its bin cell.
+// windows each.  TWO: the sum of v0 and v1, otherwise v0 alone, times `scale`.  WRAP: positions from
+// anywhere.  With `count` the new position is counted into its bin cell.
 struct InterpArgs {
     int64_t nb;
     const double* q;
     const double* q_base;
     const int32_t* box_of;
     double dt;
+    double scale;              // of the gathered sums
     double* u_out;
     double* q_out;
     BinCount bin;
 };
 
-template <typename R, int MODE, bool SPLIT, bool WRAP>
+template <typename R, int MODE, bool SPLIT, bool WRAP, bool TWO>
 __global__ void __launch_bounds__(128)
 k_interp(InterpArgs a, const R* __restrict__ v0, const R* __restrict__ v1, GridGeo g)
 {
+    dep_wait();
+    dep_release();
     __shared__ double moved[MODE == 1 && SPLIT ? 96 : 1];       // [32 blobs][3]
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t b = SPLIT ? t / 3 : t;
@@ -103,15 +106,15 @@ k_interp(InterpArgs a, const R* __restrict__ v0, const R* __restrict__ v1, GridG
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const int mask[3] = {nx - 1, ny - 1, nz - 1}, stride[3] = {1, nx, ny * nx};
     double u[3] = {0.0, 0.0, 0.0};
-    const R half = MODE == 2 && v1 ? R(0.5) : R(1);
+    const double unit = a.scale * Win<R>::UNIT;
     if (SPLIT) {
         Win<R> w[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d)
             w[d].set(p[d] * g.inv_h - (d == mine ? 0.0 : 0.5), mask[d], stride[d]);
         const size_t base = ((size_t)box * 3 + mine) * (size_t)g.N;
-        const R acc = window_sum(v0 + base, v1 ? v1 + base : nullptr, w[0], w[1], w[2]);
-        u[0] = (double)half * (double)acc;
+        const R acc = window_sum<TWO>(v0 + base, TWO ? v1 + base : nullptr, w[0], w[1], w[2]);
+        u[0] = unit * (double)acc;
     } else {
         Win<R> own[3], across[3];
 #pragma unroll
@@ -122,10 +125,10 @@ k_interp(InterpArgs a, const R* __restrict__ v0, const R* __restrict__ v1, GridG
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const size_t base = ((size_t)box * 3 + c) * (size_t)g.N;
-            const R acc = window_sum(v0 + base, v1 ? v1 + base : nullptr,
-                                     c == 0 ? own[0] : across[0], c == 1 ? own[1] : across[1],
-                                     c == 2 ? own[2] : across[2]);
-            u[c] = (double)half * (double)acc;
+            const R acc = window_sum<TWO>(v0 + base, TWO ? v1 + base : nullptr,
+                                          c == 0 ? own[0] : across[0], c == 1 ? own[1] : across[1],
+                                          c == 2 ? own[2] : across[2]);
+            u[c] = unit * (double)acc;
         }
     }
     // position updates round like the plain expression q + (c dt) u (no contraction)
@@ -155,36 +158,40 @@ k_interp(InterpArgs a, const R* __restrict__ v0, const R* __restrict__ v1, GridG
 }
 
 template <typename R>
-cudaError_t launch_interp(cudaStream_t st, int mode, int64_t nb, const double* q,
+cudaError_t launch_interp(Chain st, int mode, int64_t nb, const double* q,
                           const double* q_base, const R* v0, const R* v1,
                           const int32_t* box_of, const GridGeo& g, double dt, double* u_out,
-                          double* q_out, bool wrap, const BinCount* bin)
+                          double* q_out, bool wrap, const BinCount* bin, double scale)
 {
     if (nb <= 0) return cudaSuccess;
-    InterpArgs a{nb, q, q_base, box_of, dt, u_out, q_out, bin ? *bin : BinCount{}};
+    InterpArgs a{nb, q, q_base, box_of, dt, scale, u_out, q_out, bin ? *bin : BinCount{}};
     const bool split = split_components(nb);
     const int T = split ? 96 : blob_block(nb);           // split: 32 blobs a block
     const unsigned blocks = blocks_of(split ? 3 * nb : nb, T);
-    auto go = [&](auto k) { k<<<blocks, T, 0, st>>>(a, v0, mode == 2 ? v1 : nullptr, g); };
+    auto go = [&](auto k) { return launch_on(st, k, dim3(blocks), dim3(T), 0, a, v0, v1, g); };
     if (mode == 0) {
-        if (wrap) split ? go(k_interp<R, 0, true, true>) : go(k_interp<R, 0, false, true>);
-        else split ? go(k_interp<R, 0, true, false>) : go(k_interp<R, 0, false, false>);
-    } else if (mode == 1) {
-        if (wrap) split ? go(k_interp<R, 1, true, true>) : go(k_interp<R, 1, false, true>);
-        else split ? go(k_interp<R, 1, true, false>) : go(k_interp<R, 1, false, false>);
-    } else {
-        split ? go(k_interp<R, 2, true, false>) : go(k_interp<R, 2, false, false>);
+        if (wrap) return split ? go(k_interp<R, 0, true, true, false>) : go(k_interp<R, 0, false, true, false>);
+        return split ? go(k_interp<R, 0, true, false, false>) : go(k_interp<R, 0, false, false, false>);
     }
-    return cudaGetLastError();
+    if constexpr (sizeof(R) == 4) {
+        return cudaErrorInvalidValue;                    // FP32 grids move blobs in kernels_blob32.cu
+    } else {
+        if (mode == 1) {
+            if (wrap) return split ? go(k_interp<R, 1, true, true, false>) : go(k_interp<R, 1, false, true, false>);
+            return split ? go(k_interp<R, 1, true, false, false>) : go(k_interp<R, 1, false, false, false>);
+        }
+        if (v1) return split ? go(k_interp<R, 2, true, false, true>) : go(k_interp<R, 2, false, false, true>);
+        return split ? go(k_interp<R, 2, true, false, false>) : go(k_interp<R, 2, false, false, false>);
+    }
 }
-template cudaError_t launch_interp<float>(cudaStream_t, int, int64_t, const double*,
+template cudaError_t launch_interp<float>(Chain, int, int64_t, const double*,
                                           const double*, const float*, const float*,
                                           const int32_t*, const GridGeo&, double, double*,
-                                          double*, bool, const BinCount*);
-template cudaError_t launch_interp<double>(cudaStream_t, int, int64_t, const double*,
+                                          double*, bool, const BinCount*, double);
+template cudaError_t launch_interp<double>(Chain, int, int64_t, const double*,
                                            const double*, const double*, const double*,
                                            const int32_t*, const GridGeo&, double, double*,
-                                           double*, bool, const BinCount*);
+                                           double*, bool, const BinCount*, double);
 
 // ==========================================================================================
 // Cell binning (counting sort of blobs by bin cell, box-major): counts (by the predictor or
@@ -192,6 +199,8 @@ template cudaError_t launch_interp<double>(cudaStream_t, int, int64_t, const dou
 __global__ void k_bin_count(int64_t nb, const double* __restrict__ q,
                             const int32_t* __restrict__ box_of, BinCount c)
 {
+    dep_wait();
+    dep_release();
     const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const double p[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
@@ -219,6 +228,8 @@ k_bin_place(int64_t nb, int64_t ncells, const int32_t* __restrict__ local,
             int32_t* __restrict__ sorted, const double* __restrict__ q,
             const int32_t* __restrict__ pid, BinGeo bg, float4* __restrict__ loc)
 {
+    dep_wait();
+    dep_release();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < ncells) cell_start[i] = local[i] + tile_off[i >> BIN_SCAN_LOG];
     if (i < nb) {
@@ -235,6 +246,8 @@ __global__ void k_cell_order(int64_t ncells, const int32_t* __restrict__ cell_st
                              int32_t* __restrict__ sorted, const double* __restrict__ q,
                              const int32_t* __restrict__ pid, BinGeo bg, float4* __restrict__ loc)
 {
+    dep_wait();
+    dep_release();
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (c >= ncells) return;
     const int s = cell_start[c], e = cell_start[c + 1];
@@ -247,32 +260,35 @@ __global__ void k_cell_order(int64_t ncells, const int32_t* __restrict__ cell_st
         }
         sorted[j + 1] = key;
     }
-    if (loc)
-        for (int i = s; i < e; ++i) loc[i] = cell_local(sorted[i], (int)c, q, pid, bg);
+    for (int i = s; i < e; ++i) loc[i] = cell_local(sorted[i], (int)c, q, pid, bg);
 }
 
-cudaError_t launch_bin(cudaStream_t st, int64_t nb, const double* q, const int32_t* box_of,
+cudaError_t launch_bin(Chain st, int64_t nb, const double* q, const int32_t* box_of,
                        int B, const BinCount& c, int32_t* cell_start, int32_t* sorted,
-                       int32_t* scan_tmp, bool deterministic, const int32_t* pid, float4* loc,
+                       int32_t* scan_tmp, bool ordered, const int32_t* pid, float4* loc,
                        bool counted)
 {
     const BinGeo& bg = c.bg;
     const int64_t ncells = (int64_t)B * bg.ncell;
     cudaError_t e;
     if (!counted) {
-        e = cudaMemsetAsync(c.count, 0, sizeof(int32_t) * ncells, st);
+        e = cudaMemsetAsync(c.count, 0, sizeof(int32_t) * ncells, st.st);
         if (e != cudaSuccess) return e;
-        if (nb > 0) k_bin_count<<<blocks_of(nb, 256), 256, 0, st>>>(nb, q, box_of, c);
+        if (nb > 0) {
+            e = launch_on(st, k_bin_count, dim3(blocks_of(nb, 256)), dim3(256), 0, nb, q, box_of, c);
+            if (e != cudaSuccess) return e;
+        }
     }
     e = launch_bin_scan(st, c.count, ncells, scan_tmp, cell_start + ncells);
     if (e != cudaSuccess) return e;
-    k_bin_place<<<blocks_of(nb > ncells ? nb : ncells, 256), 256, 0, st>>>(
-        nb, ncells, c.count, scan_tmp, cell_start, c.blob_cell, c.blob_rank, sorted, q, pid, bg,
-        deterministic ? nullptr : loc);
-    if (deterministic)
-        k_cell_order<<<blocks_of(ncells, 256), 256, 0, st>>>(ncells, cell_start, sorted, q, pid, bg,
-                                                             loc);
-    return cudaGetLastError();
+    e = launch_on(st, k_bin_place, dim3(blocks_of(nb > ncells ? nb : ncells, 256)), dim3(256), 0,
+                   nb, ncells, (const int32_t*)c.count, (const int32_t*)scan_tmp, cell_start,
+                   (const int32_t*)c.blob_cell, (const int32_t*)c.blob_rank, sorted, q, pid, bg,
+                   ordered ? (float4*)nullptr : loc);
+    if (e == cudaSuccess && ordered)
+        e = launch_on(st, k_cell_order, dim3(blocks_of(ncells, 256)), dim3(256), 0, ncells,
+                       (const int32_t*)cell_start, sorted, q, pid, bg, loc);
+    return e;
 }
 
 // ==========================================================================================
@@ -303,27 +319,33 @@ __device__ __forceinline__ void block_sum3(double v[3], double* sh /*[3][32]*/)
     }
 }
 
+// The nearer image of a difference beyond half the box.  Not inlined: as predicated instructions
+// its comparisons and additions would take the FP64 pipe for every bond.
+__device__ __noinline__ double other_image(double x, double L)
+{
+    const double half = 0.5 * L;
+    return x > half ? __dsub_rn(x, L) : (x < -half ? __dadd_rn(x, L) : x);
+}
+
 // Spring force on blob b from bond (b, j): -k (|r| - r0) r/|r|, r = q_b - q_j (minimum image),
 // in FP64 with the operations in the plain order and no contraction, so that a blob's spring
 // force is the same bits however the work is scheduled.
-__device__ __forceinline__ void spring_term(const double qb[3], const double* __restrict__ qj,
-                                            double r0, double k, const double L[3], double F[3])
+__device__ __forceinline__ void spring_force(const double* __restrict__ qb,
+                                             const double* __restrict__ qj, double r0, double k,
+                                             const double L[3], double f[3])
 {
     double r[3];
     for (int d = 0; d < 3; ++d) {
         double x = __dsub_rn(qb[d], qj[d]);
         // beyond half the box (by the high words; exactly below): the other image
-        if ((__double2hiint(x) & 0x7fffffff) >= __double2hiint(L[d]) - (1 << 20)) {
-            const double half = 0.5 * L[d];
-            if (x > half) x = __dsub_rn(x, L[d]);
-            else if (x < -half) x = __dadd_rn(x, L[d]);
-        }
+        if ((__double2hiint(x) & 0x7fffffff) >= __double2hiint(L[d]) - (1 << 20))
+            x = other_image(x, L[d]);
         r[d] = x;
     }
     const Length l(__dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])),
                              __dmul_rn(r[2], r[2])));
     const double mag = l.divide(__dmul_rn(-k, __dsub_rn(l.len, r0)));
-    for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], __dmul_rn(mag, r[d]));
+    for (int d = 0; d < 3; ++d) f[d] = __dmul_rn(mag, r[d]);
 }
 
 // Repulsion k_rep (r_cut - |r|) r/|r| for |r| < r_cut, r = q_b - q_j.
@@ -342,71 +364,71 @@ __device__ __forceinline__ void pair_term(const double qb[3], const double* __re
 }
 
 // FP64 springs of a bond pattern shared by all particles (launch_springs64).  A block holds
-// whole particles (one thread per blob, blob order).  Each thread evaluates the bonds its
-// evaluation list names (spring_term on a zero sum: the force on its own blob) into its
-// shared-memory slots; after a barrier it sums ext and, in its adjacency order, its own slots
-// and the negated slots of the bonds its partners evaluated.  Negation is exact and the
-// evaluation of a bond from the other end gives the negated bits, so every sum equals the
-// per-blob adjacency sum of k_forces bit for bit.
+// whole particles.  Their bonds are spread evenly over its threads (an icosahedron's 42 over 13
+// threads' worth: evaluated at the blobs, the fullest one's four set the pace), each evaluated
+// once, as the force on its first end, into shared memory; after a barrier one thread per blob
+// and component sums ext and its bonds in adjacency order, negated where it is the other end.  Negation is
+// exact and the evaluation of a bond from the other end gives the negated bits, so every sum
+// equals the per-blob adjacency sum of k_forces bit for bit.
 __global__ void __launch_bounds__(256)
-k_springs64(int nb, int m, int S, const double* __restrict__ q, const double* __restrict__ ext,
-            const int4* __restrict__ tmpl, const int32_t* __restrict__ tstart,
-            const int32_t* __restrict__ box_of, const double* __restrict__ box_par, GridGeo g,
-            double* __restrict__ Fout)
+k_springs64(int np, int m, int nbond, int ppb, const double* __restrict__ q,
+            const double* __restrict__ ext, const int4* __restrict__ tmpl,
+            const int32_t* __restrict__ tstart, const int32_t* __restrict__ box_of,
+            const double* __restrict__ box_par, GridGeo g, double* __restrict__ Fout)
 {
-    extern __shared__ double slot_d[];                   // [blockDim][S][3]
-    const int tid = threadIdx.x;
-    const int b = blockIdx.x * blockDim.x + tid;
-    const bool live = b < nb;
-    const int l = tid % m;
-    if (live) {
-        const double qb[3] = {q[3 * b], q[3 * b + 1], q[3 * b + 2]};
-        const double k_spring = box_par[3 * (box_of ? box_of[b] : 0)];
-        const int e0 = __ldg(tstart + 2 * l), e1 = __ldg(tstart + 2 * l + 1);
-        for (int e = e0; e < e1; ++e) {
-            const int4 ad = __ldg(tmpl + e);
-            const int j = b + (int)(short)(ad.x & 0xffff);
-            const int slot = (ad.x >> 16) - 1;
-            const double r0 = __hiloint2double(ad.z, ad.y);
-            double f[3] = {0.0, 0.0, 0.0};
-            spring_term(qb, q + 3 * j, r0, k_spring, g.L, f);
-            for (int d = 0; d < 3; ++d) slot_d[(tid * S + slot) * 3 + d] = f[d];
-        }
+    dep_wait();
+    dep_release();
+    extern __shared__ double bond_f[];                   // [ppb][nbond][3]
+    const int p0 = blockIdx.x * ppb, here = min(ppb, np - p0);
+    for (int i = threadIdx.x; i < here * nbond; i += blockDim.x) {
+        const int p = i / nbond;
+        const int4 bd = __ldg(tmpl + (i - p * nbond));
+        const int base = (p0 + p) * m, a = base + (bd.x & 0xffff), b = base + (bd.x >> 16);
+        const double k_spring = box_par[3 * (box_of ? box_of[a] : 0)];
+        spring_force(q + 3 * a, q + 3 * b, __hiloint2double(bd.z, bd.y), k_spring, g.L, bond_f + 3 * i);
     }
     __syncthreads();
-    if (!live) return;
-    double F[3] = {0.0, 0.0, 0.0};
-    if (ext)
-        for (int d = 0; d < 3; ++d) F[d] = ext[3 * b + d];
-    const int c0 = __ldg(tstart + 2 * l + 1), c1 = __ldg(tstart + 2 * l + 2);
-    for (int e = c0; e < c1; ++e) {
-        const int4 ad = __ldg(tmpl + e);
-        const double* v = slot_d + ((tid + ad.x) * S + ad.y) * 3;
-        for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], ad.z > 0 ? v[d] : -v[d]);
+    for (int i = threadIdx.x; i < 3 * here * m; i += blockDim.x) {      // a component of a blob
+        const int j = i / 3, d = i - 3 * j, p = j / m, l = j - p * m;
+        const int64_t at = 3 * (int64_t)p0 * m + i;
+        double F = ext ? ext[at] : 0.0;
+        const int c0 = __ldg(tstart + l), c1 = __ldg(tstart + l + 1);
+        for (int e = c0; e < c1; ++e) {
+            const int4 ad = __ldg(tmpl + e);
+            const double v = bond_f[3 * (p * nbond + ad.x) + d];
+            F = __dadd_rn(F, ad.y > 0 ? v : -v);
+        }
+        Fout[at] = F;
     }
-    for (int d = 0; d < 3; ++d) Fout[3 * b + d] = F[d];
 }
 
-cudaError_t launch_springs64(cudaStream_t st, int64_t nb, int m, int slots, const double* q,
+cudaError_t launch_springs64(Chain st, int64_t nb, int m, int nbond, const double* q,
                              const double* ext, const int4* tmpl, const int32_t* tstart,
                              const int32_t* box_of, const double* box_par, const GridGeo& g,
                              double* Fout)
 {
     if (nb <= 0) return cudaSuccess;
-    // whole particles per block; few blobs in small blocks over more SMs
-    const int most = blob_block(nb) < 128 ? (m > 32 ? m : 32) : 256;
-    const int threads = (most / m) * m;
-    const size_t smem = sizeof(double) * 3 * (size_t)threads * (slots > 0 ? slots : 1);
-    k_springs64<<<(unsigned)((nb + threads - 1) / threads), threads, smem, st>>>(
-        (int)nb, m, slots, q, ext, tmpl, tstart, box_of, box_par, g, Fout);
-    return cudaGetLastError();
+    // about a warp of blobs a block while there are few, eight warps otherwise, within the
+    // 48 KiB of shared memory that need no opt-in (SPRINGS64_MAX_BONDS for one particle)
+    const int most = blob_block(nb) < 128 ? 32 : 256;
+    const int fit = SPRINGS64_MAX_BONDS / (nbond > 0 ? nbond : 1);
+    int ppb = most / m > 1 ? most / m : 1;
+    if (ppb > fit) ppb = fit;
+    const int np = (int)(nb / m);
+    const int threads = most == 32 ? 64 : 256;
+    return launch_on(st, k_springs64, dim3(blocks_of(np, ppb)), dim3(threads),
+                      sizeof(double) * 3 * (size_t)ppb * (nbond > 0 ? nbond : 1), np, m, nbond,
+                      ppb, q, ext, tmpl, tstart, box_of, box_par, g, Fout);
 }
 
 // Blob forces in slot order (blob order without bins: no repulsion then).
 __global__ void __launch_bounds__(256)
 k_forces(ForceArgs a, GridGeo g, BinGeo bg)
 {
+    dep_wait();
+    dep_release();
     __shared__ double sh[96];
+    __shared__ bool last;
     const int box = blockIdx.y;
     const int64_t s0 = a.box_off[box], cnt = a.box_off[box + 1] - s0;
     const int64_t local = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -427,7 +449,11 @@ k_forces(ForceArgs a, GridGeo g, BinGeo bg)
             }
             const double k_spring = a.box_par[3 * box];
             for (int e = a.adj_start[b]; e < a.adj_start[b + 1]; ++e)
-                spring_term(qb, a.q + 3 * a.adj_j[e], a.adj_rest[e], k_spring, g.L, F);
+            {
+                double f[3];
+                spring_force(qb, a.q + 3 * a.adj_j[e], a.adj_rest[e], k_spring, g.L, f);
+                for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], f[d]);
+            }
         }
         if (a.sorted && k_rep != 0.0 && r_cut > 0.0) {
             double Fp[3] = {0.0, 0.0, 0.0};
@@ -486,16 +512,29 @@ k_forces(ForceArgs a, GridGeo g, BinGeo bg)
             for (int d = 0; d < 3; ++d) F[d] = __dadd_rn(F[d], Fp[d]);
         }
         for (int d = 0; d < 3; ++d) a.F[3 * b + d] = F[d];
-        if (a.rec)
-            for (int d = 0; d < 3; ++d) {
-                a.rec[6 * slot + d] = qb[d];
-                a.rec[6 * slot + 3 + d] = F[d];
-            }
     }
+    if (!a.vbar) return;
+    // the net force: one partial sum a block; the last block of the box to finish (atomic ticket
+    // after a fence; no block waits for another) adds them in a fixed order and advances the
+    // mean velocity
     block_sum3(F, sh);
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+        for (int d = 0; d < 3; ++d) a.partial[((int64_t)box * gridDim.x + blockIdx.x) * 3 + d] = F[d];
+        __threadfence();
+        last = atomicAdd(a.ticket + box, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int c = threadIdx.x; c < (int)gridDim.x; c += blockDim.x)
+        for (int d = 0; d < 3; ++d) s[d] += __ldcg(a.partial + ((int64_t)box * gridDim.x + c) * 3 + d);
+    block_sum3(s, sh);
+    if (threadIdx.x == 0) {
         for (int d = 0; d < 3; ++d)
-            a.partial[((int64_t)box * gridDim.x + blockIdx.x) * 3 + d] = F[d];
+            a.vbar[3 * box + d] = a.mean_mode == 0 ? a.vbar[3 * box + d] + a.mean_scale * s[d] : 0.0;
+        a.ticket[box] = 0u;
+    }
 }
 
 int force_chunks(int64_t nb, int64_t max_box_blobs)
@@ -504,49 +543,13 @@ int force_chunks(int64_t nb, int64_t max_box_blobs)
     return (int)((max_box_blobs + T - 1) / T);
 }
 
-cudaError_t launch_forces(cudaStream_t st, int B, int64_t nb, int64_t max_box_blobs,
+cudaError_t launch_forces(Chain st, int B, int64_t nb, int64_t max_box_blobs,
                           const ForceArgs& a, const GridGeo& g, const BinGeo& bg)
 {
     const int chunks = force_chunks(nb, max_box_blobs);
     if (chunks <= 0) return cudaSuccess;
-    k_forces<<<dim3((unsigned)chunks, (unsigned)B), blob_block(nb), 0, st>>>(a, g, bg);
-    return cudaGetLastError();
-}
-
-// Per-box force sums in a fixed order, then the FP64 mean-velocity update.
-__global__ void __launch_bounds__(256)
-k_force_sum(int nchunk, const double* __restrict__ partial, double* __restrict__ vbar,
-            double scale, int mean_mode, double* __restrict__ fsum_out)
-{
-    __shared__ double sh[3][256];
-    const int box = blockIdx.x;
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int c = threadIdx.x; c < nchunk; c += blockDim.x)
-        for (int d = 0; d < 3; ++d) s[d] += partial[((int64_t)box * nchunk + c) * 3 + d];
-    for (int d = 0; d < 3; ++d) sh[d][threadIdx.x] = s[d];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int d = 0; d < 3; ++d) sh[d][threadIdx.x] += sh[d][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x < 3) {
-        const int d = threadIdx.x;
-        const double tot = sh[d][0];
-        if (fsum_out) fsum_out[3 * box + d] = tot;
-        if (vbar) vbar[3 * box + d] = mean_mode == 0 ? vbar[3 * box + d] + scale * tot : 0.0;
-    }
-}
-
-cudaError_t launch_force_sum(cudaStream_t st, int B, int nchunk, const double* partial,
-                             double* vbar, double scale, int mean_mode, double* fsum_out)
-{
-    if (nchunk <= 0) {
-        // no blobs anywhere: the net force is zero
-        return cudaSuccess;
-    }
-    k_force_sum<<<B, 256, 0, st>>>(nchunk, partial, vbar, scale, mean_mode, fsum_out);
-    return cudaGetLastError();
+    return launch_on(st, k_forces, dim3((unsigned)chunks, (unsigned)B), dim3(blob_block(nb)), 0, a,
+                      g, bg);
 }
 
 // ==========================================================================================
@@ -589,6 +592,8 @@ __global__ void __launch_bounds__(128)
 k_spread_atomic(int64_t nb, const double* __restrict__ q, const double* __restrict__ F,
                 const int32_t* __restrict__ box_of, GridGeo g, double scale, R* __restrict__ f)
 {
+    dep_wait();
+    dep_release();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t b = SPLIT ? t / 3 : t;
     if (b >= nb) return;
@@ -647,27 +652,29 @@ k_spread_atomic(int64_t nb, const double* __restrict__ q, const double* __restri
 }
 
 template <typename R>
-cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t nb, const double* q,
+cudaError_t launch_spread_atomic(Chain st, int B, int64_t nb, const double* q,
                                  const double* F, const int32_t* box_of, const GridGeo& g, R* f,
                                  bool zeroed, bool wrap, double scale)
 {
     if (!zeroed) {
-        const cudaError_t e = cudaMemsetAsync(f, 0, sizeof(R) * 3 * (size_t)B * g.N, st);
+        const cudaError_t e = cudaMemsetAsync(f, 0, sizeof(R) * 3 * (size_t)B * g.N, st.st);
         if (e != cudaSuccess) return e;
     }
     if (nb <= 0) return cudaSuccess;
     const bool split = split_components(nb);
     const int T = split ? 96 : blob_block(nb);
     const unsigned blocks = blocks_of(split ? 3 * nb : nb, T);
-    auto go = [&](auto k) { k<<<blocks, T, 0, st>>>(nb, q, F, box_of, g, scale, f); };
-    if (wrap) split ? go(k_spread_atomic<R, true, true>) : go(k_spread_atomic<R, false, true>);
-    else split ? go(k_spread_atomic<R, true, false>) : go(k_spread_atomic<R, false, false>);
-    return cudaGetLastError();
+    scale *= Win<R>::UNIT;
+    auto go = [&](auto k) {
+        return launch_on(st, k, dim3(blocks), dim3(T), 0, nb, q, F, box_of, g, scale, f);
+    };
+    if (wrap) return split ? go(k_spread_atomic<R, true, true>) : go(k_spread_atomic<R, false, true>);
+    return split ? go(k_spread_atomic<R, true, false>) : go(k_spread_atomic<R, false, false>);
 }
-template cudaError_t launch_spread_atomic<double>(cudaStream_t, int, int64_t, const double*,
+template cudaError_t launch_spread_atomic<double>(Chain, int, int64_t, const double*,
                                                   const double*, const int32_t*, const GridGeo&,
                                                   double*, bool, bool, double);
-template cudaError_t launch_spread_atomic<float>(cudaStream_t, int, int64_t, const double*,
+template cudaError_t launch_spread_atomic<float>(Chain, int, int64_t, const double*,
                                                  const double*, const int32_t*, const GridGeo&,
                                                  float*, bool, bool, double);
 
@@ -676,9 +683,12 @@ template cudaError_t launch_spread_atomic<float>(cudaStream_t, int, int64_t, con
 // which threads add).  The tile's scale is a power of two chosen from its largest force so that
 // no node can overflow: 2^62 over (candidates x max weight product x max |F| / h^3).
 __global__ void __launch_bounds__(256)
-k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_start, GridGeo g,
+k_spread_det(const double* __restrict__ q, const double* __restrict__ F,
+             const int32_t* __restrict__ sorted, const int32_t* __restrict__ cell_start, GridGeo g,
              BinGeo bg, int TX, int TY, int TZ, int max_ranges, double* __restrict__ f)
 {
+    dep_wait();
+    dep_release();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tileN = TX * TY * TZ;
     unsigned long long* acc = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -735,19 +745,19 @@ k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_st
     }
     __syncthreads();
     const int total = rpre[nr];
-    auto slot_of = [&](int t) {
+    auto blob_of = [&](int t) {
         int a = 0, b = nr - 1;
         while (a < b) {
             const int m = (a + b + 1) >> 1;
             if (rpre[m] <= t) a = m; else b = m - 1;
         }
-        return (int64_t)rbeg[a] + (t - rpre[a]);
+        return 3 * (int64_t)sorted[rbeg[a] + (t - rpre[a])];      // its offset in q and F
     };
     // tile scale from the largest force component among the candidates
     double fm = 0.0;
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const double* rr = rec + 6 * slot_of(t);
-        fm = fmax(fm, fmax(fabs(rr[3]), fmax(fabs(rr[4]), fabs(rr[5]))));
+        const double* Fb = F + blob_of(t);
+        fm = fmax(fm, fmax(fabs(Fb[0]), fmax(fabs(Fb[1]), fabs(Fb[2]))));
     }
     for (int o = 16; o > 0; o >>= 1) fm = fmax(fm, __shfl_down_sync(0xffffffffu, fm, o));
     if ((threadIdx.x & 31) == 0) fmax_sh[threadIdx.x >> 5] = fm;
@@ -769,8 +779,9 @@ k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_st
     for (int i = threadIdx.x; i < parts * total; i += blockDim.x) {
         const int t = i / parts, part = i - t * parts;
         const int a = part % 3, c0 = part / 3, c1 = parts == 9 ? c0 + 1 : 3;
-        const double* rr = rec + 6 * slot_of(t);
-        const double Fa = rr[3 + a] * inv_h3;
+        const int64_t at = blob_of(t);
+        const double* rr = q + at;
+        const double Fa = F[at + a] * inv_h3;
         double wx[3], wy[3], wz[3];
         const int ix = peskin_window<double>(rr[0] * g.inv_h - mac_shift(a, 0), wx) - T0[0];
         const int iy = peskin_window<double>(rr[1] * g.inv_h - mac_shift(a, 1), wy) - T0[1];
@@ -796,18 +807,33 @@ k_spread_det(const double* __restrict__ rec, const int32_t* __restrict__ cell_st
     }
     __syncthreads();
     const double inv_scale = 1.0 / scale;
+    const int lx = 31 - __clz(TX), lxy = lx + 31 - __clz(TY), lt = 31 - __clz(tileN);   // powers of two
     for (int i = threadIdx.x; i < 3 * tileN; i += blockDim.x) {
-        const int a = i / tileN, rem = i - a * tileN;
-        const int rz = rem / (TY * TX), ry = (rem / TX) % TY, rx = rem % TX;
+        const int a = i >> lt, rem = i & (tileN - 1);
+        const int rz = rem >> lxy, ry = (rem >> lx) & (TY - 1), rx = rem & (TX - 1);
         f[((size_t)box * 3 + a) * (size_t)g.N +
           ((size_t)(T0[2] + rz) * ny + (T0[1] + ry)) * nx + (T0[0] + rx)] =
             (double)(long long)acc[i] * inv_scale;
     }
 }
 
-cudaError_t launch_spread_det(cudaStream_t st, int B, const double* rec, const int32_t* cell_start,
-                              const GridGeo& g, const BinGeo& bg, const int tile[3], double* f)
+cudaError_t launch_spread_det(Chain st, int B, const double* q, const double* F,
+                              const int32_t* sorted, const int32_t* cell_start, const GridGeo& g,
+                              const BinGeo& bg, const int tile_in[3], double* f)
 {
+    // small grids: tiles halved along their longest side (whole bin cells, at least four nodes)
+    // until there are two blocks for each SM; a block's clearing and writing of its nodes, not
+    // its blobs, sets the time there
+    int tile[3] = {tile_in[0], tile_in[1], tile_in[2]};
+    const int least = bg.bs > 4 ? bg.bs : 4;
+    auto tiles = [&] { return (int64_t)(g.n[0] / tile[0]) * (g.n[1] / tile[1]) * (g.n[2] / tile[2]); };
+    while (tiles() * B < 304) {
+        int d = 0;
+        for (int e = 1; e < 3; ++e)
+            if (tile[e] > tile[d]) d = e;
+        if (tile[d] / 2 < least) break;
+        tile[d] /= 2;
+    }
     const int TX = tile[0], TY = tile[1], TZ = tile[2];
     int max_rows = 1;
     for (int d = 1; d < 3; ++d) {
@@ -824,10 +850,8 @@ cudaError_t launch_spread_det(cudaStream_t st, int B, const double* rec, const i
     static std::atomic<unsigned> attr{0};
     if (first_on_device(attr))
         cudaFuncSetAttribute(k_spread_det, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    const int ntiles = (g.n[0] / TX) * (g.n[1] / TY) * (g.n[2] / TZ);
-    k_spread_det<<<dim3((unsigned)ntiles, (unsigned)B), 256, smem, st>>>(rec, cell_start, g, bg, TX,
-                                                                         TY, TZ, max_ranges, f);
-    return cudaGetLastError();
+    return launch_on(st, k_spread_det, dim3((unsigned)tiles(), (unsigned)B), dim3(256), smem, q, F,
+                     sorted, cell_start, g, bg, TX, TY, TZ, max_ranges, f);
 }
 
 // ==========================================================================================

@@ -1174,14 +1174,14 @@ cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, 
                       dim3(256), 0, st, nb, f, g, bg);
 }
 
-cudaError_t launch_bin_scan(cudaStream_t st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
+cudaError_t launch_bin_scan(Chain st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
                             int32_t* total)
 {
     // scan_tmp: [ntiles] tile offsets, then the ticket of the last-block scan (zero between
     // launches)
     const int ntiles = (int)((ncells + (1 << BIN_SCAN_LOG) - 1) >> BIN_SCAN_LOG);
-    return launch_dep(k_bin_scan32, dim3(ntiles), dim3(BIN_SCAN_THREADS), 0, st, count, ncells,
-                      scan_tmp, total, reinterpret_cast<unsigned*>(scan_tmp + ntiles));
+    return launch_on(st, k_bin_scan32, dim3(ntiles), dim3(BIN_SCAN_THREADS), 0, count, ncells,
+                     scan_tmp, total, reinterpret_cast<unsigned*>(scan_tmp + ntiles));
 }
 
 cudaError_t launch_bin32(cudaStream_t st, int64_t nb, const float4* A, const int32_t* box_of,
@@ -1198,7 +1198,7 @@ cudaError_t launch_bin32(cudaStream_t st, int64_t nb, const float4* A, const int
             k_bin_count32<<<blocks_for(nb, 256), 256, 0, st>>>(nb, A, box_of, bg, cell_count,
                                                                blob_cell, blob_rank);
     }
-    e = launch_bin_scan(st, cell_count, ncells, scan_tmp, cell_start + ncells);
+    e = launch_bin_scan(Chain(st, true), cell_count, ncells, scan_tmp, cell_start + ncells);
     if (e != cudaSuccess) return e;
     const int64_t nthr = nb > ncells ? nb : ncells;
     return launch_dep(k_bin_place32, dim3(blocks_for(nthr, 256)), dim3(256), 0, st, nb, ncells,

@@ -622,9 +622,10 @@ k_plane_inv(FluidArgs<float> a, GridGeo g)
 }
 
 template <>
-cudaError_t launch_fluid3<float>(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<float>& a_in,
+cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const FluidArgs<float>& a_in,
                           cudaEvent_t* marks)
 {
+    cudaStream_t st = chain.st;                      // always a chain of programmatic dependents
     const FluidArgs<float> a = with_derived(a_in, g);
     constexpr int PT = 256;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;

@@ -141,7 +141,7 @@ struct mb_ctx {
     int nxh = 0;
     int tile[3] = {8, 8, 8};
 
-    DBuf v[2], vsum, f, spec, vbar, fsum, tw[3], twf[3], sym, symr, body_prof, prof_scratch;
+    DBuf v[2], vsum, f, spec, vbar, tw[3], twf[3], sym, symr, body_prof, prof_scratch;
     DBuf twk[3], symk;          // FP64 grids: twiddles and symbols in double-float
     // thermal stress (kT > 0): sigma~ of the current step [B][9][N] and the step index that
     // keys its random numbers (device memory, advanced by the step itself)
@@ -163,7 +163,7 @@ struct mb_ctx {
     int direct64 = 0;          // FP64 steps launched directly since the last rebuild
     std::vector<int64_t> box_off_h, part_off_h;
     std::vector<float> box_par32_h;                // float copy of the box parameters
-    DBuf q, qh, u, F, rec, ext, pid, box_of, adj_start, adj_j, adj_rest, part_start,
+    DBuf q, qh, u, F, ext, pid, box_of, adj_start, adj_j, adj_rest, part_start,
         part_blobs, box_off, box_par, cell_count, cell_start, blob_cell, blob_rank, sorted,
         loc, scan_tmp, partial, staging_in, staging_out, mean_scratch;
     // FP32-grid mode blob state: positions as bin cell + float-float offset (q^n and midpoint)
@@ -171,6 +171,7 @@ struct mb_ctx {
     // the bond pattern common to all particles (tmpl_m blobs each), when there is one
     DBuf tmpl32, tstart32;
     int tmpl_m = 0, tmpl_slots = 0;
+    DBuf force_ticket;  // FP64 grids: [B] tickets of the net force, zero between launches
     DBuf Fpre64;        // FP64 grids: external + spring forces of the pattern kernel [nb][3]
     // split midpoints: hA/hB[hcur] hold the predictor of the next step when pred_ready (the
     // previous step's fused corrector wrote them); hlast is the buffer of the last step's
@@ -473,7 +474,6 @@ mb_status rebuild(mb_ctx* ctx)
     MB_TRY(ensure(ctx->qh, sizeof(double) * 3 * nb, E, "q_half"));
     MB_TRY(ensure(ctx->u, sizeof(double) * 3 * nb, E, "u"));
     MB_TRY(ensure(ctx->F, sizeof(double) * 3 * nb, E, "F"));
-    MB_TRY(ensure(ctx->rec, sizeof(double) * 6 * nb, E, "rec"));
     MB_TRY(ensure(ctx->ext, sizeof(double) * 3 * nb, E, "ext"));
     MB_TRY(ensure(ctx->pid, sizeof(int32_t) * nb, E, "pid"));
     MB_TRY(ensure(ctx->box_of, sizeof(int32_t) * nb, E, "box_of"));
@@ -485,6 +485,8 @@ mb_status rebuild(mb_ctx* ctx)
     MB_TRY(ensure(ctx->box_off, sizeof(int64_t) * (B + 1), E, "box_off"));
     // [B][3] doubles, then the same rounded to float for the FP32 blob kernels
     MB_TRY(ensure(ctx->box_par, (sizeof(double) + sizeof(float)) * 3 * B, E, "box_par"));
+    MB_TRY(ensure(ctx->force_ticket, sizeof(unsigned) * B, E, "force ticket"));
+    MB_CUDA(cudaMemsetAsync(ctx->force_ticket.p, 0, sizeof(unsigned) * B, ctx->st));
     MB_TRY(ensure(ctx->cell_count, sizeof(int32_t) * ncells, E, "cell_count"));
     MB_TRY(ensure(ctx->cell_start, sizeof(int32_t) * (ncells + 1), E, "cell_start"));
     MB_TRY(ensure(ctx->blob_cell, sizeof(int32_t) * nb, E, "blob_cell"));
@@ -575,36 +577,55 @@ mb_status rebuild(mb_ctx* ctx)
     }
     // the pattern's tables: FP32 grids (k_springs32_shared) per local blob its evaluations
     // {offset | (slot + 1) << 16, r0, r0^2 hi, lo} and the slots it collects {offset, slot};
-    // FP64 grids (k_springs64) its evaluations {offset | (slot + 1) << 16, r0 low, r0 high} and
-    // its whole adjacency in order {offset of the evaluating blob, slot, sign}
+    // FP64 grids (k_springs64) the bonds {ends, r0 low, r0 high} and per local blob its whole
+    // adjacency in order {bond, sign}
+    if (pm > 0 && ctx->rsz == 8 && adj_start[pm] / 2 > SPRINGS64_MAX_BONDS) {
+        ctx->tmpl_m = 0;
+        pm = 0;
+    }
     if (pm > 0) {
         std::vector<int32_t> t_start(2 * pm + 1, 0), t;
-        for (int64_t l = 0; l < pm; ++l) {
-            for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
-                if (owner[e] != l) continue;
-                const int64_t j = adj_j[e];
-                const double r0 = adj_rest[e];
-                int32_t w[4];
-                w[0] = (int32_t)(((uint32_t)(j - l) & 0xffffu) | ((uint32_t)(slot[e] + 1) << 16));
-                if (ctx->rsz == 4) {
-                    const double r0sq = r0 * r0;
+        if (ctx->rsz == 8) {
+            std::map<std::pair<int32_t, int32_t>, int32_t> bond;       // (owner, slot) -> bond
+            for (int64_t l = 0; l < pm; ++l)
+                for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
+                    if (owner[e] != l) continue;
+                    bond[{owner[e], slot[e]}] = (int32_t)(t.size() / 4);
+                    int32_t w[4] = {(int32_t)l | (adj_j[e] << 16), 0, 0, 0};
+                    std::memcpy(&w[1], &adj_rest[e], 8);       // low word, then high word
+                    t.insert(t.end(), w, w + 4);
+                }
+            ctx->tmpl_slots = (int)(t.size() / 4);
+            t_start[0] = ctx->tmpl_slots;
+            for (int64_t l = 0; l < pm; ++l) {
+                for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
+                    const int32_t w[4] = {bond[{owner[e], slot[e]}], owner[e] == l ? 1 : -1, 0, 0};
+                    t.insert(t.end(), w, w + 4);
+                }
+                t_start[l + 1] = (int32_t)(t.size() / 4);
+            }
+        } else {
+            for (int64_t l = 0; l < pm; ++l) {
+                for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
+                    if (owner[e] != l) continue;
+                    const int64_t j = adj_j[e];
+                    const double r0 = adj_rest[e], r0sq = r0 * r0;
                     const float h = (float)r0sq, lo = (float)(r0sq - (double)h), rf = (float)r0;
+                    int32_t w[4];
+                    w[0] = (int32_t)(((uint32_t)(j - l) & 0xffffu) | ((uint32_t)(slot[e] + 1) << 16));
                     std::memcpy(&w[1], &rf, 4);
                     std::memcpy(&w[2], &h, 4);
                     std::memcpy(&w[3], &lo, 4);
-                } else {
-                    std::memcpy(&w[1], &r0, 8);            // low word, then high word
-                    w[3] = 0;
+                    t.insert(t.end(), w, w + 4);
                 }
-                t.insert(t.end(), w, w + 4);
+                t_start[2 * l + 1] = (int32_t)(t.size() / 4);
+                for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
+                    if (owner[e] == l) continue;
+                    const int32_t w[4] = {(int32_t)(owner[e] - l), slot[e], -1, 0};
+                    t.insert(t.end(), w, w + 4);
+                }
+                t_start[2 * l + 2] = (int32_t)(t.size() / 4);
             }
-            t_start[2 * l + 1] = (int32_t)(t.size() / 4);
-            for (int32_t e = adj_start[l]; e < adj_start[l + 1]; ++e) {
-                if (ctx->rsz == 4 && owner[e] == l) continue;
-                const int32_t w[4] = {(int32_t)(owner[e] - l), slot[e], owner[e] == l ? 1 : -1, 0};
-                t.insert(t.end(), w, w + 4);
-            }
-            t_start[2 * l + 2] = (int32_t)(t.size() / 4);
         }
         MB_TRY(ensure(ctx->tmpl32, sizeof(int32_t) * std::max<size_t>(t.size(), 4), E,
                       "bond pattern"));
@@ -612,6 +633,15 @@ mb_status rebuild(mb_ctx* ctx)
         MB_TRY(up(ctx->tmpl32, t.data(), sizeof(int32_t) * t.size()));
         MB_TRY(up(ctx->tstart32, t_start.data(), sizeof(int32_t) * (2 * pm + 1)));
         if (ctx->rsz == 8) MB_TRY(ensure(ctx->Fpre64, sizeof(double) * 3 * nb, E, "spring forces"));
+    }
+    // FP64 inertial steps: from one blob in 32 cells on, the inverse plane pass also writes
+    // v^n + v^{n+1}, 48 bytes a cell under its arithmetic, and saves the corrector 81 additions a
+    // blob on the narrow FP64 pipe
+    if (ctx->rsz == 8 && ctx->d.integrator == 0) {
+        if (ctx->fft_passes == 3 && 32 * nb >= B * ctx->g.N)
+            MB_TRY(ensure(ctx->vsum, grid_bytes(ctx, B), E, "v sum"));
+        else
+            MB_CUDA(dfree(ctx->vsum));
     }
     if (ctx->rsz == 4) {
         MB_TRY(ensure(ctx->sA, sizeof(float4) * nb, E, "split q"));
@@ -760,6 +790,11 @@ mb_status drain_stage_events(mb_ctx* ctx)
 // FP64 blobs: the bin cells are needed by the repulsion and by the deterministic spreading.
 bool needs_bins(const mb_ctx* ctx) { return ctx->any_rep || ctx->d.deterministic != 0; }
 
+// The chain of an FP64 step's kernels: programmatic dependents where it runs on one stream
+// without bins (rollout of 64 particles at 64^3 23.1 -> 20.9 ms); with the bins' kernels and the
+// side stream in it, the ordinary way is as fast or faster (drag at 32^3 72 against 82 us a step).
+Chain chain64(const mb_ctx* ctx) { return Chain(ctx->st, !needs_bins(ctx)); }
+
 BinCount bin_count(const mb_ctx* ctx)
 {
     return BinCount{static_cast<int32_t*>(ctx->cell_count.p),
@@ -767,25 +802,30 @@ BinCount bin_count(const mb_ctx* ctx)
                     static_cast<int32_t*>(ctx->blob_rank.p), ctx->bg};
 }
 
-// FP64 blob forces F at x (and sorted records when the spreading is deterministic).  counted:
+// FP64 blob forces F at x.  counted:
 // the blobs are in the bin counts already.  With one bond pattern for all particles the springs
 // run once per bond, summed with the external forces in the per-blob order (the same bits), on
 // the side stream beside the binning when `overlap`.
+// advance_mean: the net force advances the boxes' mean velocity.
 template <typename Mark>
 mb_status forces64(mb_ctx* ctx, const double* x, const double* ext, bool counted, bool overlap,
-                   bool det, Mark&& mark)
+                   bool det, bool advance_mean, Mark&& mark)
 {
     cudaStream_t st = ctx->st;
     const int32_t* box_of = static_cast<const int32_t*>(ctx->box_of.p);
     const bool bins = ctx->any_rep || det;
     const bool pattern = ctx->tmpl_m > 0 && !springs_per_blob();
-    auto springs = [&](cudaStream_t s2) {
+    // the springs' sums are the forces where there is no repulsion and nobody wants the net force
+    // (with mean_mode 1 the mean velocity stays zero)
+    const bool sum = advance_mean && ctx->d.mean_mode == 0;
+    const bool done = pattern && !ctx->any_rep && !sum;
+    auto springs = [&](Chain s2) {
         ctx->launches += 1;
         return launch_springs64(s2, ctx->nb, ctx->tmpl_m, ctx->tmpl_slots, x, ext,
                                 static_cast<const int4*>(ctx->tmpl32.p),
                                 static_cast<const int32_t*>(ctx->tstart32.p), box_of,
                                 static_cast<const double*>(ctx->box_par.p), ctx->g,
-                                static_cast<double*>(ctx->Fpre64.p));
+                                static_cast<double*>(done ? ctx->F.p : ctx->Fpre64.p));
     };
     const bool side = pattern && bins && overlap;
     if (side) {
@@ -796,21 +836,22 @@ mb_status forces64(mb_ctx* ctx, const double* x, const double* ext, bool counted
     }
     mark(ST_BIN);
     if (bins) {
-        MB_CUDA(launch_bin(st, ctx->nb, x, box_of, ctx->B, bin_count(ctx),
+        MB_CUDA(launch_bin(chain64(ctx), ctx->nb, x, box_of, ctx->B, bin_count(ctx),
                            static_cast<int32_t*>(ctx->cell_start.p),
                            static_cast<int32_t*>(ctx->sorted.p),
-                           static_cast<int32_t*>(ctx->scan_tmp.p), det,
+                           static_cast<int32_t*>(ctx->scan_tmp.p), det && ctx->any_rep,
                            static_cast<const int32_t*>(ctx->pid.p),
-                           static_cast<float4*>(ctx->loc.p), counted));
-        ctx->launches += (counted ? 2 : 3) + (det ? 1 : 0);
+                           ctx->any_rep ? static_cast<float4*>(ctx->loc.p) : nullptr, counted));
+        ctx->launches += (counted ? 2 : 3) + (det && ctx->any_rep ? 1 : 0);
     }
     mark(ST_FORCES);
     if (side) MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[1], 0));
-    else if (pattern) MB_CUDA(springs(st));
+    else if (pattern) MB_CUDA(springs(chain64(ctx)));
+    if (done) return MB_OK;
     ForceArgs fa{};
     fa.Fpre = pattern ? static_cast<const double*>(ctx->Fpre64.p) : nullptr;
     fa.box_off = static_cast<const int64_t*>(ctx->box_off.p);
-    fa.sorted = bins ? static_cast<const int32_t*>(ctx->sorted.p) : nullptr;
+    fa.sorted = ctx->any_rep ? static_cast<const int32_t*>(ctx->sorted.p) : nullptr;
     fa.q = x;
     fa.pid = static_cast<const int32_t*>(ctx->pid.p);
     fa.adj_start = static_cast<const int32_t*>(ctx->adj_start.p);
@@ -822,9 +863,12 @@ mb_status forces64(mb_ctx* ctx, const double* x, const double* ext, bool counted
     fa.ext = ext;
     fa.loc = static_cast<const float4*>(ctx->loc.p);
     fa.F = static_cast<double*>(ctx->F.p);
-    fa.rec = det ? static_cast<double*>(ctx->rec.p) : nullptr;
     fa.partial = static_cast<double*>(ctx->partial.p);
-    MB_CUDA(launch_forces(st, ctx->B, ctx->nb, ctx->max_box_blobs, fa, ctx->g, ctx->bg));
+    fa.ticket = static_cast<unsigned*>(ctx->force_ticket.p);
+    fa.vbar = sum ? static_cast<double*>(ctx->vbar.p) : nullptr;
+    fa.mean_scale = ctx->d.dt / (ctx->d.rho * ctx->g.L[0] * ctx->g.L[1] * ctx->g.L[2]);
+    fa.mean_mode = ctx->d.mean_mode;
+    MB_CUDA(launch_forces(chain64(ctx), ctx->B, ctx->nb, ctx->max_box_blobs, fa, ctx->g, ctx->bg));
     ctx->launches += 1;
     return MB_OK;
 }
@@ -833,11 +877,12 @@ mb_status forces64(mb_ctx* ctx, const double* x, const double* ext, bool counted
 mb_status spread64(mb_ctx* ctx, const double* x, bool det)
 {
     if (det)
-        MB_CUDA(launch_spread_det(ctx->st, ctx->B, static_cast<const double*>(ctx->rec.p),
+        MB_CUDA(launch_spread_det(chain64(ctx), ctx->B, x, static_cast<const double*>(ctx->F.p),
+                                  static_cast<const int32_t*>(ctx->sorted.p),
                                   static_cast<const int32_t*>(ctx->cell_start.p), ctx->g, ctx->bg,
                                   ctx->tile, static_cast<double*>(ctx->f.p)));
     else
-        MB_CUDA(launch_spread_atomic<double>(ctx->st, ctx->B, ctx->nb, x,
+        MB_CUDA(launch_spread_atomic<double>(chain64(ctx), ctx->B, ctx->nb, x,
                                              static_cast<const double*>(ctx->F.p),
                                              static_cast<const int32_t*>(ctx->box_of.p), ctx->g,
                                              static_cast<double*>(ctx->f.p), ctx->f_zero, false,
@@ -855,7 +900,7 @@ mb_status fluid64(mb_ctx* ctx, int boxes, FluidArgs<double> fa, bool clear_f, cu
         ctx->launches += FLUID_KERNELS;
     } else {
         if (clear_f) fa.f_clear = static_cast<double*>(ctx->f.p);
-        MB_CUDA(launch_fluid3<double>(ctx->st, boxes, ctx->g, fa, marks));
+        MB_CUDA(launch_fluid3<double>(chain64(ctx), boxes, ctx->g, fa, marks));
         ctx->launches += FLUID3_KERNELS;
     }
     ctx->f_zero = clear_f && ctx->fft_passes == 3;
@@ -885,24 +930,15 @@ mb_status do_step64(mb_ctx* ctx, const double* ext, const double* body)
         // u^n = J(q^n) v^n ; q^{n+1/2} = q^n + dt/2 u^n, counted into its bin cell on the way
         const BinCount bin = bin_count(ctx);
         if (bins) MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * B * ctx->bg.ncell, st));
-        MB_CUDA(launch_interp<double>(st, 1, ctx->nb, q, nullptr, vcur, nullptr, box_of, g,
+        MB_CUDA(launch_interp<double>(chain64(ctx), 1, ctx->nb, q, nullptr, vcur, nullptr, box_of, g,
                                       ctx->d.dt, nullptr, qh, false, bins ? &bin : nullptr));
         ctx->launches += 1;
-        MB_TRY(forces64(ctx, qh, ext, true, !ctx->timing, det, mark));
+        MB_TRY(forces64(ctx, qh, ext, true, !ctx->timing, det, true, mark));
     } else {
         mark(ST_BIN);
         mark(ST_FORCES);
     }
-    mark(ST_FORCE_SUM);
-    if (blobs) {
-        const double L3 = g.L[0] * g.L[1] * g.L[2];
-        MB_CUDA(launch_force_sum(st, B, force_chunks(ctx->nb, ctx->max_box_blobs),
-                                 static_cast<const double*>(ctx->partial.p),
-                                 static_cast<double*>(ctx->vbar.p),
-                                 ctx->d.dt / (ctx->d.rho * L3), ctx->d.mean_mode,
-                                 static_cast<double*>(ctx->fsum.p)));
-        ctx->launches += 1;
-    }
+    mark(ST_FORCE_SUM);                 // the forces' last block sums them
     mark(ST_SPREAD);
     if (blobs) MB_TRY(spread64(ctx, qh, det));
     mark(ST_STRESS);
@@ -916,14 +952,19 @@ mb_status do_step64(mb_ctx* ctx, const double* ext, const double* body)
         ctx->launches += STRESS_KERNELS;
     }
     const double* mean = ctx->d.mean_mode == 0 ? static_cast<const double*>(ctx->vbar.p) : nullptr;
-    MB_TRY(fluid64(ctx, B,
-                   fluid_args<double>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr, vnext,
-                                      ctx->body_prof.p, body, mean),
-                   blobs && !det, ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr));
+    FluidArgs<double> fa = fluid_args<double>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr,
+                                              vnext, ctx->body_prof.p, body, mean);
+    const bool vsum = blobs && ctx->vsum.p != nullptr;
+    if (vsum) {
+        fa.v_sum_base = vcur;
+        fa.v_sum_out = static_cast<double*>(ctx->vsum.p);
+    }
+    MB_TRY(fluid64(ctx, B, fa, blobs && !det, ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr));
     if (blobs) {
         // q^{n+1} = q^n + dt J(q^{n+1/2}) (v^n + v^{n+1})/2
-        MB_CUDA(launch_interp<double>(st, 2, ctx->nb, qh, q, vcur, vnext, box_of, g, ctx->d.dt,
-                                      nullptr, q));
+        MB_CUDA(launch_interp<double>(chain64(ctx), 2, ctx->nb, qh, q, vsum ? fa.v_sum_out : vcur,
+                                      vsum ? nullptr : vnext, box_of, g, ctx->d.dt, nullptr, q,
+                                      false, nullptr, 0.5));
         ctx->launches += 1;
     }
     mark(NUM_STAGES);
@@ -955,7 +996,7 @@ mb_status do_step_stokes64(mb_ctx* ctx, const double* ext, const double* body)
     auto half = [&](const double* x, bool counted, double* v_out, bool marks) -> mb_status {
         auto m = [&](int i) { if (marks) mark(i); };
         if (blobs) {
-            MB_TRY(forces64(ctx, x, ext, counted, !ctx->timing, det, m));
+            MB_TRY(forces64(ctx, x, ext, counted, !ctx->timing, det, false, m));
         } else {
             m(ST_BIN);
             m(ST_FORCES);
@@ -980,14 +1021,14 @@ mb_status do_step_stokes64(mb_ctx* ctx, const double* ext, const double* body)
         const BinCount bin = bin_count(ctx);
         if (bins)
             MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * ctx->B * ctx->bg.ncell, st));
-        MB_CUDA(launch_interp<double>(st, 1, ctx->nb, q, nullptr, v_half, nullptr, box_of, g,
+        MB_CUDA(launch_interp<double>(chain64(ctx), 1, ctx->nb, q, nullptr, v_half, nullptr, box_of, g,
                                       ctx->d.dt, nullptr, qh, false, bins ? &bin : nullptr));
         ctx->launches += 1;
     }
     MB_TRY(half(qh, true, v_full, true));
     if (blobs) {
         // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})
-        MB_CUDA(launch_interp<double>(st, 2, ctx->nb, qh, q, v_full, nullptr, box_of, g, ctx->d.dt,
+        MB_CUDA(launch_interp<double>(chain64(ctx), 2, ctx->nb, qh, q, v_full, nullptr, box_of, g, ctx->d.dt,
                                       nullptr, q));
         ctx->launches += 1;
     }
@@ -1653,10 +1694,10 @@ void release(mb_ctx* ctx)
         if (e) cudaEventDestroy(e);
         e = nullptr;
     }
-    DBuf* all[] = {&ctx->v[0], &ctx->v[1], &ctx->vsum, &ctx->f, &ctx->spec, &ctx->vbar, &ctx->fsum,
+    DBuf* all[] = {&ctx->v[0], &ctx->v[1], &ctx->vsum, &ctx->f, &ctx->spec, &ctx->vbar,
                    &ctx->tw[0], &ctx->tw[1], &ctx->tw[2], &ctx->twf[0], &ctx->twf[1],
                    &ctx->twf[2], &ctx->sym, &ctx->symr, &ctx->body_prof,
-                   &ctx->prof_scratch, &ctx->q, &ctx->qh, &ctx->u, &ctx->F, &ctx->rec,
+                   &ctx->prof_scratch, &ctx->q, &ctx->qh, &ctx->u, &ctx->F,
                    &ctx->ext, &ctx->pid, &ctx->box_of, &ctx->adj_start, &ctx->adj_j,
                    &ctx->adj_rest, &ctx->part_start, &ctx->part_blobs, &ctx->box_off,
                    &ctx->box_par, &ctx->cell_count, &ctx->cell_start, &ctx->blob_cell,
@@ -1664,7 +1705,7 @@ void release(mb_ctx* ctx)
                    &ctx->staging_in, &ctx->staging_out, &ctx->mean_scratch, 
                    &ctx->s_F, &ctx->s_g0, &ctx->s_g1, &ctx->s_g2, &ctx->s_out, &ctx->sA,
                    &ctx->sB, &ctx->hA[0], &ctx->hA[1], &ctx->hB[0], &ctx->hB[1], &ctx->F32, &ctx->rec32, &ctx->ext32,
-                   &ctx->ext_sum, &ctx->ext_ticket, &ctx->adj32, &ctx->adj32_start, &ctx->tmpl32, &ctx->tstart32, &ctx->Fpre64, &ctx->Fs32, &ctx->u32, &ctx->a_qn, &ctx->a_qh,
+                   &ctx->ext_sum, &ctx->ext_ticket, &ctx->adj32, &ctx->adj32_start, &ctx->tmpl32, &ctx->tstart32, &ctx->Fpre64, &ctx->force_ticket, &ctx->Fs32, &ctx->u32, &ctx->a_qn, &ctx->a_qh,
                    &ctx->a_gq, &ctx->a_gqh, &ctx->a_gF, &ctx->a_gu, &ctx->a_gk, &ctx->a_gU,
                    &ctx->a_vn, &ctx->a_vp, &ctx->a_gvp, &ctx->a_gvn,
                    &ctx->a_gf, &ctx->W, &ctx->step_index,
@@ -1788,7 +1829,6 @@ mb_status mb_create_grid(const mb_grid_desc* desc, void* cuda_stream, mb_ctx** o
     if ((s = ensure(ctx->f, gb, ctx->err, "f")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->spec, sb, ctx->err, "spectrum")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->vbar, sizeof(double) * 3 * ctx->B, ctx->err, "vbar")) != MB_OK) return fail(s);
-    if ((s = ensure(ctx->fsum, sizeof(double) * 3 * ctx->B, ctx->err, "fsum")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->step_index, sizeof(uint64_t), ctx->err, "step index")) != MB_OK) return fail(s);
     ctx->thermal = d.kT > 0.0;
     ctx->advect = d.advection == 1;
@@ -2261,10 +2301,10 @@ mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n
     const BinCount bin = bin_count(ctx);
     if (ctx->any_rep && nb > 0)
         MB_CUDA(cudaMemsetAsync(bin.count, 0, sizeof(int32_t) * ctx->bg.ncell, st));
-    MB_CUDA(launch_interp<double>(st, 1, nb, qn, nullptr, vn, nullptr, nullptr, g, dt, nullptr, qh,
+    MB_CUDA(launch_interp<double>(chain64(ctx), 1, nb, qn, nullptr, vn, nullptr, nullptr, g, dt, nullptr, qh,
                                   true, ctx->any_rep ? &bin : nullptr));
     if (nb > 0) {
-        MB_TRY(forces64(ctx, qh, ext, true, true, false, [](int) {}));
+        MB_TRY(forces64(ctx, qh, ext, true, true, false, false, [](int) {}));
         MB_TRY(spread64(ctx, qh, false));
     }
     MB_TRY(fluid64(ctx, 1,
@@ -2274,19 +2314,19 @@ mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n
     // ---- backward
     // corrector q^{n+1} = q^n + dt J(q^{n+1/2}) (v^n + v^{n+1})/2: half of J^T (dt gq) goes to
     // dL/dv^{n+1}, half to dL/dv^n
-    MB_CUDA(launch_spread_atomic<double>(st, 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
+    MB_CUDA(launch_spread_atomic<double>(chain64(ctx), 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
     // fluid update v^{n+1} = A v^n + T f (A, T symmetric): gf = T gv, and A gv is a stencil of gf
     FluidArgs<double> fa = fluid_args<double>(ctx, vn, gv, gf, nullptr, nullptr, nullptr);
     fa.no_v = 1;
     if (ctx->fft_passes == 5) MB_CUDA(launch_fluid<double>(st, 1, g, fa));
-    else MB_CUDA(launch_fluid3<double>(st, 1, g, fa));
-    MB_CUDA(launch_viscous_stencil(st, g, gf, ctx->d.rho / dt,
+    else MB_CUDA(launch_fluid3<double>(chain64(ctx), 1, g, fa));
+    MB_CUDA(launch_viscous_stencil(chain64(ctx), g, gf, ctx->d.rho / dt,
                                    0.5 * ctx->d.eta * g.inv_h * g.inv_h, gv));
-    MB_CUDA(launch_spread_atomic<double>(st, 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
+    MB_CUDA(launch_spread_atomic<double>(chain64(ctx), 1, nb, qh, gq, nullptr, g, gv, true, false, 0.5 * dt));
     // spreading f = S(q^{n+1/2}) F and the corrector's positions
-    MB_CUDA(launch_adjoint_midpoint(st, nb, qh, gf, F, vn, vp, gq, dt, g, gF, gqh));
+    MB_CUDA(launch_adjoint_midpoint(chain64(ctx), nb, qh, gf, F, vn, vp, gq, dt, g, gF, gqh));
     // forces F(q^{n+1/2}; k)
-    MB_CUDA(launch_force_jvp(st, nb, qh, gF, static_cast<const int32_t*>(ctx->pid.p),
+    MB_CUDA(launch_force_jvp(chain64(ctx), nb, qh, gF, static_cast<const int32_t*>(ctx->pid.p),
                              static_cast<const int32_t*>(ctx->adj_start.p),
                              static_cast<const int32_t*>(ctx->adj_j.p),
                              static_cast<const double*>(ctx->adj_rest.p), bx.k_spring, bx.k_rep,
@@ -2294,7 +2334,7 @@ mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n
                              static_cast<const int32_t*>(ctx->sorted.p),
                              static_cast<const int32_t*>(ctx->blob_cell.p), g, ctx->bg, gqh, gk_dev));
     // predictor q^{n+1/2} = q^n + dt/2 J(q^n) v^n
-    MB_CUDA(launch_adjoint_velocity(st, nb, qn, vn, gqh, 0.5 * dt, gq, gqh, g, gq, gv));
+    MB_CUDA(launch_adjoint_velocity(chain64(ctx), nb, qn, vn, gqh, 0.5 * dt, gq, gqh, g, gq, gv));
     // ---- outputs
     MB_TRY(push(ctx, grad_pos, gq, bv));
     MB_TRY(push(ctx, grad_v, gv, bg));

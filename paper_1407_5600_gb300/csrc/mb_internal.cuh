@@ -63,6 +63,13 @@ template <> struct C2<double> { using T = double2; };
 // ------------------------------------------------------------------------------------------
 // Launchers (each returns cudaGetLastError() after enqueuing).
 
+// A stream, and whether the kernels launched on it are programmatic dependents (launch_dep).
+struct Chain {
+    cudaStream_t st;
+    bool dep;
+    Chain(cudaStream_t s, bool d = false) : st(s), dep(d) {}
+};
+
 // Where blobs are counted into bin cells (a kernel that moves blobs can count them on the way);
 // count null: nowhere.  count must be zero before the first blob.
 struct BinCount {
@@ -76,30 +83,32 @@ struct BinCount {
 //   mode 0: u_out = J(q) v0
 //   mode 1: u_out = J(q) v0, q_out = wrap(q + 0.5 dt u)            (predictor); with bin, the
 //           blobs are counted into the cells of q_out
-//   mode 2: u = J(q) v with v the mean of v0 and v1 (v0 when v1 is null),
+//   mode 2: u = scale J(q) (v0 + v1) (v0 alone when v1 is null),
 //           q_out = wrap(q_base + dt u)                            (corrector)
 // wrap (modes 0 and 1): q from anywhere, taken modulo the box.
 template <typename R>
-cudaError_t launch_interp(cudaStream_t st, int mode, int64_t nb, const double* q,
+cudaError_t launch_interp(Chain st, int mode, int64_t nb, const double* q,
                           const double* q_base, const R* v0, const R* v1,
                           const int32_t* box_of, const GridGeo& g, double dt, double* u_out,
-                          double* q_out, bool wrap = false, const BinCount* bin = nullptr);
+                          double* q_out, bool wrap = false, const BinCount* bin = nullptr,
+                          double scale = 1.0);
 
-// Cell binning: count (unless the blobs are `counted` already), scan, placement (and per-cell
-// ordering when deterministic).  scan_tmp: ncells / 4096 + 2 ints, the ticket among them zero.
-cudaError_t launch_bin(cudaStream_t st, int64_t nb, const double* q, const int32_t* box_of,
+// Cell binning: count (unless the blobs are `counted` already), scan, placement, with `ordered`
+// each cell's blobs by ascending index; loc (null: not wanted) as k_forces reads it.  scan_tmp: ncells / 4096 + 2 ints, the ticket among them zero.
+cudaError_t launch_bin(Chain st, int64_t nb, const double* q, const int32_t* box_of,
                        int B, const BinCount& c, int32_t* cell_start, int32_t* sorted,
-                       int32_t* scan_tmp, bool deterministic, const int32_t* pid, float4* loc,
+                       int32_t* scan_tmp, bool ordered, const int32_t* pid, float4* loc,
                        bool counted);
 // The scan of the cell counts (kernels_blob32.cu): count scanned in place within tiles of
 // 2^BIN_SCAN_LOG cells, the tiles' offsets in scan_tmp, the grand total in *total.
 constexpr int BIN_SCAN_LOG = 12;
-cudaError_t launch_bin_scan(cudaStream_t st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
+cudaError_t launch_bin_scan(Chain st, int32_t* count, int64_t ncells, int32_t* scan_tmp,
                             int32_t* total);
 
 // FP64 blob forces at q (springs, repulsion, external) in sorted-slot order, in the plain
-// operation order without contraction; writes F (blob order), rec (sorted order: q, F) and
-// per-(box, block) partial force sums.  sorted null: blob order and no repulsion.
+// operation order without contraction; writes F (blob order) and
+// with vbar advances each box's mean velocity by the net force:
+// vbar += mean_scale * sum F (mean_mode 0) or 0.  sorted null: blob order and no repulsion.
 struct ForceArgs {
     const int64_t* box_off;    // [B+1]
     const int32_t* sorted;
@@ -114,46 +123,44 @@ struct ForceArgs {
     const double* ext;         // may be null
     const float4* loc;         // [nb] sorted-order cell-local coordinates and particle id
     double* F;
-    double* rec;               // null: not written
-    double* partial;           // [B][force_chunks][3]
+    double* partial;           // [B][force_chunks][3] scratch of the net force
+    unsigned* ticket;          // [B], zero between launches
+    double* vbar;              // [B][3], or null
+    double mean_scale;
+    int mean_mode;
     // [nb][3] external plus spring forces already summed (launch_springs64); null: the kernel
     // sums them from ext and the adjacency lists
     const double* Fpre;
 };
-cudaError_t launch_forces(cudaStream_t st, int B, int64_t nb, int64_t max_box_blobs,
+cudaError_t launch_forces(Chain st, int B, int64_t nb, int64_t max_box_blobs,
                           const ForceArgs& a, const GridGeo& g, const BinGeo& bg);
 int force_chunks(int64_t nb, int64_t max_box_blobs);     // blocks a box
 
 // FP64 spring forces when every particle shares one bond pattern (m blobs, blob l of particle
-// p is blob p m + l): each bond evaluated once, in the precise FP64 order, by the end the
-// pattern names, and each blob's sum Fout = ext + the bonds in its adjacency order, so the
-// result has the bits of the per-blob evaluation of launch_forces (the two ends' evaluations
-// are exact negatives).  tmpl: per local blob an evaluation list {offset | (slot + 1) << 16,
-// r0 low word, r0 high word, 0} and a sum list in adjacency order {offset of the evaluating
-// blob, slot, sign, 0}; tstart[2l], tstart[2l + 1], tstart[2l + 2] bound them.
-cudaError_t launch_springs64(cudaStream_t st, int64_t nb, int m, int slots, const double* q,
+// p is blob p m + l; nbond bonds): each bond evaluated once, in the precise FP64 order, and each
+// blob's sum Fout = ext + its bonds in adjacency order, so the result has the bits of the
+// per-blob evaluation of launch_forces (the two ends' evaluations are exact negatives).  tmpl:
+// the bonds {first end | second end << 16, r0 low word, r0 high word, 0}, then every local
+// blob's list {bond, +1 at the first end or -1, 0, 0}; tstart[l], tstart[l + 1] bound blob l's.
+constexpr int SPRINGS64_MAX_BONDS = 2048;               // of one particle (48 KiB of forces)
+cudaError_t launch_springs64(Chain st, int64_t nb, int m, int nbond, const double* q,
                              const double* ext, const int4* tmpl, const int32_t* tstart,
                              const int32_t* box_of, const double* box_par, const GridGeo& g,
                              double* Fout);
-
-// Sum partial forces per box (fixed order) and update the FP64 mean velocity:
-// vbar += dt * sumF / (rho L^3) when mean_mode == 0, vbar = 0 otherwise; optionally copies
-// the force sum to fsum_out [B][3].
-cudaError_t launch_force_sum(cudaStream_t st, int B, int nchunk, const double* partial,
-                             double* vbar, double scale, int mean_mode, double* fsum_out);
 
 // Blob-owner spreading with global atomic adds into f (zeroed by the launcher unless `zeroed`);
 // q, F, box_of in blob order (box_of null: one box); wrap: positions from anywhere; the node
 // sums of weights * F are multiplied by `scale` (1/h^3 for S, 1 for the transpose of J).
 template <typename R>
-cudaError_t launch_spread_atomic(cudaStream_t st, int B, int64_t nb, const double* q,
+cudaError_t launch_spread_atomic(Chain st, int B, int64_t nb, const double* q,
                                  const double* F, const int32_t* box_of, const GridGeo& g, R* f,
                                  bool zeroed, bool wrap, double scale);
 
-// Deterministic FP64 spreading from sorted records (64-bit fixed-point shared-memory
-// accumulation); writes every node of f.
-cudaError_t launch_spread_det(cudaStream_t st, int B, const double* rec, const int32_t* cell_start,
-                              const GridGeo& g, const BinGeo& bg, const int tile[3], double* f);
+// Deterministic FP64 spreading of the binned blobs (64-bit fixed-point shared-memory
+// accumulation, the same sums whatever the order of a cell's blobs); writes every node of f.
+cudaError_t launch_spread_det(Chain st, int B, const double* q, const double* F,
+                              const int32_t* sorted, const int32_t* cell_start, const GridGeo& g,
+                              const BinGeo& bg, const int tile[3], double* f);
 
 // Particle velocities U0, Omega from blob velocities (particle CSR).
 cudaError_t launch_particle_reduce(cudaStream_t st, int64_t np, const int32_t* part_start,
@@ -255,6 +262,19 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+template <typename... P, typename... A>
+inline cudaError_t launch_on(Chain c, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                             A&&... args)
+{
+    if (c.dep) return launch_dep(kernel, grid, block, smem, c.st, std::forward<A>(args)...);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.st;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 template <typename R>
 cudaError_t launch_fluid(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a,
                          cudaEvent_t* marks = nullptr);
@@ -262,13 +282,13 @@ constexpr int FLUID_KERNELS = 5;
 // Three-pass variant (plane R2C, z solve, plane C2R; FP32 grids in kernels_fft3.cu, FP64 grids
 // in kernels_fft64.cu); marks as for launch_fluid, with the y-pass marks recorded back to back.
 template <typename R>
-cudaError_t launch_fluid3(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a,
+cudaError_t launch_fluid3(Chain st, int B, const GridGeo& g, const FluidArgs<R>& a,
                           cudaEvent_t* marks = nullptr);
 template <>
-cudaError_t launch_fluid3<float>(cudaStream_t st, int B, const GridGeo& g,
+cudaError_t launch_fluid3<float>(Chain st, int B, const GridGeo& g,
                                  const FluidArgs<float>& a, cudaEvent_t* marks);
 template <>
-cudaError_t launch_fluid3<double>(cudaStream_t st, int B, const GridGeo& g,
+cudaError_t launch_fluid3<double>(Chain st, int B, const GridGeo& g,
                                   const FluidArgs<double>& a, cudaEvent_t* marks);
 constexpr int FLUID3_KERNELS = 3;
 
@@ -368,19 +388,19 @@ cudaError_t launch_forces_to_fp64(cudaStream_t st, int64_t nb, const float4* F, 
 
 // Adjoint kernels (adjoint.cu), FP64.
 // At the midpoints q: gF = h^-3 J gf and gqh = d/dq [<gf, S(q) F> + sum dt gq . J(q) (v0 + v1)/2].
-cudaError_t launch_adjoint_midpoint(cudaStream_t st, int64_t nb, const double* q, const double* gf,
+cudaError_t launch_adjoint_midpoint(Chain st, int64_t nb, const double* q, const double* gf,
                                     const double* F, const double* v0, const double* v1,
                                     const double* gq, double dt, const GridGeo& g, double* gF,
                                     double* gqh);
 // Transpose of u = J(q) v with gradient scale * gu: out = base (+ base2) + (du/dq)^T, in place if
 // out == base; gv += J(q)^T.  Positions from anywhere.
-cudaError_t launch_adjoint_velocity(cudaStream_t st, int64_t nb, const double* q, const double* v,
+cudaError_t launch_adjoint_velocity(Chain st, int64_t nb, const double* q, const double* v,
                                     const double* gu, double scale, const double* base,
                                     const double* base2, const GridGeo& g, double* out, double* gv);
 // out = a x + c (sum of the six neighbours - 6 x), one box grid.
-cudaError_t launch_viscous_stencil(cudaStream_t st, const GridGeo& g, const double* x, double a,
+cudaError_t launch_viscous_stencil(Chain st, const GridGeo& g, const double* x, double a,
                                    double c, double* out);
-cudaError_t launch_force_jvp(cudaStream_t st, int64_t nb, const double* q, const double* gF,
+cudaError_t launch_force_jvp(Chain st, int64_t nb, const double* q, const double* gF,
                              const int32_t* pid, const int32_t* adj_start, const int32_t* adj_j,
                              const double* adj_rest, double k_spring, double k_rep, double r_cut,
                              const int32_t* cell_start, const int32_t* sorted,
