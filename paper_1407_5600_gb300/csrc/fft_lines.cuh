@@ -18,7 +18,20 @@ template <typename T> __device__ __forceinline__ T cm(T a, T b)
 template <typename T> __device__ __forceinline__ T cadd(T a, T b) { return T{a.x + b.x, a.y + b.y}; }
 // Correctly rounded reciprocals (the float one is a single intrinsic instead of a division).
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// FP64: Newton's iteration from the hardware's float reciprocal (four FP64 instructions instead
+// of the division's twenty or so) where the argument is in the float range.
+__device__ __forceinline__ double recip(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    if (hi - (897u << 20) >= (253u << 20)) return 1.0 / x;
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;"
+        : "=f"(y) : "f"(__uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29))));
+    const unsigned yb = __float_as_uint(y);
+    double r = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
 template <typename T> __device__ __forceinline__ T csub(T a, T b) { return T{a.x - b.x, a.y - b.y}; }
 
 __host__ __device__ constexpr int bitrev(int i, int bits)
@@ -44,17 +57,38 @@ template <typename R> __device__ __forceinline__ R cos16(int j)
     default: return R(-0.92387953251128675613);
     }
 }
+constexpr double TAN8 = 0.41421356237309504880;      // tan(pi / 8) = sqrt(2) - 1
 // sin(2 pi j / 16) = cos(2 pi (j - 4) / 16), j < 8
 template <typename R> __device__ __forceinline__ R sin16(int j) { return cos16<R>(j < 4 ? 4 - j : j - 4); }
 
-// b W_16^j (forward) or b W_16^-j (inverse), with W_16 = exp(-2 pi i / 16); j < 8.
-template <bool INV, typename T> __device__ __forceinline__ T twiddle16(T b, int j)
+// Butterfly (a, b) -> (a + w b, a - w b), w = W_16^j (forward) or W_16^-j (inverse), with
+// W_16 = exp(-2 pi i / 16); j < 8.  The larger of w's cosine and sine is taken out (Linzer and
+// Feig): w b = c (b.x -+ r b.y, b.y +- r b.x), |r| <= 1, so that a general one takes six fused
+// operations instead of two products, two fused ones and four additions.
+template <bool INV, typename T> __device__ __forceinline__ void butterfly(T& a, T& b, int j)
 {
     using R = decltype(b.x);
-    if (j == 0) return b;
-    if (j == 4) return INV ? T{-b.y, b.x} : T{b.y, -b.x};
-    const R c = cos16<R>(j), sn = INV ? sin16<R>(j) : -sin16<R>(j);
-    return T{b.x * c - b.y * sn, b.x * sn + b.y * c};
+    T u;
+    if (j == 0) u = b;
+    else if (j == 4) u = INV ? T{-b.y, b.x} : T{b.y, -b.x};
+    if (j == 0 || j == 4) {
+        b = csub(a, u);
+        a = cadd(a, u);
+        return;
+    }
+    const R c = cos16<R>(j), s = INV ? sin16<R>(j) : -sin16<R>(j);
+    R f;                                     // the factor taken out
+    if (j < 3 || j > 5) {                    // |cos| >= |sin|
+        const R r = R((INV ? 1.0 : -1.0) * (j == 1 ? TAN8 : j == 2 ? 1.0 : j == 6 ? -1.0 : -TAN8));
+        u = T{b.x - r * b.y, b.y + r * b.x};
+        f = c;
+    } else {                                 // j = 3, 5: w b = s (r b.x - b.y, r b.y + b.x)
+        const R r = R((INV ? 1.0 : -1.0) * (j == 3 ? TAN8 : -TAN8));
+        u = T{r * b.x - b.y, r * b.y + b.x};
+        f = s;
+    }
+    b = T{a.x - f * u.x, a.y - f * u.y};
+    a = T{a.x + f * u.x, a.y + f * u.y};
 }
 
 // One radix-2 stage (butterfly span LEN) of an in-register DIT DFT, then the next stage.  The
@@ -68,10 +102,7 @@ __device__ __forceinline__ void dft_stage(T (&x)[P])
     for (int s0 = 0; s0 < P; s0 += LEN) {
 #pragma unroll
         for (int m = 0; m < HALF; ++m) {
-            const T b = twiddle16<INV>(x[s0 + m + HALF], m * (16 / LEN));
-            const T a = x[s0 + m];
-            x[s0 + m] = cadd(a, b);
-            x[s0 + m + HALF] = csub(a, b);
+            butterfly<INV>(x[s0 + m], x[s0 + m + HALF], m * (16 / LEN));
         }
     }
     if constexpr (LEN < P) dft_stage<P, 2 * LEN, INV>(x);
@@ -102,7 +133,6 @@ template <> struct Split<16> { static constexpr int N1 = 4, N2 = 4; };
 template <> struct Split<32> { static constexpr int N1 = 8, N2 = 4; };
 template <> struct Split<64> { static constexpr int N1 = 8, N2 = 8; };
 template <> struct Split<128> { static constexpr int N1 = 16, N2 = 8; };
-template <> struct Split<256> { static constexpr int N1 = 16, N2 = 16; };
 
 // FFTs of `lines` lines of N points held in shared memory; element j of line l is at
 // buf[idx(l, j)].  All threads of the block call this; lines are spread over warps with the
@@ -154,6 +184,41 @@ __device__ __forceinline__ void lines_fft(T* buf, int lines, Idx idx, const T* _
     }
 }
 
+// 256-point lines (16 x 16) whose element j is at (j + (j >> 4)) CL from the line's first, CL a
+// compile-time stride: every element of thread t is then a base plus a compile-time offset
+// (16 n + t at 17 n + t, 16 t + n at 17 t + n), so the transform spends no instructions on
+// indexing.  (With run-time layouts the 256^3 passes issued 145 instructions a point, 43% of
+// them integer.)  The 32 lanes of a warp are lane = 2 t + line of two consecutive lines.
+constexpr int LINE256 = 272;                    // elements of a padded line
+__device__ __forceinline__ int pad256(int j) { return j + (j >> 4); }
+template <bool INV, int CL, typename T>
+__device__ __forceinline__ void line256(T* line, int t, const T* __restrict__ tw)
+{
+    T* b1 = line + t * CL;
+    const T* b2 = line + 17 * CL * t;
+    T a[16];
+#pragma unroll
+    for (int n = 0; n < 16; ++n) a[n] = b1[17 * CL * n];
+    reg_dft<16, INV>(a);
+#pragma unroll
+    for (int k = 1; k < 16; ++k) {
+        T w = tw[t * k];
+        if (INV) w.y = -w.y;
+        a[k] = cm(a[k], w);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) b1[17 * CL * k] = a[k];
+    __syncwarp();
+#pragma unroll
+    for (int n = 0; n < 16; ++n) a[n] = b2[CL * n];
+    reg_dft<16, INV>(a);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) b1[17 * CL * k] = a[k];
+    __syncwarp();
+}
+
 template <bool INV, typename T, typename Idx>
 __device__ __forceinline__ void lines_fft_n(int n, T* buf, int lines, Idx idx, const T* tw)
 {
@@ -163,8 +228,7 @@ __device__ __forceinline__ void lines_fft_n(int n, T* buf, int lines, Idx idx, c
     case 16: lines_fft<16, INV>(buf, lines, idx, tw); break;
     case 32: lines_fft<32, INV>(buf, lines, idx, tw); break;
     case 64: lines_fft<64, INV>(buf, lines, idx, tw); break;
-    case 128: lines_fft<128, INV>(buf, lines, idx, tw); break;
-    default: lines_fft<256, INV>(buf, lines, idx, tw); break;
+    default: lines_fft<128, INV>(buf, lines, idx, tw); break;
     }
 }
 
@@ -209,5 +273,57 @@ __device__ __forceinline__ void store4(double* p, const double v[4])
     reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
     reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
 }
+// Adds mih D.T (mih = -1/h) on the faces of component `comp` at the cells x0 .. x0+3 of the rows
+// (y0, z) and (y0 + 1, z) to r0 and r1: T is the staggered stress [9][N] of kernels_noise.cu,
+// backward differences of T_aa, forward ones of T_ab.
+template <typename R>
+__device__ __forceinline__ void stress_rows(const R* __restrict__ T, int comp, const GridGeo& g,
+                                            int x0, int y0, int z, R mih, R r0[4], R r1[4])
+{
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const int zr = z * ny, o0 = (zr + y0) * nx, o1 = o0 + nx;
+    R c0[4], c1[4], e[4];
+    {
+        const R* t = T + (size_t)(3 * comp) * g.N;
+        load4(t + o0 + x0, c0);
+        load4(t + o1 + x0, c1);
+        const bool back = comp == 0;
+        const int xn = back ? (x0 - 1) & (nx - 1) : (x0 + 4) & (nx - 1);
+        const R n0 = t[o0 + xn], n1 = t[o1 + xn];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const R d0 = back ? c0[i] - (i == 0 ? n0 : c0[i - 1]) : (i == 3 ? n0 : c0[i + 1]) - c0[i];
+            const R d1 = back ? c1[i] - (i == 0 ? n1 : c1[i - 1]) : (i == 3 ? n1 : c1[i + 1]) - c1[i];
+            r0[i] += mih * d0;
+            r1[i] += mih * d1;
+        }
+    }
+    {
+        const R* t = T + (size_t)(3 * comp + 1) * g.N;
+        const bool back = comp == 1;
+        load4(t + o0 + x0, c0);
+        load4(t + o1 + x0, c1);
+        load4(t + (zr + ((back ? y0 - 1 : y0 + 2) & (ny - 1))) * nx + x0, e);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            r0[i] += mih * (back ? c0[i] - e[i] : c1[i] - c0[i]);
+            r1[i] += mih * (back ? c1[i] - c0[i] : e[i] - c1[i]);
+        }
+    }
+    {
+        const R* t = T + (size_t)(3 * comp + 2) * g.N;
+        const bool back = comp == 2;
+        const int zn = (((back ? z - 1 : z + 1) & (nz - 1)) * ny + y0) * nx + x0;
+        load4(t + o0 + x0, c0);
+        load4(t + zn, e);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r0[i] += mih * (back ? c0[i] - e[i] : e[i] - c0[i]);
+        load4(t + o1 + x0, c1);
+        load4(t + zn + nx, e);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r1[i] += mih * (back ? c1[i] - e[i] : e[i] - c1[i]);
+    }
+}
+
 }  // namespace
 }  // namespace mbk

@@ -150,7 +150,7 @@ template <> struct PlaneSlots<Skew128> { static size_t count(int, int) { return 
 // Pass A.  Plane buffer P[p][pad(j)], p < ny/2: first rows 2p, 2p+1 packed as re + i im; after
 // the row FFT and the in-place separation, logical slot 2k + e of row p holds X_{2p+e}[k],
 // k <= nx/2.  pad(j) = j + (j >> pad_shift(nx)).
-template <typename L>
+template <typename L, bool STRESS>
 __global__ void __launch_bounds__(256, 3)
 k_plane_fwd(FluidArgs<float> a, GridGeo g)
 {
@@ -247,6 +247,8 @@ k_plane_fwd(FluidArgs<float> a, GridGeo g)
                 store4(pclr + (size_t)y1 * nx + x0, zero);
             }
         }
+        if (STRESS)
+            stress_rows(a.W + (size_t)(bc / 3) * 9 * g.N, comp, g, x0, y0, z, -a.inv_h32, r0, r1);
         if (body) {
             for (int i = 0; i < 4; ++i) {
                 const int x = x0 + i;
@@ -258,6 +260,8 @@ k_plane_fwd(FluidArgs<float> a, GridGeo g)
         for (int i = 0; i < 4; ++i) rowp[lay.off(x0 + i)] = float2{r0[i], r1[i]};
     }
     __syncthreads();
+    if (STRESS && a.step_index && (blockIdx.x | blockIdx.y | threadIdx.x) == 0)
+        *a.step_index += 1;                // the stress of this step has been drawn
     lay.template rows<false>(P, twx);
     __syncthreads();
     // separate the two real rows of each packed row (one warp per packed row, in place)
@@ -633,11 +637,13 @@ cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const Flu
     static std::atomic<unsigned> attr{0};     // per instantiation
     if (first_on_device(attr)) {
         const int lim = 200 * 1024;
-        cudaFuncSetAttribute(k_plane_fwd<PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_fwd<PadPlane, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_fwd<PadPlane, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zsolve<CZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zsolve<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_plane_inv<PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_fwd<Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_fwd<Skew128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_plane_fwd<Skew128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_plane_inv<Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     }
     // FP32 planes of 128 x 128 take the conflict-free layout (MB_PLANE_LAYOUT=pad keeps the
@@ -655,8 +661,9 @@ cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const Flu
     mark(0);
     cudaError_t e;
     const dim3 gp(nz, 3 * B), gz(ny / C, nxh, B);
-    if (skew) e = launch_dep(k_plane_fwd<Skew128>, gp, dim3(PT), smem_plane, st, a, g);
-    else e = launch_dep(k_plane_fwd<PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
+    auto fwd = a.W ? (skew ? k_plane_fwd<Skew128, true> : k_plane_fwd<PadPlane, true>)
+                   : (skew ? k_plane_fwd<Skew128, false> : k_plane_fwd<PadPlane, false>);
+    e = launch_dep(fwd, gp, dim3(PT), smem_plane, st, a, g);
     if (e != cudaSuccess) return e;
     mark(1);
     mark(2);

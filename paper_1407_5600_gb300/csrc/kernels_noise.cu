@@ -19,10 +19,12 @@
 // v_a averaged along b times v_b averaged along a (the conservative centred form), explicit
 // at v^n, so one divergence serves both stresses.
 //
-// Two launches per step: k_stress forms sigma~ + rho v v into a [B][9][N] buffer (one thread
-// per group of four cells, each Philox block computed once, vector stores), k_stress_div adds -D.(sigma~ + rho v v) to the force-density grid
-// and advances the step index held in device memory (when drawing noise), so captured CUDA
-// graphs draw fresh noise on every replay.
+// k_stress forms sigma~ + rho v v into a [B][9][N] buffer (one thread per group of four cells,
+// each Philox block computed once, vector stores).  Its divergence joins the right-hand side in
+// the first FFT pass (stress_rows), which also advances the step index held in device memory
+// (when drawing noise), so captured CUDA graphs draw fresh noise on every replay.  The FP64
+// three-pass FFT, whose first pass is bound by arithmetic, takes it from k_stress_div instead,
+// through the force-density grid.
 #include "mb_internal.cuh"
 #include "fft_lines.cuh"
 
@@ -120,7 +122,7 @@ __device__ __forceinline__ void convective(const GridGeo& g, const R* __restrict
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
 k_stress(int B, GridGeo g, uint64_t seed, const uint64_t* __restrict__ step_index, R amp,
          const R* __restrict__ v, R rho, R* __restrict__ W)
 {
@@ -248,10 +250,10 @@ cudaError_t launch_fluid_stress(cudaStream_t st, int B, const GridGeo& g, uint64
 {
     const int64_t total = (int64_t)B * g.N;
     if (total <= 0) return cudaSuccess;
-    const unsigned blocks = noise_blocks(total);
+    const unsigned blocks = noise_blocks(total / 4);           // four cells a thread
     if (parts & 1) k_stress<R><<<blocks, 256, 0, st>>>(B, g, seed, step_index, R(amp), v, R(rho), W);
-    if (parts & 2)
-        k_stress_div<R><<<blocks, 256, 0, st>>>(B, g, W, f, accumulate ? 1 : 0,
+    if constexpr (sizeof(R) == 8)
+        if (parts & 2) k_stress_div<R><<<blocks, 256, 0, st>>>(B, g, W, f, accumulate ? 1 : 0,
                                                 amp != 0.0 ? step_index : nullptr);
     return cudaGetLastError();
 }

@@ -768,6 +768,13 @@ FluidArgs<R> fluid_args(mb_ctx* ctx, const void* v, const void* f, void* v_out,
     return a;
 }
 
+// The step's stress in W joins the right-hand side of the FFT's first pass.
+template <typename R> void set_stress(mb_ctx* ctx, FluidArgs<R>& a)
+{
+    a.W = static_cast<const R*>(ctx->W.p);
+    a.step_index = ctx->thermal ? static_cast<uint64_t*>(ctx->step_index.p) : nullptr;
+}
+
 // Accumulates the stage times of every recorded step (waits for the last one).
 mb_status drain_stage_events(mb_ctx* ctx)
 {
@@ -942,18 +949,22 @@ mb_status do_step64(mb_ctx* ctx, const double* ext, const double* body)
     mark(ST_SPREAD);
     if (blobs) MB_TRY(spread64(ctx, qh, det));
     mark(ST_STRESS);
-    const bool stress = ctx->thermal || ctx->advect;
+    // thermal and convective stress: its divergence joins the five-pass right-hand side, or goes
+    // through f for the three-pass one
+    const bool stress = ctx->thermal || ctx->advect, through_f = stress && ctx->fft_passes == 3;
     if (stress) {
         MB_CUDA(launch_fluid_stress<double>(st, B, g, ctx->d.seed,
                                             static_cast<uint64_t*>(ctx->step_index.p),
                                             ctx->thermal_amp, ctx->advect ? vcur : nullptr,
                                             ctx->d.rho, static_cast<double*>(ctx->W.p),
-                                            static_cast<double*>(ctx->f.p), blobs));
-        ctx->launches += STRESS_KERNELS;
+                                            static_cast<double*>(ctx->f.p), blobs,
+                                            through_f ? 3 : 1));
+        ctx->launches += through_f ? 2 : 1;
     }
     const double* mean = ctx->d.mean_mode == 0 ? static_cast<const double*>(ctx->vbar.p) : nullptr;
-    FluidArgs<double> fa = fluid_args<double>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr,
+    FluidArgs<double> fa = fluid_args<double>(ctx, vcur, blobs || through_f ? ctx->f.p : nullptr,
                                               vnext, ctx->body_prof.p, body, mean);
+    if (stress && !through_f) set_stress(ctx, fa);
     const bool vsum = blobs && ctx->vsum.p != nullptr;
     if (vsum) {
         fa.v_sum_base = vcur;
@@ -1137,8 +1148,8 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
             MB_CUDA(launch_fluid_stress<float>(ctx->side, B, g, ctx->d.seed,
                                                static_cast<uint64_t*>(ctx->step_index.p),
                                                ctx->thermal_amp, ctx->advect ? vcur : nullptr,
-                                               ctx->d.rho, static_cast<float*>(ctx->W.p),
-                                               static_cast<float*>(ctx->f.p), blobs, 1));
+                                               ctx->d.rho, static_cast<float*>(ctx->W.p), nullptr,
+                                               false, 1));
             MB_CUDA(cudaEventRecord(ctx->fork[2], ctx->side));
         }
     }
@@ -1208,17 +1219,19 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
     mark(ST_STRESS);
     const bool stress = ctx->thermal || ctx->advect;
     if (stress) {
-        if (overlap) MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[2], 0));
-        MB_CUDA(launch_fluid_stress<float>(st, B, g, ctx->d.seed,
-                                           static_cast<uint64_t*>(ctx->step_index.p),
-                                           ctx->thermal_amp, ctx->advect ? vcur : nullptr,
-                                           ctx->d.rho, static_cast<float*>(ctx->W.p),
-                                           static_cast<float*>(ctx->f.p), blobs,
-                                           overlap ? 2 : 3));
-        ctx->launches += STRESS_KERNELS;
+        if (overlap)
+            MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[2], 0));
+        else
+            MB_CUDA(launch_fluid_stress<float>(st, B, g, ctx->d.seed,
+                                               static_cast<uint64_t*>(ctx->step_index.p),
+                                               ctx->thermal_amp, ctx->advect ? vcur : nullptr,
+                                               ctx->d.rho, static_cast<float*>(ctx->W.p), nullptr,
+                                               false, 1));
+        ctx->launches += 1;
     }
-    FluidArgs<float> fa = fluid_args<float>(ctx, vcur, blobs || stress ? ctx->f.p : nullptr,
+    FluidArgs<float> fa = fluid_args<float>(ctx, vcur, blobs ? ctx->f.p : nullptr,
                                             vnext, ctx->body_prof.p, body, nullptr);
+    if (stress) set_stress(ctx, fa);
     if (ctx->d.mean_mode == 0) {
         const double L3 = g.L[0] * g.L[1] * g.L[2];
         if (ctx->fft_passes == 3) {
@@ -1821,7 +1834,8 @@ mb_status mb_create_grid(const mb_grid_desc* desc, void* cuda_stream, mb_ctx** o
         return s;
     };
     const size_t gb = grid_bytes(ctx, ctx->B);
-    const size_t sb = (size_t)ctx->B * 3 * ns[2] * ns[1] * ctx->nxh * 2 * ctx->rsz;
+    const size_t sb = (size_t)ctx->B * 3 * ns[2] * ns[1] *
+                      (ctx->fft_passes == 5 ? spec_row(ns[0]) : ctx->nxh) * 2 * ctx->rsz;
     mb_status s;
     if ((s = ensure(ctx->v[0], gb, ctx->err, "v")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->v[1], gb, ctx->err, "v")) != MB_OK) return fail(s);
@@ -2551,23 +2565,28 @@ mb_status mb_fluid_update(mb_ctx* ctx, const void* v_in, const void* f, const do
     const void *vd = nullptr, *fd = nullptr;
     if (!stokes) MB_TRY(stage_in(ctx, v_in, by, ctx->s_g1, &vd, "v_in"));
     if (f) MB_TRY(stage_in(ctx, f, by, ctx->s_g2, &fd, "f"));
+    // - rho D.(v_in v_in): from the stress itself in the first FFT pass, or for the FP64 three-pass
+    // FFT through the library's own copy of f (the caller's f is not written)
+    const bool through_f = ctx->advect && ctx->rsz == 8 && ctx->fft_passes == 3;
     if (ctx->advect) {
-        // f - rho D.(v_in v_in) in the library's own copy (the caller's f is not written)
-        MB_TRY(ensure(ctx->s_g2, by, ctx->err, "f"));
-        if (fd && fd != ctx->s_g2.p)
-            MB_CUDA(cudaMemcpyAsync(ctx->s_g2.p, fd, by, cudaMemcpyDeviceToDevice, ctx->st));
         MB_TRY(ensure(ctx->W, 3 * by, ctx->err, "fluid stress"));
-        if (ctx->rsz == 4)
+        if (ctx->rsz == 4) {
             MB_CUDA(launch_fluid_stress<float>(ctx->st, 1, ctx->g, 0, nullptr, 0.0,
                                                static_cast<const float*>(vd), ctx->d.rho,
-                                               static_cast<float*>(ctx->W.p),
-                                               static_cast<float*>(ctx->s_g2.p), fd != nullptr));
-        else
+                                               static_cast<float*>(ctx->W.p), nullptr, false, 1));
+        } else {
+            if (through_f) {
+                MB_TRY(ensure(ctx->s_g2, by, ctx->err, "f"));
+                if (fd && fd != ctx->s_g2.p)
+                    MB_CUDA(cudaMemcpyAsync(ctx->s_g2.p, fd, by, cudaMemcpyDeviceToDevice, ctx->st));
+            }
             MB_CUDA(launch_fluid_stress<double>(ctx->st, 1, ctx->g, 0, nullptr, 0.0,
                                                 static_cast<const double*>(vd), ctx->d.rho,
                                                 static_cast<double*>(ctx->W.p),
-                                                static_cast<double*>(ctx->s_g2.p), fd != nullptr));
-        fd = ctx->s_g2.p;
+                                                static_cast<double*>(ctx->s_g2.p), fd != nullptr,
+                                                through_f ? 3 : 1));
+            if (through_f) fd = ctx->s_g2.p;
+        }
     }
     if (body_force) MB_TRY(set_body(ctx, body_force, ctx->prof_scratch, false));
     void* dst;
@@ -2582,11 +2601,13 @@ mb_status mb_fluid_update(mb_ctx* ctx, const void* v_in, const void* f, const do
     if (ctx->rsz == 4) {
         FluidArgs<float> a = fluid_args<float>(ctx, vd, fd, dst, ctx->prof_scratch.p, body_force, nullptr);
         if (stokes) stokes_args(a);
+        if (ctx->advect) a.W = static_cast<const float*>(ctx->W.p);
         if (ctx->fft_passes == 5) MB_CUDA(launch_fluid<float>(ctx->st, 1, ctx->g, a));
         else MB_CUDA(launch_fluid3<float>(ctx->st, 1, ctx->g, a));
     } else {
         FluidArgs<double> a = fluid_args<double>(ctx, vd, fd, dst, ctx->prof_scratch.p, body_force, nullptr);
         if (stokes) stokes_args(a);
+        if (ctx->advect && !through_f) a.W = static_cast<const double*>(ctx->W.p);
         if (ctx->fft_passes == 5) MB_CUDA(launch_fluid<double>(ctx->st, 1, ctx->g, a));
         else MB_CUDA(launch_fluid3<double>(ctx->st, 1, ctx->g, a));
     }

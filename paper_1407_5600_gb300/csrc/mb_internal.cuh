@@ -172,12 +172,15 @@ cudaError_t launch_particle_mean_adjoint(cudaStream_t st, int64_t np, const int3
                                          const int32_t* part_blobs, const double* gU,
                                          double* gu);
 
+// Values in a row of the five-pass spectrum: nx/2 + 1 rounded up to whole 64-byte runs.
+__host__ __device__ inline int spec_row(int nx) { return (nx / 2 + 8) & ~7; }
+
 // Fluid update pipeline on B boxes.
 template <typename R>
 struct FluidArgs {
     const R* v;            // [B][3][N]
     const R* f;            // [B][3][N] or null
-    typename C2<R>::T* spec;   // [B][3][nz][ny][nx/2+1]
+    typename C2<R>::T* spec;   // half spectrum; five passes: [B][3][nz][ny][spec_row(nx)]
     R* v_out;
     const R* tw[3];        // twiddles per dimension, n/2 complex each (interleaved re, im)
     const R* twf[3];       // full tables W_n^j, j < n, per dimension (interleaved re, im)
@@ -204,7 +207,11 @@ struct FluidArgs {
     double* mean_state;
     const double* mean_force;
     double mean_scale;
-    int no_v;              // three-pass FFT: right-hand side f (+ body) only (Stokes limit)
+    int no_v;              // right-hand side f (+ body) only (Stokes limit)
+    // fluid stress [B][9][N] whose divergence -D.W joins the right-hand side (not in the FP64
+    // three-pass FFT), and the step index it was drawn with, advanced then; either may be null
+    const R* W;
+    uint64_t* step_index;
 };
 // marks: null, or 6 events recorded before pass 1 and after each of the 5 passes.
 // The derived launch constants of a FluidArgs (1/h, 1/h^2, 1/N and the float roundings), set
@@ -294,7 +301,8 @@ constexpr int FLUID3_KERNELS = 3;
 
 // Thermal and convective stress (kernels_noise.cu): W = amp * normals of step *step_index
 // (amp != 0) + rho v v (v != NULL) [parts & 1], then f (+)= -D.W and *step_index += 1
-// (amp != 0) [parts & 2].  W is [B][9][N], v and f [B][3][N].
+// (amp != 0) [parts & 2, FP64 only].  parts & 4: other kernels run beside it.  W is [B][9][N],
+// v and f [B][3][N].
 template <typename R>
 cudaError_t launch_fluid_stress(cudaStream_t st, int B, const GridGeo& g, uint64_t seed,
                                 uint64_t* step_index, double amp, const R* v, double rho, R* W,
