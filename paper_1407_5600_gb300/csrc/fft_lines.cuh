@@ -133,6 +133,7 @@ template <> struct Split<16> { static constexpr int N1 = 4, N2 = 4; };
 template <> struct Split<32> { static constexpr int N1 = 8, N2 = 4; };
 template <> struct Split<64> { static constexpr int N1 = 8, N2 = 8; };
 template <> struct Split<128> { static constexpr int N1 = 16, N2 = 8; };
+template <> struct Split<256> { static constexpr int N1 = 16, N2 = 16; };
 
 // FFTs of `lines` lines of N points held in shared memory; element j of line l is at
 // buf[idx(l, j)].  All threads of the block call this; lines are spread over warps with the
@@ -184,39 +185,56 @@ __device__ __forceinline__ void lines_fft(T* buf, int lines, Idx idx, const T* _
     }
 }
 
-// 256-point lines (16 x 16) whose element j is at (j + (j >> 4)) CL from the line's first, CL a
-// compile-time stride: every element of thread t is then a base plus a compile-time offset
-// (16 n + t at 17 n + t, 16 t + n at 17 t + n), so the transform spends no instructions on
-// indexing.  (With run-time layouts the 256^3 passes issued 145 instructions a point, 43% of
-// them integer.)  The 32 lanes of a warp are lane = 2 t + line of two consecutive lines.
-constexpr int LINE256 = 272;                    // elements of a padded line
-__device__ __forceinline__ int pad256(int j) { return j + (j >> 4); }
-template <bool INV, int CL, typename T>
-__device__ __forceinline__ void line256(T* line, int t, const T* __restrict__ tw)
+// One line of N = N1 N2 points at compile-time offsets: thread t (of N2) finds element N2 n1 + t
+// at b1[c1(n1)], element (t + N2 m) N2 + n2 at b2[c2(m, n2)] and element t + N2 m + N1 k2 at
+// b1[c3(m, k2)], so the transform spends no instructions on indexing.  (With run-time layouts the
+// 256^3 passes issued 145 instructions a point, 43% of them integer.)
+template <int N, bool INV, typename T, typename F1, typename F2, typename F3>
+__device__ __forceinline__ void line_core(T* b1, const T* b2, int t, const T* __restrict__ tw, F1 c1,
+                                          F2 c2, F3 c3)
 {
-    T* b1 = line + t * CL;
-    const T* b2 = line + 17 * CL * t;
-    T a[16];
+    constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, M = N1 / N2;
+    T a[N1];
 #pragma unroll
-    for (int n = 0; n < 16; ++n) a[n] = b1[17 * CL * n];
-    reg_dft<16, INV>(a);
+    for (int n = 0; n < N1; ++n) a[n] = b1[c1(n)];
+    reg_dft<N1, INV>(a);
 #pragma unroll
-    for (int k = 1; k < 16; ++k) {
-        T w = tw[t * k];
+    for (int k = 1; k < N1; ++k) {
+        T w = tw[(t * k) & (N - 1)];
         if (INV) w.y = -w.y;
         a[k] = cm(a[k], w);
     }
     __syncwarp();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) b1[17 * CL * k] = a[k];
+    for (int k = 0; k < N1; ++k) b1[c1(k)] = a[k];
+    __syncwarp();
+    T b[M][N2];
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int n = 0; n < N2; ++n) b[m][n] = b2[c2(m, n)];
+#pragma unroll
+    for (int m = 0; m < M; ++m) reg_dft<N2, INV>(b[m]);
     __syncwarp();
 #pragma unroll
-    for (int n = 0; n < 16; ++n) a[n] = b2[CL * n];
-    reg_dft<16, INV>(a);
-    __syncwarp();
+    for (int m = 0; m < M; ++m)
 #pragma unroll
-    for (int k = 0; k < 16; ++k) b1[17 * CL * k] = a[k];
+        for (int k = 0; k < N2; ++k) b1[c3(m, k)] = b[m][k];
     __syncwarp();
+}
+
+// Lines whose element j is at (j + j / N2) CL from the line's first, CL a compile-time stride:
+// N2 n + t at (N2 + 1) n + t, and so on.
+template <int N> __host__ __device__ constexpr int padded_line() { return N + N / Split<N>::N2; }
+template <int N> __host__ __device__ __forceinline__ int pad_line(int j) { return j + j / Split<N>::N2; }
+template <int N, bool INV, int CL, typename T>
+__device__ __forceinline__ void line_fft(T* line, int t, const T* __restrict__ tw)
+{
+    constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
+    line_core<N, INV>(
+        line + t * CL, line + (N2 + 1) * CL * t, t, tw, [](int n) { return (N2 + 1) * CL * n; },
+        [](int m, int n) { return ((N2 + 1) * N2 * m + n) * CL; },
+        [](int m, int k) { return (N2 + 1) * (m + N1 / N2 * k) * CL; });
 }
 
 template <bool INV, typename T, typename Idx>

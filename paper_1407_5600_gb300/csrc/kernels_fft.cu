@@ -17,7 +17,7 @@
 // on a sector: at nx/2 + 1 values a row a chunk of 8 touched three sectors instead of two.  A
 // block has as many threads as its lines need (n / N1 each, lines_threads): with 256 threads
 // whatever the sides, the 64-point passes left six of eight warps without a line.  256-point
-// lines have layouts of their own with compile-time offsets (line256).  Times before and after:
+// lines have layouts of their own with compile-time offsets (line_fft).  Times before and after:
 // FP32 256^3 rhs (with the stress divergence, a pass of its own before) 165 + 180 -> 250 us,
 // y 134 -> 78, z and solve 275 -> 167, c2r 196 -> 110; FP64 256 x 64 x 64 800 -> 582 us in all.
 #include "mb_internal.cuh"
@@ -64,7 +64,7 @@ k_rhs_fft_x(FluidArgs<R> a, GridGeo g, int RP)
     T* sb = reinterpret_cast<T*>(smem_raw);
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], ld_s = spec_row(nx);
     const int sx = pad_shift(nx), ld = L256 ? Lay256<R>::ROW : padded_len(nx) + 1;
-    auto px = [sx](int j) { return L256 ? pad256(j) : pj(j, sx); };
+    auto px = [sx](int j) { return L256 ? pad_line<256>(j) : pj(j, sx); };
     const int yp0 = blockIdx.x * RP;
     const int z = blockIdx.y;
     const int bc = blockIdx.z;
@@ -134,7 +134,7 @@ k_rhs_fft_x(FluidArgs<R> a, GridGeo g, int RP)
     }
     __syncthreads();
     if constexpr (L256)
-        line256<false, 1>(sb + (2 * (threadIdx.x >> 5) + (threadIdx.x & 1)) * ld, (threadIdx.x & 31) >> 1,
+        line_fft<256, false, 1>(sb + (2 * (threadIdx.x >> 5) + (threadIdx.x & 1)) * ld, (threadIdx.x & 31) >> 1,
                        reinterpret_cast<const T*>(a.twf[0]));
     else
         lines_fft_n<false>(nx, sb, RP, [ld, sx](int l, int j) { return l * ld + pj(j, sx); },
@@ -171,7 +171,7 @@ k_fft_y(typename C2<R>::T* spec, const R* twy, GridGeo g, int lc)
     const int C = 1 << lc, kx0 = blockIdx.x * C;
     const int cw = min(C, nxh - kx0);
     const int sy = pad_shift(ny), CL = L256 ? Lay256<R>::YS : C + 1;
-    auto at = [=](int y, int c) { return (L256 ? pad256(y) : pj(y, sy)) * CL + c; };
+    auto at = [=](int y, int c) { return (L256 ? pad_line<256>(y) : pj(y, sy)) * CL + c; };
     T* plane = spec + ((size_t)blockIdx.z * nz + blockIdx.y) * (size_t)ny * ld_s + kx0;
     // every copy of a thread in flight at once (columns past the last kx are transformed as
     // garbage and not stored).  256 points, sixteen threads a column: a thread's elements y0 + 16 j
@@ -194,7 +194,7 @@ k_fft_y(typename C2<R>::T* spec, const R* twy, GridGeo g, int lc)
     __syncthreads();
     const T* tw = reinterpret_cast<const T*>(twy);
     if constexpr (L256)
-        line256<INV, Lay256<R>::YS>(sb + 2 * (threadIdx.x >> 5) + (threadIdx.x & 1),
+        line_fft<256, INV, Lay256<R>::YS>(sb + 2 * (threadIdx.x >> 5) + (threadIdx.x & 1),
                                     (threadIdx.x & 31) >> 1, tw);
     else
         lines_fft_n<INV>(ny, sb, C, [CL, sy](int l, int j) { return pj(j, sy) * CL + l; }, tw);
@@ -233,8 +233,8 @@ k_fft_z_solve(FluidArgs<R> a, GridGeo g, int LC)
     T* col[3];
     for (int c = 0; c < 3; ++c)
         col[c] = a.spec + ((size_t)(box * 3 + c) * nz) * zstride + (size_t)ky * ld_s + kx0;
-    const int sz = pad_shift(nz), PZ = L256 ? LINE256 : padded_len(nz), CL = L256 ? Lay256<R>::ZS : C + 1;
-    auto at = [=](int c, int z, int k) { return (c * PZ + (L256 ? pad256(z) : pj(z, sz))) * CL + k; };
+    const int sz = pad_shift(nz), PZ = L256 ? padded_line<256>() : padded_len(nz), CL = L256 ? Lay256<R>::ZS : C + 1;
+    auto at = [=](int c, int z, int k) { return (c * PZ + (L256 ? pad_line<256>(z) : pj(z, sz))) * CL + k; };
     // z twiddles in shared memory, after the three component columns (ready at the barrier
     // that follows the column copies)
     T* twz = sb + 3 * PZ * CL;
@@ -245,7 +245,7 @@ k_fft_z_solve(FluidArgs<R> a, GridGeo g, int LC)
     // 256 points: thread (row r = tid / CZ, column k) moves the elements z = r % 16 + 16 j of
     // component r / 16, at fixed strides on both sides
     const int fk = threadIdx.x & (Lay256<R>::CZ - 1), fr = threadIdx.x >> Lay256<R>::ZL;
-    T* fs = sb + ((fr >> 4) * LINE256 + (fr & 15)) * Lay256<R>::ZS + fk;
+    T* fs = sb + ((fr >> 4) * padded_line<256>() + (fr & 15)) * Lay256<R>::ZS + fk;
     T* fg = a.spec + ((size_t)(box * 3 + (fr >> 4)) * nz + (fr & 15)) * zstride + (size_t)ky * ld_s + kx0 + fk;
     if constexpr (L256) {
         if (fk < cw) {
@@ -264,8 +264,8 @@ k_fft_z_solve(FluidArgs<R> a, GridGeo g, int LC)
     // 256 points: two lines a warp
     auto idx = [=](int l, int j) { return at(l >> LC, j, l & (C - 1)); };
     const int l2 = 2 * (threadIdx.x >> 5) + (threadIdx.x & 1);
-    T* mine = sb + (l2 >> Lay256<R>::ZL) * (LINE256 * Lay256<R>::ZS) + (l2 & (Lay256<R>::CZ - 1));
-    if constexpr (L256) line256<false, Lay256<R>::ZS>(mine, (threadIdx.x & 31) >> 1, twz);
+    T* mine = sb + (l2 >> Lay256<R>::ZL) * (padded_line<256>() * Lay256<R>::ZS) + (l2 & (Lay256<R>::CZ - 1));
+    if constexpr (L256) line_fft<256, false, Lay256<R>::ZS>(mine, (threadIdx.x & 31) >> 1, twz);
     else lines_fft_n<false>(nz, sb, 3 * C, idx, twz);
     __syncthreads();
 
@@ -324,7 +324,7 @@ k_fft_z_solve(FluidArgs<R> a, GridGeo g, int LC)
         for (int c = 0; c < 3; ++c) sb[at(c, kz, k)] = W[c];
     }
     __syncthreads();
-    if constexpr (L256) line256<true, Lay256<R>::ZS>(mine, (threadIdx.x & 31) >> 1, twz);
+    if constexpr (L256) line_fft<256, true, Lay256<R>::ZS>(mine, (threadIdx.x & 31) >> 1, twz);
     else lines_fft_n<true>(nz, sb, 3 * C, idx, twz);
     __syncthreads();
     if constexpr (L256) {
@@ -351,7 +351,7 @@ k_fft_x_c2r(FluidArgs<R> a, GridGeo g, int RP)
     T* sb = reinterpret_cast<T*>(smem_raw);
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], ld_s = spec_row(nx);
     const int sx = pad_shift(nx), ld = L256 ? Lay256<R>::ROW : padded_len(nx) + 1;
-    auto px = [sx](int j) { return L256 ? pad256(j) : pj(j, sx); };
+    auto px = [sx](int j) { return L256 ? pad_line<256>(j) : pj(j, sx); };
     const int yp0 = blockIdx.x * RP;
     const int z = blockIdx.y;
     const int bc = blockIdx.z;
@@ -374,7 +374,7 @@ k_fft_x_c2r(FluidArgs<R> a, GridGeo g, int RP)
     }
     __syncthreads();
     if constexpr (L256)
-        line256<true, 1>(sb + (2 * (threadIdx.x >> 5) + (threadIdx.x & 1)) * ld, (threadIdx.x & 31) >> 1,
+        line_fft<256, true, 1>(sb + (2 * (threadIdx.x >> 5) + (threadIdx.x & 1)) * ld, (threadIdx.x & 31) >> 1,
                        reinterpret_cast<const T*>(a.twf[0]));
     else
         lines_fft_n<true>(nx, sb, RP, [ld, sx](int l, int j) { return l * ld + pj(j, sx); },
@@ -434,8 +434,8 @@ cudaError_t launch_fluid(cudaStream_t st, int B, const GridGeo& g, const FluidAr
     const int Cz = z256 ? L::CZ : lines_per_block(nz, 64, nxh);
     auto log2i = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
     const size_t smem_x = (size_t)RP * (x256 ? L::ROW : padded_len(nx) + 1) * sizeof(T);
-    const size_t smem_y = (y256 ? (size_t)LINE256 * L::YS : (size_t)padded_len(ny) * (Cy + 1)) * sizeof(T);
-    const size_t smem_z = ((z256 ? (size_t)3 * LINE256 * L::ZS : (size_t)3 * padded_len(nz) * (Cz + 1)) + nz) *
+    const size_t smem_y = (y256 ? (size_t)padded_line<256>() * L::YS : (size_t)padded_len(ny) * (Cy + 1)) * sizeof(T);
+    const size_t smem_z = ((z256 ? (size_t)3 * padded_line<256>() * L::ZS : (size_t)3 * padded_len(nz) * (Cz + 1)) + nz) *
                           sizeof(T);
     const dim3 gx(ny / 2 / RP, nz, 3 * B), gy((nxh + Cy - 1) / Cy, nz, 3 * B),
         gz((nxh + Cz - 1) / Cz, ny, B);

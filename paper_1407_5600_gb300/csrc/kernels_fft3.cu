@@ -14,6 +14,7 @@
 // Real rows are packed two per complex row and separated after the row transform.
 #include <cstdlib>
 #include <string>
+#include <type_traits>
 
 #include "mb_internal.cuh"
 #include "fft_lines.cuh"
@@ -142,16 +143,65 @@ struct Skew128 {
     }
 };
 
+// PlaneT: the other planes with sides of 32, 64 and 128, at compile-time offsets.  One pad slot
+// every N2 slots (of the row lines); rows differ by S = 4 (mod 16) slots, or 2 for 32-point rows,
+// and by a skew per N2/2 packed rows, so that the lanes of a half-warp (4 rows x 4 threads, 2
+// columns x 8) fall on different 8-byte banks in both stages of the line transforms.
+template <int NX, int NY> struct PlaneT {
+    static constexpr int X2 = Split<NX>::N2, Y2 = Split<NY>::N2, G = Y2 / 2;
+    static constexpr int RAW = NX + 2 + (NX + 1) / X2 + 14;                  // pads and skew
+    static constexpr int S = RAW + ((NX >= 64 ? 4 : 2) - RAW % 16 + 16) % 16;
+    static constexpr unsigned SKW = Y2 == 8 ? (NX >= 64 ? 0xDC985410u : 0x55441100u)
+                                            : (NX >= 64 ? 0x11001100u : 0u);
+    __host__ __device__ static constexpr int sk(int i) { return (int)((SKW >> (4 * (i & 7))) & 15u); }
+    __device__ PlaneT(int, int) {}
+    __device__ __forceinline__ int row(int p) const { return p * S + sk(p / G); }
+    __device__ __forceinline__ int off(int j) const { return j + j / X2; }
+    __device__ __forceinline__ int at(int p, int j) const { return row(p) + off(j); }
+    template <bool INV> __device__ __forceinline__ void rows(float2* P, const float2* tw) const
+    {
+        constexpr int LPW = 32 / X2;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        for (int l0 = warp * LPW; l0 < NY / 2; l0 += nw * LPW)
+            line_fft<NX, INV, 1>(P + row(l0 + lane % LPW), lane / LPW, tw);
+    }
+    template <bool INV> __device__ __forceinline__ void cols(float2* P, const float2* tw) const
+    {
+        constexpr int LPW = 32 / Y2, N1 = Split<NY>::N1;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        const int t = lane % Y2;
+        // element y of column k: slot 2k + (y & 1) of packed row y / 2
+        for (int k0 = warp * LPW; k0 < NX / 2; k0 += nw * LPW) {
+            const int c = off(2 * (k0 + lane / Y2));
+            line_core<NY, INV>(
+                P + (t >> 1) * S + (t & 1) + c, P + G * t * S + sk(t) + c, t, tw,
+                [](int n) { return G * n * S + sk(n); },
+                [](int m, int n) { return (G * Y2 * m + (n >> 1)) * S + (n & 1); },
+                [](int m, int k) { return (G * m + N1 / 2 * k) * S + sk(m + N1 / Y2 * k); });
+        }
+    }
+};
+
+// Blocks an SM: four (64 registers a thread) where no line is longer than 64 points (32 boxes of
+// 64^3: forward 100 -> 90 us); lines of 128 spill at that (64 x 128 x 32: 16.4 -> 18.4).
+template <typename L> struct PlaneBlocks { static constexpr int N = 3; };
+template <int NX, int NY> struct PlaneBlocks<PlaneT<NX, NY>> {
+    static constexpr int N = NX > 64 || NY > 64 ? 3 : 4;
+};
+
 template <typename L> struct PlaneSlots;
 template <> struct PlaneSlots<PadPlane> { static size_t count(int nx, int ny) { return (size_t)(ny / 2) * plane_ld(nx); } };
 template <> struct PlaneSlots<Skew128> { static size_t count(int, int) { return 64 * (size_t)Skew128::S; } };
+template <int NX, int NY> struct PlaneSlots<PlaneT<NX, NY>> {
+    static size_t count(int, int) { return (size_t)(NY / 2) * PlaneT<NX, NY>::S; }
+};
 
 // ------------------------------------------------------------------------------------------
 // Pass A.  Plane buffer P[p][pad(j)], p < ny/2: first rows 2p, 2p+1 packed as re + i im; after
 // the row FFT and the in-place separation, logical slot 2k + e of row p holds X_{2p+e}[k],
 // k <= nx/2.  pad(j) = j + (j >> pad_shift(nx)).
 template <typename L, bool STRESS>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, PlaneBlocks<L>::N)
 k_plane_fwd(FluidArgs<float> a, GridGeo g)
 {
     dep_wait();
@@ -171,8 +221,10 @@ k_plane_fwd(FluidArgs<float> a, GridGeo g)
     const float* pz = vc + (size_t)z * ny * nx;
     const float* pzp = vc + (size_t)((z + 1) & (nz - 1)) * ny * nx;
     const float* pzm = vc + (size_t)((z - 1) & (nz - 1)) * ny * nx;
-    const float* pf = fc ? fc + (size_t)z * ny * nx : nullptr;
-    float* pclr = a.f_clear && fc ? a.f_clear + (size_t)bc * g.N + (size_t)z * ny * nx : nullptr;
+    // planes that nothing was spread into are zero: neither read nor cleared
+    const bool spread = fc && !(a.f_dirty && a.f_dirty[(bc / 3) * nz + z] == 0);
+    const float* pf = spread ? fc + (size_t)z * ny * nx : nullptr;
+    float* pclr = a.f_clear && spread ? a.f_clear + (size_t)bc * g.N + (size_t)z * ny * nx : nullptr;
     // each work unit: 4 consecutive x of the two rows 2p, 2p+1
     const int qx = nx / 4, lq = 31 - __clz(qx);   // nx is a power of two
     for (int u = threadIdx.x; u < qx * (ny / 2) && a.no_v; u += blockDim.x) {
@@ -336,83 +388,45 @@ k_plane_fwd(FluidArgs<float> a, GridGeo g)
     }
 }
 
-// 128-point z-lines of the pass-B buffer (FP32, C = 8 columns): element z of line l (component
-// l / 8, column l % 8) is at ((l / 8) 144 + z + (z >> 3)) 12 + l % 8.  Same 16 x 8 split as
-// lines_fft; thread t of a line addresses a per-thread base plus compile-time offsets (z =
-// 8 n1 + t pads to 9 n1 + t, 8 (t + 8 m) + n2 to 9 t + 72 m + n2, t + 8 m + 16 k2 to
-// t + 9 m + 18 k2), so the transforms spend no instructions on indexing.
-template <bool INV>
-__device__ __forceinline__ void zlines128(float2* Bf, const float2* tw)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int sub = lane & 3, t = lane >> 2;
-    for (int l0 = warp * 4; l0 < 24; l0 += nw * 4) {
-        const int l = l0 + sub, c = l >> 3, k = l & 7;
-        float2* b1 = Bf + (c * 144 + t) * 12 + k;
-        float2* b2 = Bf + (c * 144 + 9 * t) * 12 + k;
-        float2 a[16];
-#pragma unroll
-        for (int n1 = 0; n1 < 16; ++n1) a[n1] = b1[108 * n1];
-        reg_dft<16, INV>(a);
-#pragma unroll
-        for (int k1 = 1; k1 < 16; ++k1) {
-            float2 w = tw[(t * k1) & 127];
-            if (INV) w.y = -w.y;
-            a[k1] = cm(a[k1], w);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < 16; ++k1) b1[108 * k1] = a[k1];
-        __syncwarp();
-        float2 b[2][8];
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int n2 = 0; n2 < 8; ++n2) b[m][n2] = b2[(72 * m + n2) * 12];
-#pragma unroll
-        for (int m = 0; m < 2; ++m) reg_dft<8, INV>(b[m]);
-        __syncwarp();
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2) b1[(9 * m + 18 * k2) * 12] = b[m][k2];
-        __syncwarp();
-    }
-}
-
 // ------------------------------------------------------------------------------------------
-// Pass B.  CTA = (ky block of width C, kx, box); shared buffer [3][pad(nz)][C + 4].  C is a
-// compile-time width (16 FP32, 8 FP64) and the block has 3 C N2 threads, one round of lines.
-template <int C>
+// Pass B.  CTA = (ky block of width C, kx, box).  NZ: the line length where the kernel has it at
+// compile time (NZ / N1 threads a line, 3 C of them one round; element z of component c, column k
+// at ((c * padded_line + z + z / N2) * CL + k), or 0 for any length, buffer [3][pad(nz)][C + 4].
+template <int C, int NZ>
 __global__ void __launch_bounds__(3 * C * 8, 768 / (3 * C * 8))
 k_zsolve(FluidArgs<float> a, GridGeo g)
 {
-    constexpr int Cp = C + 4;                    // 4 z-rows x 4 lines per half-warp: distinct banks
+    constexpr bool FIX = NZ != 0;
+    constexpr int NL = FIX ? NZ : 4, Z2 = Split<NL>::N2, ZP = padded_line<NL>();
+    // half-warps of 4 lines x 4 threads (strides of 12 slots) or 8 x 2 (8 slots) on different banks
+    constexpr int CL = FIX && Z2 == 4 ? 8 : C + 4, LPW = 32 / Z2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
+    const int nx = g.n[0], ny = g.n[1], nz = FIX ? NZ : g.n[2], nxh = nx / 2 + 1;
     const int lz = 31 - __clz(nz);
-    const int sz = pad_shift(nz), nzp = padded_len(nz);
+    const int sz = pad_shift(nz), nzp = FIX ? ZP : padded_len(nz);
     float2* Bf = reinterpret_cast<float2*>(smem_raw);
-    float2* twz = Bf + 3 * nzp * Cp;
+    float2* twz = Bf + 3 * nzp * CL;
     load_table(twz, reinterpret_cast<const float2*>(a.twk[2]), nz);   // set up once: no wait
     dep_wait();
     dep_release();
     const int ky0 = blockIdx.x * C, kx = blockIdx.y, box = blockIdx.z;
+    if (a.f_dirty && blockIdx.x == 0 && kx == 0)          // pass A has read them
+        for (int i = threadIdx.x; i < nz; i += blockDim.x) a.f_dirty[box * nz + i] = 0;
     const size_t zstride = (size_t)nxh * ny;
     const size_t cstride = (size_t)nz * zstride;
     float2* base = reinterpret_cast<float2*>(a.spec) + (size_t)(box * 3) * cstride + (size_t)kx * ny + ky0;
-    auto at = [=](int c, int z, int k) { return (c * nzp + z + (z >> sz)) * Cp + k; };
+    auto at = [=](int c, int z, int k) {
+        return (c * nzp + (FIX ? pad_line<NL>(z) : z + (z >> sz))) * CL + k;
+    };
     const int total = 3 * nz * C;
-    constexpr bool z128 = C == 8;
-    // 128-point z-lines with 192 threads: thread (zr = tid / 8, k = tid % 8) moves the elements
-    // (c = zr / 8, z = zr % 8 + 8 j, k), j < 16, at a fixed stride on both sides
-    const bool fast = z128 && nz == 128 && blockDim.x == 3 * 8 * C;
-    if (fast) {
-        const int k = threadIdx.x & 7, zr = threadIdx.x >> 3, c = zr >> 3, z0 = zr & 7;
-        float2* sb = Bf + (c * 144 + z0) * 12 + k;
-        const float2* gb = base + c * cstride + (size_t)z0 * zstride + k;
+    // compile-time lines: thread (row r = tid / C, column k) moves the elements z = r % N2 + N2 j of
+    // component r / N2, at fixed strides on both sides
+    const int fk = threadIdx.x % C, fr = threadIdx.x / C;
+    float2* fs = Bf + (fr / Z2 * ZP + fr % Z2) * CL + fk;
+    float2* fg = base + fr / Z2 * cstride + (size_t)(fr % Z2) * zstride + fk;
+    if constexpr (FIX) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) async_copy(sb + 108 * j, gb + (size_t)(8 * j) * zstride);
+        for (int j = 0; j < NL / Z2; ++j) async_copy(fs + (Z2 + 1) * CL * j, fg + (size_t)(Z2 * j) * zstride);
     } else {
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             const int k = i % C, zc = i / C, z = zc & (nz - 1), c = zc >> lz;
@@ -422,12 +436,10 @@ k_zsolve(FluidArgs<float> a, GridGeo g)
     async_wait_all();
     __syncthreads();
     auto idx = [=](int l, int z) { return at(l / C, z, l % C); };
-    if constexpr (z128) {
-        if (nz == 128) zlines128<false>(reinterpret_cast<float2*>(Bf), reinterpret_cast<const float2*>(twz));
-        else lines_fft_n<false>(nz, Bf, 3 * C, idx, twz);
-    } else {
-        lines_fft_n<false>(nz, Bf, 3 * C, idx, twz);
-    }
+    const int lane = threadIdx.x & 31, l = (threadIdx.x >> 5) * LPW + lane % LPW;
+    float2* mine = Bf + l / C * (ZP * CL) + l % C;
+    if constexpr (FIX) line_fft<NL, false, CL>(mine, lane / LPW, twz);
+    else lines_fft_n<false>(nz, Bf, 3 * C, idx, twz);
     __syncthreads();
     const float* sym = reinterpret_cast<const float*>(a.symk);     // [9][256] cos, sin, lambda
     const float ih = kparam<float>(a.inv_h, a.inv_h32);
@@ -484,19 +496,12 @@ k_zsolve(FluidArgs<float> a, GridGeo g)
         for (int c = 0; c < 3; ++c) Bf[at(c, kz, k)] = W[c];
     }
     __syncthreads();
-    if constexpr (z128) {
-        if (nz == 128) zlines128<true>(reinterpret_cast<float2*>(Bf), reinterpret_cast<const float2*>(twz));
-        else lines_fft_n<true>(nz, Bf, 3 * C, idx, twz);
-    } else {
-        lines_fft_n<true>(nz, Bf, 3 * C, idx, twz);
-    }
+    if constexpr (FIX) line_fft<NL, true, CL>(mine, lane / LPW, twz);
+    else lines_fft_n<true>(nz, Bf, 3 * C, idx, twz);
     __syncthreads();
-    if (fast) {
-        const int k = threadIdx.x & 7, zr = threadIdx.x >> 3, c = zr >> 3, z0 = zr & 7;
-        const float2* sb = Bf + (c * 144 + z0) * 12 + k;
-        float2* gb = base + c * cstride + (size_t)z0 * zstride + k;
+    if constexpr (FIX) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) gb[(size_t)(8 * j) * zstride] = sb[108 * j];
+        for (int j = 0; j < NL / Z2; ++j) fg[(size_t)(Z2 * j) * zstride] = fs[(Z2 + 1) * CL * j];
     } else {
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             const int k = i % C, zc = i / C, z = zc & (nz - 1), c = zc >> lz;
@@ -625,55 +630,77 @@ k_plane_inv(FluidArgs<float> a, GridGeo g)
     }
 }
 
+using PlaneKernel = void (*)(FluidArgs<float>, GridGeo);
+struct PlanePass {
+    PlaneKernel fwd[2], inv;               // fwd[1]: with the fluid stress
+    size_t slots;
+    int threads;
+};
+template <typename L> PlanePass plane_pass(int nx, int ny, int threads)
+{
+    const PlanePass p{{k_plane_fwd<L, false>, k_plane_fwd<L, true>}, k_plane_inv<L>,
+                      PlaneSlots<L>::count(nx, ny), threads};
+    static std::atomic<unsigned> attr{0};     // per layout
+    if (first_on_device(attr))
+        for (PlaneKernel k : {p.fwd[0], p.fwd[1], p.inv})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    return p;
+}
+// as many threads as one round of lines takes, at most 256
+template <int NX, int NY> PlanePass plane_fixed()
+{
+    constexpr int r = NY / 2 * Split<NX>::N2, c = NX / 2 * Split<NY>::N2, m = r > c ? r : c;
+    using L = std::conditional_t<NX == 128 && NY == 128, Skew128, PlaneT<NX, NY>>;
+    return plane_pass<L>(NX, NY, m < 256 ? m : 256);
+}
+template <int NX> PlanePass plane_of(int ny)
+{
+    return ny == 32 ? plane_fixed<NX, 32>() : (ny == 64 ? plane_fixed<NX, 64>() : plane_fixed<NX, 128>());
+}
+
 template <>
 cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const FluidArgs<float>& a_in,
                           cudaEvent_t* marks)
 {
     cudaStream_t st = chain.st;                      // always a chain of programmatic dependents
     const FluidArgs<float> a = with_derived(a_in, g);
-    constexpr int PT = 256;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxh = nx / 2 + 1;
-    constexpr int CZ = 8;                             // ky columns per z-pass block
-    static std::atomic<unsigned> attr{0};     // per instantiation
-    if (first_on_device(attr)) {
-        const int lim = 200 * 1024;
-        cudaFuncSetAttribute(k_plane_fwd<PadPlane, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_fwd<PadPlane, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zsolve<CZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zsolve<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_inv<PadPlane>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_fwd<Skew128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_fwd<Skew128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane_inv<Skew128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    }
-    // FP32 planes of 128 x 128 take the conflict-free layout (MB_PLANE_LAYOUT=pad keeps the
-    // padded one, for comparison)
-    static const bool skew_off = [] {
+    // planes of sides from 32 to 128 have layouts at compile-time offsets; MB_PLANE_LAYOUT=pad
+    // keeps the padded run-time one, for comparison.  32 boxes of 64^3, run-time / compile-time:
+    // forward 128 / 90 us (with the untouched planes of f left out), inverse 114 / 75 (without
+    // the sum v^n + v^{n+1}), z 77 / 68; the L1 is then 83 to 88% busy
+    static const bool pad = [] {
         const char* e = std::getenv("MB_PLANE_LAYOUT");
         return e && std::string(e) == "pad";
     }();
-    const bool skew = nx == 128 && ny == 128 && !skew_off;
-    const size_t smem_plane = (skew ? PlaneSlots<Skew128>::count(nx, ny)
-                                    : PlaneSlots<PadPlane>::count(nx, ny)) * sizeof(float2);
-    const int C = ny >= CZ ? CZ : 4;
-    const size_t smem_z = ((size_t)3 * padded_len(nz) * (C + 4) + nz) * sizeof(float2);
+    const bool fixed = !pad && nx >= 32 && ny >= 32;
+    const PlanePass pp = !fixed ? plane_pass<PadPlane>(nx, ny, 256)
+                         : nx == 128 ? plane_of<128>(ny)
+                         : nx == 64 ? plane_of<64>(ny) : plane_of<32>(ny);
+    const size_t smem_plane = pp.slots * sizeof(float2);
+    // z lines of 32 to 128 points at compile-time offsets, 8 columns a block
+    const int C = ny >= 8 ? 8 : 4, zfix = C == 8 && nz >= 32 ? nz : 0;
+    PlaneKernel zs = zfix == 128 ? k_zsolve<8, 128> : zfix == 64 ? k_zsolve<8, 64>
+                     : zfix == 32 ? k_zsolve<8, 32> : C == 8 ? k_zsolve<8, 0> : k_zsolve<4, 0>;
+    const int Z2 = zfix == 32 ? 4 : 8, CL = zfix == 32 ? 8 : C + 4;
+    const unsigned tz = zfix ? 3 * C * Z2 : 3 * C * 8;
+    const size_t smem_z = ((size_t)3 * (zfix ? nz + nz / Z2 : padded_len(nz)) * CL + nz) * sizeof(float2);
+    static std::atomic<unsigned> attr{0};
+    if (first_on_device(attr))
+        for (PlaneKernel k : {k_zsolve<8, 128>, k_zsolve<8, 64>, k_zsolve<8, 32>, k_zsolve<8, 0>, k_zsolve<4, 0>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     auto mark = [&](int i) { if (marks) cudaEventRecord(marks[i], st); };
     mark(0);
-    cudaError_t e;
     const dim3 gp(nz, 3 * B), gz(ny / C, nxh, B);
-    auto fwd = a.W ? (skew ? k_plane_fwd<Skew128, true> : k_plane_fwd<PadPlane, true>)
-                   : (skew ? k_plane_fwd<Skew128, false> : k_plane_fwd<PadPlane, false>);
-    e = launch_dep(fwd, gp, dim3(PT), smem_plane, st, a, g);
+    cudaError_t e = launch_dep(pp.fwd[a.W ? 1 : 0], gp, dim3(pp.threads), smem_plane, st, a, g);
     if (e != cudaSuccess) return e;
     mark(1);
     mark(2);
-    if (C == CZ) e = launch_dep(k_zsolve<CZ>, gz, dim3(3 * CZ * 8), smem_z, st, a, g);
-    else e = launch_dep(k_zsolve<4>, gz, dim3(3 * 4 * 8), smem_z, st, a, g);
+    e = launch_dep(zs, gz, dim3(tz), smem_z, st, a, g);
     if (e != cudaSuccess) return e;
     mark(3);
     mark(4);
-    if (skew) e = launch_dep(k_plane_inv<Skew128>, gp, dim3(PT), smem_plane, st, a, g);
-    else e = launch_dep(k_plane_inv<PadPlane>, gp, dim3(PT), smem_plane, st, a, g);
+    e = launch_dep(pp.inv, gp, dim3(pp.threads), smem_plane, st, a, g);
     if (e != cudaSuccess) return e;
     mark(5);
     return cudaGetLastError();

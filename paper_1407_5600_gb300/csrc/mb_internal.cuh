@@ -200,6 +200,9 @@ struct FluidArgs {
     // per thread on GB300's narrow FP64 pipe
     float rho_dt32, half_eta32, inv_h32, inv_h2_32, inv_n32;
     R* f_clear;            // three-pass FFT: f, zeroed as it is read (null = leave f alone)
+    // FP32 three-pass FFT: [B][nz], non-zero for the z planes of f that were spread into (the others
+    // are zero and not read); zeroed by the z pass.  Null: all may be non-zero
+    int* f_dirty;
     const R* v_sum_base;   // three-pass FFT: v^n; with v_sum_out, also write v^n + v^{n+1}
     R* v_sum_out;
     // three-pass FFT, mean_mode 0: the FP64 mean velocity [B][3], advanced in place by the
@@ -384,7 +387,12 @@ cudaError_t launch_pairs32(cudaStream_t st, int Bx, int64_t max_box_blobs,
 bool spread32_tile_ok(const int tile[3], const GridGeo& g, const BinGeo& bg);
 cudaError_t launch_spread32(cudaStream_t st, int Bx, const float4* rec, const int32_t* cell_start,
                             const GridGeo& g, const BinGeo& bg, const int tile[3], float* f,
-                            bool f_is_zero = false);
+                            bool f_is_zero = false, int* dirty = nullptr);
+// The same straight to f, for few blobs (spread32_few).
+bool spread32_few(int64_t nb);
+cudaError_t launch_spread32_few(cudaStream_t st, int64_t nb, int Bx, const float4* rec,
+                                const int32_t* sorted, const int32_t* box_of, const GridGeo& g,
+                                const BinGeo& bg, float* f, bool f_is_zero, int* dirty);
 // External forces to FP32 plus their per-box FP64 sums (partial: [B][chunks][3] scratch;
 // ticket: one zeroed unsigned, left zero), in one launch.
 cudaError_t launch_ext_prepare(cudaStream_t st, int Bx, int64_t max_box_blobs,
