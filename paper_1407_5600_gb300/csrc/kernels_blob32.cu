@@ -169,7 +169,8 @@ __global__ void k_unsplit(int64_t nb, const float4* __restrict__ A, const float4
 }
 
 // ------------------------------------------------------------------------------------------
-// Interpolation J from the split positions (mode 0: u only; 1: predictor; 2: corrector).
+// Interpolation J from the split positions (mode 0: u only; 1: predictor; 2: corrector with the
+// mean of two fields; 3: corrector with one field).
 // The x nodes ix, ix + 1, ix + 2 (periodic) of a window lie in the two aligned node pairs that
 // start at a = ix & ~1 and at (a + 2) mod nx: each row of a window is read with two 8-byte loads
 // instead of three 4-byte ones (a third fewer L1 sector lookups per gather), and the three
@@ -236,6 +237,8 @@ k_interp32(int64_t nb, const float4* __restrict__ A, const float4* __restrict__ 
            int32_t* __restrict__ count, int32_t* __restrict__ blob_cell,
            int32_t* __restrict__ blob_rank)
 {
+    dep_wait();
+    dep_release();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= nb) return;
     // blobs in cell order (when known) so that neighbouring threads gather neighbouring nodes
@@ -407,57 +410,68 @@ k_interp32_fused(int64_t nb, FusedArgs f, GridGeo g, BinGeo bg)
 // One thread / nine lanes a blob, 128^3: 19.6 / 8.1 us of 4,095 blobs, 20.0 / 9.7 of 8,190,
 // 20.5 / 13.4 of 16,380, 21.0 / 22.8 of 32,760.
 constexpr int64_t FEW_BLOBS = 24576;
+struct Lane9 {
+    int j, comp, cz, t;        // blob of the warp, component, z node; sorted position
+    bool writer;
+};
+__device__ __forceinline__ Lane9 lane9(int nb)
+{
+    const int lane = threadIdx.x & 31, warp = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int j = min(lane / 9, 2), k = lane - 9 * j, t = 3 * warp + j;
+    return {j, min(k / 3, 2), k % 3, min(t, nb - 1), k == 0 && t < nb};
+}
+// J (v0 + v1) (v1 may be null) at cell c, offset hi: this lane's rows, then every lane sums its
+// blob's; all lanes of the warp call it.
+__device__ __forceinline__ void gather9(const Lane9& l, const int c[3], const float hi[3],
+                                        const float* v0, const float* v1, int box, const Geo32& G,
+                                        float u[3])
+{
+    const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
+    const size_t base = ((size_t)box * 3 + l.comp) * (size_t)G.N;
+    float wx[3], wy[3], wz[3];
+    const int ix = window32(c[0], G.bs, hi[0], G.inv_h, l.comp == 0 ? 0.f : 0.5f, wx);
+    const int iy = window32(c[1], G.bs, hi[1], G.inv_h, l.comp == 1 ? 0.f : 0.5f, wy);
+    const int iz = window32(c[2], G.bs, hi[2], G.inv_h, l.comp == 2 ? 0.f : 0.5f, wz);
+    const float w = l.cz == 0 ? wz[0] : (l.cz == 1 ? wz[1] : wz[2]);
+    const XPair xp = xpair(ix, nx, wx);
+    const int zo = ((iz + l.cz) & (nz - 1)) * (ny * nx);
+    float acc = 0.0f;
+#pragma unroll
+    for (int cy = 0; cy < 3; ++cy)
+        acc += wy[cy] * w * xrow(v0 + base, v1 ? v1 + base : nullptr,
+                                 zo + ((iy + cy) & (ny - 1)) * nx, xp);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        float s = 0.0f;
+#pragma unroll
+        for (int z = 0; z < 3; ++z) s += __shfl_sync(0xffffffffu, acc, 9 * l.j + 3 * d + z);
+        u[d] = s;
+    }
+}
+
 __global__ void __launch_bounds__(128)
 k_interp32_fused9(int nb, FusedArgs f, GridGeo g, BinGeo bg)
 {
     dep_wait();
     dep_release();
     const Geo32 G = geo32(g, bg);
-    const int lane = threadIdx.x & 31, warp = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (3 * warp >= nb) return;
-    const int j = min(lane / 9, 2), k = lane - 9 * j, comp = min(k / 3, 2), cz = k % 3;
-    const int t = 3 * warp + j;
-    const bool writer = k == 0 && t < nb;
-    const int64_t b = f.order ? f.order[min(t, nb - 1)] : min(t, nb - 1);
+    const Lane9 l = lane9(nb);
+    const int64_t b = f.order ? f.order[l.t] : l.t;
     const int box = f.box_of ? f.box_of[b] : 0;
-    const size_t base = ((size_t)box * 3 + comp) * (size_t)G.N;
-    const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
-    // u = J (v0 + v1) at cell c, offset hi: this lane's rows, then every lane sums its blob's
-    auto gather = [&](const int c[3], const float hi[3], const float* v0, const float* v1, float u[3]) {
-        float wx[3], wy[3], wz[3];
-        const int ix = window32(c[0], G.bs, hi[0], G.inv_h, comp == 0 ? 0.f : 0.5f, wx);
-        const int iy = window32(c[1], G.bs, hi[1], G.inv_h, comp == 1 ? 0.f : 0.5f, wy);
-        const int iz = window32(c[2], G.bs, hi[2], G.inv_h, comp == 2 ? 0.f : 0.5f, wz);
-        const float w = cz == 0 ? wz[0] : (cz == 1 ? wz[1] : wz[2]);
-        const XPair xp = xpair(ix, nx, wx);
-        const int zo = ((iz + cz) & (nz - 1)) * (ny * nx);
-        float acc = 0.0f;
-#pragma unroll
-        for (int cy = 0; cy < 3; ++cy)
-            acc += wy[cy] * w * xrow(v0 + base, v1 ? v1 + base : nullptr,
-                                     zo + ((iy + cy) & (ny - 1)) * nx, xp);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            float s = 0.0f;
-#pragma unroll
-            for (int z = 0; z < 3; ++z) s += __shfl_sync(0xffffffffu, acc, 9 * j + 3 * d + z);
-            u[d] = s;
-        }
-    };
     const float4 a = f.A[b], ab = f.A_base[b], lb = f.B_base[b];
     const int pk = __float_as_int(a.w), pb = __float_as_int(ab.w);
     const int c[3] = {cell_unpack(pk, 0), cell_unpack(pk, 1), cell_unpack(pk, 2)};
     const float hi[3] = {a.x, a.y, a.z};
     int cc[3] = {cell_unpack(pb, 0), cell_unpack(pb, 1), cell_unpack(pb, 2)};
     float h2[3] = {ab.x, ab.y, ab.z}, l2[3] = {lb.x, lb.y, lb.z}, u[3];
-    gather(c, hi, f.v0, f.v1, u);
+    gather9(l, c, hi, f.v0, f.v1, box, G, u);
     for (int d = 0; d < 3; ++d) ff_move(cc[d], h2[d], l2[d], f.dt * (0.5f * u[d]), G.w, G.nc[d]);
-    if (writer) {
+    if (l.writer) {
         f.A_out[b] = make_float4(h2[0], h2[1], h2[2], __int_as_float(cell_pack(cc[0], cc[1], cc[2])));
         f.B_out[b] = make_float4(l2[0], l2[1], l2[2], 0.0f);
     }
-    gather(cc, h2, f.vp, nullptr, u);
-    if (!writer) return;
+    gather9(l, cc, h2, f.vp, nullptr, box, G, u);
+    if (!l.writer) return;
     f.u_out[b] = make_float4(u[0], u[1], u[2], 0.0f);
     for (int d = 0; d < 3; ++d) ff_move(cc[d], h2[d], l2[d], 0.5f * f.dt * u[d], G.w, G.nc[d]);
     f.Ah_out[b] = make_float4(h2[0], h2[1], h2[2], __int_as_float(cell_pack(cc[0], cc[1], cc[2])));
@@ -465,6 +479,39 @@ k_interp32_fused9(int nb, FusedArgs f, GridGeo g, BinGeo bg)
     const int cell = (int)(box * G.ncell) + (cc[2] * G.nc[1] + cc[1]) * G.nc[0] + cc[0];
     f.blob_cell[b] = cell;
     f.blob_rank[b] = atomicAdd(f.count + cell, 1);
+}
+
+// Modes 1 (A, B the base position) and 3 of k_interp32 with nine lanes a blob.  A_out may be A_base:
+// every lane has read its blob's before the sums meet.
+template <int MODE>
+__global__ void __launch_bounds__(128)
+k_interp32_few(int nb, const float4* A, const float* v0, const int32_t* box_of, GridGeo g, BinGeo bg,
+               float dt, const float4* A_base, const float4* B_base, float4* A_out, float4* B_out,
+               const int32_t* order, int32_t* count, int32_t* blob_cell, int32_t* blob_rank)
+{
+    dep_wait();
+    dep_release();
+    const Geo32 G = geo32(g, bg);
+    const Lane9 l = lane9(nb);
+    const int64_t b = order ? order[l.t] : l.t;
+    const int box = box_of ? box_of[b] : 0;
+    const float4 a = A[b], ab = A_base[b], lb = B_base[b];
+    const int pk = __float_as_int(a.w), pb = __float_as_int(ab.w);
+    const int c[3] = {cell_unpack(pk, 0), cell_unpack(pk, 1), cell_unpack(pk, 2)};
+    const float hi[3] = {a.x, a.y, a.z};
+    int cc[3] = {cell_unpack(pb, 0), cell_unpack(pb, 1), cell_unpack(pb, 2)};
+    float h2[3] = {ab.x, ab.y, ab.z}, l2[3] = {lb.x, lb.y, lb.z}, u[3];
+    gather9(l, c, hi, v0, nullptr, box, G, u);
+    if (!l.writer) return;
+    const float scale = MODE == 1 ? 0.5f * dt : dt;
+    for (int d = 0; d < 3; ++d) ff_move(cc[d], h2[d], l2[d], scale * u[d], G.w, G.nc[d]);
+    A_out[b] = make_float4(h2[0], h2[1], h2[2], __int_as_float(cell_pack(cc[0], cc[1], cc[2])));
+    B_out[b] = make_float4(l2[0], l2[1], l2[2], 0.0f);
+    if (MODE == 1 && count) {
+        const int cell = (int)(box * G.ncell) + (cc[2] * G.nc[1] + cc[1]) * G.nc[0] + cc[0];
+        blob_cell[b] = cell;
+        blob_rank[b] = atomicAdd(count + cell, 1);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -894,8 +941,8 @@ k_forces32(Force32Args a, GridGeo g, BinGeo bg)
 // least 2 h wide), so the bound is a bound on the sum of the blobs' largest force components
 // over any 3 x 3 x 3 block of the tile's cells, times the kernel's largest weight (2/3)^3.  The
 // block then adds the copy to f (zeroed beforehand) with vector atomics, skipping all-zero
-// chunks; nodes shared with neighbouring tiles receive every tile's part.  dirty (or null; grids of
-// up to 128 planes): [box][nz], set for the z planes added to.  TXc = 0 takes the
+// chunks; nodes shared with neighbouring tiles receive every tile's part.  dirty (or null): [box][nz],
+// set for the z planes that the tile may add to.  TXc = 0 takes the
 // tile from the arguments (small grids).
 template <int TXc, int TYc, int TZc>
 __global__ void __launch_bounds__(256)
@@ -905,13 +952,16 @@ k_spread32(const float4* __restrict__ rec, const int32_t* __restrict__ cell_star
     dep_wait();
     dep_release();
     const int TX = TXc ? TXc : TXr, TY = TYc ? TYc : TYr, TZ = TZc ? TZc : TZr;
-    const int SXC = TX / 4 + 2, SX = 4 * SXC, SY = TY + 3, SZ = TZ + 3;
-    const int SN = SX * SY * SZ;
+    // Rows of TX + 4 words: a row's chunks start at T0 - 4, of which only the node T0 - 1 is ever
+    // added to, and end with that of T0 + TX and T0 + TX + 1; so the last chunk of a row is the
+    // first of the next.  The 32 x 8 x 8 copy then takes 52 KiB and four blocks an SM (128^3,
+    // 244,504 blobs: 29.7 -> 28.7 us; three blocks with rows of TX + 8).
+    const int SXC = TX / 4 + 2, SX = TX + 4, SY = TY + 3, SZ = TZ + 3;
+    const int SN = SX * SY * SZ + 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* acc = reinterpret_cast<int*>(smem_raw);                 // [3][SZ][SY][SX]
     __shared__ int rb[64], rp[65];
     __shared__ float wmax[8];
-    __shared__ int plane[132];                                   // (dirty) planes of the copy added to
     const Geo32 G = geo32(g, bg);
     const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
     const int box = blockIdx.y;
@@ -944,16 +994,17 @@ k_spread32(const float4* __restrict__ rec, const int32_t* __restrict__ cell_star
         if (r == 31) carry0 = x;
         if (r == 63) rp[64] = x;               // the second warp's total (carry added below)
     }
-    if (dirty && threadIdx.x < 132) plane[threadIdx.x] = 0;
     const int ncell = ncx * rows;
     float* cf = reinterpret_cast<float*>(acc + 3 * SN);          // [ncz][ncy][ncx] force sums
-    if (!__syncthreads_or(any)) return;                          // no blobs in the tile
     {
         int4* a4 = reinterpret_cast<int4*>(acc);
         for (int i = threadIdx.x; i < 3 * SN / 4; i += blockDim.x) a4[i] = make_int4(0, 0, 0, 0);
         for (int i = threadIdx.x; i < ncell; i += blockDim.x) cf[i] = 0.0f;
     }
-    __syncthreads();
+    if (!__syncthreads_or(any)) return;                          // no blobs in the tile
+    if (dirty)
+        for (int i = threadIdx.x; i < SZ; i += blockDim.x)
+            dirty[box * nz + ((T0[2] - 1 + i) & (nz - 1))] = 1;
     if (threadIdx.x >= 32 && threadIdx.x < 65) rp[threadIdx.x] += carry0;
     __syncthreads();
     const int total = rp[rows];
@@ -1021,7 +1072,7 @@ k_spread32(const float4* __restrict__ rec, const int32_t* __restrict__ cell_star
             const int sxs = comp == 0 ? 0 : 1, sys = comp == 1 ? 0 : 1, szs = comp == 2 ? 0 : 1;
             // window starts in the copy: [3, TX + 3] and [0, T] for blobs of the tile (offsets
             // in [0, w)); clamped so that no offset can address outside the copy
-            const int lx = min(max(wx.i0[sxs] - ox, 0), SX - 3);
+            const int lx = min(max(wx.i0[sxs] - ox, 3), TX + 3);
             const int ly = min(max(wy.i0[sys] - oy, 0), SY - 3);
             const int lz = min(max(wz.i0[szs] - oz, 0), SZ - 3);
             int* a0 = acc + comp * SN + (lz * SY + ly) * SX + lx;
@@ -1045,21 +1096,17 @@ k_spread32(const float4* __restrict__ rec, const int32_t* __restrict__ cell_star
     const int N32 = (int)G.N;
     const float unscale = 1.0f / scale;
     for (int i = threadIdx.x; i < 3 * SY * SZ * SXC; i += blockDim.x) {
-        const int4 q = a4[i];
-        if ((q.x | q.y | q.z | q.w) == 0) continue;
         const int row = i / SXC, cx = i - row * SXC;
         const int comp = row / (SY * SZ), rr = row - comp * (SY * SZ);
+        int4 q = a4[comp * (SN / 4) + rr * (SX / 4) + cx];
+        if (cx == 0) q.x = q.y = q.z = 0;               // the rest of these is the row's before
+        if (cx == SXC - 1) q.z = q.w = 0;               // and the row's after
+        if ((q.x | q.y | q.z | q.w) == 0) continue;
         const int sz = rr / SY, sy = rr - sz * SY;
         const int gx = (ox + 4 * cx) & (nx - 1), gy = (oy + sy) & (ny - 1), gz = (oz + sz) & (nz - 1);
         float* dst = fb + (comp * N32 + (gz * ny + gy) * nx + gx);
         atomicAdd(reinterpret_cast<float4*>(dst),
                   make_float4(q.x * unscale, q.y * unscale, q.z * unscale, q.w * unscale));
-        if (dirty) plane[sz] = 1;
-    }
-    if (dirty) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < SZ; i += blockDim.x)
-            if (plane[i]) dirty[box * nz + ((oz + i) & (nz - 1))] = 1;
     }
 }
 
@@ -1259,18 +1306,16 @@ cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4*
                             int32_t* count, int32_t* blob_cell, int32_t* blob_rank)
 {
     if (nb <= 0) return cudaSuccess;
-    const unsigned nbk = blocks_for(nb, 256);
-    if (mode == 0)
-        k_interp32<0><<<nbk, 256, 0, st>>>(nb, A, B, v0, v1, box_of, g, bg, dt, A_base, B_base,
-                                           A_out, B_out, u_out, order, nullptr, nullptr, nullptr);
-    else if (mode == 1)
-        k_interp32<1><<<nbk, 256, 0, st>>>(nb, A, B, v0, v1, box_of, g, bg, dt, A_base, B_base,
-                                           A_out, B_out, u_out, order, count, blob_cell,
-                                           blob_rank);
-    else
-        k_interp32<2><<<nbk, 256, 0, st>>>(nb, A, B, v0, v1, box_of, g, bg, dt, A_base, B_base,
-                                           A_out, B_out, u_out, order, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    if ((mode == 1 || mode == 3) && nb <= FEW_BLOBS)
+        return launch_dep(mode == 1 ? k_interp32_few<1> : k_interp32_few<3>,
+                          dim3((unsigned)((nb + 11) / 12)), dim3(128), 0, st, (int)nb, A, v0, box_of, g,
+                          bg, dt, mode == 1 ? A : A_base, mode == 1 ? B : B_base, A_out, B_out, order,
+                          count, blob_cell, blob_rank);
+    const auto k = mode == 0 ? k_interp32<0> : mode == 1 ? k_interp32<1>
+                   : mode == 2 ? k_interp32<2> : k_interp32<3>;
+    return launch_dep(k, dim3(blocks_for(nb, 256)), dim3(256), 0, st, nb, A, B, v0, v1, box_of, g, bg, dt,
+                      A_base, B_base, A_out, B_out, u_out, order, mode == 1 ? count : nullptr,
+                      blob_cell, blob_rank);
 }
 
 cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, const float* v0,
@@ -1377,7 +1422,7 @@ cudaError_t launch_pairs32(cudaStream_t st, int Bx, int64_t max_box_blobs,
 // The shared copy (3 components, 16-byte chunks along x) and one force sum per bin cell.
 size_t spread32_smem(const int tile[3], int bs)
 {
-    return (size_t)3 * (tile[0] + 8) * (tile[1] + 3) * (tile[2] + 3) * sizeof(float) +
+    return (size_t)3 * ((tile[0] + 4) * (tile[1] + 3) * (tile[2] + 3) + 4) * sizeof(float) +
            (size_t)(tile[0] / bs) * (tile[1] / bs) * (tile[2] / bs) * sizeof(float);
 }
 
@@ -1407,7 +1452,6 @@ cudaError_t launch_spread32(cudaStream_t st, int Bx, const float4* rec, const in
                             const GridGeo& g, const BinGeo& bg, const int tile[3], float* f,
                             bool f_is_zero, int* dirty)
 {
-    if (g.n[2] > 128) dirty = nullptr;
     if (!spread32_tile_ok(tile, g, bg)) return cudaErrorInvalidValue;
     if (!f_is_zero) {
         const cudaError_t e = cudaMemsetAsync(f, 0, sizeof(float) * 3 * (size_t)Bx * g.N, st);

@@ -1061,8 +1061,14 @@ void finish_step64(mb_ctx* ctx)
     ctx->steps_taken++;
 }
 
-// One time step of every box in FP32-grid mode: blob positions as bin cell + float-float
-// offset, forces and weights on the FP32 pipes, the k = 0 mode from the FP64 external force sum.
+// The marks of the z planes of f that are spread into, where most planes may stay untouched:
+// with many blobs none does, and the right-hand side would wait for its mark in vain (128^3,
+// 244,504 blobs: 33.7 -> 34.4 us).
+int* f_planes(mb_ctx* ctx)
+{
+    return spread32_few(ctx->nb) ? static_cast<int*>(ctx->f_dirty.p) : nullptr;
+}
+
 // Host-side state after an FP32-grid step has been enqueued (directly or as a graph replay).
 void finish_fast_step(mb_ctx* ctx)
 {
@@ -1078,6 +1084,8 @@ void finish_fast_step(mb_ctx* ctx)
     }
 }
 
+// One time step of every box in FP32-grid mode: blob positions as bin cell + float-float
+// offset, forces and weights on the FP32 pipes, the k = 0 mode from the FP64 external force sum.
 mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
 {
     cudaStream_t st = ctx->st;
@@ -1216,12 +1224,12 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
             MB_CUDA(launch_spread32_few(st, ctx->nb, B, static_cast<const float4*>(ctx->rec32.p),
                                         static_cast<const int32_t*>(ctx->sorted.p), box_of, g,
                                         ctx->bg, static_cast<float*>(ctx->f.p), ctx->f_zero,
-                                        static_cast<int*>(ctx->f_dirty.p)));
+                                        f_planes(ctx)));
         else
             MB_CUDA(launch_spread32(st, B, static_cast<const float4*>(ctx->rec32.p),
                                     static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
                                     ctx->tile, static_cast<float*>(ctx->f.p), ctx->f_zero,
-                                    static_cast<int*>(ctx->f_dirty.p)));
+                                    f_planes(ctx)));
         ctx->launches += 1;
     }
     mark(ST_STRESS);
@@ -1256,7 +1264,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
     }
     if (blobs && ctx->fft_passes == 3) {
         fa.f_clear = static_cast<float*>(ctx->f.p);
-        fa.f_dirty = static_cast<int*>(ctx->f_dirty.p);
+        fa.f_dirty = f_planes(ctx);
     }
     // the sum v^n + v^{n+1} costs the plane pass a read and a write of the grid and saves the
     // corrector half its gathers.  128^3, plane pass and corrector without / with the sum: 53 / 54 us
@@ -1328,10 +1336,20 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
     }
     auto mark = [&](int i) { if (ctx->timing) cudaEventRecord(ctx->ev[i], st); };
     const float dt = (float)ctx->d.dt;
+    const bool overlap = blobs && !ctx->timing;
     // forces at (A, B) (binned already when `counted`), spreading, steady flow into v_out
     auto half = [&](const float4* A, const float4* Bp, bool counted, float* v_out,
                     bool marks) -> mb_status {
         if (marks) mark(ST_BIN);
+        // as in the inertial step, the springs run beside the binning
+        if (overlap) {
+            MB_CUDA(cudaEventRecord(ctx->fork[0], st));
+            MB_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork[0], 0));
+            MB_CUDA(launch_springs32(ctx->side, ctx->nb, A, Bp, springs32(ctx), box_of,
+                                     box_par32(ctx), g, ctx->bg,
+                                     static_cast<float4*>(ctx->Fs32.p)));
+            MB_CUDA(cudaEventRecord(ctx->fork[1], ctx->side));
+        }
         if (blobs) {
             MB_CUDA(launch_bin32(st, ctx->nb, A, box_of, B, ctx->bg,
                                  static_cast<int32_t*>(ctx->cell_count.p),
@@ -1347,18 +1365,30 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
         }
         if (marks) mark(ST_FORCES);
         if (blobs) {
-            MB_CUDA(launch_forces32(st, B, ctx->nb, ctx->max_box_blobs,
-                                    static_cast<const int64_t*>(ctx->box_off.p),
-                                    static_cast<const int32_t*>(ctx->sorted.p), A, Bp,
-                                    static_cast<const float4*>(ctx->loc.p), springs32(ctx),
-                                    box_of,
-                                    box_par32(ctx),
-                                    static_cast<const int32_t*>(ctx->cell_start.p),
-                                    static_cast<const int32_t*>(ctx->blob_cell.p),
-                                    ext ? static_cast<const float4*>(ctx->ext32.p) : nullptr,
-                                    static_cast<float4*>(ctx->Fs32.p),
-                                    static_cast<float4*>(ctx->F32.p),
-                                    static_cast<float4*>(ctx->rec32.p), g, ctx->bg));
+            const int64_t* box_off = static_cast<const int64_t*>(ctx->box_off.p);
+            const float4* ext4 = ext ? static_cast<const float4*>(ctx->ext32.p) : nullptr;
+            if (overlap) {
+                MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[1], 0));
+                MB_CUDA(launch_pairs32(st, B, ctx->max_box_blobs, box_off,
+                                       static_cast<const int32_t*>(ctx->sorted.p), A, Bp,
+                                       static_cast<const float4*>(ctx->loc.p), box_of,
+                                       box_par32(ctx),
+                                       static_cast<const int32_t*>(ctx->cell_start.p),
+                                       static_cast<const int32_t*>(ctx->blob_cell.p), ext4,
+                                       static_cast<float4*>(ctx->Fs32.p),
+                                       static_cast<float4*>(ctx->F32.p),
+                                       static_cast<float4*>(ctx->rec32.p), g, ctx->bg));
+            } else {
+                MB_CUDA(launch_forces32(st, B, ctx->nb, ctx->max_box_blobs, box_off,
+                                        static_cast<const int32_t*>(ctx->sorted.p), A, Bp,
+                                        static_cast<const float4*>(ctx->loc.p), springs32(ctx),
+                                        box_of, box_par32(ctx),
+                                        static_cast<const int32_t*>(ctx->cell_start.p),
+                                        static_cast<const int32_t*>(ctx->blob_cell.p), ext4,
+                                        static_cast<float4*>(ctx->Fs32.p),
+                                        static_cast<float4*>(ctx->F32.p),
+                                        static_cast<float4*>(ctx->rec32.p), g, ctx->bg));
+            }
             ctx->launches += 2;
         }
         if (marks) mark(ST_FORCE_SUM);
@@ -1366,8 +1396,8 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
         if (blobs) {
             MB_CUDA(launch_spread32(st, B, static_cast<const float4*>(ctx->rec32.p),
                                     static_cast<const int32_t*>(ctx->cell_start.p), g, ctx->bg,
-                                    ctx->tile, static_cast<float*>(ctx->f.p), false,
-                                    static_cast<int*>(ctx->f_dirty.p)));
+                                    ctx->tile, static_cast<float*>(ctx->f.p), ctx->f_zero,
+                                    f_planes(ctx)));
             ctx->launches += 1;
         }
         if (marks) mark(ST_STRESS);
@@ -1377,6 +1407,10 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
         fa.rho_dt = 0.0;
         fa.half_eta = ctx->d.eta;
         fa.mean_mode = 1;
+        if (blobs && ctx->fft_passes == 3) {        // the plane pass leaves f zeroed
+            fa.f_clear = static_cast<float*>(ctx->f.p);
+            fa.f_dirty = f_planes(ctx);
+        }
         cudaEvent_t* fm = marks && ctx->timing ? ctx->ev + ST_FLUID_X_FWD : nullptr;
         if (ctx->fft_passes == 5) {
             MB_CUDA(launch_fluid<float>(st, B, g, fa, fm));
@@ -1385,6 +1419,7 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
             MB_CUDA(launch_fluid3<float>(st, B, g, fa, fm));
             ctx->launches += FLUID3_KERNELS;
         }
+        if (blobs) ctx->f_zero = ctx->fft_passes == 3;
         return MB_OK;
     };
     mark(ST_INTERP_PREDICT);
@@ -1402,8 +1437,8 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
     }
     MB_TRY(half(hA, hB, true, v_full, true));
     if (blobs) {
-        // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})  (the mean of a field with itself)
-        MB_CUDA(launch_interp32(st, 2, ctx->nb, hA, hB, v_full, v_full, box_of, g, ctx->bg, dt,
+        // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})
+        MB_CUDA(launch_interp32(st, 3, ctx->nb, hA, hB, v_full, nullptr, box_of, g, ctx->bg, dt,
                                 sA, sB, sA, sB, nullptr,
                                 static_cast<const int32_t*>(ctx->sorted.p)));
         ctx->launches += 1;
@@ -1413,7 +1448,6 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
     ctx->hcur = 0;
     ctx->hlast = 0;
     ctx->pred_ready = false;
-    ctx->f_zero = false;
     ctx->steps_taken++;
     return MB_OK;
 }
@@ -1421,11 +1455,12 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
 // Times each candidate spreading tile on the current binned records (the first step after
 // the blobs were set) and keeps the fastest; choices are cached per geometry and blob count.
 struct TuneKey {
-    int n[3], B, bs;
+    int n[3], B, bs, integrator;
     int64_t nb;
     bool operator<(const TuneKey& o) const
     {
-        return std::tie(n[0], n[1], n[2], B, bs, nb) < std::tie(o.n[0], o.n[1], o.n[2], o.B, o.bs, o.nb);
+        return std::tie(n[0], n[1], n[2], B, bs, integrator, nb) <
+               std::tie(o.n[0], o.n[1], o.n[2], o.B, o.bs, o.integrator, o.nb);
     }
 };
 std::map<TuneKey, std::array<int, 3>> g_tile_cache;
@@ -1435,7 +1470,7 @@ mb_status autotune_spread(mb_ctx* ctx)
 {
     ctx->tuned = true;
     if (!ctx->autotune || ctx->nb == 0) return MB_OK;
-    const TuneKey key{{ctx->g.n[0], ctx->g.n[1], ctx->g.n[2]}, ctx->B, ctx->bg.bs, ctx->nb};
+    const TuneKey key{{ctx->g.n[0], ctx->g.n[1], ctx->g.n[2]}, ctx->B, ctx->bg.bs, ctx->d.integrator, ctx->nb};
     {
         std::lock_guard<std::mutex> lock(g_tile_mu);
         auto it = g_tile_cache.find(key);
@@ -1450,6 +1485,9 @@ mb_status autotune_spread(mb_ctx* ctx)
     MB_CUDA(cudaEventCreate(&e1));
     // rounds over the candidates (the first warms up), each candidate's fastest launch kept:
     // the candidates differ by a few percent, about the spread of single launches
+    // (Stokes-limit steps amplify the spreading's rounding in the lowest modes, and a tile's
+    // fixed-point step grows with its densest spot: 3.5e-6 / 4.0e-6 of the dense 128^3 flow in
+    // tiles of 1024 / 2048 nodes, 6e-6 in larger ones, for 2% of the spreading's time)
     constexpr int NCAND = sizeof(cand) / sizeof(cand[0]), ROUNDS = 7;
     float fastest[NCAND];
     for (int i = 0; i < NCAND; ++i) fastest[i] = 1e30f;
@@ -1457,6 +1495,7 @@ mb_status autotune_spread(mb_ctx* ctx)
         for (int i = 0; i < NCAND; ++i) {
             const int t[3] = {cand[i][0], cand[i][1], cand[i][2]};
             if (!spread32_tile_ok(t, ctx->g, ctx->bg)) continue;
+            if (ctx->d.integrator == 1 && t[0] * t[1] * t[2] > 2048) continue;
             MB_CUDA(cudaEventRecord(e0, ctx->st));
             MB_CUDA(launch_spread32(ctx->st, ctx->B, static_cast<const float4*>(ctx->rec32.p),
                                     static_cast<const int32_t*>(ctx->cell_start.p), ctx->g,
@@ -1579,7 +1618,9 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
 {
     const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0;
     for (int s = 0; s < n_steps; ++s) {
-        if (!graphs || !ctx->tuned) {
+        // direct also from a state of f that steps do not leave behind (after a rebuild or a tile
+        // timing): the graph is that of the steps after
+        if (!graphs || !ctx->tuned || ctx->f_zero != (ctx->fft_passes == 3)) {
             MB_TRY(do_step_stokes_fast(ctx, ext, body));
             if (!ctx->tuned) MB_TRY(autotune_spread(ctx));
             continue;
@@ -1592,7 +1633,7 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
         // the state changes of do_step_stokes_fast
         ctx->hcur = ctx->hlast = 0;
         ctx->pred_ready = false;
-        ctx->f_zero = false;
+        ctx->f_zero = ctx->fft_passes == 3;
         ctx->sorted_valid = true;
         ctx->steps_taken++;
         ctx->launches += ctx->graph_launches;

@@ -91,3 +91,48 @@ def test_fp32_steps_at_the_edges_of_the_few_blob_kernels(nblobs, mean_mode):
                                    0.0, 0.0, 0.0, ext=F[b])
         assert rel_l2(v[b], v_ref) < 6e-6
         assert_positions(q[lo:lo + n[b]], q_ref, q0[b], g.L, 3, 2e-5)
+
+
+@pytest.mark.parametrize("nblobs", [1, 4, 13, 24576, 24577])
+def test_fp32_stokes_steps_at_the_edges_of_the_few_blob_kernels(nblobs):
+    """Two boxes, a direct step, then graph replays that clear the force grid as they read it."""
+    g = oracle.Grid(32, 16, 64, dt=0.05, mean_mode=1)
+    d = mb.GridDesc(32, 16, 64, dt=0.05, precision=0, mean_mode=1, integrator=1, batch=2)
+    rng = np.random.default_rng(nblobs)
+    none = (np.zeros((0, 2), np.int32), np.zeros(0))
+    n = [nblobs // 3, nblobs - nblobs // 3]
+    q0 = [rng.random((k, 3)) * [32, 16, 64] for k in n]
+    F = [rng.normal(size=(k, 3)) for k in n]
+    with mb.Multiblob(d) as sim:
+        for b in range(2):
+            sim.set_particles(b, q0[b], np.arange(n[b], dtype=np.int32), *none, 0.0)
+        sim.step(4, ext_blob_force=np.concatenate(F))
+        v, q = to_np(sim.velocity_field()), to_np(sim.blob_positions())
+    for b, lo in ((0, 0), (1, n[0])):
+        if n[b] == 0:
+            continue
+        q_ref, v_ref = oracle.stokes_step(g, 4, q0[b], np.arange(n[b], dtype=np.int32), *none,
+                                          0.0, 0.0, 0.0, ext=F[b])
+        assert rel_l2(v[b], v_ref) < 1e-5            # the repository's bound for FP32 Stokes steps
+        assert_positions(q[lo:lo + n[b]], q_ref, q0[b], g.L, 4, 2e-5)
+
+
+@pytest.mark.parametrize("n", [(8, 256, 8), (16, 16, 64)])
+def test_fp32_stokes_replays_after_the_tile_timing(n):
+    """Stokes steps in both numbers of passes whose first, direct step times the spreading tiles
+    and leaves the force grid cleared: the replays after it clear it themselves where due."""
+    g = oracle.Grid(*n, dt=0.3, mean_mode=1)
+    d = mb.GridDesc(*n, dt=0.3, precision=0, mean_mode=1, integrator=1)
+    rng = np.random.default_rng(n[1])
+    none = (np.zeros((0, 2), np.int32), np.zeros(0))
+    for nblobs in (7, 19):                    # a tile choice of their own each
+        q0, F = rng.random((nblobs, 3)) * n, rng.normal(size=(nblobs, 3))
+        F -= F.mean(0)
+        pid = np.arange(nblobs, dtype=np.int32)
+        with mb.Multiblob(d) as sim:
+            sim.set_particles(0, q0, pid, *none, 0.0)
+            sim.step(5, ext_blob_force=F)
+            v, q = to_np(sim.velocity_field())[0], to_np(sim.blob_positions())
+        q_ref, v_ref = oracle.stokes_step(g, 5, q0, pid, *none, 0.0, 0.0, 0.0, ext=F)
+        assert rel_l2(v, v_ref) < 1e-5
+        assert_positions(q, q_ref, q0, g.L, 5, 2e-5)
