@@ -250,10 +250,16 @@ mb_status mb_set_positions(mb_ctx* ctx, const double* pos);
  * so its transpose reuses the forward solver; the blob-force transpose is the force Hessian
  * applied to the incoming gradient (forces derive from a potential).  Provided for FP64
  * contexts (precision 1) with batch 1, integrator 0, kT = 0 and advection = 0; MB_EINVAL
- * otherwise.  Arrays may be host or device. */
+ * otherwise.  Arrays may be host or device.  With grad_k_spring the results are complete on
+ * return. */
 mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n,
                           const double* ext_blob_force, const double* body_force,
                           double* grad_pos, void* grad_v, double* grad_k_spring);
+/* The same, complete in the order of the context's stream only (device arrays stay the caller's
+ * to keep until then). */
+mb_status mb_adjoint_step_async(mb_ctx* ctx, const double* pos_n, const void* grid_v_n,
+                                const double* ext_blob_force, const double* body_force,
+                                double* grad_pos, void* grad_v, double* grad_k_spring);
 
 /* Adjoint of the blob velocities u = J(q) v (Eq. ju) at positions pos and field grid_v:
  * grad_pos += (du/dq)^T grad_u and grad_v += J^T grad_u = h^3 S(q) grad_u.  FP64 contexts with

@@ -109,6 +109,7 @@ def load_library(path: str | None = None):
         "mb_set_positions": [P, P],
         "mb_get_tuning": [P, P, P],
         "mb_adjoint_step": [P, P, P, P, P, P, P, P],
+        "mb_adjoint_step_async": [P, P, P, P, P, P, P, P],
         "mb_velocity_adjoint": [P, P, P, P, P, P],
         "mb_particle_velocity_adjoint": [P, P, P, P, P, P],
         "mb_get_stage_times": [P, I, P, P, ctypes.POINTER(I)],
@@ -278,10 +279,16 @@ def get_step_index(ctx):
 def adjoint_step(ctx, pos_n, grid_v_n, ext_blob_force, body_force, grad_pos, grad_v,
                  grad_k_spring=None):
     """mb_adjoint_step: overwrites grad_pos and grad_v in place, adds to grad_k_spring[0]."""
+    _adjoint_step(load_library().mb_adjoint_step, ctx, pos_n, grid_v_n, ext_blob_force, body_force,
+                  grad_pos, grad_v, grad_k_spring)
+
+
+def _adjoint_step(entry, ctx, pos_n, grid_v_n, ext_blob_force, body_force, grad_pos, grad_v,
+                  grad_k_spring):
     body = None
     if body_force is not None:
         body = np.ascontiguousarray(np.asarray(body_force, dtype=np.float64).reshape(4))
-    _check(ctx, load_library().mb_adjoint_step(
+    _check(ctx, entry(
         ctx, _ptr(pos_n, np.float64), _ptr(grid_v_n), _ptr(ext_blob_force, np.float64),
         _ptr(body), _ptr(grad_pos, np.float64), _ptr(grad_v),
         _ptr(grad_k_spring, np.float64) if grad_k_spring is not None else None))

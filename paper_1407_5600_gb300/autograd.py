@@ -15,7 +15,7 @@ from __future__ import annotations
 import numpy as np
 import torch
 
-from . import (Multiblob, adjoint_step, particle_velocity_adjoint, set_positions,
+from . import (Multiblob, _adjoint_step, load_library, particle_velocity_adjoint, set_positions,
                set_velocity_field, step)
 
 
@@ -47,7 +47,12 @@ class _Rollout(torch.autograd.Function):
         particle_velocity_adjoint(sim.ctx, fctx.qK, fctx.vK,
                                   gU.to(dtype=torch.float64, device=sim.device).contiguous(),
                                   gq, gv)
-        # on the device, so that no step of the backward pass waits for the host
+        # on the device, and on the context's own stream with steps that are complete in its order
+        # only, so that no step of the backward pass waits for the host (64 particles at 64^3, 50
+        # steps: 20.3 ms, 21.4 with a wait a step)
+        lib = load_library()
+        own = torch.cuda.current_stream(sim.device) == sim.stream
+        entry = lib.mb_adjoint_step_async if own else lib.mb_adjoint_step
         gk = torch.zeros(1, dtype=torch.float64, device=sim.device)
         K, chk_every = fctx.K, fctx.checkpoint
         for seg in reversed(range(len(fctx.chk))):
@@ -60,7 +65,7 @@ class _Rollout(torch.autograd.Function):
                 states.append((sim.blob_positions(), sim.velocity_field()))
                 step(sim.ctx, 1, fctx.ext, fctx.body)
             for qn, vn in reversed(states):
-                adjoint_step(sim.ctx, qn, vn, fctx.ext, fctx.body, gq, gv, gk)
+                _adjoint_step(entry, sim.ctx, qn, vn, fctx.ext, fctx.body, gq, gv, gk)
         return gq, gk[0], None, None, None, None, None, None
 
 

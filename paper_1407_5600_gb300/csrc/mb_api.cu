@@ -2207,6 +2207,7 @@ mb_status mb_set_positions(mb_ctx* ctx, const double* pos)
     ctx->sorted_valid = false;
     ctx->pred_ready = false;
     ctx->steps_taken = 0;
+    MB_CUDA(cudaStreamSynchronize(ctx->st));      // the caller's array is free on return
     return MB_OK;
 }
 
@@ -2327,6 +2328,19 @@ mb_status mb_particle_velocity_adjoint(mb_ctx* ctx, const double* pos, const voi
 mb_status mb_adjoint_step(mb_ctx* ctx, const double* pos_n, const void* grid_v_n,
                           const double* ext_blob_force, const double* body_force,
                           double* grad_pos, void* grad_v, double* grad_k_spring)
+{
+    MB_TRY(mb_adjoint_step_async(ctx, pos_n, grid_v_n, ext_blob_force, body_force, grad_pos, grad_v,
+                                 grad_k_spring));
+    if (grad_k_spring) {
+        DeviceGuard dg(ctx->device);
+        MB_CUDA(cudaStreamSynchronize(ctx->st));
+    }
+    return MB_OK;
+}
+
+mb_status mb_adjoint_step_async(mb_ctx* ctx, const double* pos_n, const void* grid_v_n,
+                                const double* ext_blob_force, const double* body_force,
+                                double* grad_pos, void* grad_v, double* grad_k_spring)
 {
     if (!ctx) return MB_EINVAL;
     DeviceGuard dg(ctx->device);
@@ -2551,6 +2565,7 @@ mb_status mb_set_velocity_field(mb_ctx* ctx, const void* grid_v)
     ctx->pred_ready = false;              // the next predictor must see the new field
     if (ctx->d.mean_mode == 1) {
         MB_CUDA(cudaMemsetAsync(ctx->vbar.p, 0, sizeof(double) * 3 * ctx->B, ctx->st));
+        MB_CUDA(cudaStreamSynchronize(ctx->st));  // the caller's array is free on return
         return MB_OK;
     }
     MB_TRY(ensure(ctx->mean_scratch, sizeof(double) * 3 * ctx->B * grid_mean_chunks(ctx->g.N),
@@ -2562,6 +2577,7 @@ mb_status mb_set_velocity_field(mb_ctx* ctx, const void* grid_v)
     else
         MB_CUDA(launch_grid_mean<double>(ctx->st, ctx->B, ctx->g, static_cast<const double*>(ctx->v[ctx->cur].p),
                                          static_cast<double*>(ctx->vbar.p), partial));
+    MB_CUDA(cudaStreamSynchronize(ctx->st));
     return MB_OK;
 }
 

@@ -99,3 +99,37 @@ def test_adjoint_arrays_in_place_and_staged(k_rep):
     for r in res[1:]:
         for a, b in zip(r, res[0]):
             assert rel_l2(a, b) < 1e-10
+
+
+@pytest.mark.parametrize("prec", [1, 0])
+def test_state_arrays_are_free_on_return(prec):
+    """Page-locked host arrays given to set_positions and set_velocity_field behind a queue of
+    steps may be overwritten as soon as the calls return; so may a device array by another
+    stream's work."""
+    d = mb.GridDesc(32, 32, 32, precision=prec, mean_mode=1, dt=0.01)
+    rng = np.random.default_rng(5)
+    none = (np.zeros((0, 2), np.int32), np.zeros(0))
+    q0 = rng.random((200, 3)) * 32
+    v0 = wl.random_field((32, 32, 32), 6).astype(d.grid_dtype)[None]
+    dev = torch.tensor(q0, device="cuda")
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with mb.Multiblob(d) as sim:
+        sim.set_particles(0, rng.random((200, 3)) * 32, np.arange(200, dtype=np.int32), *none, 0.0)
+        for kind in ("pinned", "device"):
+            sim.step(200, body_force=(0.1, 0, 1, 1))
+            if kind == "pinned":
+                q, v = torch.tensor(q0).pin_memory(), torch.tensor(v0).pin_memory()
+                mb.set_positions(sim.ctx, q.numpy())
+                q.zero_()
+                sim.step(200)
+                mb.set_velocity_field(sim.ctx, v.numpy())
+                v.zero_()
+                assert np.array_equal(to_np(sim.velocity_field()), v0)
+                sim.step(200)
+                mb.set_positions(sim.ctx, torch.tensor(q0).pin_memory().numpy())
+            else:
+                mb.set_positions(sim.ctx, dev)
+                with torch.cuda.stream(other):
+                    dev.zero_()
+            assert np.max(np.abs(to_np(sim.blob_positions()) - q0)) < 1e-12
