@@ -412,14 +412,20 @@ k_zsolve(FluidArgs<float> a, GridGeo g)
         return (c * nzp + (FIX ? pad_line<NL>(z) : z + (z >> sz))) * CL + k;
     };
     const int total = 3 * nz * C;
-    // compile-time lines: thread (row r = tid / C, column k) moves the elements z = r % N2 + N2 j of
-    // component r / N2, at fixed strides on both sides
-    const int fk = threadIdx.x % C, fr = threadIdx.x / C;
-    float2* fs = Bf + (fr / Z2 * ZP + fr % Z2) * CL + fk;
-    float2* fg = base + fr / Z2 * cstride + (size_t)(fr % Z2) * zstride + fk;
+    // compile-time lines: thread (row r = 2 tid / C, columns k, k + 1) moves 16 bytes of the elements
+    // z = z0 + 2 N2 j of component r / (2 N2), at fixed strides on both sides; z0 = r % (2 N2) with
+    // its low bits swapped, so that the two rows of a quarter-warp (CL = 12: 96 bytes apart for
+    // neighbours, 64 mod 128 for every other) fall on different banks.  8 -> 16 bytes: 32 boxes of
+    // 64^3 68.2 -> 64.0 us, 128^3 20.4 -> 19.2
+    const int fk = 2 * (threadIdx.x % (C / 2)), fr = threadIdx.x / (C / 2), f0 = fr % (2 * Z2);
+    const int fz = Z2 == 4 ? f0 : (f0 & ~3) | (f0 & 1) << 1 | (f0 >> 1 & 1);
+    float2* fs = Bf + (fr / (2 * Z2) * ZP + pad_line<NL>(fz)) * CL + fk;
+    float2* fg = base + fr / (2 * Z2) * cstride + (size_t)fz * zstride + fk;
     if constexpr (FIX) {
 #pragma unroll
-        for (int j = 0; j < NL / Z2; ++j) async_copy(fs + (Z2 + 1) * CL * j, fg + (size_t)(Z2 * j) * zstride);
+        for (int j = 0; j < NL / (2 * Z2); ++j)
+            async_copy(reinterpret_cast<float4*>(fs + 2 * (Z2 + 1) * CL * j),
+                       reinterpret_cast<const float4*>(fg + (size_t)(2 * Z2 * j) * zstride));
     } else {
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             const int k = i % C, zc = i / C, z = zc & (nz - 1), c = zc >> lz;
@@ -494,7 +500,9 @@ k_zsolve(FluidArgs<float> a, GridGeo g)
     __syncthreads();
     if constexpr (FIX) {
 #pragma unroll
-        for (int j = 0; j < NL / Z2; ++j) fg[(size_t)(Z2 * j) * zstride] = fs[(Z2 + 1) * CL * j];
+        for (int j = 0; j < NL / (2 * Z2); ++j)
+            *reinterpret_cast<float4*>(fg + (size_t)(2 * Z2 * j) * zstride) =
+                *reinterpret_cast<const float4*>(fs + 2 * (Z2 + 1) * CL * j);
     } else {
         for (int i = threadIdx.x; i < total; i += blockDim.x) {
             const int k = i % C, zc = i / C, z = zc & (nz - 1), c = zc >> lz;
@@ -661,7 +669,7 @@ cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const Flu
     // planes of sides from 32 to 128 have layouts at compile-time offsets; MB_PLANE_LAYOUT=pad
     // keeps the padded run-time one, for comparison.  32 boxes of 64^3, run-time / compile-time:
     // forward 128 / 90 us (with the untouched planes of f left out), inverse 114 / 75 (without
-    // the sum v^n + v^{n+1}), z 77 / 68; the L1 is then 83 to 88% busy
+    // the sum v^n + v^{n+1}), z 77 / 64; the L1 is then 83 to 88% busy
     static const bool pad = [] {
         const char* e = std::getenv("MB_PLANE_LAYOUT");
         return e && std::string(e) == "pad";
