@@ -1202,6 +1202,21 @@ k_ext_prepare(const int64_t* __restrict__ box_off, const double* __restrict__ ex
     __syncthreads();
     if (!last) return;
     __threadfence();
+    // few partials a box, or many boxes: a warp a box (32 boxes of one chunk each: 12 us; box after
+    // box by the whole block with its barriers: 65)
+    if (nchunk <= 64 || gridDim.y >= 8) {
+        for (int bx = warp; bx < (int)gridDim.y; bx += (int)(blockDim.x >> 5)) {
+            double t[3] = {0.0, 0.0, 0.0};
+            for (int c = lane; c < nchunk; c += 32)
+                for (int d = 0; d < 3; ++d) t[d] += __ldcg(partial + ((int64_t)bx * nchunk + c) * 3 + d);
+            for (int o = 16; o > 0; o >>= 1)
+                for (int d = 0; d < 3; ++d) t[d] += __shfl_down_sync(0xffffffffu, t[d], o);
+            if (lane == 0)
+                for (int d = 0; d < 3; ++d) ext_sum[3 * bx + d] = t[d];
+        }
+        if (threadIdx.x == 0) *ticket = 0u;
+        return;
+    }
     for (int bx = 0; bx < (int)gridDim.y; ++bx) {
         double t[3] = {0.0, 0.0, 0.0};
         for (int c = threadIdx.x; c < nchunk; c += blockDim.x)

@@ -635,14 +635,22 @@ mb_status rebuild(mb_ctx* ctx)
         MB_TRY(up(ctx->tstart32, t_start.data(), sizeof(int32_t) * (2 * pm + 1)));
         if (ctx->rsz == 8) MB_TRY(ensure(ctx->Fpre64, sizeof(double) * 3 * nb, E, "spring forces"));
     }
-    // FP64 inertial steps: from one blob in 32 cells on, the inverse plane pass also writes
-    // v^n + v^{n+1}, 48 bytes a cell under its arithmetic, and saves the corrector 81 additions a
-    // blob on the narrow FP64 pipe
-    if (ctx->rsz == 8 && ctx->d.integrator == 0) {
-        if (ctx->fft_passes == 3 && 32 * nb >= B * ctx->g.N)
+    // Inertial steps: with many blobs the inverse plane pass also writes v^n + v^{n+1}.  FP64: from
+    // one blob in 32 cells on; 48 bytes a cell under the pass's arithmetic save the corrector 81
+    // additions a blob on the narrow FP64 pipe.  FP32: from one in 10 on; a read and a write of the
+    // grid save the corrector half its gathers (128^3, plane pass and corrector without / with the
+    // sum: 53 / 54 us of 104,000 blobs, 65 / 66 of 156,000, 74 / 72 of 244,504)
+    if (ctx->d.integrator == 0) {
+        const int64_t cells = ctx->rsz == 8 ? 32 : (ctx->fuse_interp ? 10 : 0);
+        if (nb > 0 && ctx->fft_passes == 3 && cells * nb >= B * ctx->g.N)
             MB_TRY(ensure(ctx->vsum, grid_bytes(ctx, B), E, "v sum"));
         else
             MB_CUDA(dfree(ctx->vsum));
+    }
+    if (ctx->rsz == 4 && ctx->fft_passes == 3 && spread32_few(nb)) {
+        const size_t by = sizeof(int) * (size_t)B * ctx->g.n[2];
+        MB_TRY(ensure(ctx->f_dirty, by, E, "planes of f"));
+        MB_CUDA(cudaMemsetAsync(ctx->f_dirty.p, 0, by, ctx->st));
     }
     if (ctx->rsz == 4) {
         MB_TRY(ensure(ctx->sA, sizeof(float4) * nb, E, "split q"));
@@ -1266,11 +1274,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
         fa.f_clear = static_cast<float*>(ctx->f.p);
         fa.f_dirty = f_planes(ctx);
     }
-    // the sum v^n + v^{n+1} costs the plane pass a read and a write of the grid and saves the
-    // corrector half its gathers.  128^3, plane pass and corrector without / with the sum: 53 / 54 us
-    // of 104,000 blobs, 65 / 66 of 156,000, 74 / 72 of 244,504
-    const bool vsum = blobs && ctx->fuse_interp && ctx->fft_passes == 3 &&
-                      10 * ctx->nb >= B * g.N;
+    const bool vsum = blobs && ctx->vsum.p != nullptr;
     if (vsum) {
         fa.v_sum_base = vcur;
         fa.v_sum_out = static_cast<float*>(ctx->vsum.p);
@@ -1896,13 +1900,7 @@ mb_status mb_create_grid(const mb_grid_desc* desc, void* cuda_stream, mb_ctx** o
     mb_status s;
     if ((s = ensure(ctx->v[0], gb, ctx->err, "v")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->v[1], gb, ctx->err, "v")) != MB_OK) return fail(s);
-    if (ctx->rsz == 4 && (s = ensure(ctx->vsum, gb, ctx->err, "v sum")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->f, gb, ctx->err, "f")) != MB_OK) return fail(s);
-    if (ctx->rsz == 4 && ctx->fft_passes == 3) {
-        const size_t db = sizeof(int) * (size_t)ctx->B * ns[2];
-        if ((s = ensure(ctx->f_dirty, db, ctx->err, "planes of f")) != MB_OK) return fail(s);
-        cudaMemsetAsync(ctx->f_dirty.p, 0, db, ctx->st);
-    }
     if ((s = ensure(ctx->spec, sb, ctx->err, "spectrum")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->vbar, sizeof(double) * 3 * ctx->B, ctx->err, "vbar")) != MB_OK) return fail(s);
     if ((s = ensure(ctx->step_index, sizeof(uint64_t), ctx->err, "step index")) != MB_OK) return fail(s);
