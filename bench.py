@@ -35,21 +35,22 @@ DENSE128_BLOBS, DENSE128_PARTICLES = 244504, 18808      # the recipe's counts at
 
 # What bounds each FP64-grid kernel below the HBM roofline (ncu, dense 128^3 workload).
 FP64_LIMITERS = {
-    "spread": "FP64 shared-memory atomic adds (one per node contribution)",
+    "spread": "FP64 global atomic adds (one per node contribution)",
     "forces": "FP64 arithmetic of the bond and repulsion forces",
     "fluid_x_fwd": "FP32-pipe issue of the double-float FFT arithmetic",
     "fluid_z_solve": "FP32-pipe issue of the double-float FFT arithmetic",
     "fluid_x_inv": "FP32-pipe issue of the double-float FFT arithmetic",
-    "interp_correct": "gather latency (L1 sectors per request)",
-    "interp_predict": "gather latency (L1 sectors per request)",
+    "interp_correct": "FP64 arithmetic of the weights and sums",
+    "interp_predict": "FP64 arithmetic of the weights and sums",
 }
 
 # Algorithmic bytes moved by each stage per step, per unit:
 #   grid real = 4 B (FP32) / 8 B (FP64); half-spectrum complex = 2 reals; blob FP64 vec = 24 B.
 def stage_model(n, nb, rsz, ncell, thermal=False):
     """Algorithmic bytes per stage.  FP32 grids (rsz = 4) fuse the next step's predictor into
-    the corrector pass, whose grid v^n + v^{n+1} the inverse plane pass writes; FP64 grids
-    (rsz = 8) run the predictor as its own pass and the corrector reads v^n and v^{n+1}."""
+    the corrector pass; FP64 grids (rsz = 8) run the predictor as its own pass.  With this many
+    blobs the corrector of both reads v^n + v^{n+1}, which the inverse plane pass writes.
+    thermal: the 256^3 workload, whose first FFT pass reads the nine stress grids."""
     N = n ** 3
     grid = 3 * N * rsz                                  # one 3-component grid
     spec = 3 * n * n * (n // 2 + 1) * 2 * rsz           # one 3-component half spectrum
@@ -66,8 +67,8 @@ def stage_model(n, nb, rsz, ncell, thermal=False):
             "fluid_y_fwd": ("hbm", 0),
             "fluid_z_solve": ("hbm", 2 * spec),
             "fluid_y_inv": ("hbm", 0),
-            "fluid_x_inv": ("hbm", spec + grid),        # read spectrum; write v^{n+1}
-            "interp_correct": ("hbm", 2 * grid + 3 * vec),   # read v^n, v^{n+1}, q_half, q; write q
+            "fluid_x_inv": ("hbm", spec + 3 * grid),    # as below
+            "interp_correct": ("hbm", grid + 3 * vec),  # read v^n + v^{n+1}, q_half, q; write q
         }
     return {
         # the predictor of step n+1 runs inside step n's corrector pass (same gathered nodes)
@@ -79,10 +80,10 @@ def stage_model(n, nb, rsz, ncell, thermal=False):
         "forces": ("hbm", nb * (24 + 4 + 4 + 24 + 48)),
         "force_sum": ("hbm", 0),
         "spread": ("hbm", 48 * nb + grid),               # sorted (q, F) records; write f
-        # thermal / convective stress (kT > 0 or advection only): write 9 stress grids, read
-        # them and f, write f
-        "fluid_stress": ("hbm", 3 * grid + 3 * grid + 2 * grid if thermal else 0),
-        "fluid_x_fwd": ("hbm", 2 * grid + spec),         # read v, f; write spectrum
+        # thermal / convective stress (kT > 0 or advection only): write 9 stress grids
+        "fluid_stress": ("hbm", 3 * grid if thermal else 0),
+        # read v, f (and the stress); write spectrum
+        "fluid_x_fwd": ("hbm", (5 if thermal else 2) * grid + spec),
         "fluid_y_fwd": ("hbm", 0),                       # no kernel in the three-pass FFT
         "fluid_z_solve": ("hbm", 2 * spec),
         "fluid_y_inv": ("hbm", 0),                       # no kernel in the three-pass FFT
