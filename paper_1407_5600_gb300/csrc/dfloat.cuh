@@ -144,10 +144,6 @@ __host__ __device__ __forceinline__ dfloat operator*(dfloat a, dfloat b)
     return dd_fast_two_sum(p, e);
 }
 
-__host__ __device__ __forceinline__ dfloat& operator+=(dfloat& a, dfloat b) { return a = a + b; }
-__host__ __device__ __forceinline__ dfloat& operator-=(dfloat& a, dfloat b) { return a = a - b; }
-__host__ __device__ __forceinline__ dfloat& operator*=(dfloat& a, dfloat b) { return a = a * b; }
-
 // 1 / x: the float reciprocal refined by one Newton step in double-float.
 __host__ __device__ __forceinline__ dfloat dd_recip(dfloat x)
 {

@@ -6,7 +6,6 @@
 // (X[k1 + N1 k2] = sum_n2 W_N2^{n2 k2} W_N^{n2 k1} sum_n1 x[N2 n1 + n2] W_N1^{n1 k1}).
 #pragma once
 #include "mb_internal.cuh"
-#include "dfloat.cuh"
 
 namespace mbk {
 namespace {
