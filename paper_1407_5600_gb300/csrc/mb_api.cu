@@ -267,38 +267,49 @@ mb_status invalid(mb_ctx* ctx, const std::string& msg)
 
 size_t grid_bytes(const mb_ctx* ctx, int boxes) { return (size_t)boxes * 3 * ctx->g.N * ctx->rsz; }
 
-// Copies an input array to the device if it lives in host memory.
+// Whether kernels may access a device array in vectors of `align` bytes.
+bool aligned(const void* p, size_t align) { return (reinterpret_cast<uintptr_t>(p) & (align - 1)) == 0; }
+
+// Copies an input array to the device if it lives in host memory, or in device memory at an
+// address that its kernels' loads of `align` bytes cannot take.
 mb_status stage_in(mb_ctx* ctx, const void* p, size_t bytes, DBuf& buf, const void** out,
-                   const char* what)
+                   const char* what, size_t align = 1)
 {
-    if (is_device_ptr(p)) {
+    const bool device = is_device_ptr(p);
+    if (device && aligned(p, align)) {
         *out = p;
         return MB_OK;
     }
     MB_TRY(ensure(buf, bytes, ctx->err, what));
-    MB_CUDA(cudaMemcpyAsync(buf.p, p, bytes, cudaMemcpyHostToDevice, ctx->st));
+    MB_CUDA(cudaMemcpyAsync(buf.p, p, bytes,
+                            device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->st));
     *out = buf.p;
     return MB_OK;
 }
 
-// Device destination for an output: the caller's pointer, or a staging buffer.
-mb_status out_target(mb_ctx* ctx, void* p, size_t bytes, DBuf& buf, void** dev, bool* host,
-                     const char* what)
+// Device destination for an output: the caller's pointer, or a staging buffer for host memory and
+// for addresses that stores of `align` bytes cannot take.
+mb_status out_target(mb_ctx* ctx, void* p, size_t bytes, DBuf& buf, void** dev, bool* staged,
+                     const char* what, size_t align = 1)
 {
-    if (is_device_ptr(p)) {
+    if (is_device_ptr(p) && aligned(p, align)) {
         *dev = p;
-        *host = false;
+        *staged = false;
         return MB_OK;
     }
     MB_TRY(ensure(buf, bytes, ctx->err, what));
     *dev = buf.p;
-    *host = true;
+    *staged = true;
     return MB_OK;
 }
 
-mb_status finish_out(mb_ctx* ctx, void* p, const void* dev, size_t bytes, bool host)
+mb_status finish_out(mb_ctx* ctx, void* p, const void* dev, size_t bytes, bool staged)
 {
-    if (!host) return MB_OK;
+    if (!staged) return MB_OK;
+    if (is_device_ptr(p)) {
+        MB_CUDA(cudaMemcpyAsync(p, dev, bytes, cudaMemcpyDeviceToDevice, ctx->st));
+        return MB_OK;
+    }
     MB_CUDA(cudaMemcpyAsync(p, dev, bytes, cudaMemcpyDeviceToHost, ctx->st));
     MB_CUDA(cudaStreamSynchronize(ctx->st));
     return MB_OK;
@@ -2592,7 +2603,8 @@ mb_status mb_spread(mb_ctx* ctx, int64_t n, const double* pos, const double* F, 
     const size_t by = grid_bytes(ctx, 1);
     void* dst;
     bool host;
-    MB_TRY(out_target(ctx, grid_out, by, ctx->s_out, &dst, &host, "grid_out"));
+    // FP32 rows are added in pairs of nodes (k_spread_atomic), each pair on 8 bytes
+    MB_TRY(out_target(ctx, grid_out, by, ctx->s_out, &dst, &host, "grid_out", ctx->rsz == 4 ? 8 : 1));
     const double scale = ctx->g.inv_h * ctx->g.inv_h * ctx->g.inv_h;
     if (ctx->rsz == 4)
         MB_CUDA(launch_spread_atomic<float>(ctx->st, 1, n, static_cast<const double*>(qd),
