@@ -2222,16 +2222,17 @@ mb_status mb_set_positions(mb_ctx* ctx, const double* pos)
 
 namespace {
 
-// A caller array as device memory of this context: itself when it is there, otherwise (host
-// memory, another GPU) a copy in buf.
+// A caller array as device memory of this context at a multiple of `align` bytes: itself when it
+// is that, otherwise (host memory, another GPU, another address) a copy in buf.
 mb_status pull(mb_ctx* ctx, DBuf& buf, const void* src, size_t bytes, const char* what,
-               const double** out)
+               const double** out, size_t align = sizeof(double))
 {
     cudaPointerAttributes at;
     const bool known = cudaPointerGetAttributes(&at, src) == cudaSuccess;
     if (!known) cudaGetLastError();
-    if (known && (at.type == cudaMemoryTypeManaged ||
-                  (at.type == cudaMemoryTypeDevice && at.device == ctx->device))) {
+    if (known && aligned(src, align) &&
+        (at.type == cudaMemoryTypeManaged ||
+         (at.type == cudaMemoryTypeDevice && at.device == ctx->device))) {
         *out = static_cast<const double*>(src);
         return MB_OK;
     }
@@ -2248,7 +2249,7 @@ struct Span {
     size_t bytes;
 };
 mb_status pull_inout(mb_ctx* ctx, DBuf& buf, void* p, size_t bytes, const char* what,
-                     const std::vector<Span>& inputs, double** out)
+                     const std::vector<Span>& inputs, double** out, size_t align = sizeof(double))
 {
     const double* dev = nullptr;
     bool shared = false;
@@ -2256,7 +2257,7 @@ mb_status pull_inout(mb_ctx* ctx, DBuf& buf, void* p, size_t bytes, const char* 
         if (s.p)
             shared = shared || ((const char*)p < (const char*)s.p + s.bytes &&
                                 (const char*)s.p < (const char*)p + bytes);
-    if (!shared) MB_TRY(pull(ctx, buf, p, bytes, what, &dev));
+    if (!shared) MB_TRY(pull(ctx, buf, p, bytes, what, &dev, align));
     if (shared) {
         MB_TRY(ensure(buf, bytes, ctx->err, what));
         MB_CUDA(cudaMemcpyAsync(buf.p, p, bytes, cudaMemcpyDefault, ctx->st));
@@ -2372,11 +2373,13 @@ mb_status mb_adjoint_step_async(mb_ctx* ctx, const double* pos_n, const void* gr
                                {has_ext ? ext_blob_force : nullptr, bv}};
     const double *qn, *vn, *ext = nullptr;
     double *gq, *gv;
+    // the five-pass FFT loads its grids in pairs of doubles, all other kernels value by value
+    const size_t wide = ctx->fft_passes == 5 ? sizeof(double2) : sizeof(double);
     MB_TRY(pull(ctx, ctx->a_qn, pos_n, bv, "adjoint q", &qn));
-    MB_TRY(pull(ctx, ctx->a_vn, grid_v_n, bg, "adjoint v", &vn));
+    MB_TRY(pull(ctx, ctx->a_vn, grid_v_n, bg, "adjoint v", &vn, wide));
     if (has_ext) MB_TRY(pull(ctx, ctx->ext, ext_blob_force, bv, "adjoint ext", &ext));
     MB_TRY(pull_inout(ctx, ctx->a_gq, grad_pos, bv, "adjoint gq", in, &gq));
-    MB_TRY(pull_inout(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv", in, &gv));
+    MB_TRY(pull_inout(ctx, ctx->a_gvn, grad_v, bg, "adjoint gv", in, &gv, wide));
     for (DBuf* b : {&ctx->a_qh, &ctx->a_gqh, &ctx->a_gF}) MB_TRY(ensure(*b, bv, E, "adjoint blobs"));
     for (DBuf* b : {&ctx->a_vp, &ctx->a_gf}) MB_TRY(ensure(*b, bg, E, "adjoint grids"));
     // dL/dk: added straight to device memory of this context, through a device scalar otherwise

@@ -49,3 +49,58 @@ def test_spread_into_an_odd_offset(n, nblobs, prec, off):
         mb.spread(sim.ctx, pos, F, out)
     assert rel_l2(to_np(out), to_np(want)) < (1e-12 if prec else 1e-5)
     assert _untouched(store, off, out.numel())
+
+
+def _particles(n, seed):
+    """Two icosahedra at random places of a box of sides n."""
+    rng = np.random.default_rng(seed)
+    L = np.array(n, dtype=np.float64)
+    return wl.build_particles(rng.random((2, 3)) * L, 0.9, rng, L), rng
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+@pytest.mark.parametrize("n", [(8, 8, 256), (256, 4, 8), (16, 8, 32)])
+def test_step_adjoint_on_odd_offsets(n, off):
+    """Velocity and gradients at an odd element (the field behind the positions in one flat state,
+    say), with five FFT passes and with three, against arrays of their own; and that gradient
+    against central differences of the step."""
+    s, rng = _particles(n, off)
+    shape = (1, 3, n[2], n[1], n[0])
+    body = (1e-3, 0, 2, 1)
+
+    def dev(x):
+        return torch.as_tensor(x, device="cuda")
+
+    q, ext = dev(s.pos), dev(rng.normal(scale=1e-3, size=s.pos.shape))
+    v = dev(rng.normal(scale=1e-3, size=shape))
+    cq, cv = dev(rng.normal(size=s.pos.shape)), dev(rng.normal(size=shape))
+    L = dev(np.array(n, dtype=np.float64))
+    with mb.Multiblob(mb.GridDesc(*n, precision=1, dt=0.05)) as sim:
+        sim.set_particles(0, s.pos, s.pid, s.bonds, s.rest, 100.0)
+        gq, gv, gk = cq.clone(), cv.clone(), torch.zeros(1, dtype=torch.float64, device="cuda")
+        mb.adjoint_step(sim.ctx, q, v, ext, body, gq, gv, gk)
+        vo, _ = _odd(shape, torch.float64, off, v)
+        qo, _ = _odd(s.pos.shape, torch.float64, off, q)
+        go, store = _odd(shape, torch.float64, off, cv)
+        gqo, qstore = _odd(s.pos.shape, torch.float64, off, cq)
+        gko = torch.zeros(1, dtype=torch.float64, device="cuda")
+        mb.adjoint_step(sim.ctx, qo, vo, ext, body, gqo, go, gko)
+        for a, b in ((gqo, gq), (go, gv), (gko, gk)):
+            assert rel_l2(to_np(a), to_np(b)) < 1e-12
+        assert _untouched(store, off, v.numel()) and _untouched(qstore, off, q.numel())
+        assert torch.equal(vo, v) and torch.equal(qo, q)
+
+        def loss(qq, vv):
+            sim.set_positions(qq)
+            sim.set_velocity_field(vv)
+            sim.step(1, ext_blob_force=ext, body_force=body)
+            dq = sim.blob_positions() - q
+            dq -= torch.round(dq / L) * L
+            return float((cq * dq).sum() + (cv * sim.velocity_field()).sum())
+
+        eps = 1e-6
+        for dq, dv, g in ((dev(rng.normal(size=s.pos.shape)), 0.0 * v, gq),
+                          (0.0 * q, dev(rng.normal(size=shape)), gv)):
+            fd = (loss(q + eps * dq, v + eps * dv) - loss(q - eps * dq, v - eps * dv)) / (2 * eps)
+            an = float((g * (dv if g is gv else dq)).sum())
+            assert abs(an - fd) < 1e-6 * max(1.0, abs(fd)), (an, fd)
