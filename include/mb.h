@@ -19,7 +19,9 @@
  *    FP32-grid mb_step reads page-locked external forces directly instead).  Input arrays in
  *    device or page-locked memory are read in stream order, like cudaMemcpyAsync: keep them
  *    unchanged until the stream has reached the call.  The caller owns every array it
- *    passes; no caller pointer is used by work enqueued after the call returns.
+ *    passes; no caller pointer is used by work enqueued after the call returns.  Arrays need
+ *    the alignment of their elements only; device grids that are not on 16 bytes may be copied
+ *    through the library's buffers.
  *  - Environment (read when a context is created; for comparisons and tuning, the defaults
  *    are the fast path): MB_FFT_PASSES=5 runs the fluid solve as five one-axis passes instead
  *    of three; MB_NO_GRAPH=1 launches every step directly instead of replaying its captured CUDA

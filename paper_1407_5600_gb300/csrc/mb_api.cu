@@ -2654,8 +2654,10 @@ mb_status mb_fluid_update(mb_ctx* ctx, const void* v_in, const void* f, const do
     if ((!v_in && !stokes) || !v_out) return invalid(ctx, "v_in and v_out must be non-null");
     const size_t by = grid_bytes(ctx, 1);
     const void *vd = nullptr, *fd = nullptr;
-    if (!stokes) MB_TRY(stage_in(ctx, v_in, by, ctx->s_g1, &vd, "v_in"));
-    if (f) MB_TRY(stage_in(ctx, f, by, ctx->s_g2, &fd, "f"));
+    // the FP32 passes and the five FP64 ones load and store 16 bytes at a time
+    const size_t wide = ctx->rsz == 4 || ctx->fft_passes == 5 ? 16 : 1;
+    if (!stokes) MB_TRY(stage_in(ctx, v_in, by, ctx->s_g1, &vd, "v_in", wide));
+    if (f) MB_TRY(stage_in(ctx, f, by, ctx->s_g2, &fd, "f", wide));
     // - rho D.(v_in v_in): from the stress itself in the first FFT pass, or for the FP64 three-pass
     // FFT through the library's own copy of f (the caller's f is not written)
     const bool through_f = ctx->advect && ctx->rsz == 8 && ctx->fft_passes == 3;
@@ -2682,7 +2684,7 @@ mb_status mb_fluid_update(mb_ctx* ctx, const void* v_in, const void* f, const do
     if (body_force) MB_TRY(set_body(ctx, body_force, ctx->prof_scratch, false));
     void* dst;
     bool host;
-    MB_TRY(out_target(ctx, v_out, by, ctx->s_out, &dst, &host, "v_out"));
+    MB_TRY(out_target(ctx, v_out, by, ctx->s_out, &dst, &host, "v_out", wide));
     auto stokes_args = [&](auto& a) {
         a.v = a.v_out;                      // unread: the right-hand side is f + f_body
         a.no_v = 1;

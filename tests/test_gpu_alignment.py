@@ -104,3 +104,22 @@ def test_step_adjoint_on_odd_offsets(n, off):
             fd = (loss(q + eps * dq, v + eps * dv) - loss(q - eps * dq, v - eps * dv)) / (2 * eps)
             an = float((g * (dv if g is gv else dq)).sum())
             assert abs(an - fd) < 1e-6 * max(1.0, abs(fd)), (an, fd)
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+@pytest.mark.parametrize("prec,n", [(0, (16, 8, 32)), (0, (32, 64, 4)), (0, (8, 8, 256)),
+                                    (1, (16, 8, 32)), (1, (256, 8, 4))])
+@pytest.mark.parametrize("advection", [0, 1])
+def test_fluid_update_on_odd_offsets(prec, n, advection, off):
+    dt = torch.float64 if prec else torch.float32
+    shape = (1, 3, n[2], n[1], n[0])
+    g = torch.Generator(device="cuda").manual_seed(off)
+    v, f = (torch.randn(shape, generator=g, device="cuda", dtype=dt) for _ in range(2))
+    with mb.Multiblob(mb.GridDesc(*n, precision=prec, advection=advection)) as sim:
+        want = sim.fluid_update(v, f)
+        (vo, _), (fo, _), (out, store) = (_odd(shape, dt, off, x) for x in (v, f, None))
+        mb.fluid_update(sim.ctx, vo, fo, out)
+        assert torch.equal(out, want) and _untouched(store, off, v.numel())
+        assert torch.equal(vo, v) and torch.equal(fo, f)
+        mb.fluid_update(sim.ctx, vo, None, vo)             # in place, without a force
+        assert torch.equal(vo, sim.fluid_update(v))
