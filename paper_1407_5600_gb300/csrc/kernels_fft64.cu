@@ -132,9 +132,12 @@ template <bool INV> __device__ __forceinline__ void plane_cols(dc* P, int nx, in
 }  // namespace
 
 // Pass A: right-hand side and 2-D R2C transform of one (box, component, z) plane.  Half of the
-// Laplacian's neighbours (z and the outer y) are summed on the FP64 pipe, four additions a row
-// pair, while the FP32 pipes convert and add the rest in double-float: all of it in FP64 would
-// hold this phase for 41k cycles a 128 x 128 plane, all of it in double-float for 24k.
+// Laplacian's neighbours (z and the outer y) and -6 times the centre are summed on the FP64 pipe, six
+// instructions a row pair, while the FP32 pipes convert and add the rest in double-float: all of it
+// in FP64 would hold this phase for 41k cycles a 128 x 128 plane, all of it in double-float for 24k.
+// The centre goes in before the sum is scaled: with a weight of rho/dt - 3 eta/h^2 for the centre
+// instead, the roundings of the weights did not cancel on smooth fields and scaled every low mode
+// the same way each step (1.2e-12 at eta dt / (rho h^2) = 183; 4e-15 to 2e-14 now, for 8 us of a dense 128^3 step of 900).
 __global__ void __launch_bounds__(1024, 1)
 k_plane_fwd64(FluidArgs<double> a, GridGeo g)
 {
@@ -157,9 +160,7 @@ k_plane_fwd64(FluidArgs<double> a, GridGeo g)
     const double* f = a.f ? a.f + (size_t)bc * g.N + z * plane : nullptr;
     double* fclr = a.f_clear && f ? a.f_clear + (size_t)bc * g.N + z * plane : nullptr;
     const bool body = a.body_prof && comp == a.body_axis;
-    // rhs = (rho/dt - 6 c) v + c (sum of the six neighbours) + f,  c = (eta/2) / h^2
-    const double c = a.half_eta * a.inv_h2;
-    const dfloat alpha(a.rho_dt - 6.0 * c), beta(c);
+    const dfloat rho_dt(a.rho_dt), beta(a.half_eta * a.inv_h2);
     for (int i = threadIdx.x; i < (ny / 2) * nx; i += blockDim.x) {
         const int x = i & (nx - 1), p = i >> lx;
         const int o0 = 2 * p * nx + x, o1 = o0 + nx;
@@ -178,13 +179,15 @@ k_plane_fwd64(FluidArgs<double> a, GridGeo g)
         }
         const int xm = ((x - 1) & (nx - 1)) - x, xp = ((x + 1) & (nx - 1)) - x;
         const int om = ((2 * p - 1) & (ny - 1)) * nx + x, op = ((2 * p + 2) & (ny - 1)) * nx + x;
-        const double s0 = (vzp[o0] + vzm[o0]) + vz[om], s1 = (vzp[o1] + vzm[o1]) + vz[op];
-        const dc cc = dc_make(dfloat(vz[o0]), dfloat(vz[o1]));
+        const double c0 = vz[o0], c1 = vz[o1];
+        const double s0 = fma(-6.0, c0, (vzp[o0] + vzm[o0]) + vz[om]);
+        const double s1 = fma(-6.0, c1, (vzp[o1] + vzm[o1]) + vz[op]);
+        const dc cc = dc_make(dfloat(c0), dfloat(c1));
         // the row pair's other row: c1 is a neighbour of row 0, c0 of row 1
         dc lap = cadd(dc_make(dfloat(s0), dfloat(s1)), cswap(cc));
         lap = cadd(lap, cadd(dc_make(dfloat(vz[o0 + xm]), dfloat(vz[o1 + xm])),
                              dc_make(dfloat(vz[o0 + xp]), dfloat(vz[o1 + xp]))));
-        dc v = cadd(cscale(cc, dr_make(alpha)), cscale(lap, dr_make(beta)));
+        dc v = cadd(cscale(cc, dr_make(rho_dt)), cscale(lap, dr_make(beta)));
         if (f || body) v = cadd(v, dc_make(dfloat(r0), dfloat(r1)));
         P[p * S + x] = v;
     }
