@@ -19,13 +19,25 @@ from . import (Multiblob, _adjoint_step, load_library, particle_velocity_adjoint
                set_velocity_field, step)
 
 
+def _streams(sim):
+    """PyTorch's current stream, which makes and reads the tensors here, and the context's, which
+    the library works on."""
+    own = sim.stream
+    if not isinstance(own, torch.cuda.Stream):
+        own = torch.cuda.ExternalStream(int(own), device=sim.device)
+    return torch.cuda.current_stream(sim.device), own
+
+
 class _Rollout(torch.autograd.Function):
     @staticmethod
     def forward(fctx, q0, k_spring, sim, topo, K, checkpoint, ext, body):
         pid, bonds, rest, k_rep, r_cut = topo
-        sim.set_particles(0, q0.detach(), pid, bonds, rest, float(k_spring), k_rep, r_cut)
         dev, dt = sim.device, sim.grid_dtype
+        q = q0.detach().to(device=dev, dtype=torch.float64).contiguous()
         v0 = torch.zeros(sim.grid_shape(), dtype=dt, device=dev)
+        current, own = _streams(sim)
+        own.wait_stream(current)
+        sim.set_particles(0, q, pid, bonds, rest, float(k_spring), k_rep, r_cut)
         set_velocity_field(sim.ctx, v0)
         chk = []
         for s in range(K):
@@ -37,6 +49,7 @@ class _Rollout(torch.autograd.Function):
         fctx.ext, fctx.body, fctx.chk = ext, body, chk
         fctx.qK = sim.blob_positions()
         fctx.vK = sim.velocity_field()
+        current.wait_stream(own)
         return U
 
     @staticmethod
@@ -44,16 +57,17 @@ class _Rollout(torch.autograd.Function):
         sim = fctx.sim
         gq = torch.zeros_like(fctx.qK)
         gv = torch.zeros_like(fctx.vK)
-        particle_velocity_adjoint(sim.ctx, fctx.qK, fctx.vK,
-                                  gU.to(dtype=torch.float64, device=sim.device).contiguous(),
-                                  gq, gv)
-        # on the device, and on the context's own stream with steps that are complete in its order
+        gk = torch.zeros(1, dtype=torch.float64, device=sim.device)
+        gU = gU.to(dtype=torch.float64, device=sim.device).contiguous()
+        # the library adds to the zeros above and reads gU on its own stream
+        current, own = _streams(sim)
+        own.wait_stream(current)
+        particle_velocity_adjoint(sim.ctx, fctx.qK, fctx.vK, gU, gq, gv)
+        # gk on the device, and on the context's own stream steps that are complete in its order
         # only, so that no step of the backward pass waits for the host (64 particles at 64^3, 50
         # steps: 20.3 ms, 21.4 with a wait a step)
         lib = load_library()
-        own = torch.cuda.current_stream(sim.device) == sim.stream
-        entry = lib.mb_adjoint_step_async if own else lib.mb_adjoint_step
-        gk = torch.zeros(1, dtype=torch.float64, device=sim.device)
+        entry = lib.mb_adjoint_step_async if current == own else lib.mb_adjoint_step
         K, chk_every = fctx.K, fctx.checkpoint
         for seg in reversed(range(len(fctx.chk))):
             q_s, v_s = fctx.chk[seg]
@@ -66,6 +80,7 @@ class _Rollout(torch.autograd.Function):
                 step(sim.ctx, 1, fctx.ext, fctx.body)
             for qn, vn in reversed(states):
                 _adjoint_step(entry, sim.ctx, qn, vn, fctx.ext, fctx.body, gq, gv, gk)
+        current.wait_stream(own)
         return gq, gk[0], None, None, None, None, None, None
 
 

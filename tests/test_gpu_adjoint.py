@@ -197,3 +197,31 @@ def test_differentiable_workload_64cube_k50():
         an = float((q0.grad * dq).sum())
         assert abs(an - fd) < 1e-5 * abs(fd), (an, fd)
         assert abs(float(k0.grad) - fdk) < 1e-5 * abs(fdk), (float(k0.grad), fdk)
+
+
+def test_rollout_gradient_off_the_contexts_stream():
+    """A context on a stream of its own, called from another one that is still busy: the tensors
+    made there (inputs, zeroed gradients) are ready before the library works on them, and its
+    results before they are read there.  FP64 atomics in any order: 1e-10, as the other rollouts."""
+    s, ext = _two_particles(n=16, seed=23)
+    gU = torch.tensor(np.random.default_rng(4).normal(size=(s.n_particles, 3)), device="cuda")
+
+    def run(stream, busy):
+        d = mb.GridDesc(16, 16, 16, precision=1, dt=0.05, mean_mode=0)
+        with mb.Multiblob(d, stream=stream) as sim:
+            torch.cuda.synchronize()
+            busy()
+            q0 = torch.tensor(s.pos, device="cuda").add_(0.0).requires_grad_()
+            k = torch.tensor(100.0, dtype=torch.float64, device="cuda", requires_grad=True)
+            U = rollout_particle_velocities(sim, q0, k, s.pid, s.bonds, s.rest, K=5, checkpoint=2,
+                                            ext_blob_force=torch.tensor(ext, device="cuda"))
+            U = 1.0 * U
+            busy()
+            gq, gk = torch.autograd.grad(U, (q0, k), grad_outputs=gU)
+            return [x.detach().cpu().numpy() for x in (1.0 * U, 1.0 * gq, 1.0 * gk)]
+
+    want = run(None, lambda: None)
+    side = torch.cuda.Stream()
+    for stream in (side, side.cuda_stream):
+        for a, b in zip(run(stream, lambda: torch.cuda._sleep(100_000_000)), want):
+            assert np.linalg.norm(a - b) < 1e-10 * np.linalg.norm(b)
