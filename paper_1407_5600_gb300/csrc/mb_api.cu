@@ -1656,16 +1656,29 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
     return MB_OK;
 }
 
+// Whether the caller is capturing the context's stream into a graph of its own.
+bool being_captured(const mb_ctx* ctx)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->st, &s) != cudaSuccess) cudaGetLastError();
+    return s != cudaStreamCaptureStatusNone;
+}
+
 // n_steps FP64 steps: the first two after a rebuild launched directly (a capture costs as much
-// as a few steps), then replays of the captured graph of each velocity-buffer parity.
+// as a few steps), then replays of the captured graph of each velocity-buffer parity.  Into a
+// caller's graph every step goes directly, and clears f itself: what ran before that graph, or
+// whether it runs at all, is not known here.
 mb_status run_steps64(mb_ctx* ctx, int n_steps, const double* ext, const double* body)
 {
-    const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0;
+    const bool captured = being_captured(ctx);
+    const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0 && !captured;
     for (int s = 0; s < n_steps; ++s) {
+        if (captured) ctx->f_zero = false;
         if (!graphs || ctx->direct64 < 2) {
             MB_TRY(enqueue_step64(ctx, ext, body));
             finish_step64(ctx);
-            ctx->direct64++;
+            if (captured) ctx->f_zero = false;
+            else ctx->direct64++;
             continue;
         }
         const int c = ctx->cur;
