@@ -118,6 +118,17 @@ void* mapped_host_ptr(const void* p)
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
+// A captured step.  Its kernels hold the velocity-buffer parity, whether there are external forces,
+// and the axis and wave direction of the body force (or none), which choose its place (graph_of),
+// so that calls which alternate in these replay it; the rest is checked before a replay.
+struct StepGraph {
+    cudaGraphExec_t exec = nullptr;
+    const double* ext_src = nullptr;
+    int hcur = 0;
+    bool fz = false, fz_after = false;     // f_zero before and after (the latter of FP64 steps)
+    int64_t launches = 0;                  // kernels a replay
+};
+
 struct BoxData {
     bool set = false;
     std::vector<double> pos;
@@ -187,8 +198,8 @@ struct mb_ctx {
     // spreading tile picked by timing candidate shapes on the first FP32-grid step
     bool autotune = true, tuned = false;
     float tile_ms = 0.f;
-    // CUDA graphs of one FP32-grid step, one per velocity-buffer parity
     bool use_graph = true;
+    StepGraph graph[2][2][10];       // [parity][external forces][body force: none, 1 + 3 axis + wave]
     cudaStream_t cap_stream = nullptr;
     // second stream for the spring forces, which overlap the binning (fork/join events)
     cudaStream_t side = nullptr;
@@ -200,13 +211,6 @@ struct mb_ctx {
     // device-readable external forces of the current single-step call, converted inside the
     // step beside the binning (null: ext32 already holds them or there are none)
     const double* ext_src = nullptr;
-    const double* graph_ext_src[2] = {nullptr, nullptr};
-    cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
-    bool graph_ext[2] = {false, false}, graph_body[2] = {false, false};
-    int graph_hcur[2] = {0, 0};
-    bool graph_fz[2] = {false, false};
-    bool graph_fz_after = false;       // f_zero after a replay (FP64 steps)
-    int64_t graph_launches = 0;        // kernels per graph launch
     // adjoint scratch: blob vectors and grids (FP64 contexts)
     DBuf a_qn, a_qh, a_gq, a_gqh, a_gF, a_gu, a_gk, a_gU;
     DBuf a_vn, a_vp, a_gvp, a_gvn, a_gf;
@@ -396,18 +400,25 @@ void pick_tile(mb_ctx* ctx)
         ctx->tile[d] = std::min(std::max(std::min(want[d], ctx->g.n[d]), ctx->bg.bs), ctx->g.n[d]);
 }
 
-void drop_graph(mb_ctx* ctx)
+void drop_graphs(mb_ctx* ctx)
 {
-    for (cudaGraphExec_t& g : ctx->graph_exec) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
-    }
+    for (auto& parity : ctx->graph)
+        for (auto& ext : parity)
+            for (StepGraph& g : ext) {
+                if (g.exec) cudaGraphExecDestroy(g.exec);
+                g.exec = nullptr;
+            }
+}
+
+StepGraph& graph_of(mb_ctx* ctx, bool ext, const double* body)
+{
+    return ctx->graph[ctx->cur][ext][body ? 1 + 3 * (int)body[1] + (int)body[2] : 0];
 }
 
 // Concatenates the boxes' blobs into the device arrays used by the step.
 mb_status rebuild(mb_ctx* ctx)
 {
-    drop_graph(ctx);
+    drop_graphs(ctx);
     const int B = ctx->B;
     ctx->box_off_h.assign(B + 1, 0);
     ctx->part_off_h.assign(B + 1, 0);
@@ -1543,11 +1554,11 @@ mb_status autotune_spread(mb_ctx* ctx)
 
 // Captures one step from the current velocity buffer into a CUDA graph (on a private
 // stream; nothing executes during the capture).
-mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
+mb_status capture_graph(mb_ctx* ctx, StepGraph& sg, bool ext, const double* body)
 {
     const int cur0 = ctx->cur;
-    if (ctx->graph_exec[cur0]) cudaGraphExecDestroy(ctx->graph_exec[cur0]);
-    ctx->graph_exec[cur0] = nullptr;
+    if (sg.exec) cudaGraphExecDestroy(sg.exec);
+    sg.exec = nullptr;
     if (!ctx->cap_stream)
         MB_CUDA(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
     cudaStream_t user = ctx->st;
@@ -1572,10 +1583,10 @@ mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
     ctx->hcur = hcur0;
     ctx->hlast = hlast0;
     ctx->pred_ready = ready0;
-    ctx->graph_fz_after = ctx->f_zero;
+    sg.fz_after = ctx->f_zero;
     ctx->f_zero = fz0;
     ctx->sorted_valid = sorted0;
-    ctx->graph_launches = ctx->launches - l0;
+    sg.launches = ctx->launches - l0;
     ctx->launches = l0;
     if (s != MB_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -1586,23 +1597,21 @@ mb_status capture_graph(mb_ctx* ctx, bool ext, const double* body)
         ctx->err = std::string("graph capture: ") + cudaGetErrorString(e);
         return MB_ECUDA;
     }
-    e = cudaGraphInstantiate(&ctx->graph_exec[cur0], graph, 0);
+    e = cudaGraphInstantiate(&sg.exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        ctx->graph_exec[cur0] = nullptr;
+        sg.exec = nullptr;
         ctx->err = std::string("graph instantiate: ") + cudaGetErrorString(e);
         return MB_ECUDA;
     }
-    ctx->graph_ext[cur0] = ext;
-    ctx->graph_ext_src[cur0] = ctx->ext_src;
-    ctx->graph_body[cur0] = body != nullptr;
-    ctx->graph_hcur[cur0] = hcur0;
-    ctx->graph_fz[cur0] = ctx->f_zero;
+    sg.ext_src = ctx->ext_src;
+    sg.hcur = hcur0;
+    sg.fz = fz0;
     return MB_OK;
 }
 
-// n_steps FP32-grid steps, each replaying the captured graph of its parity (stage timing off).
+// n_steps FP32-grid steps, each replaying its captured graph (stage timing off).
 mb_status run_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double* body)
 {
     const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0;
@@ -1614,21 +1623,18 @@ mb_status run_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double* body)
             if (!ctx->tuned) MB_TRY(autotune_spread(ctx));
             continue;
         }
-        const int c = ctx->cur;
-        if (!ctx->graph_exec[c] || ctx->graph_ext[c] != ext ||
-            ctx->graph_ext_src[c] != ctx->ext_src ||
-            ctx->graph_body[c] != (body != nullptr) || ctx->graph_hcur[c] != ctx->hcur ||
-            ctx->graph_fz[c] != ctx->f_zero)
-            MB_TRY(capture_graph(ctx, ext, body));
-        MB_CUDA(cudaGraphLaunch(ctx->graph_exec[c], ctx->st));
+        StepGraph& sg = graph_of(ctx, ext, body);
+        if (!sg.exec || sg.ext_src != ctx->ext_src || sg.hcur != ctx->hcur || sg.fz != ctx->f_zero)
+            MB_TRY(capture_graph(ctx, sg, ext, body));
+        MB_CUDA(cudaGraphLaunch(sg.exec, ctx->st));
         finish_fast_step(ctx);
-        ctx->launches += ctx->graph_launches;
+        ctx->launches += sg.launches;
     }
     return MB_OK;
 }
 
 // Stokes-limit steps in FP32-grid mode: direct launches until the spreading tile is tuned,
-// then replays of a captured graph of one step (keyed by external forces and body force).
+// then replays of a captured graph of one step.
 mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double* body)
 {
     const bool graphs = ctx->use_graph && !ctx->timing && ctx->nb > 0;
@@ -1640,18 +1646,16 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
             if (!ctx->tuned) MB_TRY(autotune_spread(ctx));
             continue;
         }
-        const int c = ctx->cur;
-        if (!ctx->graph_exec[c] || ctx->graph_ext[c] != ext ||
-            ctx->graph_body[c] != (body != nullptr))
-            MB_TRY(capture_graph(ctx, ext, body));
-        MB_CUDA(cudaGraphLaunch(ctx->graph_exec[c], ctx->st));
+        StepGraph& sg = graph_of(ctx, ext, body);
+        if (!sg.exec) MB_TRY(capture_graph(ctx, sg, ext, body));
+        MB_CUDA(cudaGraphLaunch(sg.exec, ctx->st));
         // the state changes of do_step_stokes_fast
         ctx->hcur = ctx->hlast = 0;
         ctx->pred_ready = false;
         ctx->f_zero = ctx->fft_passes == 3;
         ctx->sorted_valid = true;
         ctx->steps_taken++;
-        ctx->launches += ctx->graph_launches;
+        ctx->launches += sg.launches;
     }
     return MB_OK;
 }
@@ -1681,14 +1685,12 @@ mb_status run_steps64(mb_ctx* ctx, int n_steps, const double* ext, const double*
             else ctx->direct64++;
             continue;
         }
-        const int c = ctx->cur;
-        if (!ctx->graph_exec[c] || ctx->graph_ext[c] != (ext != nullptr) ||
-            ctx->graph_body[c] != (body != nullptr) || ctx->graph_fz[c] != ctx->f_zero)
-            MB_TRY(capture_graph(ctx, ext != nullptr, body));
-        MB_CUDA(cudaGraphLaunch(ctx->graph_exec[c], ctx->st));
+        StepGraph& sg = graph_of(ctx, ext != nullptr, body);
+        if (!sg.exec || sg.fz != ctx->f_zero) MB_TRY(capture_graph(ctx, sg, ext != nullptr, body));
+        MB_CUDA(cudaGraphLaunch(sg.exec, ctx->st));
         finish_step64(ctx);
-        ctx->f_zero = ctx->graph_fz_after;
-        ctx->launches += ctx->graph_launches;
+        ctx->f_zero = sg.fz_after;
+        ctx->launches += sg.launches;
     }
     return MB_OK;
 }
@@ -1781,7 +1783,7 @@ mb_status upload_tables(mb_ctx* ctx)
 
 void release(mb_ctx* ctx)
 {
-    drop_graph(ctx);
+    drop_graphs(ctx);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     ctx->cap_stream = nullptr;
     if (ctx->side) cudaStreamDestroy(ctx->side);
@@ -2040,12 +2042,9 @@ mb_status mb_step(mb_ctx* ctx, int n_steps, const double* ext_blob_force,
     if (n_steps < 0) return invalid(ctx, "n_steps must be >= 0");
     MB_TRY(ensure_ready(ctx));
     if (body_force) {
-        // captured steps hold the profile's buffer, axis and wave direction
         const void* before = ctx->body_prof.p;
-        const double axis = ctx->body_cached[1], dir = ctx->body_cached[2];
         MB_TRY(set_body(ctx, body_force, ctx->body_prof, true));
-        if (ctx->body_prof.p != before || ctx->body_cached[1] != axis || ctx->body_cached[2] != dir)
-            drop_graph(ctx);
+        if (ctx->body_prof.p != before) drop_graphs(ctx);      // captured steps hold the old buffer
     }
     const double* ext = nullptr;
     if (ctx->d.integrator == 1 && ctx->rsz == 4) {

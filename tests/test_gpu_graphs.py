@@ -1,4 +1,6 @@
-"""FP64 steps captured into a caller's CUDA graph: accepted before any step and after the library
+"""Steps and CUDA graphs.
+
+FP64 steps captured into a caller's CUDA graph: accepted before any step and after the library
 has graphs of its own, replayed any number of times, with the library's own steps before, between
 and after; the same states as steps taken one by one.
 
@@ -8,7 +10,7 @@ over a dozen steps (the forces differ by the rounding of at most a few hundred t
 import numpy as np
 import pytest
 
-from helpers import rel_l2, to_np
+from helpers import assert_positions, rel_l2, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -50,3 +52,31 @@ def test_steps_in_a_callers_graph(integrator, deterministic, n, warm):
             assert torch.equal(a.last_forces()[0], b.last_forces()[0])
             assert torch.equal(a.blob_positions(), b.blob_positions())
             assert torch.equal(a.velocity_field(), b.velocity_field())
+
+
+@pytest.mark.parametrize("prec,integrator", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_steps_that_alternate_in_their_forces(prec, integrator, monkeypatch):
+    """Calls with and without external forces and with body forces along different axes in turn,
+    each from the captured step of its own kind, against direct launches.  The same kernels in the
+    same order: FP64 1e-12 (atomics in any order), FP32 1e-5 (the repository's bound)."""
+    n = 16
+    rng = np.random.default_rng(31)
+    s = wl.build_particles(rng.random((2, 3)) * n, 1.5, rng, (n, n, n))
+    ext = torch.as_tensor(rng.normal(scale=1e-2, size=s.pos.shape), device="cuda")
+    d = mb.GridDesc(n, n, n, precision=prec, integrator=integrator, mean_mode=integrator)
+    kinds = [(e, b) for e in (None, ext) for b in (None, (1e-2, 0, 2, 1), (2e-2, 1, 0, 1), (1e-2, 0, 1, 2))]
+
+    def run():
+        with mb.Multiblob(d) as sim:
+            sim.set_particles(0, s.pos, s.pid, s.bonds, s.rest, 20.0, 10.0, 1.0)
+            for i in range(40):
+                e, b = kinds[(5 * i) % len(kinds)]
+                sim.step(1 + i % 3, ext_blob_force=e, body_force=b)
+            return to_np(sim.blob_positions()), to_np(sim.velocity_field())
+
+    q, v = run()
+    monkeypatch.setenv("MB_NO_GRAPH", "1")
+    q_ref, v_ref = run()
+    tol = 1e-12 if prec else 1e-5
+    assert rel_l2(v, v_ref) < tol
+    assert_positions(q, q_ref, s.pos, (n, n, n), 80, tol)
