@@ -23,8 +23,9 @@ def _streams(sim):
     """PyTorch's current stream, which makes and reads the tensors here, and the context's, which
     the library works on."""
     own = sim.stream
-    if not isinstance(own, torch.cuda.Stream):
-        own = torch.cuda.ExternalStream(int(own), device=sim.device)
+    if not isinstance(own, torch.cuda.Stream):      # a handle; 0 is the default stream's
+        own = (torch.cuda.ExternalStream(int(own), device=sim.device) if own
+               else torch.cuda.default_stream(sim.device))
     return torch.cuda.current_stream(sim.device), own
 
 

@@ -222,6 +222,8 @@ def test_rollout_gradient_off_the_contexts_stream():
 
     want = run(None, lambda: None)
     side = torch.cuda.Stream()
-    for stream in (side, side.cuda_stream):
-        for a, b in zip(run(stream, lambda: torch.cuda._sleep(100_000_000)), want):
-            assert np.linalg.norm(a - b) < 1e-10 * np.linalg.norm(b)
+    for stream, current in ((side, torch.cuda.default_stream()), (side.cuda_stream, torch.cuda.default_stream()),
+                            (0, side)):
+        with torch.cuda.stream(current):
+            for a, b in zip(run(stream, lambda: torch.cuda._sleep(100_000_000)), want):
+                assert np.linalg.norm(a - b) < 1e-10 * np.linalg.norm(b)
