@@ -29,6 +29,12 @@ def _streams(sim):
     return torch.cuda.current_stream(sim.device), own
 
 
+def _after(first, then):
+    """Work on `then` from here on comes after that on `first` up to here."""
+    if then != first:
+        then.wait_stream(first)
+
+
 class _Rollout(torch.autograd.Function):
     @staticmethod
     def forward(fctx, q0, k_spring, sim, topo, K, checkpoint, ext, body):
@@ -37,7 +43,7 @@ class _Rollout(torch.autograd.Function):
         q = q0.detach().to(device=dev, dtype=torch.float64).contiguous()
         v0 = torch.zeros(sim.grid_shape(), dtype=dt, device=dev)
         current, own = _streams(sim)
-        own.wait_stream(current)
+        _after(current, own)
         sim.set_particles(0, q, pid, bonds, rest, float(k_spring), k_rep, r_cut)
         set_velocity_field(sim.ctx, v0)
         chk = []
@@ -50,7 +56,7 @@ class _Rollout(torch.autograd.Function):
         fctx.ext, fctx.body, fctx.chk = ext, body, chk
         fctx.qK = sim.blob_positions()
         fctx.vK = sim.velocity_field()
-        current.wait_stream(own)
+        _after(own, current)
         return U
 
     @staticmethod
@@ -62,7 +68,7 @@ class _Rollout(torch.autograd.Function):
         gU = gU.to(dtype=torch.float64, device=sim.device).contiguous()
         # the library adds to the zeros above and reads gU on its own stream
         current, own = _streams(sim)
-        own.wait_stream(current)
+        _after(current, own)
         particle_velocity_adjoint(sim.ctx, fctx.qK, fctx.vK, gU, gq, gv)
         # gk on the device, and on the context's own stream steps that are complete in its order
         # only, so that no step of the backward pass waits for the host (64 particles at 64^3, 50
@@ -81,7 +87,7 @@ class _Rollout(torch.autograd.Function):
                 step(sim.ctx, 1, fctx.ext, fctx.body)
             for qn, vn in reversed(states):
                 _adjoint_step(entry, sim.ctx, qn, vn, fctx.ext, fctx.body, gq, gv, gk)
-        current.wait_stream(own)
+        _after(own, current)
         return gq, gk[0], None, None, None, None, None, None
 
 
