@@ -285,6 +285,24 @@ inline cudaError_t launch_on(Chain c, void (*kernel)(P...), dim3 grid, dim3 bloc
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// Whether a kernel of a chain is to be a programmatic dependent.  The blocks of a dependent are
+// placed while the kernel before it drains, as many to an SM as fit, on the SMs that empty first; a
+// grid that would lie thinner over all the SMs is launched the ordinary way.  resident: blocks of it
+// that fit an SM (resident_blocks).
+inline bool start_early(int64_t blocks, int resident) { return (blocks + 151) / 152 >= resident; }
+template <typename... P>
+inline int resident_blocks(std::atomic<int>& cached, void (*kernel)(P...), int threads, size_t smem)
+{
+    int n = cached.load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        n = 1;
+    }
+    cached.store(n > 0 ? n : 1, std::memory_order_relaxed);
+    return n > 0 ? n : 1;
+}
+
 template <typename R>
 cudaError_t launch_fluid(cudaStream_t st, int B, const GridGeo& g, const FluidArgs<R>& a,
                          cudaEvent_t* marks = nullptr);
