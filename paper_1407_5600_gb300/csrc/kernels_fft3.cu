@@ -696,8 +696,13 @@ cudaError_t launch_fluid3<float>(Chain chain, int B, const GridGeo& g, const Flu
     mark(0);
     const dim3 gp(nz, 3 * B), gz(ny / C, nxh, B);
     // Steps with this pass always a dependent / as the rule says, 4,160 blobs: 128 x 128 x 32
-    // 79.5 / 54.9 us, 128 x 128 x 64 82.9 / 70.1, 64^3 46.6 / 41.4
-    cudaError_t e = launch_on(Chain(st, start_early((int64_t)nz * 3 * B, pp.resident)),
+    // 79.5 / 54.9 us, 128 x 128 x 64 82.9 / 70.1, 64^3 46.6 / 41.4.  Planes of less than 64 x 64 gain by
+    // lying evenly only behind the nine-lane spreading, which ends at once (64 x 32 x 32 38.7 / 35.4; behind
+    // the tiles, which hold all SMs, the early start hides the launch: two boxes of 32^3, 20,000 blobs
+    // 48.0 / 52.3), those of 16 x 16 not even there (four boxes, 4,160 blobs 32.8 / 34.2).
+    const int cells = nx * ny;
+    const bool even = cells >= 64 * 64 || (a.after_short && cells >= 32 * 32);
+    cudaError_t e = launch_on(Chain(st, !even || start_early((int64_t)nz * 3 * B, pp.resident)),
                               pp.fwd[a.W ? 1 : 0], gp, dim3(pp.threads), smem_plane, a, g);
     if (e != cudaSuccess) return e;
     mark(1);

@@ -1295,6 +1295,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
     if (blobs && ctx->fft_passes == 3) {
         fa.f_clear = static_cast<float*>(ctx->f.p);
         fa.f_dirty = f_planes(ctx);
+        fa.after_short = spread32_few(ctx->nb);
     }
     const bool vsum = blobs && ctx->vsum.p != nullptr;
     if (vsum) {

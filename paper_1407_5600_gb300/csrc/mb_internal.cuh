@@ -203,6 +203,7 @@ struct FluidArgs {
     // FP32 three-pass FFT: [B][nz], non-zero for the z planes of f that were spread into (the others
     // are zero and not read); zeroed by the z pass.  Null: all may be non-zero
     int* f_dirty;
+    bool after_short;      // FP32 three-pass FFT: the kernel before is the nine-lane spreading
     const R* v_sum_base;   // three-pass FFT: v^n; with v_sum_out, also write v^n + v^{n+1}
     R* v_sum_out;
     // three-pass FFT, mean_mode 0: the FP64 mean velocity [B][3], advanced in place by the
