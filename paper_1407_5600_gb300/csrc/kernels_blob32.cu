@@ -408,8 +408,11 @@ k_interp32_fused(int64_t nb, FusedArgs f, GridGeo g, BinGeo bg)
 // warp): each lane gathers three rows and the sums meet in shuffles.  One thread a blob leaves
 // most SMs without a warp there and has each thread wait for its 54 to 108 loads in turn.
 // One thread / nine lanes a blob, 128^3: 19.6 / 8.1 us of 4,095 blobs, 20.0 / 9.7 of 8,190,
-// 20.5 / 13.4 of 16,380, 21.0 / 22.8 of 32,760.
-constexpr int64_t FEW_BLOBS = 24576;
+// 20.5 / 13.4 of 16,380, 21.0 / 22.8 of 32,760.  In smaller boxes one thread's gathers meet more in
+// the caches and the two cross earlier: at 18,000 to 22,000 blobs in 2^15 to 2^19 cells (steps of
+// 20,000: 64^3 52.9 / 56.2 us, 128 x 64 x 64 68.2 / 67.5, 128 x 128 x 64 87.8 / 85.3).
+constexpr int64_t FEW_MOST = 24576;
+inline bool gather_few(int64_t nb, int64_t cells) { return nb <= FEW_MOST && nb <= 16384 + cells / 256; }
 struct Lane9 {
     int j, comp, cz, t;        // blob of the warp, component, z node; sorted position
     bool writer;
@@ -1114,6 +1117,11 @@ k_spread32(const float4* __restrict__ rec, const int32_t* __restrict__ cell_star
 // (zeroed beforehand) and marks its z plane dirty (or null).  The tiles spend their time on
 // clearing and adding shared copies that hold next to nothing.  Tiles / nine lanes a blob, 128^3:
 // 11.1 / 3.4 us of 1,040 blobs, 15.5 / 5.2 of 4,095, 22.8 / 12.4 of 16,380, 24.1 / 23.9 of 32,760.
+// A tile costs the same whatever the box, so in smaller boxes fewer blobs make the tiles faster
+// (spread32_few: 10,240 blobs, or one in 64 cells where that is more; up to 16,384 cells there are
+// too few tiles for the SMs, 16 x 16 x 32 with 16,380 blobs 66.0 / 50.1).  Steps with tiles / nine lanes:
+// 32^3 41.4 / 38.5 us of 8,190 blobs, 43.8 / 44.7 of 12,000, 53.5 / 64.8 of 24,570; 64^3 46.2 / 44.1,
+// 47.9 / 50.0 and 56.2 / 69.0; 128 x 128 x 64 81.3 / 81.9 of 14,000, 82.5 / 88.5 of 16,380.
 // Inertial steps only: the Stokes limit amplifies the error of the net force, which the tiles'
 // fixed-point sums keep smaller.
 __global__ void __launch_bounds__(128)
@@ -1313,7 +1321,7 @@ cudaError_t launch_unsplit(cudaStream_t st, int64_t nb, const float4* A, const f
     return cudaGetLastError();
 }
 
-cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4* A,
+cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, int Bx, const float4* A,
                             const float4* B, const float* v0, const float* v1,
                             const int32_t* box_of, const GridGeo& g, const BinGeo& bg, float dt,
                             const float4* A_base, const float4* B_base, float4* A_out,
@@ -1321,7 +1329,7 @@ cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4*
                             int32_t* count, int32_t* blob_cell, int32_t* blob_rank)
 {
     if (nb <= 0) return cudaSuccess;
-    if ((mode == 1 || mode == 3) && nb <= FEW_BLOBS)
+    if ((mode == 1 || mode == 3) && gather_few(nb, Bx * g.N))
         return launch_dep(mode == 1 ? k_interp32_few<1> : k_interp32_few<3>,
                           dim3((unsigned)((nb + 11) / 12)), dim3(128), 0, st, (int)nb, A, v0, box_of, g,
                           bg, dt, mode == 1 ? A : A_base, mode == 1 ? B : B_base, A_out, B_out, order,
@@ -1333,7 +1341,7 @@ cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4*
                       blob_cell, blob_rank);
 }
 
-cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, const float* v0,
+cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, int Bx, const float4* A, const float* v0,
                                   const float* v1, const float* vp, const int32_t* box_of,
                                   const GridGeo& g,
                                   const BinGeo& bg, float dt, const float4* A_base,
@@ -1345,7 +1353,7 @@ cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, 
     if (nb <= 0) return cudaSuccess;
     const FusedArgs f{A, v0, v1, vp, box_of, dt, A_base, B_base, A_out, B_out, Ah_out, Bh_out,
                       order, count, blob_cell, blob_rank, u_out};
-    if (nb <= FEW_BLOBS)
+    if (gather_few(nb, Bx * g.N))
         return launch_dep(k_interp32_fused9, dim3((unsigned)((nb + 11) / 12)), dim3(128), 0, st,
                           (int)nb, f, g, bg);
     static std::atomic<unsigned> attr{0};
@@ -1487,7 +1495,10 @@ cudaError_t launch_spread32(cudaStream_t st, int Bx, const float4* rec, const in
     return launch_spread32_t<0, 0, 0>(st, Bx, rec, cell_start, g, bg, tile, f, dirty);
 }
 
-bool spread32_few(int64_t nb) { return nb <= FEW_BLOBS; }
+bool spread32_few(int64_t nb, int64_t cells)
+{
+    return nb <= FEW_MOST && (nb <= 10240 || 64 * nb <= cells || cells <= 16384);
+}
 cudaError_t launch_spread32_few(cudaStream_t st, int64_t nb, int Bx, const float4* rec,
                                 const int32_t* sorted, const int32_t* box_of, const GridGeo& g,
                                 const BinGeo& bg, float* f, bool f_is_zero, int* dirty)

@@ -669,7 +669,7 @@ mb_status rebuild(mb_ctx* ctx)
         else
             MB_CUDA(dfree(ctx->vsum));
     }
-    if (ctx->rsz == 4 && ctx->fft_passes == 3 && spread32_few(nb)) {
+    if (ctx->rsz == 4 && ctx->fft_passes == 3 && spread32_few(nb, B * ctx->g.N)) {
         const size_t by = sizeof(int) * (size_t)B * ctx->g.n[2];
         MB_TRY(ensure(ctx->f_dirty, by, E, "planes of f"));
         MB_CUDA(cudaMemsetAsync(ctx->f_dirty.p, 0, by, ctx->st));
@@ -1096,7 +1096,7 @@ void finish_step64(mb_ctx* ctx)
 // 244,504 blobs: 33.7 -> 34.4 us).
 int* f_planes(mb_ctx* ctx)
 {
-    return spread32_few(ctx->nb) ? static_cast<int*>(ctx->f_dirty.p) : nullptr;
+    return spread32_few(ctx->nb, ctx->B * ctx->g.N) ? static_cast<int*>(ctx->f_dirty.p) : nullptr;
 }
 
 // Host-side state after an FP32-grid step has been enqueued (directly or as a graph replay).
@@ -1140,7 +1140,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
         // the predictor also bins the midpoint positions (counts per cell); the previous
         // step's cell order still groups neighbouring blobs
         MB_CUDA(cudaMemsetAsync(ctx->cell_count.p, 0, sizeof(int32_t) * B * ctx->bg.ncell, st));
-        MB_CUDA(launch_interp32(st, 1, ctx->nb, sA, sB, vcur, nullptr, box_of, g, ctx->bg, dt,
+        MB_CUDA(launch_interp32(st, 1, ctx->nb, B, sA, sB, vcur, nullptr, box_of, g, ctx->bg, dt,
                                 nullptr, nullptr, hA, hB, nullptr,
                                 ctx->sorted_valid ? static_cast<const int32_t*>(ctx->sorted.p)
                                                   : nullptr,
@@ -1250,7 +1250,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
     mark(ST_FORCE_SUM);                 // the mean momentum advances inside the z pass
     mark(ST_SPREAD);
     if (blobs) {
-        if (spread32_few(ctx->nb))
+        if (spread32_few(ctx->nb, ctx->B * ctx->g.N))
             MB_CUDA(launch_spread32_few(st, ctx->nb, B, static_cast<const float4*>(ctx->rec32.p),
                                         static_cast<const int32_t*>(ctx->sorted.p), box_of, g,
                                         ctx->bg, static_cast<float*>(ctx->f.p), ctx->f_zero,
@@ -1295,7 +1295,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
     if (blobs && ctx->fft_passes == 3) {
         fa.f_clear = static_cast<float*>(ctx->f.p);
         fa.f_dirty = f_planes(ctx);
-        fa.after_short = spread32_few(ctx->nb);
+        fa.after_short = spread32_few(ctx->nb, ctx->B * ctx->g.N);
     }
     const bool vsum = blobs && ctx->vsum.p != nullptr;
     if (vsum) {
@@ -1316,7 +1316,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
             // with the bin counts the next step sorts by)
             if (clear_side) MB_CUDA(cudaStreamWaitEvent(st, ctx->fork[5], 0));
             else MB_CUDA(cudaMemsetAsync(ctx->cell_count.p, 0, sizeof(int32_t) * B * ctx->bg.ncell, st));
-            MB_CUDA(launch_interp32_fused(st, ctx->nb, hA, vsum ? static_cast<const float*>(ctx->vsum.p) : vcur,
+            MB_CUDA(launch_interp32_fused(st, ctx->nb, B, hA, vsum ? static_cast<const float*>(ctx->vsum.p) : vcur,
                                           vsum ? nullptr : vnext, vnext, box_of, g, ctx->bg, dt, sA,
                                           sB, sA, sB,
                                           static_cast<float4*>(ctx->hA[ctx->hcur ^ 1].p),
@@ -1327,7 +1327,7 @@ mb_status do_step_fast(mb_ctx* ctx, bool ext, const double* body)
                                           static_cast<int32_t*>(ctx->blob_rank.p),
                                           static_cast<float4*>(ctx->u32.p)));
         } else {
-            MB_CUDA(launch_interp32(st, 2, ctx->nb, hA, hB, vcur, vnext, box_of, g, ctx->bg, dt,
+            MB_CUDA(launch_interp32(st, 2, ctx->nb, B, hA, hB, vcur, vnext, box_of, g, ctx->bg, dt,
                                     sA, sB, sA, sB, nullptr,
                                     static_cast<const int32_t*>(ctx->sorted.p)));
         }
@@ -1454,7 +1454,7 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
     if (blobs) {
         // q^{n+1/2} = q^n + dt/2 J(q^n) v(q^n), binned on the way
         MB_CUDA(cudaMemsetAsync(ctx->cell_count.p, 0, sizeof(int32_t) * B * ctx->bg.ncell, st));
-        MB_CUDA(launch_interp32(st, 1, ctx->nb, sA, sB, v_half, nullptr, box_of, g, ctx->bg, dt,
+        MB_CUDA(launch_interp32(st, 1, ctx->nb, B, sA, sB, v_half, nullptr, box_of, g, ctx->bg, dt,
                                 nullptr, nullptr, hA, hB, nullptr,
                                 static_cast<const int32_t*>(ctx->sorted.p),
                                 static_cast<int32_t*>(ctx->cell_count.p),
@@ -1465,7 +1465,7 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
     MB_TRY(half(hA, hB, true, v_full, true));
     if (blobs) {
         // q^{n+1} = q^n + dt J(q^{n+1/2}) v(q^{n+1/2})
-        MB_CUDA(launch_interp32(st, 3, ctx->nb, hA, hB, v_full, nullptr, box_of, g, ctx->bg, dt,
+        MB_CUDA(launch_interp32(st, 3, ctx->nb, B, hA, hB, v_full, nullptr, box_of, g, ctx->bg, dt,
                                 sA, sB, sA, sB, nullptr,
                                 static_cast<const int32_t*>(ctx->sorted.p)));
         ctx->launches += 1;
@@ -2487,7 +2487,7 @@ static mb_status blob_velocities(mb_ctx* ctx)
         MB_CUDA(launch_forces_to_fp64(ctx->st, ctx->nb, static_cast<const float4*>(ctx->u32.p),
                                       static_cast<double*>(ctx->u.p)));
     else if (ctx->rsz == 4)
-        MB_CUDA(launch_interp32(ctx->st, 0, ctx->nb, static_cast<const float4*>(ctx->sA.p),
+        MB_CUDA(launch_interp32(ctx->st, 0, ctx->nb, ctx->B, static_cast<const float4*>(ctx->sA.p),
                                 static_cast<const float4*>(ctx->sB.p),
                                 static_cast<const float*>(ctx->v[ctx->cur].p), nullptr,
                                 static_cast<const int32_t*>(ctx->box_of.p), ctx->g, ctx->bg,

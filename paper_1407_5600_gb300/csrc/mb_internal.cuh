@@ -337,7 +337,7 @@ cudaError_t launch_split(cudaStream_t st, int64_t nb, const double* q, const Gri
                          const BinGeo& bg, float4* A, float4* B);
 cudaError_t launch_unsplit(cudaStream_t st, int64_t nb, const float4* A, const float4* B,
                            const GridGeo& g, const BinGeo& bg, double* q);
-cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4* A,
+cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, int Bx, const float4* A,
                             const float4* B, const float* v0, const float* v1,
                             const int32_t* box_of, const GridGeo& g, const BinGeo& bg, float dt,
                             const float4* A_base, const float4* B_base, float4* A_out,
@@ -348,7 +348,7 @@ cudaError_t launch_interp32(cudaStream_t st, int mode, int64_t nb, const float4*
 // which must be zero).  Mode-2 + mode-1 semantics of launch_interp32: the corrector gathers
 // (v0 + v1) / 2 (v1 may be null when v0 already holds v^n + v^{n+1}), the predictor vp; the
 // predictor's velocities (those of the new state) go to u_out.
-cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, const float4* A, const float* v0,
+cudaError_t launch_interp32_fused(cudaStream_t st, int64_t nb, int Bx, const float4* A, const float* v0,
                                   const float* v1, const float* vp, const int32_t* box_of,
                                   const GridGeo& g,
                                   const BinGeo& bg, float dt, const float4* A_base,
@@ -407,8 +407,8 @@ bool spread32_tile_ok(const int tile[3], const GridGeo& g, const BinGeo& bg);
 cudaError_t launch_spread32(cudaStream_t st, int Bx, const float4* rec, const int32_t* cell_start,
                             const GridGeo& g, const BinGeo& bg, const int tile[3], float* f,
                             bool f_is_zero = false, int* dirty = nullptr);
-// The same straight to f, for few blobs (spread32_few).
-bool spread32_few(int64_t nb);
+// The same straight to f, for few blobs (spread32_few of the blobs and cells of all boxes).
+bool spread32_few(int64_t nb, int64_t cells);
 cudaError_t launch_spread32_few(cudaStream_t st, int64_t nb, int Bx, const float4* rec,
                                 const int32_t* sorted, const int32_t* box_of, const GridGeo& g,
                                 const BinGeo& bg, float* f, bool f_is_zero, int* dirty);

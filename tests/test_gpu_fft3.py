@@ -136,3 +136,27 @@ def test_fp32_stokes_replays_after_the_tile_timing(n):
         q_ref, v_ref = oracle.stokes_step(g, 5, q0, pid, *none, 0.0, 0.0, 0.0, ext=F)
         assert rel_l2(v, v_ref) < 1e-5
         assert_positions(q, q_ref, q0, g.L, 5, 2e-5)
+
+
+@pytest.mark.parametrize("integrator", [0, 1])
+@pytest.mark.parametrize("nblobs", [10240, 10241, 16512, 16513])
+def test_fp32_steps_at_the_edges_of_the_few_blob_rules(nblobs, integrator):
+    """32^3 cells: nine lanes a blob up to 10240 (spreading) and 16384 + cells / 256
+    (interpolation) blobs."""
+    g = oracle.Grid(32, 32, 32, dt=0.1, mean_mode=1)
+    d = mb.GridDesc(32, 32, 32, dt=0.1, precision=0, mean_mode=1, integrator=integrator)
+    rng = np.random.default_rng(nblobs)
+    none = (np.zeros((0, 2), np.int32), np.zeros(0))
+    q0, F = rng.random((nblobs, 3)) * 32, rng.normal(size=(nblobs, 3))
+    F -= F.mean(0)
+    pid = np.arange(nblobs, dtype=np.int32)
+    with mb.Multiblob(d) as sim:
+        sim.set_particles(0, q0, pid, *none, 0.0)
+        sim.step(3, ext_blob_force=F)
+        v, q = to_np(sim.velocity_field())[0], to_np(sim.blob_positions())
+    if integrator:
+        q_ref, v_ref = oracle.stokes_step(g, 3, q0, pid, *none, 0.0, 0.0, 0.0, ext=F)
+    else:
+        q_ref, v_ref = oracle.step(g, 3, q0, g.zeros(), pid, *none, 0.0, 0.0, 0.0, ext=F)
+    assert rel_l2(v, v_ref) < (1e-5 if integrator else 6e-6)
+    assert_positions(q, q_ref, q0, g.L, 3, 2e-5)
