@@ -1481,6 +1481,7 @@ mb_status do_step_stokes_fast(mb_ctx* ctx, bool ext, const double* body)
 
 // Times each candidate spreading tile on the current binned records (the first step after
 // the blobs were set) and keeps the fastest; choices are cached per geometry and blob count.
+// Inertial steps of few blobs spread without tiles and time none.
 struct TuneKey {
     int n[3], B, bs, integrator;
     int64_t nb;
@@ -1496,7 +1497,10 @@ std::mutex g_tile_mu;
 mb_status autotune_spread(mb_ctx* ctx)
 {
     ctx->tuned = true;
-    if (!ctx->autotune || ctx->nb == 0) return MB_OK;
+    ctx->tile_ms = 0.f;
+    if (!ctx->autotune || ctx->nb == 0 ||
+        (ctx->d.integrator == 0 && spread32_few(ctx->nb, ctx->B * ctx->g.N)))
+        return MB_OK;
     const TuneKey key{{ctx->g.n[0], ctx->g.n[1], ctx->g.n[2]}, ctx->B, ctx->bg.bs, ctx->d.integrator, ctx->nb};
     {
         std::lock_guard<std::mutex> lock(g_tile_mu);

@@ -160,3 +160,18 @@ def test_fp32_steps_at_the_edges_of_the_few_blob_rules(nblobs, integrator):
         q_ref, v_ref = oracle.step(g, 3, q0, g.zeros(), pid, *none, 0.0, 0.0, 0.0, ext=F)
     assert rel_l2(v, v_ref) < (1e-5 if integrator else 6e-6)
     assert_positions(q, q_ref, q0, g.L, 3, 2e-5)
+
+
+@pytest.mark.parametrize("integrator,nblobs,timed", [(0, 13, False), (0, 10240, False), (0, 10241, True),
+                                                     (1, 13, True)])
+def test_tiles_are_timed_where_they_are_used(integrator, nblobs, timed):
+    """Inertial steps of few blobs spread without tiles, and none is timed then (32,768 cells: up to
+    10,240 blobs).  Grid and blob counts of no other test, whose choice would be taken over."""
+    rng = np.random.default_rng(nblobs)
+    none = (np.zeros((0, 2), np.int32), np.zeros(0))
+    d = mb.GridDesc(16, 64, 32, dt=0.05, mean_mode=1, integrator=integrator)
+    with mb.Multiblob(d) as sim:
+        sim.set_particles(0, rng.random((nblobs, 3)) * [16, 64, 32], np.arange(nblobs, dtype=np.int32), *none, 0.0)
+        sim.step(4, ext_blob_force=rng.normal(size=(nblobs, 3)))
+        tile, ms = mb.get_tuning(sim.ctx)
+    assert len(tile) == 3 and (ms > 0.0) == timed
