@@ -319,11 +319,13 @@ __device__ __forceinline__ void block_sum3(double v[3], double* sh /*[3][32]*/)
     }
 }
 
-// The nearer image of a difference beyond half the box.  Not inlined: as predicated instructions
-// its comparisons and additions would take the FP64 pipe for every bond.
+// The nearest image of a difference beyond half the box: one box on, or more where a midpoint moved
+// by more than the box.  Not inlined: as predicated instructions its comparisons and additions
+// would take the FP64 pipe for every bond.
 __device__ __noinline__ double other_image(double x, double L)
 {
     const double half = 0.5 * L;
+    if (fabs(x) >= L) return __dsub_rn(x, __dmul_rn(L, rint(__ddiv_rn(x, L))));
     return x > half ? __dsub_rn(x, L) : (x < -half ? __dadd_rn(x, L) : x);
 }
 

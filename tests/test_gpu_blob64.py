@@ -133,3 +133,25 @@ def test_state_arrays_are_free_on_return(prec):
                 with torch.cuda.stream(other):
                     dev.zero_()
             assert np.max(np.abs(to_np(sim.blob_positions()) - q0)) < 1e-12
+
+
+@pytest.mark.parametrize("pattern", [True, False])
+def test_springs_of_blobs_that_move_by_more_than_the_box(pattern):
+    """A field under which half a step carries the ends of a bond several boxes apart: the spring is
+    that of the nearest images, as for any two positions (1e-9: the differences of positions of up
+    to ten boxes are rounded at 1e-15 of them, the spring multiplies the bond's by a few)."""
+    n, L = 8, 8.0
+    pos = np.array([[1.0, 1.0, 1.0], [1.8, 5.5, 1.5], [4.0, 2.0, 6.0], [4.9, 6.0, 6.5]])
+    pid, bonds = np.array([0, 0, 1, 1], np.int32), np.array([[0, 1], [2, 3]], np.int32)
+    rest = np.array([3.0, 3.0 if pattern else 3.1])
+    v = np.zeros((1, 3, n, n, n))
+    v[0, 0, :, 4:, :] = 900.0                     # 2.8 boxes in half a step, in half of the box
+    d = mb.GridDesc(n, n, n, precision=1, dt=0.05)
+    with mb.Multiblob(d) as sim:
+        sim.set_particles(0, pos, pid, bonds, rest, 40.0)
+        sim.set_velocity_field(v)
+        sim.step(1)
+        F, qh = (to_np(x) for x in sim.last_forces())
+    assert np.min(np.max(np.abs(qh[bonds[:, 0]] - qh[bonds[:, 1]]), axis=1)) > 1.5 * L
+    F_ref = oracle.bond_forces(oracle.Grid(n, n, n, dt=0.05), qh, bonds, rest, 40.0)
+    assert rel_l2(F, F_ref) < 1e-9
