@@ -15,14 +15,15 @@ template <typename T> __device__ __forceinline__ T cm(T a, T b)
     return T{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
 template <typename T> __device__ __forceinline__ T cadd(T a, T b) { return T{a.x + b.x, a.y + b.y}; }
-// Correctly rounded reciprocals (the float one is a single intrinsic instead of a division).
+// The correctly rounded float reciprocal (a single intrinsic instead of a division).
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 // FP64: Newton's iteration from the hardware's float reciprocal (four FP64 instructions instead
-// of the division's twenty or so) where the argument is in the float range.
+// of the division's twenty or so) where argument and reciprocal are normal floats: 2^-126 <= x < 2^126.
+// Good to 2^-85 before its rounding, so one in 2^32 may round to the other neighbour.
 __device__ __forceinline__ double recip(double x)
 {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    if (hi - (897u << 20) >= (253u << 20)) return 1.0 / x;
+    if (hi - (897u << 20) >= (252u << 20)) return 1.0 / x;
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;"
         : "=f"(y) : "f"(__uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29))));
