@@ -26,7 +26,10 @@
  *    are the fast path): MB_FFT_PASSES=5 runs the fluid solve as five one-axis passes instead
  *    of three; MB_NO_GRAPH=1 launches every step directly instead of replaying its captured CUDA
  *    graph; MB_NO_AUTOTUNE=1 keeps the default spreading tile;
- *    MB_NO_FUSE_INTERP=1 runs the corrector and the next predictor as separate passes.
+ *    MB_NO_FUSE_INTERP=1 runs the corrector and the next predictor as separate passes.  Read once
+ *    by the process: MB_PDL=0 launches the kernels of a step the ordinary way instead of as
+ *    programmatic dependents, MB_SPRINGS=list keeps per-blob bond lists where all particles share
+ *    a bond pattern, MB_PLANE_LAYOUT=pad keeps the run-time layout of the FP32 plane passes.
  *    MB_FAULT_ALLOC=k makes the k-th device allocation fail (tests of the error paths).
  *  - Layouts: blob arrays are [n][3] row-major FP64 (x, y, z).  A velocity or force grid of
  *    one box is 3 component arrays stored one after another, each [nz][ny][nx] with x
@@ -285,7 +288,10 @@ mb_status mb_particle_velocity_adjoint(mb_ctx* ctx, const double* pos, const voi
  * mb_set_particles times a set of candidate tile shapes on the actual blob distribution, in
  * several rounds, and keeps the one with the fastest launch (synchronising the stream after
  * each timed launch; set MB_NO_AUTOTUNE=1 to keep the default); choices are cached per
- * geometry and blob count for the life of the process. */
+ * geometry and blob count for the life of the process.  Inertial FP32 steps of few blobs
+ * (10,240, or one in 64 cells where that is more, at most 24,576, which also holds up to 16,384
+ * cells) spread without tiles: none is timed for them, and the tile
+ * returned is the default.  So it is for FP64 steps, whose deterministic spreading may halve it. */
 mb_status mb_get_tuning(const mb_ctx* ctx, int* spread_tile, float* spread_ms);
 
 /* Number of blobs and particles of all boxes together. */

@@ -193,7 +193,6 @@ struct mb_ctx {
     DBuf f_dirty;               // [B][nz]: z planes of f spread into (FP32 three-pass grids; others are zero)
     bool f_zero = false;        // ctx->f holds zeros (cleared by the last plane pass)
 
-    bool ext_present = false;
     bool sorted_valid = false;     // `sorted` holds a permutation of the current blobs
     // spreading tile picked by timing candidate shapes on the first FP32-grid step
     bool autotune = true, tuned = false;
@@ -213,7 +212,7 @@ struct mb_ctx {
     const double* ext_src = nullptr;
     // adjoint scratch: blob vectors and grids (FP64 contexts)
     DBuf a_qn, a_qh, a_gq, a_gqh, a_gF, a_gu, a_gk, a_gU;
-    DBuf a_vn, a_vp, a_gvp, a_gvn, a_gf;
+    DBuf a_vn, a_vp, a_gvn, a_gf;
     // standalone-operator scratch
     DBuf s_F, s_g0, s_g1, s_g2, s_out;
 
@@ -720,7 +719,6 @@ mb_status rebuild(mb_ctx* ctx)
         MB_TRY(up(ctx->adj32_start, s32.data(), sizeof(int32_t) * (nb + 1)));
         MB_CUDA(launch_split(st, nb, static_cast<const double*>(ctx->q.p), ctx->g, ctx->bg,
                              static_cast<float4*>(ctx->sA.p), static_cast<float4*>(ctx->sB.p)));
-        ctx->ext_present = false;
         ctx->sorted_valid = false;
         ctx->pred_ready = false;
         ctx->tuned = false;
@@ -1812,7 +1810,7 @@ void release(mb_ctx* ctx)
                    &ctx->sB, &ctx->hA[0], &ctx->hA[1], &ctx->hB[0], &ctx->hB[1], &ctx->F32, &ctx->rec32, &ctx->ext32,
                    &ctx->ext_sum, &ctx->ext_ticket, &ctx->adj32, &ctx->adj32_start, &ctx->tmpl32, &ctx->tstart32, &ctx->Fpre64, &ctx->force_ticket, &ctx->Fs32, &ctx->u32, &ctx->a_qn, &ctx->a_qh,
                    &ctx->a_gq, &ctx->a_gqh, &ctx->a_gF, &ctx->a_gu, &ctx->a_gk, &ctx->a_gU,
-                   &ctx->a_vn, &ctx->a_vp, &ctx->a_gvp, &ctx->a_gvn,
+                   &ctx->a_vn, &ctx->a_vp, &ctx->a_gvn,
                    &ctx->a_gf, &ctx->W, &ctx->step_index,
                    &ctx->twk[0], &ctx->twk[1], &ctx->twk[2], &ctx->symk};
     for (DBuf* b : all) dfree(*b);

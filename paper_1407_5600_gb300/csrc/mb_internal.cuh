@@ -323,13 +323,12 @@ constexpr int FLUID3_KERNELS = 3;
 
 // Thermal and convective stress (kernels_noise.cu): W = amp * normals of step *step_index
 // (amp != 0) + rho v v (v != NULL) [parts & 1], then f (+)= -D.W and *step_index += 1
-// (amp != 0) [parts & 2, FP64 only].  parts & 4: other kernels run beside it.  W is [B][9][N],
+// (amp != 0) [parts & 2, FP64 only].  W is [B][9][N],
 // v and f [B][3][N].
 template <typename R>
 cudaError_t launch_fluid_stress(cudaStream_t st, int B, const GridGeo& g, uint64_t seed,
                                 uint64_t* step_index, double amp, const R* v, double rho, R* W,
                                 R* f, bool accumulate, int parts = 3);
-constexpr int STRESS_KERNELS = 2;
 
 // FP32-grid blob pipeline (kernels_blob32.cu): positions as bin cell + float-float offset,
 // A = {hi.xyz, packed cell}, B = {lo.xyz, 0} per blob.
