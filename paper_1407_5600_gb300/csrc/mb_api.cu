@@ -1667,7 +1667,10 @@ mb_status run_stokes_fast_steps(mb_ctx* ctx, int n_steps, bool ext, const double
 bool being_captured(const mb_ctx* ctx)
 {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->st, &s) != cudaSuccess) cudaGetLastError();
+    if (cudaStreamIsCapturing(ctx->st, &s) != cudaSuccess) {
+        cudaGetLastError();        // the default stream while another one is captured
+        return false;
+    }
     return s != cudaStreamCaptureStatusNone;
 }
 
