@@ -18,8 +18,8 @@
 // block has as many threads as its lines need (n / N1 each, lines_threads): with 256 threads
 // whatever the sides, the 64-point passes left six of eight warps without a line.  256-point
 // lines have layouts of their own with compile-time offsets (line_fft).  Times before and after:
-// FP32 256^3 rhs (with the stress divergence, a pass of its own before) 165 + 180 -> 250 us,
-// y 134 -> 78, z and solve 275 -> 167, c2r 196 -> 110; FP64 256 x 64 x 64 800 -> 582 us in all.
+// FP32 256^3 rhs (with the stress divergence, a pass of its own before) 165 + 180 -> 258 us,
+// y 134 -> 78, z and solve 275 -> 167, c2r 196 -> 110; FP64 256 x 64 x 64 800 -> 590 us in all.
 #include "mb_internal.cuh"
 #include "fft_lines.cuh"
 
@@ -427,7 +427,7 @@ cudaError_t launch_fluid(cudaStream_t st, int B, const GridGeo& g, const FluidAr
     }
     // Block sizes (times at 256^3, FP32): x passes of one warp (two 256-point row pairs) keep
     // more blocks in different phases on an SM than wider ones: 276 / 126 us with 256 threads,
-    // 258 / 112 with 64, 250 / 110 with 32.  y blocks of 8 columns (64-byte runs) 78 us, of 16
+    // 258 / 112 with 64, 250 / 110 with 32 (before the centre's own instruction).  y blocks of 8 columns (64-byte runs) 78 us, of 16
     // 87 us; z blocks of 8 columns 167 us, of 4 (32-byte runs) 178 us.  FP64 blocks are bound by
     // the FP64 pipe (80-84% busy) at four warps.
     const int rp = lines_per_block(nx, sizeof(R) == 4 ? 32 : 128, ny / 2), RP = rp < ny / 2 ? rp : ny / 2;

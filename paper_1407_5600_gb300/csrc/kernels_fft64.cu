@@ -14,7 +14,7 @@
 // Now the FP32 pipes bound them (ncu at 128^3: math-pipe throttle, 48-56% issue of two-cycle
 // instructions).  Launch times (ncu), plane forward / z / plane inverse: 32^3 37.3 / 35.4 / 34.1
 // -> 11.8 / 9.5 / 8.5 us, 64^3 47.8 / 40.4 / 50.5 -> 21.2 / 18.7 / 24.3 us, 128^3 254 / 197 / 179
-// -> 165 / 100 / 133 us.  The error against 64 bits stays what it was (1.04e-14 at 128^3).
+// -> 165 / 100 / 133 us (forward 8 us more with the centre in the sum, below).  The error against 64 bits stays what it was (1.04e-14 at 128^3).
 //
 // Shared layout of a plane: packed row p holds nx values, stride S = nx + 5; after the
 // separation the even row's columns at k and the odd row's at nx/2 + 4 + k.  Consecutive lanes

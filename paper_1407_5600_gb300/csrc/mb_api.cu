@@ -660,7 +660,9 @@ mb_status rebuild(mb_ctx* ctx)
     // one blob in 32 cells on; 48 bytes a cell under the pass's arithmetic save the corrector 81
     // additions a blob on the narrow FP64 pipe.  FP32: from one in 10 on; a read and a write of the
     // grid save the corrector half its gathers (128^3, plane pass and corrector without / with the
-    // sum: 53 / 54 us of 104,000 blobs, 65 / 66 of 156,000, 74 / 72 of 244,504)
+    // sum: 53 / 54 us of 104,000 blobs, 65 / 66 of 156,000, 74 / 72 of 244,504; steps of other boxes: 64^3
+    // 59.7 / 61.1 at one in 8, 66.3 / 65.8 at one in 5, eight of them 138.9 / 139.1 at one in 20, 170.5 /
+    // 168.3 at one in 10, 32^3 33.8 / 34.1 at one in 10, 42.8 / 41.0 at one in 3)
     if (ctx->d.integrator == 0) {
         const int64_t cells = ctx->rsz == 8 ? 32 : (ctx->fuse_interp ? 10 : 0);
         if (nb > 0 && ctx->fft_passes == 3 && cells * nb >= B * ctx->g.N)
